@@ -138,17 +138,23 @@ class _OtherRanks:
         return self.gathered[len([x for x in self.sent if x.dtype == torch.bfloat16]) - 1]
 
 
-def _phi(c, x, w):
-    """The feature map of rows x [B, H, n, d] in fp32, for the other ranks' share of the state."""
-    a = torch.relu(x.float() @ w["wk"].float().transpose(-1, -2) + (w["biases"]["bk1"].float()[:, None] if c["bias"] else 0.0))
+def _phi(c, x, w, side, dtype=torch.float32, slope=False):
+    """The feature map of rows x [B, H, n, d], of the queries ("q") or the keys ("k"); with `slope` its derivative w.r.t. the last
+    layer's sums beside it."""
+    a = x.to(dtype) @ w["w" + side].to(dtype).transpose(-1, -2) + (w["biases"]["b%s1" % side].to(dtype)[:, None] if c["bias"] else 0.0)
     if c["hidden"]:
-        a = torch.relu(a @ w["wk2"].float().transpose(-1, -2) + (w["biases"]["bk2"].float()[:, None] if c["bias"] else 0.0))
-    part = c["F"] // c["degree"]
-    return torch.cat([a[..., p * part:(p + 1) * part] ** (p + 1) for p in range(c["degree"])], dim=-1)
+        a = torch.relu(a) @ w["w%s2" % side].to(dtype).transpose(-1, -2)
+        a = a + (w["biases"]["b%s2" % side].to(dtype)[:, None] if c["bias"] else 0.0)
+    r, part = torch.relu(a), c["F"] // c["degree"]
+    cols = [slice(p * part, (p + 1) * part) for p in range(c["degree"])]
+    phi = torch.cat([r[..., x] ** (p + 1) for p, x in enumerate(cols)], dim=-1)
+    if not slope:
+        return phi
+    return phi, torch.cat([(a[..., x] > 0) * (p + 1) * r[..., x] ** p for p, x in enumerate(cols)], dim=-1)
 
 
-def prepare(case, seed):
-    c, s = case, _State()
+def _inputs(c, seed):
+    """(q, k, v, weights, teacher's output or None) of a case: whole layers, on the GPU."""
     B, H, N, d, F = c["B"], c["H"], _n_tokens(c), c["d"], c["F"]
     g = torch.Generator(device="cuda").manual_seed(seed)
 
@@ -179,6 +185,14 @@ def prepare(case, seed):
         if c["rate"] > 0:
             last = "bq2" if c["hidden"] else "bq1"
             w["biases"][last] = (w["biases"][last].float() * 2e-3).bfloat16()
+    teacher = (0.5 * torch.randn((B, H, N, d), device="cuda", generator=g)).bfloat16() if c["use"] == "step" else None
+    return q, k, v, w, teacher
+
+
+def prepare(case, seed):
+    c, s = case, _State()
+    B, H, N, d, F = c["B"], c["H"], _n_tokens(c), c["d"], c["F"]
+    q, k, v, w, s.teacher = _inputs(c, seed)
     s.use, s.w = c["use"], w
     kw = {"phi_dim": F, "poly_degree": c["degree"], "stab_mode": AS_STAB_EXACT if c["exact"] else AS_STAB_PAPER,
           "phi_layers": 2 if c["hidden"] else 1, "phi_hidden": c["hidden"] or None}
@@ -192,7 +206,7 @@ def prepare(case, seed):
         if len(idx) < N:
             linear = torch.ones(N, device="cuda")
             linear[at] = 0
-            phi = _phi(c, k, w) * linear[:, None]
+            phi = _phi(c, k, w, "k") * linear[:, None]
             totals = {3: (phi.transpose(-1, -2) @ v.float()).reshape(B * H, F, d), 2: phi.sum(dim=2).reshape(B * H, F)}
         s.comm = _OtherRanks(totals, gathered)
         s.op = SeqShardedAttention(B, H, N, d, idx, c["ranks"] // 2, c["ranks"], comm=s.comm, **kw)
@@ -201,7 +215,6 @@ def prepare(case, seed):
         q, k, v = (x.cpu().pin_memory() for x in (q, k, v))
         s.out = torch.empty_like(q).pin_memory()
     if c["use"] == "step":
-        s.teacher = (0.5 * torch.randn((B, H, N, d), device="cuda", generator=g)).bfloat16()
         s.aux = torch.empty((B, H, N, 3), dtype=torch.float32, device="cuda")
     s.q, s.k, s.v = q, k, v
     return s
@@ -249,3 +262,99 @@ def tolerance(case):
         # loss |y - y_hat| has a kink, and where another rounding of y_hat falls on the other side of y a whole unit changes sign
         return {"rel": 0.03}
     return {"rel": 0.01}
+
+
+def _softmax_mask(c):
+    """True for the softmax tokens: the raster index inside the token's block, clipped at the grid's border, is a multiple of the rate."""
+    sides = [torch.arange(n, device="cuda") for n in (c["gt"], c["gh"], c["gw"])]
+    blocks, grid = (c["bt"], c["bh"], c["bw"]), (c["gt"], c["gh"], c["gw"])
+    inner = [x % b for x, b in zip(sides, blocks)]
+    extent = [torch.clamp(n - x // b * b, max=b) for x, b, n in zip(sides, blocks, grid)]
+    at = (inner[0][:, None, None] * extent[1][None, :, None] + inner[1][None, :, None]) * extent[2][None, None, :] + inner[2][None, None, :]
+    return (at.reshape(-1) % c["rate"] == 0) if c["rate"] else torch.zeros(_n_tokens(c), dtype=torch.bool, device="cuda")
+
+
+def exact(case, seed):
+    """What `run` returns, in 64 bits from the method's equations."""
+    c, f64 = case, torch.float64
+    B, H, N, d, F = c["B"], c["H"], _n_tokens(c), c["d"], c["F"]
+    q, k, v, w, teacher = _inputs(c, seed)
+    soft = _softmax_mask(c)
+    lin = ~soft
+    n_s = int(soft.sum())
+    n0, n1 = 0, N
+    if c["ranks"] > 1:                                       # contiguous near-equal ranges, the first ones a token longer
+        rank, (base, extra) = c["ranks"] // 2, divmod(N, c["ranks"])
+        n0 = rank * base + min(rank, extra)
+        n1 = n0 + base + (rank < extra)
+    mine = torch.zeros_like(soft)
+    mine[n0:n1] = True
+    out = torch.empty((B, H, n1 - n0, d), dtype=f64, device="cuda")
+    aux = torch.zeros((B, H, N, 3), dtype=f64, device="cuda") if c["use"] == "step" else None
+    part = []
+    dw = [torch.zeros((H, F, d), dtype=f64, device="cuda") for _ in range(2)]
+    loss = torch.zeros(1, dtype=f64, device="cuda")
+    step = max(1, (1 << 26) // max(n_s, 4 * F))
+    for b in range(B):
+        for h in range(H):
+            wh = {n: ({m: y[h:h + 1] for m, y in x.items()} if n == "biases" else x[h:h + 1]) for n, x in w.items()}
+            phi_of = lambda x, side, **kw: _phi(c, x[None, None], wh, side, f64, **kw)
+            ks, vs = k[b, h][soft].to(f64), v[b, h][soft].to(f64)
+            S, z, pS, pz = (torch.zeros(x, dtype=f64, device="cuda") for x in ((F, d), (F,), (F, d), (F,)))
+            for i in range(0, N, step):
+                rows = lin[i:i + step, None].to(f64)
+                phi, val = phi_of(k[b, h, i:i + step], "k")[0, 0] * rows, v[b, h, i:i + step].to(f64)
+                S += phi.T @ val
+                z += phi.sum(dim=0)
+                if c["use"] == "shard":
+                    phi = phi * mine[i:i + step, None].to(f64)
+                    pS += phi.T @ val
+                    pz += phi.sum(dim=0)
+            part.append((pS, pz))
+            dS, dz = torch.zeros_like(S), torch.zeros_like(z)
+            for i in range(n0, n1, step):
+                j = min(n1, i + step)
+                x = q[b, h, i:j]
+                num, den, top = torch.zeros((j - i, d), dtype=f64, device="cuda"), torch.zeros(j - i, dtype=f64, device="cuda"), None
+                if n_s:
+                    e = (x.to(f64) @ ks.T) / math.sqrt(d)
+                    top = e.max(dim=1).values
+                    e = torch.exp_(e.sub_(top[:, None]))
+                    num, den = e @ vs, e.sum(dim=1)
+                    del e
+                lam = torch.exp(-top) if n_s and c["exact"] else torch.ones_like(den)
+                if aux is not None:
+                    aux[b, h, i:j, 1] = den
+                    if n_s:
+                        aux[b, h, i:j, 0] = top
+                if n_s < N:
+                    phi, slope = (y[0, 0] for y in phi_of(x, "q", slope=True))
+                    num = num + lam[:, None] * (phi @ S)
+                    den = den + lam * (phi @ z)
+                    if aux is not None:
+                        aux[b, h, i:j, 2] = phi @ z
+                y = num / den[:, None]
+                out[b, h, i - n0:j - n0] = y
+                if c["use"] == "step":
+                    diff = y - teacher[b, h, i:j].to(f64)
+                    loss += diff.abs().sum()
+                    gy = diff.sign()
+                    if n_s < N:
+                        g, sden = gy / den[:, None], -(gy * y).sum(dim=1) / den
+                        dphi = lam[:, None] * (g @ S.T + sden[:, None] * z)
+                        dw[0][h] += (dphi * slope).T @ x.to(f64)
+                        phi = lam[:, None] * phi
+                        dS += phi.T @ g
+                        dz += phi.T @ sden
+            if c["use"] == "step" and n_s < N:
+                for i in range(0, N, step):
+                    x = k[b, h, i:i + step]
+                    slope = phi_of(x, "k", slope=True)[1][0, 0] * lin[i:i + step, None]
+                    dw[1][h] += ((v[b, h, i:i + step].to(f64) @ dS.T + dz) * slope).T @ x.to(f64)
+    if c["use"] == "step":
+        return {"out": out, "aux": aux, "dwq": dw[0], "dwk": dw[1], "loss": loss}
+    if c["use"] == "shard":
+        sent = [torch.stack([x[n] for x in part]) for n in (0, 1)] if n_s < N else []
+        own = [x[:, :, soft & mine].reshape(B * H, -1, d).to(f64) for x in (k, v)]
+        return [out] + sent + own
+    return out.cpu() if c["use"] == "host" else out
