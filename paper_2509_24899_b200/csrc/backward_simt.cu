@@ -1,8 +1,9 @@
 // Gradient of the value-distillation loss L = sum |y - y_hat| ("Attention Distillation", value-distillation
 // loss; Algorithm 1 updates the feature maps only) w.r.t. the feature-map weights W_q, W_k of one hybrid
-// attention layer, in fp32 on CUDA cores: one-layer feature maps with F == d and no bias.  (With d = F = 128 on the tensor
-// path the products run on the tensor cores instead, backward_tensor.cu; this file keeps the reductions, the layout
-// of the partial results and the entry points.)
+// attention layer, in fp32 on CUDA cores: one-layer feature maps with F == d and no bias.  (On the tensor path the products
+// run on the tensor cores instead: d = F = 128 in backward_tensor.cu, d = F = 64 in backward_tensor_d64.cu.  This file
+// keeps the check path, the d = 64 layers whose tensors TMA cannot address, the reductions, the layout of the partial
+// results and the entry points.)
 //
 // With y_hat_i = num_i / den_i, num_i = N_i + lambda_i phi_q,i S, den_i = D_i + lambda_i phi_q,i . z (N_i, D_i: the
 // softmax branch, independent of the weights) the chain rule gives, per (batch, head):
@@ -377,12 +378,21 @@ as_status_t as_hybrid_attn_backward_phi(as_hybrid_attn_t h, const void* q, const
 
   const int BH = d.B * d.H, D = d.d;
   const dim3 grid(L.chunks, BH), rgrid((D * D + D + 255) / 256, std::max(BH, d.H), 2);
+  // TMA wants 16-byte aligned tensors; at d = 64 the CUDA-core kernels (eleven times slower) take what is not
+  const bool aligned = (((uintptr_t)q | (uintptr_t)k | (uintptr_t)v | (uintptr_t)w->wq1 | (uintptr_t)w->wk1 | (uintptr_t)y_teacher |
+                         (uintptr_t)y_hat) & 15) == 0;
   cudaError_t e = cudaSuccess;
   if (D == 128 && d.phi_dim == 128 && d.kernel_path == AS_PATH_TENSOR) {
     // the products on the tensor cores; the same fixed-order reductions
     if ((e = as_bw_tensor_init()) == cudaSuccess && (e = as_bw_tensor_query(p, st)) == cudaSuccess) {
       bw_reduce_kernel<<<rgrid, 256, 0, st>>>(p, D, 0);
       if ((e = as_bw_tensor_key(p, st)) == cudaSuccess) bw_reduce_kernel<<<rgrid, 256, 0, st>>>(p, D, 1);
+    }
+  } else if (D == 64 && d.kernel_path == AS_PATH_TENSOR && aligned) {
+    // the products on the tensor cores, fp32 operands in three bf16 pieces
+    if ((e = as_bw_tensor_d64_init()) == cudaSuccess && (e = as_bw_tensor_d64_query(p, st)) == cudaSuccess) {
+      bw_reduce_kernel<<<rgrid, 256, 0, st>>>(p, D, 0);
+      if ((e = as_bw_tensor_d64_key(p, st)) == cudaSuccess) bw_reduce_kernel<<<rgrid, 256, 0, st>>>(p, D, 1);
     }
   } else if (D == 128) {
     if ((e = cudaFuncSetAttribute(bw_query_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BwSmem<128>::BYTES)) == cudaSuccess &&

@@ -48,8 +48,7 @@ def _run(wl, mode, gain, margin, simt=False):
     y_bits = _teacher_with_margin(wl, oracle_inputs(data), mode) if margin else W.teacher_output(wl)
     dev = {k: to_cuda_bf16(v) for k, v in data.items()}
     y_dev = to_cuda_bf16(y_bits)
-    # (with d = F = 128 the default path runs the products on the tensor cores; the fp32 CUDA-core kernels take every
-    # other shape, and d = F = 128 as well when the handle is on the check path)
+    # (the default path runs the products on the tensor cores; the fp32 CUDA-core kernels are the check path)
     kw = {"kernel_path": binding.AS_PATH_SIMT} if simt else {}
     op = HybridAttention.from_workload(wl, stab_mode=mode, **kw)
     aux = torch.empty((wl.B, wl.H, wl.N, 3), dtype=torch.float32, device="cuda")
@@ -93,6 +92,62 @@ def test_phi_weight_gradients_on_the_cuda_core_path(name):
              "loss_rel_err": abs(loss - ref_loss) / ref_loss})
     assert eq <= 5e-3 and ek <= 5e-3, (eq, ek)
     assert abs(loss - ref_loss) <= 2e-3 * ref_loss
+
+
+# B, H, grid, block, rate, degree, stab_mode: less than a tile, one row past a tile, whole tiles, several tiles a chunk (odd
+# and even counts), more (batch, head) pairs than SMs, no softmax tokens
+D64_SHAPES = [(1, 1, (1, 7, 9), (1, 4, 4), 2, 2, O.STAB_PAPER), (1, 2, (1, 3, 43), (1, 4, 4), 0, 1, O.STAB_PAPER),
+              (1, 1, (1, 16, 16), (1, 4, 4), 4, 2, O.STAB_EXACT), (2, 40, (2, 20, 21), (1, 4, 4), 8, 2, O.STAB_EXACT),
+              (3, 60, (1, 29, 31), (1, 4, 4), 32, 1, O.STAB_PAPER), (1, 30, (2, 30, 52), (1, 6, 8), 0, 2, O.STAB_PAPER)]
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("shape", D64_SHAPES, ids=str)
+def test_narrow_head_gradient_has_the_precision_of_the_cuda_core_kernels(shape, offset):
+    """d = 64: the tensor-core kernels (three bf16 pieces) next to the fp32 kernels of the check path, on the same y_hat, row
+    statistics and state, and against the chain rule in 64 bits on those.  Sums over up to 3120 tokens in fp32, in blocks of 128:
+    a few times 2^-24 sqrt(log2(3120)) each, so 1e-6 (the fp32 kernels: up to 6e-7 here).  `offset`: a teacher tensor that starts
+    2 bytes off, which TMA cannot address."""
+    import torch
+    from paper_2509_24899_b200 import HybridAttention, binding
+    B, H, grid, block, rate, degree, mode = shape
+    N, d = int(np.prod(grid)), 64
+    wl = W.Workload("bw_d64", B=B, H=H, d=d, F=d, grid=grid, block=block, rate=rate, seed=67, degree=degree)
+    dev = {k: to_cuda_bf16(v) for k, v in W.generate(wl, wq_gain=2e-3 if rate else 1.0).items()}
+    flat = torch.empty(B * H * N * d + 8, dtype=torch.bfloat16, device="cuda")
+    y = flat[offset:offset + B * H * N * d].view(B, H, N, d)
+    y.copy_(to_cuda_bf16(W.teacher_output(wl)))
+    ops = [HybridAttention.from_workload(wl, stab_mode=mode, kernel_path=k) for k in (binding.AS_PATH_TENSOR, binding.AS_PATH_SIMT)]
+    aux = torch.empty((B, H, N, 3), dtype=torch.float32, device="cuda")
+    args = [dev[n] for n in ("q", "k", "v", "wq", "wk")]
+    y_hat = ops[0].forward(*args, aux=aux)
+    ops[1]._ws = ops[0].workspace()                     # S and z of the tensor path's forward
+    got = [op.backward_phi(*args, y, y_hat, aux) for op in ops]
+    S, z = (x.double() for x in ops[0].linear_state())
+    assert ops[0].last_status() == 0
+
+    def phi(x, w):
+        a = x.double() @ w.double().transpose(-1, -2)
+        power = torch.arange(d, device="cuda") // (d // degree)
+        return a.relu() ** (power + 1), (a > 0) * (power + 1) * a.relu() ** power
+
+    q, k, v, wq, wk = args
+    lam = torch.exp(-aux[..., 0].double()) if mode == O.STAB_EXACT and rate else torch.ones_like(aux[..., 0], dtype=torch.float64)
+    w = (lam / (aux[..., 1].double() + lam * aux[..., 2].double()))[..., None]
+    diff = y_hat.double() - y.double()
+    G = diff.sign()
+    t = -(G * y_hat.double()).sum(-1, keepdim=True)
+    phi_q, slope_q = phi(q, wq)
+    dwq = ((w * (G @ S.transpose(-1, -2) + z[:, :, None] * t) * slope_q).transpose(-1, -2) @ q.double()).sum(0)
+    dS, dz = (w * phi_q).transpose(-1, -2) @ G, (w * phi_q * t).sum(2)
+    linear = torch.from_numpy(~oracle_mask(wl)).cuda()[:, None]
+    dwk = (((v.double() @ dS.transpose(-1, -2) + dz[:, :, None]) * phi(k, wk)[1] * linear).transpose(-1, -2) @ k.double()).sum(0)
+    for dq, dk, loss in got:
+        # a pre-activation whose rounding changes its sign flips a slope of one: one row of one token, so the median over the features
+        for a, r in ((dq, dwq), (dk, dwk)):
+            err = (a.double() - r).norm(dim=-1) / r.norm(dim=-1)
+            assert err.median() <= 1e-6 and (err > 1e-5).sum() <= 2, err.max()
+        assert abs(loss.item() - diff.abs().sum().item()) <= 1e-5 * diff.abs().sum().item()
 
 
 def test_backward_argument_errors_and_zero_gradient_without_linear_tokens():
