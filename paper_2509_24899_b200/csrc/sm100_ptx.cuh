@@ -133,6 +133,19 @@ AS_DEV void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t i
       : "memory");
 }
 
+// One lane of a converged warp (the same one every time).  MMAs issued behind this test take their operands from uniform
+// registers; behind a comparison of the lane index every operand is moved over from a vector register first (measured
+// alone on an SM: eight MMAs and a commit 400 clk to issue against 540).
+AS_DEV bool elect_one() {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok));
+  return ok != 0;
+}
+
 // Instruction descriptor for kind::f16 with bf16 operands and fp32 accumulation.
 // a_mn / b_mn: 1 when the operand is MN-major (its M/N index is the contiguous one in smem).
 __host__ __device__ constexpr uint32_t make_idesc(int M, int N, int a_mn, int b_mn) {

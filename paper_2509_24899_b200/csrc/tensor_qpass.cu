@@ -114,8 +114,10 @@ struct QRing {
   //   two layers:  W1[0], V_last, W1[1 .. nh-1], then W2[c, j] (c slow), then S[0 .. fc-1]
   // addresses and waits only (the key loop needs nothing else)
   AS_DEV explicit QRing(const QCtx& c_) : c(c_), nkv(0), lin(0), two(0), fc(0), nh(0), vl(0), n_stream(0), n_items(0), n_s(0), n_p(0), n_pf(0) {}
-  AS_DEV QRing(const QParams& p, const QCtx& c_)
-      : c(c_), nkv(p.nkv), lin(p.lin), two(p.lin && p.layers == 2), fc(p.lin ? p.fc : 0), nh(p.nh), vl(p.nkv > 0 ? 1 : 0) {
+  // `uniform`: for warps that issue MMAs, addresses that the compiler can see to be the same in all lanes
+  AS_DEV QRing(const QParams& p, const QCtx& c_, bool uniform = false)
+      : c(uniform ? QCtx{__shfl_sync(0xffffffffu, c_.sbase, 0), __shfl_sync(0xffffffffu, c_.tmem, 0), c_.wc} : c_),
+        nkv(p.nkv), lin(p.lin), two(p.lin && p.layers == 2), fc(p.lin ? p.fc : 0), nh(p.nh), vl(p.nkv > 0 ? 1 : 0) {
     n_stream = nkv > 0 ? 2 * nkv - 1 : 0;
     n_items = n_stream + vl + (two ? nh + fc * nh + fc : 2 * fc);
     n_s = nkv + (two ? nh + fc : fc);
@@ -141,20 +143,7 @@ struct QRing {
   AS_DEV uint32_t tO(int g) const { return c.tmem + 256u + 128u * g; }
   AS_DEV bool wait(int b, int phase) const { return mbar_wait_warp(bar(b), phase & 1, c.wc); }
   AS_DEV void release(int item) const { tc_commit(bar(B_EMPTY + item % KV_STAGES)); }
-  // single-thread forms for the issuing thread (no warp vote): a wait that is already satisfied still
-  // costs a round trip to shared memory, so barriers needed together are probed together
-  AS_DEV bool wait1(int b, int phase) const { return mbar_wait(bar(b), phase & 1, c.wc); }
-  AS_DEV bool probe(int b, int phase) const { return mbar_try_wait(bar(b), phase & 1); }
-  AS_DEV bool wait_full(int item) const { return wait1(B_FULL + item % KV_STAGES, item / KV_STAGES); }
-  // barrier b0 and, when use1, the ring item's full barrier
-  AS_DEV bool wait2(int b0, int ph0, bool use1, int item) const {
-    const int b1 = B_FULL + item % KV_STAGES, ph1 = item / KV_STAGES;
-    const bool r0 = probe(b0, ph0);
-    const bool r1 = use1 ? probe(b1, ph1) : true;
-    if (r0 && r1) return true;
-    if (!r1 && !wait1(b1, ph1)) return false;
-    return r0 || wait1(b0, ph0);
-  }
+  AS_DEV bool wait_full(int item) const { return wait(B_FULL + item % KV_STAGES, item / KV_STAGES); }
 };
 
 // ---------------------------------------------------------------- TMA producer, one unit
@@ -215,20 +204,20 @@ __device__ __noinline__ bool q_produce_unit(const QParams& p, const QCtx& c, con
 }
 
 // ---------------------------------------------------------------- MMA issuers, one unit
-// Two issuing threads (lane 0 of warps 9 and 10; the other lanes wait at the end of the role): one issues
-// what writes the score columns (Q K^T per tile, Phi at the end) as soon as the softmax threads have read
-// them out, the other what accumulates into O (P V per tile, phi_q S at the end) as soon as P is in
-// shared memory.  The two streams touch different TMEM columns and release different ring items, so they
-// need no ordering between them; each thread's commits cover its own MMAs.  An issuing thread is the
-// busiest resource of the CTA - every clock it spends outside the MMA instructions is a clock the tensor
-// pipe may idle - so it takes no warp votes or warp barriers, probes the barriers it needs together, and
-// has its operands ready before it looks at a barrier.
+// Two issuing warps (9 and 10): one issues what writes the score columns (Q K^T per tile, Phi at the end) as soon as
+// the softmax threads have read them out, the other what accumulates into O (P V per tile, phi_q S at the end) as soon as
+// P is in shared memory.  The two streams touch different TMEM columns and release different ring items, so they
+// need no ordering between them; each warp's commits cover its own MMAs.  The whole warp walks the loop and one elected
+// lane issues: from converged code the operands of an MMA sit in uniform registers.  With a single thread in a branch of
+// its own, eight MMAs took 630 - 700 clk to issue beside the softmax warps (N = 64, d = 64: as long, though they execute in
+// 380); now 320 - 380 (130 for the four of Q K^T at d = 64).  N = 7800: 96.3 -> 93.7 us, headline layer 838 -> 830 us
+// (sustained), two-layer map 1203 -> 1176 us.
 template <int D, bool TWO, bool GEN>
 __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u) {
   using R = QRing<D>;
   constexpr uint32_t ID_QK = make_idesc(128, 128, 0, 0);      // S = Q K^T      (N = 128 keys)
   const int nkv = p.nkv, lin = p.lin;
-  const R q(p, c);
+  const R q(p, c, true);
   const uint32_t id_phi = make_idesc(128, D == 128 ? 128 : p.fcw, 0, 0);   // Phi_c = X W^T  (N = features of a chunk; 128 at d = 128)
   constexpr uint32_t ID_HID = make_idesc(128, D, 0, 0);       // hidden slice = Q W_1[j]^T (N = D hidden units)
   const int base = u * q.n_items, ps = u * q.n_s;             // first ring item / first score-column phase of the unit
@@ -242,20 +231,23 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
   }
   // The i-th product of the unit into a group's score columns overwrites what the threads read last: the
   // (i-1)-th use, or the previous unit's last one.
-  auto s_free = [&](int g, int i) -> bool { return (u == 0 && i == 0) ? true : q.wait1(R::B_SF + g, ps + i - 1); };
+  auto s_free = [&](int g, int i) -> bool { return (u == 0 && i == 0) ? true : q.wait(R::B_SF + g, ps + i - 1); };
 
   // ---- first key tile (its product opens the unit)
   if (nkv > 0) {
     for (int g = 0; g < ng; ++g) {
       if (!s_free(g, 0)) return false;
-      if (!q.wait2(R::B_Q0 + g, u, g == 0, base)) return false;
+      if (g == 0 && !q.wait_full(base)) return false;
+      if (!q.wait(R::B_Q0 + g, u)) return false;
       tc_fence_after();
       const uint64_t k0 = kmajor_desc(q.sKV(base));
+      if (elect_one()) {
 #pragma unroll
-      for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tS(g), dq[g][kk], k0 + kstep_kmajor(kk), ID_QK, kk > 0 ? 1u : 0u);
-      tc_commit(q.bar(R::B_S + g));
-      if (g == ng - 1) q.release(base);
-      if (nkv == 1 && !lin) tc_commit(q.bar(R::B_QF + g));
+        for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tS(g), dq[g][kk], k0 + kstep_kmajor(kk), ID_QK, kk > 0 ? 1u : 0u);
+        tc_commit(q.bar(R::B_S + g));
+        if (g == ng - 1) q.release(base);
+        if (nkv == 1 && !lin) tc_commit(q.bar(R::B_QF + g));
+      }
     }
   }
   // ---- as soon as the groups have read their score rows: the next tile's Q K^T
@@ -265,14 +257,17 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
 #pragma unroll
     for (int g = 0; g < 2; ++g) {
       if (g >= ng) break;
-      if (!q.wait2(R::B_SF + g, ps + j, g == 0, ik)) return false;
+      if (g == 0 && !q.wait_full(ik)) return false;
+      if (!q.wait(R::B_SF + g, ps + j)) return false;
       tc_fence_after();
+      if (elect_one()) {
 #pragma unroll
-      for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tS(g), dq[g][kk], k0 + kstep_kmajor(kk), ID_QK, kk > 0 ? 1u : 0u);
-      tc_commit(q.bar(R::B_S + g));
-      if (j + 2 == nkv && !lin) tc_commit(q.bar(R::B_QF + g));   // the unit's last read of the Q tile
+        for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tS(g), dq[g][kk], k0 + kstep_kmajor(kk), ID_QK, kk > 0 ? 1u : 0u);
+        tc_commit(q.bar(R::B_S + g));
+        if (j + 2 == nkv && !lin) tc_commit(q.bar(R::B_QF + g));   // the unit's last read of the Q tile
+      }
     }
-    q.release(ik);
+    if (elect_one()) q.release(ik);
   }
   if (!lin) return true;
 
@@ -284,15 +279,17 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
       const uint64_t w0 = kmajor_desc(q.sKV(iw));
       for (int g = 0; g < ng; ++g) {
         if (!s_free(g, nkv + ch)) return false;
-        if (nkv == 0 && ch == 0 && !q.wait1(R::B_Q0 + g, u)) return false;
+        if (nkv == 0 && ch == 0 && !q.wait(R::B_Q0 + g, u)) return false;
         if (g == 0 && !q.wait_full(iw)) return false;
         tc_fence_after();
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tS(g), dq[g][kk], w0 + kstep_kmajor(kk), id_phi, kk > 0 ? 1u : 0u);
-        tc_commit(q.bar(R::B_S + g));
-        if (ch == q.fc - 1) tc_commit(q.bar(R::B_QF + g));     // nothing of this unit reads the group's Q tile any more
+          for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tS(g), dq[g][kk], w0 + kstep_kmajor(kk), id_phi, kk > 0 ? 1u : 0u);
+          tc_commit(q.bar(R::B_S + g));
+          if (ch == q.fc - 1) tc_commit(q.bar(R::B_QF + g));     // nothing of this unit reads the group's Q tile any more
+        }
       }
-      q.release(iw);
+      if (elect_one()) q.release(iw);
     }
     return true;
   } else {
@@ -303,15 +300,17 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
     const uint64_t w0 = kmajor_desc(q.sKV(iw));
     for (int g = 0; g < ng; ++g) {
       if (!s_free(g, nkv + j)) return false;
-      if (nkv == 0 && j == 0 && !q.wait1(R::B_Q0 + g, u)) return false;
+      if (nkv == 0 && j == 0 && !q.wait(R::B_Q0 + g, u)) return false;
       if (g == 0 && !q.wait_full(iw)) return false;
       tc_fence_after();
+      if (elect_one()) {
 #pragma unroll
-      for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tS(g), dq[g][kk], w0 + kstep_kmajor(kk), ID_HID, kk > 0 ? 1u : 0u);
-      tc_commit(q.bar(R::B_S + g));
-      if (q.nh == 1 && q.fc == 1) tc_commit(q.bar(R::B_QF + g));   // the Q tile is not reused as a buffer in this shape
+        for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tS(g), dq[g][kk], w0 + kstep_kmajor(kk), ID_HID, kk > 0 ? 1u : 0u);
+        tc_commit(q.bar(R::B_S + g));
+        if (q.nh == 1 && q.fc == 1) tc_commit(q.bar(R::B_QF + g));   // the Q tile is not reused as a buffer in this shape
+      }
     }
-    q.release(iw);
+    if (elect_one()) q.release(iw);
   }
   for (int ch = 0; ch < q.fc; ++ch) {
     for (int j = 0; j < q.nh; ++j) {
@@ -321,20 +320,22 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
       for (int g = 0; g < ng; ++g) {
         if (j == 0) {
           if (!s_free(g, nkv + q.nh + ch)) return false;
-          if (ch == 0 && !q.wait1(R::B_H + g, u)) return false;   // the group's hidden activations are in shared memory
+          if (ch == 0 && !q.wait(R::B_H + g, u)) return false;   // the group's hidden activations are in shared memory
         }
         tc_fence_after();
         const uint64_t a0 = kmajor_desc(j == 0 ? q.sP(g) : q.sQ(g));
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk)
-          mma_ss(q.tS(g), a0 + kstep_kmajor(kk), w0 + kstep_kmajor(kk), id_phi, (j > 0 || kk > 0) ? 1u : 0u);
-        if (j == q.nh - 1) {
-          tc_commit(q.bar(R::B_S + g));
-          // two hidden slices, one feature chunk: this was the last read of the Q tile (as a buffer)
-          if (q.nh == 2 && q.fc == 1) tc_commit(q.bar(R::B_QF + g));
+          for (int kk = 0; kk < D / 16; ++kk)
+            mma_ss(q.tS(g), a0 + kstep_kmajor(kk), w0 + kstep_kmajor(kk), id_phi, (j > 0 || kk > 0) ? 1u : 0u);
+          if (j == q.nh - 1) {
+            tc_commit(q.bar(R::B_S + g));
+            // two hidden slices, one feature chunk: this was the last read of the Q tile (as a buffer)
+            if (q.nh == 2 && q.fc == 1) tc_commit(q.bar(R::B_QF + g));
+          }
         }
       }
-      q.release(iw);
+      if (elect_one()) q.release(iw);
     }
   }
   return true;
@@ -346,7 +347,7 @@ __device__ __noinline__ bool q_accum_unit(const QParams& p, const QCtx& c, int u
   using R = QRing<D>;
   constexpr uint32_t ID_PV = make_idesc(128, D, 0, 1);        // O += P V and O += phi_q S  (V, S are MN-major)
   const int nkv = p.nkv, lin = p.lin;
-  const R q(p, c);
+  const R q(p, c, true);
   const int base = u * q.n_items, pp = u * q.n_p;             // first ring item / first P hand-over phase of the unit
   const int ng = q_unit(p, u).ng;
   uint64_t dp[2][8];                                          // the P tiles never move
@@ -364,14 +365,17 @@ __device__ __noinline__ bool q_accum_unit(const QParams& p, const QCtx& c, int u
 #pragma unroll
     for (int g = 0; g < 2; ++g) {
       if (g >= ng) break;
-      if (!q.wait2(R::B_P + g, pp + j, g == 0, iv)) return false;
+      if (g == 0 && !q.wait_full(iv)) return false;
+      if (!q.wait(R::B_P + g, pp + j)) return false;
       tc_fence_after();
+      if (elect_one()) {
 #pragma unroll
-      for (int kk = 0; kk < 8; ++kk) mma_ss(q.tO(g), dp[g][kk], v0 + kstep_mnmajor(kk), ID_PV, (j > 0 || kk > 0) ? 1u : 0u);
-      tc_commit(q.bar(R::B_PF + g));
-      if (last && !lin) tc_commit(q.bar(R::B_O + g));
+        for (int kk = 0; kk < 8; ++kk) mma_ss(q.tO(g), dp[g][kk], v0 + kstep_mnmajor(kk), ID_PV, (j > 0 || kk > 0) ? 1u : 0u);
+        tc_commit(q.bar(R::B_PF + g));
+        if (last && !lin) tc_commit(q.bar(R::B_O + g));
+      }
     }
-    q.release(iv);
+    if (elect_one()) q.release(iv);
   }
   if (!lin) return true;
   // O += phi_q,c S_c per feature chunk: phi_q sits where P sits (two layers, second chunk: in the Q tile),
@@ -382,19 +386,22 @@ __device__ __noinline__ bool q_accum_unit(const QParams& p, const QCtx& c, int u
     const uint64_t s0 = mnmajor_desc(q.sKV(is));
     const bool in_q_tile = TWO && ch == 1;
     for (int g = 0; g < ng; ++g) {
-      if (!q.wait2(R::B_P + g, pp + nkv + ch, g == 0, is)) return false;
+      if (g == 0 && !q.wait_full(is)) return false;
+      if (!q.wait(R::B_P + g, pp + nkv + ch)) return false;
       tc_fence_after();
       const uint64_t a0 = in_q_tile ? kmajor_desc(q.sQ(g)) : dp[g][0];
+      if (elect_one()) {
 #pragma unroll
-      for (int kk = 0; kk < 8; ++kk)
-        if (kk < ksteps) mma_ss(q.tO(g), a0 + kstep_kmajor(kk), s0 + kstep_mnmajor(kk), ID_PV, (nkv > 0 || ch > 0 || kk > 0) ? 1u : 0u);
-      if (!in_q_tile) tc_commit(q.bar(R::B_PF + g));           // a reader of the P tile has completed
-      if (ch == q.fc - 1) {
-        tc_commit(q.bar(R::B_O + g));
-        if (in_q_tile) tc_commit(q.bar(R::B_QF + g));          // ... and the last reader of the Q tile
+        for (int kk = 0; kk < 8; ++kk)
+          if (kk < ksteps) mma_ss(q.tO(g), a0 + kstep_kmajor(kk), s0 + kstep_mnmajor(kk), ID_PV, (nkv > 0 || ch > 0 || kk > 0) ? 1u : 0u);
+        if (!in_q_tile) tc_commit(q.bar(R::B_PF + g));           // a reader of the P tile has completed
+        if (ch == q.fc - 1) {
+          tc_commit(q.bar(R::B_O + g));
+          if (in_q_tile) tc_commit(q.bar(R::B_QF + g));          // ... and the last reader of the Q tile
+        }
       }
     }
-    q.release(is);
+    if (elect_one()) q.release(is);
   }
   return true;
 }
@@ -946,17 +953,11 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     for (int u = 0; u < n_mine; ++u)
       if (!q_produce_unit<D, false, GEN>(p, c, &tmQ, &tmQ, &tmQ, &tmW, &tmSt, &tmW, u)) break;
   } else if (warp == 17) {
-    if ((threadIdx.x & 31) == 0) {
-      for (int u = 0; u < n_mine; ++u)
-        if (!q_score_unit<D, false, GEN>(p, c, u)) break;
-    }
-    __syncwarp();
+    for (int u = 0; u < n_mine; ++u)
+      if (!q_score_unit<D, false, GEN>(p, c, u)) break;
   } else if (warp == 18) {
-    if ((threadIdx.x & 31) == 0) {
-      for (int u = 0; u < n_mine; ++u)
-        if (!q_accum_unit<D, false, GEN>(p, c, u)) break;
-    }
-    __syncwarp();
+    for (int u = 0; u < n_mine; ++u)
+      if (!q_accum_unit<D, false, GEN>(p, c, u)) break;
   } else {
     const int g = (warp >> 2) & 1;
     // a unit worked on by one group only (a left-over half) is the CTA's last one: group 1 stops before it
@@ -1020,17 +1021,11 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     for (int u = 0; u < n_mine; ++u)
       if (!q_produce_unit<D, TWO, GEN>(p, c, &tmQ, &tmK, &tmV, &tmW, &tmSt, &tmW1, u)) break;
   } else if (warp == 9) {
-    if ((threadIdx.x & 31) == 0) {
-      for (int u = 0; u < n_mine; ++u)
-        if (!q_score_unit<D, TWO, GEN>(p, c, u)) break;
-    }
-    __syncwarp();
+    for (int u = 0; u < n_mine; ++u)
+      if (!q_score_unit<D, TWO, GEN>(p, c, u)) break;
   } else if (warp == 10) {
-    if ((threadIdx.x & 31) == 0) {
-      for (int u = 0; u < n_mine; ++u)
-        if (!q_accum_unit<D, TWO, GEN>(p, c, u)) break;
-    }
-    __syncwarp();
+    for (int u = 0; u < n_mine; ++u)
+      if (!q_accum_unit<D, TWO, GEN>(p, c, u)) break;
   } else {
     // a unit worked on by one group only (a left-over half) is the CTA's last one: group 1 stops before it
     const int n_grp = (n_mine > p.n_rounds && p.split_last && warp >= 4) ? p.n_rounds : n_mine;
