@@ -22,7 +22,6 @@ struct KParams {
   int N, n_s, n_chunks, chunk_tiles, P, F, H;
   const int32_t* sm_rank;              // [N (+ padding)]: position in T_S, or -1 for a linear token
   __nv_bfloat16 *ks_w, *vs_w;          // compact softmax K / V (nullptr when nothing is gathered)
-  const __nv_bfloat16* k;              // two-layer maps gather the softmax K rows from here (no K tile in the ring)
   const __nv_bfloat16* bias;           // last-layer bias [H][F], or nullptr
   float *part_s, *part_z;
   float *S, *z;                        // [B*H][F][D], [B*H][F]: the chunks' partials added up ...
@@ -243,6 +242,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
         for (int i = 0; i < IPT; ++i) {
           const int it = t * IPT + i;
           ok = ok && mbar_wait_warp(bar(B_FULL + it % SLOTS), (it / SLOTS) & 1, wc);
+          if (LAYERS == 2 && i < NX && ok && lane == 0) mbar_arrive(bar(B_EMPTY + it % SLOTS));   // a hidden slice: not read here
         }
         if (!ok) break;
         const uint8_t* kt = LAYERS == 1 ? smem + L::RING_OFF + ((t * IPT) % SLOTS) * L::TILE : nullptr;
@@ -255,17 +255,11 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
             bits &= bits - 1;
             const int rank = __shfl_sync(0xffffffffu, rk[e], src);
             const uint32_t rrow = gw * 64 + e * 32 + src;
-            // lanes [0, CH) move the K row, lanes [16, 16 + CH) the V row
+            // lanes [0, CH) move the K row (two layers: phi1_kernel has done that), lanes [16, 16 + CH) the V row
             const int c = lane & 15;
-            if (c < CH) {
-              uint4 val;
-              if (lane < 16 && LAYERS == 2) {
-                const size_t n = (size_t)(t_begin + t) * 128 + rrow;
-                val = *reinterpret_cast<const uint4*>(p.k + ((size_t)bh * p.N + n) * D + c * 8);
-              } else {
-                const uint8_t* tile = (lane < 16) ? kt : vt;
-                val = *reinterpret_cast<const uint4*>(tile + (c / 8) * BOX_BYTES + swz128_chunk_offset(rrow, c % 8));
-              }
+            if (c < CH && (LAYERS == 1 || lane >= 16)) {
+              const uint8_t* tile = (lane < 16) ? kt : vt;
+              const uint4 val = *reinterpret_cast<const uint4*>(tile + (c / 8) * BOX_BYTES + swz128_chunk_offset(rrow, c % 8));
               __nv_bfloat16* dst = ((lane < 16) ? p.ks_w : p.vs_w) + ((size_t)bh * p.n_s + rank) * D + c * 8;
               *reinterpret_cast<uint4*>(dst) = val;
             }
@@ -273,7 +267,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
         }
         __syncwarp();
         if (lane == 0)
-          for (int i = 0; i < IPT; ++i) mbar_arrive(bar(B_EMPTY + (t * IPT + i) % SLOTS));
+          for (int i = LAYERS == 1 ? 0 : NX; i < IPT; ++i) mbar_arrive(bar(B_EMPTY + (t * IPT + i) % SLOTS));
       }
     }
     named_barrier_arrive(2, K_FEATURE_THREADS + 64);           // the feature warps may reuse the ring for the partial S
@@ -442,8 +436,12 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
 // ======================================================================================
 // First layer of a two-layer feature map for the keys ("Characterization of phi": the embedding
 // network): h1 = relu(k W_1^T + b_1), [B*H, N, hidden] bf16.  One 128-token tile per CTA, all hidden slices.
+// The softmax rows of K are copied to K_S here, where the K tile is in shared memory, by the warps that otherwise only wait
+// for the product.  (The K pass, which has h1 tiles in its ring instead, fetched them from global memory one row after
+// the other and held its slots of the ring meanwhile: the whole key side 338 us against 181 at N = 32760, rate 1/8, hidden =
+// F = 256, the layer 1182 against 1071.)
 // ======================================================================================
-struct P1Params { int H, hid; const __nv_bfloat16* bias; uint32_t* status; };
+struct P1Params { int H, hid, N, n_s; const __nv_bfloat16* bias; const int32_t* sm_rank; __nv_bfloat16* ks_w; uint32_t* status; };
 constexpr int P1_THREADS = 160;          // warps 0-3: epilogue (one thread per token row); warp 4: TMA + MMA
 
 template <int D, int NH>
@@ -513,7 +511,32 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
   } else {
     const int r = warp * 32 + lane;
     const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
-    bool ok = mbar_wait_warp(bar_done, 0, wc);
+    bool ok = true;
+    if (p.ks_w != nullptr) {
+      // this warp's 32 rows of the K tile (which its threads overwrite below, each its own row); D / 8 lanes a row
+      constexpr int CH = D / 8, RPI = 32 / CH;
+      const int rank = row0 + r < p.N ? p.sm_rank[row0 + r] : -1;
+      uint32_t bits = __ballot_sync(0xffffffffu, rank >= 0);
+      if (bits) ok = mbar_wait_warp(bar_full, 0, wc);
+      while (ok && bits) {
+        int src = -1;
+#pragma unroll
+        for (int i = 0; i < RPI; ++i) {
+          if (bits) {
+            if (lane / CH == i) src = __ffs(bits) - 1;
+            bits &= bits - 1;
+          }
+        }
+        const int to = __shfl_sync(0xffffffffu, rank, src < 0 ? 0 : src);
+        if (src >= 0) {
+          const int c = lane % CH;
+          const uint4 val = *reinterpret_cast<const uint4*>(smem + L::X_OFF + (c / 8) * BOX_BYTES + swz128_chunk_offset(warp * 32 + src, c % 8));
+          *reinterpret_cast<uint4*>(p.ks_w + ((size_t)bh * p.n_s + to) * D + c * 8) = val;
+        }
+      }
+      __syncwarp();
+    }
+    if (ok) ok = mbar_wait_warp(bar_done, 0, wc);
     if (ok) {
       tc_fence_after();
       uint32_t x[32];
@@ -585,7 +608,7 @@ cudaError_t as_tensor_phi1(const as_launch_args& a, cudaStream_t st) {
   if (!make_map(&tmX, a.k, a.d, a.N, BH, 128) || !make_map(&tmW, a.wk, a.d, a.hid, a.H, 128) ||
       !make_map(&tmH, a.h1k, a.hid, a.N, BH, 128))
     return cudaErrorInvalidValue;
-  P1Params p{a.H, a.hid, a.bk1, a.status};
+  P1Params p{a.H, a.hid, a.N, a.n_s, a.bk1, a.sm_rank, a.ks_w, a.status};
   dim3 grid((a.N + 127) / 128, BH, 1);
   if (a.d == 128 && a.hid == 256) phi1_kernel<128, 2><<<grid, P1_THREADS, P1Layout<128, 2>::TOTAL, st>>>(tmX, tmW, tmH, p);
   else if (a.d == 128) phi1_kernel<128, 1><<<grid, P1_THREADS, P1Layout<128, 1>::TOTAL, st>>>(tmX, tmW, tmH, p);
@@ -604,7 +627,7 @@ cudaError_t as_tensor_kpass(const as_launch_args& a, cudaStream_t st) {
   else tmH = tmK;               // never used with a one-layer map
   KParams p{};
   p.N = a.N; p.n_s = a.n_s; p.n_chunks = a.n_chunks; p.chunk_tiles = a.chunk_tiles; p.P = a.P; p.F = a.F;
-  p.H = a.H; p.sm_rank = a.sm_rank; p.ks_w = a.ks_w; p.vs_w = a.vs_w; p.k = a.k;
+  p.H = a.H; p.sm_rank = a.sm_rank; p.ks_w = a.ks_w; p.vs_w = a.vs_w;
   p.bias = two ? a.bk2 : a.bk1;
   p.part_s = a.part_s; p.part_z = a.part_z; p.status = a.status;
   p.S = a.S; p.z = a.z; p.Sb = a.Sb; p.counters = a.counters;
