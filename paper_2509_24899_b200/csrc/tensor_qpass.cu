@@ -32,9 +32,10 @@ struct QParams {
   int nh;                    // two layers: slices of the hidden width (each D wide)
   const __nv_bfloat16* b1;   // two layers: first-layer bias of this launch's first head [H][hidden], or nullptr
   const __nv_bfloat16* b2;   // last-layer bias [H][F], or nullptr
-  int nx, n_units;           // 256-row units per (batch, head); units over all (batch, head) pairs
-  int n_rounds;              // rounds in which every CTA has a unit (n_units / gridDim.x)
-  int split_last;            // 1: the units left over after those rounds are cut in two 128-row halves, one per CTA
+  int nx, n_pairs;           // two-tile units per (batch, head); over all (batch, head) pairs
+  int n_single;              // units of a (batch, head)'s last tile alone: one per (batch, head) or none
+  int n_rounds;              // rounds in which every CTA has a two-tile unit (n_pairs / gridDim.x)
+  int split_last;            // 1: the two-tile units left over after those rounds are cut in two, one tile per CTA
   float scale_log2;          // softmax scale * log2(e)
   const float* z;            // [B*H][F]
   float* aux;                // [B*H][N][3] or nullptr
@@ -75,24 +76,26 @@ struct QCtx {
   WaitCtx wc;
 };
 
-// Unit u of this CTA: which 256-row unit, which row it starts at, and how many of the two 128-row groups
-// work on it.  In the rounds every CTA takes part in, CTA c has unit c + u * gridDim.x.  What is left
-// over afterwards would keep less than half of the SMs busy for a whole unit's time; a single group, which
-// has the tensor and XU pipes to itself, needs little more than half of that, so the left-over units are
-// cut into their two 128-row halves and spread over twice as many CTAs.
-struct QUnit { int w, row0, ng; };
+// Unit u of this CTA: which (batch, head), the row it starts at, and how many of the two 128-row groups work on it.  In
+// the rounds every CTA takes part in, CTA c has two-tile unit c + u * gridDim.x.  Last, each CTA takes at most one of what
+// is left: two-tile units - cut into their two tiles where CTAs enough are left for that - and the last tiles of heads with
+// an odd number of them (see plan_units).  A group that has the tensor and XU pipes to itself needs about two thirds of
+// the time that the two of a two-tile unit take.
+struct QUnit { int bh, row0, ng; };
 AS_DEV QUnit q_unit(const QParams& p, int u) {
   const int c = (int)blockIdx.x, n = (int)gridDim.x;
-  if (u < p.n_rounds) { const int w = c + u * n; return QUnit{w, (w % p.nx) * 256, 2}; }
-  if (p.split_last) { const int w = p.n_rounds * n + (c >> 1); return QUnit{w, (w % p.nx) * 256 + (c & 1) * 128, 1}; }
-  const int w = p.n_rounds * n + c;
-  return QUnit{w, (w % p.nx) * 256, 2};
+  int w = c + u * n, half = 0, ng = 2;
+  if (u >= p.n_rounds) {
+    const int left = p.n_pairs - p.n_rounds * n, cut = p.split_last ? 2 * left : left;
+    if (c >= cut) return QUnit{c - cut, p.nx * 256, 1};
+    if (p.split_last) { w = p.n_rounds * n + (c >> 1); half = (c & 1) * 128; ng = 1; }
+  }
+  return QUnit{w / p.nx, (w % p.nx) * 256 + half, ng};
 }
 // number of units CTA c walks over
 AS_DEV int q_units_of_cta(const QParams& p) {
-  const int left = p.n_units - p.n_rounds * (int)gridDim.x;
-  const int extra = p.split_last ? ((int)blockIdx.x < 2 * left) : ((int)blockIdx.x < left);
-  return p.n_rounds + (extra ? 1 : 0);
+  const int left = p.n_pairs - p.n_rounds * (int)gridDim.x;
+  return p.n_rounds + ((int)blockIdx.x < (p.split_last ? 2 * left : left) + p.n_single ? 1 : 0);
 }
 
 template <int D>
@@ -157,7 +160,7 @@ __device__ __noinline__ bool q_produce_unit(const QParams& p, const QCtx& c, con
   const R q(p, c);
   const int lane = threadIdx.x & 31;
   const QUnit un = q_unit(p, u);
-  const int bh = un.w / p.nx, h = bh % p.H, row0 = un.row0;
+  const int bh = un.bh, h = bh % p.H, row0 = un.row0;
   const int base = u * q.n_items;
   const int q_at = nkv > 0 ? 1 : 0;                   // the Q tiles are requested right after the unit's first K tile
   for (int it = 0; it < q.n_items; ++it) {
@@ -725,7 +728,7 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
   }
 
   const QUnit un = q_unit(p, u);
-  const int bh = un.w / p.nx;
+  const int bh = un.bh;
   const int row = un.row0 + g * 128 + r;
   float den = l, den_l_out = 0.f;
   if (p.lin) {
@@ -815,7 +818,7 @@ __device__ __noinline__ bool q_linear_unit(const QParams& p, const QCtx& c, cons
   const int fcw = D == 128 ? 128 : p.fcw;           // width of a feature chunk; this thread takes columns [hf, hf + 1) * half
   const int half = fcw / 2;
   const QUnit un = q_unit(p, u);
-  const int bh = un.w / p.nx, row = un.row0 + g * 128 + r;
+  const int bh = un.bh, row = un.row0 + g * 128 + r;
   const int part = p.F / p.P;
   uint32_t x[32];
   float dl = 0.f;
@@ -960,8 +963,8 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       if (!q_accum_unit<D, false, GEN>(p, c, u)) break;
   } else {
     const int g = (warp >> 2) & 1;
-    // a unit worked on by one group only (a left-over half) is the CTA's last one: group 1 stops before it
-    const int n_grp = (n_mine > p.n_rounds && p.split_last && g == 1) ? p.n_rounds : n_mine;
+    // a unit worked on by one group only is the CTA's last one: group 1 stops before it
+    const int n_grp = (n_mine > p.n_rounds && g == 1 && q_unit(p, p.n_rounds).ng == 1) ? p.n_rounds : n_mine;
     for (int u = 0; u < n_grp; ++u)
       if (!q_linear_unit<D, GEN>(p, c, &tmO, smem, sDl, u)) break;
     if ((threadIdx.x & 31) == 0) tma_store_wait_read();
@@ -1027,8 +1030,8 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     for (int u = 0; u < n_mine; ++u)
       if (!q_accum_unit<D, TWO, GEN>(p, c, u)) break;
   } else {
-    // a unit worked on by one group only (a left-over half) is the CTA's last one: group 1 stops before it
-    const int n_grp = (n_mine > p.n_rounds && p.split_last && warp >= 4) ? p.n_rounds : n_mine;
+    // a unit worked on by one group only is the CTA's last one: group 1 stops before it
+    const int n_grp = (n_mine > p.n_rounds && warp >= 4 && q_unit(p, p.n_rounds).ng == 1) ? p.n_rounds : n_mine;
     for (int u = 0; u < n_grp; ++u)
       if (!q_softmax_unit<D, TWO, GEN>(p, c, &tmO, smem, u)) break;
     if ((threadIdx.x & 31) == 0) tma_store_wait_read();  // this warp's output stores have read their rows (the writes land by the end of the kernel)
@@ -1061,6 +1064,33 @@ cudaError_t as_tensor_init_qpass() {
   if ((e = opt_in_smem(qlin_kernel<64, true>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
   return cudaSuccess;
 }
+
+// How the 128-row tiles of a launch are dealt out to the CTAs: full rounds of two-tile units, then one last round.  A head
+// with an odd number of tiles either has its last tile in a unit of its own, or in a two-tile unit whose other half is
+// past the end; which is better depends on what the last round comes to (N = 7800, 61 tiles in each of 12 heads, 148 SMs:
+// 360 units and 12 single tiles are two rounds and 140 tiles alone, 372 units are two rounds and 76 units: layer 92.8 -> 88.6
+// us; N = 1024 with 2 heads on 16 CTAs instead of 8: 22.5 -> 21.4).  Returns the
+// number of CTAs.
+namespace {
+int plan_units(QParams& p, int BH, int sms) {
+  const int tiles = (p.N + 127) / 128;
+  double best = 0.;
+  int grid = 0;
+  for (int alone = 0; alone <= (tiles & 1); ++alone) {
+    const int nx = (tiles + 1 - alone) / 2, pairs = nx * BH, single = alone * BH;
+    const int rounds = pairs / sms, left = pairs - rounds * sms;
+    const bool cut = 2 * left + single <= sms;
+    const int last = (cut ? 2 * left : left) + single;
+    if (last > sms) continue;                        // one last round only
+    const double t = rounds + (last == 0 ? 0. : (cut || left == 0) ? 0.7 : 1.);
+    if (grid != 0 && t > best) continue;             // (no worse: without empty tiles)
+    best = t;
+    p.nx = nx; p.n_pairs = pairs; p.n_single = single; p.n_rounds = rounds; p.split_last = cut ? 1 : 0;
+    grid = rounds > 0 ? sms : last;
+  }
+  return grid;
+}
+}  // namespace
 
 cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   if (as_tensor_qstream_handles(a)) return as_tensor_qstream(a, st);   // no softmax tokens, the common feature map
@@ -1095,17 +1125,11 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   p.b2 = two ? a.bq2 : a.bq1;
   p.scale_log2 = a.scale * 1.4426950408889634f;
   p.z = a.z; p.aux = a.aux; p.status = a.status;
-  p.nx = (a.N + 255) / 256;
-  p.n_units = p.nx * BH;
   // persistent: one CTA per SM (the kernel's shared memory and its 512 TMEM columns allow no second one)
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
     return cudaErrorInvalidValue;
-  dim3 grid(p.n_units < sms ? p.n_units : sms, 1, 1);
-  p.n_rounds = p.n_units / (int)grid.x;
-  const int left = p.n_units - p.n_rounds * (int)grid.x;
-  // left-over units as 128-row halves when twice their number still fits the grid
-  p.split_last = (left > 0 && 2 * left <= (int)grid.x) ? 1 : 0;
+  const dim3 grid(plan_units(p, BH, sms), 1, 1);
   // the general kernels carry the bias and the powers beyond 2; the common case does without them
   const bool gen = lin && (a.P > 2 || p.b1 != nullptr || p.b2 != nullptr);
   if (p.nkv == 0 && lin && !two) {
