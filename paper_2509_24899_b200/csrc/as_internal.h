@@ -92,5 +92,18 @@ cudaError_t as_tensor_init();
 // Test aid: a kernel whose bounded wait (the one every kernel here uses) runs out after `limit_cycles`.
 cudaError_t as_tensor_expire_wait(uint32_t* status, long long limit_cycles, cudaStream_t st);
 
+// Launches a kernel that begins with griddep_wait after its set-up (barriers, tensor memory): its CTAs may start, and
+// set up, while the kernel before it in the stream drains.
+template <typename... P, typename... A>
+cudaError_t as_launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cfg.attrs = &attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Status bits written by kernels into as_launch_args::status.
 constexpr uint32_t AS_DEV_TIMEOUT = 1u;

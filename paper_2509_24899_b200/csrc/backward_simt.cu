@@ -19,6 +19,7 @@
 
 #include "as_internal.h"
 #include "backward_common.h"
+#include "sm100_ptx.cuh"
 
 namespace {
 
@@ -238,6 +239,8 @@ __global__ void __launch_bounds__(BW_THREADS, 1) bw_key_kernel(BwParams p) {
 // Fixed-order sums.  stage 0 (after the query side): dS, dz per (batch, head); dW_q per head over batch and
 // chunks; the loss.  stage 1 (after the key side): dW_k per head.
 __global__ void bw_reduce_kernel(BwParams p, int D, int stage) {
+  sm100::griddep_launch();
+  sm100::griddep_wait();
   const int F = D;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;          // entry of an [F][D] matrix, then of an [F] vector
   const int bh = blockIdx.y;                                    // stage 0, blockIdx.z == 0: per (batch, head)
@@ -381,19 +384,18 @@ as_status_t as_hybrid_attn_backward_phi(as_hybrid_attn_t h, const void* q, const
   // TMA wants 16-byte aligned tensors; at d = 64 the CUDA-core kernels (eleven times slower) take what is not
   const bool aligned = (((uintptr_t)q | (uintptr_t)k | (uintptr_t)v | (uintptr_t)w->wq1 | (uintptr_t)w->wk1 | (uintptr_t)y_teacher |
                          (uintptr_t)y_hat) & 15) == 0;
+  auto reduce = [&](int stage) { return as_launch_dependent(bw_reduce_kernel, rgrid, dim3(256), 0, st, p, D, stage); };
   cudaError_t e = cudaSuccess;
   if (D == 128 && d.phi_dim == 128 && d.kernel_path == AS_PATH_TENSOR) {
     // the products on the tensor cores; the same fixed-order reductions
-    if ((e = as_bw_tensor_init()) == cudaSuccess && (e = as_bw_tensor_query(p, st)) == cudaSuccess) {
-      bw_reduce_kernel<<<rgrid, 256, 0, st>>>(p, D, 0);
-      if ((e = as_bw_tensor_key(p, st)) == cudaSuccess) bw_reduce_kernel<<<rgrid, 256, 0, st>>>(p, D, 1);
-    }
+    if ((e = as_bw_tensor_init()) == cudaSuccess && (e = as_bw_tensor_query(p, st)) == cudaSuccess && (e = reduce(0)) == cudaSuccess &&
+        (e = as_bw_tensor_key(p, st)) == cudaSuccess)
+      e = reduce(1);
   } else if (D == 64 && d.kernel_path == AS_PATH_TENSOR && aligned) {
     // the products on the tensor cores, fp32 operands in three bf16 pieces
-    if ((e = as_bw_tensor_d64_init()) == cudaSuccess && (e = as_bw_tensor_d64_query(p, st)) == cudaSuccess) {
-      bw_reduce_kernel<<<rgrid, 256, 0, st>>>(p, D, 0);
-      if ((e = as_bw_tensor_d64_key(p, st)) == cudaSuccess) bw_reduce_kernel<<<rgrid, 256, 0, st>>>(p, D, 1);
-    }
+    if ((e = as_bw_tensor_d64_init()) == cudaSuccess && (e = as_bw_tensor_d64_query(p, st)) == cudaSuccess && (e = reduce(0)) == cudaSuccess &&
+        (e = as_bw_tensor_d64_key(p, st)) == cudaSuccess)
+      e = reduce(1);
   } else if (D == 128) {
     if ((e = cudaFuncSetAttribute(bw_query_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BwSmem<128>::BYTES)) == cudaSuccess &&
         (e = cudaFuncSetAttribute(bw_key_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BwSmem<128>::BYTES)) == cudaSuccess) {

@@ -116,10 +116,6 @@ btq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
   const int tok_end = min(p.N, tok_begin + p.chunk_tokens);
   const int nt = (tok_end - tok_begin + 127) / 128;
 
-  __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
-  __syncthreads();
-  if (s_skip != 0u) return;
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
     mbar_init(bar(B_WFULL), 1); mbar_init(bar(B_FULL), 1); mbar_init(bar(B_ARDY), 1); mbar_init(bar(B_GRDY), BT_COMPUTE);
@@ -128,9 +124,18 @@ btq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     fence_proxy_async();
   }
   if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
+  griddep_launch();
+  griddep_wait();                                    // the set-up above ran beside the kernel before this one
+  // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
+  __shared__ uint32_t s_skip;
+  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (s_skip != 0u) {
+    if (warp == 16) tmem_dealloc(*tmem_slot, 512);
+    return;
+  }
   const uint32_t tmem = *tmem_slot;
   const uint32_t tA = tmem, tU = tmem + 128, tdS = tmem + 256, tdW = tmem + 384;
   const WaitCtx wc{p.status, abort_flag};
@@ -330,10 +335,6 @@ btk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
   const int tok_end = min(p.N, tok_begin + p.chunk_tokens);
   const int nt = (tok_end - tok_begin + 127) / 128;
 
-  __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
-  __syncthreads();
-  if (s_skip != 0u) return;
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
     mbar_init(bar(B_WFULL), 1); mbar_init(bar(B_FULL), 1); mbar_init(bar(B_FULL1), 1); mbar_init(bar(B_ARDY), 1);
@@ -342,9 +343,18 @@ btk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
     fence_proxy_async();
   }
   if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
+  griddep_launch();
+  griddep_wait();                                    // the set-up above ran beside the kernel before this one
+  // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
+  __shared__ uint32_t s_skip;
+  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (s_skip != 0u) {
+    if (warp == 16) tmem_dealloc(*tmem_slot, 512);
+    return;
+  }
   const uint32_t tmem = *tmem_slot;
   const uint32_t tA = tmem, tT = tmem + 128, tdW = tmem + 256;
   const WaitCtx wc{p.status, abort_flag};
@@ -466,8 +476,7 @@ cudaError_t as_bw_tensor_query(const BwParams& p, cudaStream_t st) {
       !make_map(&tmH, p.yhat, 128, p.N, BH, 128) || !make_map(&tmW, p.wq, 128, 128, p.H, 128) ||
       !make_map(&tmS, p.Sb, 128, 128, BH, 128))
     return cudaErrorInvalidValue;
-  btq_kernel<<<dim3(p.chunks, BH), BT_THREADS, BtLayout::TOTAL, st>>>(tmQ, tmY, tmH, tmW, tmS, p);
-  return cudaGetLastError();
+  return as_launch_dependent(btq_kernel, dim3(p.chunks, BH), dim3(BT_THREADS), BtLayout::TOTAL, st, tmQ, tmY, tmH, tmW, tmS, p);
 }
 
 cudaError_t as_bw_tensor_key(const BwParams& p, cudaStream_t st) {
@@ -476,6 +485,5 @@ cudaError_t as_bw_tensor_key(const BwParams& p, cudaStream_t st) {
   if (!make_map(&tmK, p.k, 128, p.N, BH, 128) || !make_map(&tmV, p.v, 128, p.N, BH, 128) ||
       !make_map(&tmW, p.wk, 128, 128, p.H, 128) || !make_map(&tmS, p.dSb, 128, 128, BH, 128))
     return cudaErrorInvalidValue;
-  btk_kernel<<<dim3(p.chunks, BH), BT_THREADS, BtLayout::TOTAL, st>>>(tmK, tmV, tmW, tmS, p);
-  return cudaGetLastError();
+  return as_launch_dependent(btk_kernel, dim3(p.chunks, BH), dim3(BT_THREADS), BtLayout::TOTAL, st, tmK, tmV, tmW, tmS, p);
 }

@@ -77,8 +77,8 @@ AS_DEV void st_shared4(uint32_t addr, const uint32_t* w) {
 // The three pieces of a [64 x 64] fp32 matrix as swizzled K-major tiles, by the 512 compute threads.
 AS_DEV void split_matrix(const float* src, uint32_t dst, int tid) {
   const int f = tid >> 3, c = tid & 7;
-  const float4 a = __ldg(reinterpret_cast<const float4*>(src + f * 64 + c * 8));
-  const float4 b = __ldg(reinterpret_cast<const float4*>(src + f * 64 + c * 8) + 1);
+  const float4 a = *reinterpret_cast<const float4*>(src + f * 64 + c * 8);
+  const float4 b = *(reinterpret_cast<const float4*>(src + f * 64 + c * 8) + 1);
   uint32_t w[3][4];
   split3(a.x, a.y, w[0][0], w[1][0], w[2][0]);
   split3(a.z, a.w, w[0][1], w[1][1], w[2][1]);
@@ -163,10 +163,6 @@ bsq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
   const int tok_end = min(p.N, tok_begin + p.chunk_tokens);
   const int nt = (tok_end - tok_begin + 127) / 128;
 
-  __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
-  __syncthreads();
-  if (s_skip != 0u) return;
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
     mbar_init(bar(Q_WFULL), 1); mbar_init(bar(Q_FULL), 1); mbar_init(bar(Q_FULL + 1), 1); mbar_init(bar(Q_GRDY), BS_COMPUTE);
@@ -175,9 +171,18 @@ bsq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     fence_proxy_async();
   }
   if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 256); tmem_relinquish(); }
+  griddep_launch();
+  griddep_wait();                                    // the set-up above ran beside the kernel before this one
+  // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
+  __shared__ uint32_t s_skip;
+  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (s_skip != 0u) {
+    if (warp == 16) tmem_dealloc(*tmem_slot, 256);
+    return;
+  }
   const uint32_t tmem = *tmem_slot;
   const uint32_t tA = tmem, tU = tmem + 64, tAcc = tmem + 128;
   const WaitCtx wc{p.status, abort_flag};
@@ -382,10 +387,6 @@ bsk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
   const int tok_end = min(p.N, tok_begin + p.chunk_tokens);
   const int nt = (tok_end - tok_begin + 127) / 128;
 
-  __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
-  __syncthreads();
-  if (s_skip != 0u) return;
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
     mbar_init(bar(K_WFULL), 1); mbar_init(bar(K_SRDY), BS_COMPUTE);
@@ -396,9 +397,18 @@ bsk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
     fence_proxy_async();
   }
   if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
+  griddep_launch();
+  griddep_wait();                                    // the set-up above ran beside the kernel before this one
+  // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
+  __shared__ uint32_t s_skip;
+  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (s_skip != 0u) {
+    if (warp == 16) tmem_dealloc(*tmem_slot, 512);
+    return;
+  }
   const uint32_t tmem = *tmem_slot;
   // per tile parity: A, T and two accumulators: lanes 0-63 of the first hold the product of the hi pieces, lanes 64-127 of
   // the mid pieces; lanes 64-127 of the second of the lo pieces (its lower half repeats the mid pieces and is not read)
@@ -534,8 +544,7 @@ cudaError_t as_bw_tensor_d64_query(const BwParams& p, cudaStream_t st) {
   if (!make_map(&tmQ, p.q, 64, p.N, BH, 128) || !make_map(&tmY, p.y, 64, p.N, BH, 128) ||
       !make_map(&tmH, p.yhat, 64, p.N, BH, 128) || !make_map(&tmW, p.wq, 64, 64, p.H, 64))
     return cudaErrorInvalidValue;
-  bsq_kernel<<<dim3(p.chunks, BH), BS_THREADS, BsqLayout::TOTAL, st>>>(tmQ, tmY, tmH, tmW, p);
-  return cudaGetLastError();
+  return as_launch_dependent(bsq_kernel, dim3(p.chunks, BH), dim3(BS_THREADS), BsqLayout::TOTAL, st, tmQ, tmY, tmH, tmW, p);
 }
 
 cudaError_t as_bw_tensor_d64_key(const BwParams& p, cudaStream_t st) {
@@ -543,6 +552,5 @@ cudaError_t as_bw_tensor_d64_key(const BwParams& p, cudaStream_t st) {
   CUtensorMap tmK, tmV, tmW;
   if (!make_map(&tmK, p.k, 64, p.N, BH, 128) || !make_map(&tmV, p.v, 64, p.N, BH, 128) || !make_map(&tmW, p.wk, 64, 64, p.H, 64))
     return cudaErrorInvalidValue;
-  bsk_kernel<<<dim3(p.chunks, BH), BS_THREADS, BskLayout::TOTAL, st>>>(tmK, tmV, tmW, p);
-  return cudaGetLastError();
+  return as_launch_dependent(bsk_kernel, dim3(p.chunks, BH), dim3(BS_THREADS), BskLayout::TOTAL, st, tmK, tmV, tmW, p);
 }

@@ -4,6 +4,7 @@
 // The SIMT kernels are the on-device cross-check of the tensor-core path: same inputs, same
 // workspace layout, every product and sum in fp32, no tensor cores, no TMA.
 #include "as_internal.h"
+#include "sm100_ptx.cuh"
 
 namespace {
 
@@ -128,6 +129,7 @@ __global__ void reduce_state_kernel(as_launch_args a) {
 }
 
 __global__ void round_state_kernel(const float* S, __nv_bfloat16* Sb, size_t n) {
+  sm100::griddep_launch();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) Sb[i] = __float2bfloat16_rn(S[i]);
 }

@@ -72,6 +72,13 @@ AS_DEV bool mbar_wait_warp(uint32_t bar, uint32_t parity, const WaitCtx& w) {
   return __all_sync(0xffffffffu, ok);
 }
 
+// ---------------------------------------------------------------- dependent launches
+// A kernel launched by as_launch_dependent may start while the kernel before it in the stream is still running, once
+// every CTA of that one has called griddep_launch or ended.  griddep_wait returns when that kernel has completed and
+// its writes are visible: no access to global memory comes before it.
+AS_DEV void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+AS_DEV void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------- TMA
 AS_DEV void tma_prefetch_desc(const CUtensorMap* m) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");

@@ -103,6 +103,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   const WaitCtx wc{p.status, abort_flag};
   const bool gathers = (p.ks_w != nullptr) && fc == 0;       // this CTA copies the softmax rows out
 
+  griddep_launch();                                          // the query stage's CTAs may set up as these ones end
   __shared__ uint32_t s_skip;
   if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
   __syncthreads();

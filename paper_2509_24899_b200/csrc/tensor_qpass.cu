@@ -927,11 +927,6 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   const int warp = threadIdx.x >> 5;
   __shared__ float sDl[2 * 128];                     // per group and row: share of phi_q . z, then the denominator
 
-  __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
-  __syncthreads();
-  if (s_skip != 0u) return;
-
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
     mbar_init(bar(R::B_Q0), 1); mbar_init(bar(R::B_Q0 + 1), 1);
@@ -945,9 +940,18 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     fence_proxy_async();
   }
   if (warp == 17) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
+  griddep_launch();
+  griddep_wait();                                    // the set-up above ran beside the kernel before this one
+  // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
+  __shared__ uint32_t s_skip;
+  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (s_skip != 0u) {
+    if (warp == 17) tmem_dealloc(*tmem_slot, 512);
+    return;
+  }
   const QCtx c{sbase, *tmem_slot, WaitCtx{p.status, abort_flag}};
   const int n_mine = q_units_of_cta(p);
 
@@ -994,12 +998,6 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   auto bar = [&](int i) { return sbase + L::BAR_OFF + 8 * i; };
   const int warp = threadIdx.x >> 5;
 
-  // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
-  __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
-  __syncthreads();
-  if (s_skip != 0u) return;
-
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
     mbar_init(bar(R::B_Q0), 1); mbar_init(bar(R::B_Q0 + 1), 1);
@@ -1013,9 +1011,18 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     fence_proxy_async();
   }
   if (warp == 9) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
+  griddep_launch();
+  griddep_wait();                                    // the set-up above ran beside the kernel before this one
+  // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
+  __shared__ uint32_t s_skip;
+  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (s_skip != 0u) {
+    if (warp == 9) tmem_dealloc(*tmem_slot, 512);
+    return;
+  }
   const QCtx c{sbase, *tmem_slot, WaitCtx{p.status, abort_flag}};
   const int n_mine = q_units_of_cta(p);               // units of this CTA
 
@@ -1134,17 +1141,14 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   const bool gen = lin && (a.P > 2 || p.b1 != nullptr || p.b2 != nullptr);
   if (p.nkv == 0 && lin && !two) {
     // no softmax tokens, one-layer map: the variant with sixteen compute warps
-    if (a.d == 128) {
-      if (gen) qlin_kernel<128, true><<<grid, QL_THREADS, QLayout<128>::TOTAL, st>>>(tmQ, tmW, tmSt, tmO, p);
-      else qlin_kernel<128, false><<<grid, QL_THREADS, QLayout<128>::TOTAL, st>>>(tmQ, tmW, tmSt, tmO, p);
-    } else {
-      if (gen) qlin_kernel<64, true><<<grid, QL_THREADS, QLayout<64>::TOTAL, st>>>(tmQ, tmW, tmSt, tmO, p);
-      else qlin_kernel<64, false><<<grid, QL_THREADS, QLayout<64>::TOTAL, st>>>(tmQ, tmW, tmSt, tmO, p);
-    }
-    return cudaGetLastError();
+#define AS_LAUNCH_QL(D_, GEN_) \
+  return as_launch_dependent(qlin_kernel<D_, GEN_>, grid, dim3(QL_THREADS), QLayout<D_>::TOTAL, st, tmQ, tmW, tmSt, tmO, p)
+    if (a.d == 128) { if (gen) AS_LAUNCH_QL(128, true); else AS_LAUNCH_QL(128, false); }
+    if (gen) AS_LAUNCH_QL(64, true); else AS_LAUNCH_QL(64, false);
+#undef AS_LAUNCH_QL
   }
 #define AS_LAUNCH_Q(D_, TWO_, GEN_) \
-  qpass_kernel<D_, TWO_, GEN_><<<grid, Q_THREADS, QLayout<D_>::TOTAL, st>>>(tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO, p)
+  return as_launch_dependent(qpass_kernel<D_, TWO_, GEN_>, grid, dim3(Q_THREADS), QLayout<D_>::TOTAL, st, tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO, p)
   if (a.d == 128) {
     if (two) { if (gen) AS_LAUNCH_Q(128, true, true); else AS_LAUNCH_Q(128, true, false); }
     else { if (gen) AS_LAUNCH_Q(128, false, true); else AS_LAUNCH_Q(128, false, false); }
@@ -1153,5 +1157,4 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
     else { if (gen) AS_LAUNCH_Q(64, false, true); else AS_LAUNCH_Q(64, false, false); }
   }
 #undef AS_LAUNCH_Q
-  return cudaGetLastError();
 }

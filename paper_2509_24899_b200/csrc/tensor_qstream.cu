@@ -218,12 +218,6 @@ qstream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + QSLayout::BAR_OFF + 8 * B_COUNT + 4);
   const int warp = threadIdx.x >> 5;
 
-  // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
-  __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
-  __syncthreads();
-  if (s_skip != 0u) return;
-
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
     auto bar = [&](int i) { return sbase + QSLayout::BAR_OFF + 8 * i; };
@@ -237,9 +231,18 @@ qstream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     fence_proxy_async();
   }
   if (warp == 9) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
+  griddep_launch();
+  griddep_wait();                                    // the set-up above ran beside the kernel before this one
+  // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
+  __shared__ uint32_t s_skip;
+  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (s_skip != 0u) {
+    if (warp == 9) tmem_dealloc(*tmem_slot, 512);
+    return;
+  }
   // Every CTA gets a contiguous run of tiles.  With at least as many CTAs as (batch, head) pairs no run crosses a
   // pair (a change of pair stalls the pipeline while W and S are replaced): the pairs get floor or ceil(G / pairs)
   // CTAs each, which share the pair's tiles evenly.  Otherwise the tiles of all pairs are cut into G near-equal runs.
@@ -303,6 +306,5 @@ cudaError_t as_tensor_qstream(const as_launch_args& a, cudaStream_t st) {
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
     return cudaErrorInvalidValue;
   const dim3 grid((unsigned)(p.tiles < sms ? p.tiles : sms), 1, 1);   // persistent: one CTA per SM
-  qstream_kernel<<<grid, QS_THREADS, QSLayout::TOTAL, st>>>(tmQ, tmW, tmSt, tmO, p);
-  return cudaGetLastError();
+  return as_launch_dependent(qstream_kernel, grid, dim3(QS_THREADS), QSLayout::TOTAL, st, tmQ, tmW, tmSt, tmO, p);
 }
