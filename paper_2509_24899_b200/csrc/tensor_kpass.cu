@@ -370,7 +370,9 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   // a (batch, head, feature chunk) takes a slice of the [F x (D + 1)] entries once all of them have stored theirs.
   // The CTAs of one launch are resident together (one per SM, a cooperative launch when there is more than one
   // chunk), so the wait ends; it is bounded like every other wait.  The second counter tells the last CTA to finish
-  // its slice that both counters can go back to zero for the next launch.
+  // its slice that both counters can go back to zero for the next launch.  This is a chain of L2 round trips: the loads of all
+  // chunks at once instead of four by four, and no sleep between two looks at the counter, took N = 7800 from 87.5 to 86.3 us
+  // and N = 1024 with 2 heads from 19.5 to 18.5 us.
   __shared__ uint32_t s_go;
   uint32_t* cnt = p.counters + 2 * ((size_t)bh * gridDim.z + fc);
   const uint32_t n_ctas = gridDim.x;
@@ -380,14 +382,12 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     uint32_t go = 1u, it = 0;
     long long t0 = 0;
     while (*reinterpret_cast<volatile uint32_t*>(cnt) < n_ctas) {
-      __nanosleep(100);
-      if ((++it & 63u) == 0u) {
-        const long long now = clock64();
-        if (t0 == 0) t0 = now;
-        if (*abort_flag != 0u || now - t0 > kWaitLimitCycles) { atomicOr(p.status, 1u); go = 0u; break; }
-      }
-      // a CTA that found the status word set never arrives: the others stop waiting as soon as they see it too
+      if ((++it & 15u) != 0u) continue;                        // a look at the counter is a round trip to L2: no need to sleep between
+      // a CTA that found the status word set never arrives: the others stop waiting when they see it too
       if (*reinterpret_cast<volatile uint32_t*>(p.status) != 0u) { go = 0u; break; }
+      const long long now = clock64();
+      if (t0 == 0) t0 = now;
+      if (*abort_flag != 0u || now - t0 > kWaitLimitCycles) { atomicOr(p.status, 1u); go = 0u; break; }
     }
     s_go = go;
   }
@@ -405,16 +405,14 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     for (int i = chunk * per + (int)threadIdx.x; i < i_end; i += K_THREADS) {
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
       int c = 0;
-      for (; c + 4 <= p.n_chunks; c += 4) {                    // four chunks' loads in flight, added in chunk order
-        float4 v[4];
+      for (; c < p.n_chunks; c += 12) {                        // up to twelve chunks' loads in flight, added in chunk order
+        float4 v[12];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) v[j] = __ldcg(reinterpret_cast<const float4*>(src + (c + j) * pitch) + i);
+        for (int j = 0; j < 12; ++j)
+          if (c + j < p.n_chunks) v[j] = __ldcg(reinterpret_cast<const float4*>(src + (c + j) * pitch) + i);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) { acc.x += v[j].x; acc.y += v[j].y; acc.z += v[j].z; acc.w += v[j].w; }
-      }
-      for (; c < p.n_chunks; ++c) {
-        const float4 v = __ldcg(reinterpret_cast<const float4*>(src + c * pitch) + i);
-        acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+        for (int j = 0; j < 12; ++j)
+          if (c + j < p.n_chunks) { acc.x += v[j].x; acc.y += v[j].y; acc.z += v[j].z; acc.w += v[j].w; }
       }
       reinterpret_cast<float4*>(dS)[i] = acc;
       reinterpret_cast<uint2*>(dSb)[i] = make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
@@ -422,7 +420,14 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     if (chunk == 0) {
       for (int f = threadIdx.x; f < nf; f += K_THREADS) {
         float acc = 0.f;
-        for (int c = 0; c < p.n_chunks; ++c) acc += __ldcg(p.part_z + ((size_t)bh * p.n_chunks + c) * p.F + f0 + f);
+        for (int c = 0; c < p.n_chunks; c += 12) {
+          float v[12];
+#pragma unroll
+          for (int j = 0; j < 12; ++j) v[j] = c + j < p.n_chunks ? __ldcg(p.part_z + ((size_t)bh * p.n_chunks + c + j) * p.F + f0 + f) : 0.f;
+#pragma unroll
+          for (int j = 0; j < 12; ++j)
+            if (c + j < p.n_chunks) acc += v[j];
+        }
         p.z[(size_t)bh * p.F + f0 + f] = acc;
       }
     }
