@@ -150,6 +150,46 @@ def test_narrow_head_gradient_has_the_precision_of_the_cuda_core_kernels(shape, 
         assert abs(loss.item() - diff.abs().sum().item()) <= 1e-5 * diff.abs().sum().item()
 
 
+# less than a tile of 64, whole tiles, one row more, an odd number of tiles, more tiles a chunk than the ring has slots; every power
+@pytest.mark.parametrize("B,H,N,rate,degree,mode", [(1, 1, 40, 2, 2, O.STAB_PAPER), (1, 2, 64, 0, 1, O.STAB_PAPER), (1, 2, 65, 4, 4, O.STAB_EXACT),
+                                                    (1, 3, 192, 3, 2, O.STAB_EXACT), (2, 75, 700, 4, 4, O.STAB_PAPER), (1, 150, 321, 0, 2, O.STAB_PAPER)])
+def test_gradient_at_the_edges_of_tiles(B, H, N, rate, degree, mode):
+    """d = 128: the tensor-core kernels next to the fp32 ones on the same y_hat, row statistics and state.  Their operands g, lambda phi_q,
+    dL/da, S, dS are rounded to bf16 (2^-9 each, at random): 2e-3 to 4e-3 in relative L2; 6e-3 asserted."""
+    import torch
+    from paper_2509_24899_b200 import HybridAttention, binding
+    wl = W.Workload("bw_edges", B=B, H=H, d=128, F=128, grid=(1, 1, N), block=(1, 1, N), rate=rate, seed=68, degree=degree)
+    dev = {k: to_cuda_bf16(v) for k, v in W.generate(wl, wq_gain=2e-3 if rate else 1.0).items()}
+    y = to_cuda_bf16(W.teacher_output(wl))
+    ops = [HybridAttention.from_workload(wl, stab_mode=mode) for _ in range(2)]
+    aux = torch.empty((B, H, N, 3), dtype=torch.float32, device="cuda")
+    args = [dev[n] for n in ("q", "k", "v", "wq", "wk")]
+    y_hat = ops[0].forward(*args, aux=aux)
+    got = ops[0].backward_phi(*args, y, y_hat, aux)
+    S, z = (x.double() for x in ops[0].linear_state())
+    assert ops[0].last_status() == 0
+    q, k, v, wq, wk = (x.double() for x in args)
+    power = torch.arange(128, device="cuda") // (128 // degree)
+
+    def phi(x, w):
+        a = x @ w.transpose(-1, -2)
+        return a.relu() ** (power + 1), (a > 0) * (power + 1) * a.relu() ** power
+
+    lam = torch.exp(-aux[..., 0].double()) if mode == O.STAB_EXACT and rate else torch.ones_like(aux[..., 0], dtype=torch.float64)
+    w = (lam / (aux[..., 1].double() + lam * aux[..., 2].double()))[..., None]
+    diff = y_hat.double() - y.double()
+    G = diff.sign()
+    t = -(G * y_hat.double()).sum(-1, keepdim=True)
+    phi_q, slope_q = phi(q, wq)
+    dwq = ((w * (G @ S.transpose(-1, -2) + z[:, :, None] * t) * slope_q).transpose(-1, -2) @ q).sum(0)
+    dS, dz = (w * phi_q).transpose(-1, -2) @ G, (w * phi_q * t).sum(2)
+    linear = torch.from_numpy(~oracle_mask(wl)).cuda()[:, None]
+    dwk = (((v @ dS.transpose(-1, -2) + dz[:, :, None]) * phi(k, wk)[1] * linear).transpose(-1, -2) @ k).sum(0)
+    for a, r in ((got[0], dwq), (got[1], dwk)):
+        assert float((a.double() - r).norm() / r.norm()) <= 6e-3
+    assert abs(got[2].item() - diff.abs().sum().item()) <= 1e-5 * diff.abs().sum().item()
+
+
 def test_backward_argument_errors_and_zero_gradient_without_linear_tokens():
     import torch
     from paper_2509_24899_b200 import HybridAttention, binding, AsError
