@@ -20,50 +20,10 @@ namespace {
 using namespace as_tc;
 
 constexpr int BT_COMPUTE = 512;          // warps 0-15
-constexpr int BT_THREADS = BT_COMPUTE + 32;   // key side: row = thread % 128, column quarter = thread / 128; warp 16: TMA + MMA issue (lane 0)
 constexpr int TILE = 128 * 128 * 2;      // bytes of a [128 x 128] bf16 tile
-constexpr uint32_t ID_KK = make_idesc(128, 128, 0, 0);      // both operands K-major
-constexpr uint32_t ID_MM = make_idesc(128, 128, 1, 1);      // both operands MN-major (token rows are the K index)
 
-// barriers of the key side (per-tile ones are used once per tile: phase = tile index; B_FULL: one per K/V set)
-constexpr int B_WFULL = 0, B_FULL = 1, B_FULL1 = 2, B_ARDY = 3, B_PRDY = 4, B_DONE = 5, B_COUNT = 6;
-
-// Key side: K and V tiles of 128 tokens in two sets, one tile's products issued while the next tile arrives.
-struct BtLayout {
-  static constexpr int W_OFF = 0;                 // W_k [F][d]
-  static constexpr int S_OFF = TILE;              // dS in bf16 [F][d]
-  static constexpr int X_OFF = 2 * TILE;          // K tile of the even set
-  static constexpr int Y_OFF = 3 * TILE;          // V tile of the even set, then dL/da_k in place
-  static constexpr int H_OFF = 4 * TILE;          // K tile of the odd set
-  static constexpr int A_OFF = 5 * TILE;          // V tile of the odd set, then dL/da_k in place
-  static constexpr int BAR_OFF = 6 * TILE;
-  static constexpr int ZVEC_OFF = BAR_OFF + 128;  // 128 floats: dz
-  static constexpr int TOTAL = ZVEC_OFF + 512 + 1024;   // + slack for the 1024-byte alignment
-};
-
-// phi = r^p and its slope p r^(p-1) for r = relu(a); the power is a compile-time constant (a thread's 32 features
-// belong to one part of the feature map)
-template <int PW>
-AS_DEV void bt_poly(float a, float& phi, float& slope) {
-  const float r = fmaxf(a, 0.f);
-  float rp1 = 1.f;                                // r^(p-1)
-#pragma unroll
-  for (int i = 1; i < PW; ++i) rp1 *= r;
-  phi = rp1 * r;
-  slope = a > 0.f ? (float)PW * rp1 : 0.f;
-}
-// Key side, 32 features of one row: dL/da_k = (T + dz) phi' on linear tokens, zero on softmax tokens.
-template <int PW>
-AS_DEV void bt_k_features(const uint32_t (&xa)[32], const uint32_t (&xt)[32], const float* zv, bool lin, uint32_t (&wa)[16]) {
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    float ph0, sl0, ph1, sl1;
-    bt_poly<PW>(__uint_as_float(xa[2 * i]), ph0, sl0);
-    bt_poly<PW>(__uint_as_float(xa[2 * i + 1]), ph1, sl1);
-    const float t0 = (__uint_as_float(xt[2 * i]) + zv[2 * i]) * sl0, t1 = (__uint_as_float(xt[2 * i + 1]) + zv[2 * i + 1]) * sl1;
-    wa[i] = lin ? pack_bf16(t0, t1) : 0u;
-  }
-}
+AS_DEV float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
+AS_DEV float bf_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 AS_DEV uint32_t sub_bf16x2(uint32_t a, uint32_t b) {
   uint32_t r;
   asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
@@ -75,8 +35,6 @@ AS_DEV uint32_t ne_bf16x2(uint32_t a, uint32_t b) {
   asm("set.neu.u32.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
   return r;
 }
-AS_DEV float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
-AS_DEV float bf_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
 // Writes 32 columns of one accumulator row (TMEM lane = feature row) to dst.
 AS_DEV void bt_store_acc(uint32_t tacc, float* dst) {
@@ -420,27 +378,64 @@ btq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
 }
 
 // ---------------------------------------------------------------------------------------------- key side
-__global__ void __launch_bounds__(BT_THREADS, 1)
+// As the query side: A^T = W_k K^T and T^T = dS V^T with TMEM lane = feature, dL/da_k written back over A^T as packed bf16,
+// dW_k += (dL/da_k)^T K with that as the A operand.  Two groups of eight warps take turns at the tiles, each with columns
+// of its own.  (Before: 128-token tiles, all sixteen warps on one, dL/da_k through shared memory.  Whole gradient 136.9 -> 130.5
+// us at the headline shape, 63.1 -> 61.9 at N = 7800.)
+struct BtkLayout {
+  static constexpr int QTILE = BtqLayout::QTILE;
+  static constexpr int SLOTS = 5;
+  static constexpr int W_OFF = 0;                 // W_k [F][d]
+  static constexpr int S_OFF = TILE;              // dS in bf16 [F][d]
+  static constexpr int KV_OFF = 2 * TILE;         // ring of [k | v]
+  static constexpr int BAR_OFF = KV_OFF + SLOTS * 2 * QTILE;
+  static constexpr int TOTAL = BAR_OFF + 192;     // (the array is aligned to 1024 bytes)
+};
+enum { K_WFULL = 0, K_FULL = 1, K_AT = K_FULL + BtkLayout::SLOTS, K_PRDY = K_AT + 2, K_DONE = K_PRDY + 2, K_END = K_DONE + BtkLayout::SLOTS, K_BARS };
+constexpr int BTK_THREADS = BT_COMPUTE + 64;      // warps 0-15: features; 16: MMA issue; 17: loads
+
+// One feature of 32 tokens: dL/da_k = (T + dz) phi' on linear tokens (bits of `linear`), zero on the others.
+template <int PW>
+AS_DEV void btk_features(const uint32_t (&xa)[32], const uint32_t (&xt)[32], float dz, uint32_t linear, uint32_t (&wa)[16]) {
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const float a0 = __uint_as_float(xa[2 * i]), a1 = __uint_as_float(xa[2 * i + 1]);
+    float2 t = __fadd2_rn(make_float2(__uint_as_float(xt[2 * i]), __uint_as_float(xt[2 * i + 1])), make_float2(dz, dz));
+    if (PW == 1) {
+      t = make_float2(a0 > 0.f ? t.x : 0.f, a1 > 0.f ? t.y : 0.f);
+    } else {
+      const float2 r = make_float2(fmaxf(a0, 0.f), fmaxf(a1, 0.f));
+      float2 rp = r;                                 // r^(p-1)
+#pragma unroll
+      for (int e = 2; e < PW; ++e) rp = __fmul2_rn(rp, r);
+      t = __fmul2_rn(__fmul2_rn(t, rp), make_float2((float)PW, (float)PW));
+    }
+    wa[i] = pack_bf16((linear >> (2 * i)) & 1u ? t.x : 0.f, (linear >> (2 * i + 1)) & 1u ? t.y : 0.f);
+  }
+}
+
+__global__ void __launch_bounds__(BTK_THREADS, 1)
 btk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmW,
            const __grid_constant__ CUtensorMap tmS, const __grid_constant__ BwParams p) {
-  using L = BtLayout;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  using L = BtkLayout;
+  extern __shared__ __align__(1024) uint8_t btq_smem[];
+  uint8_t* smem = btq_smem;
   const uint32_t sbase = smem_u32(smem);
   auto bar = [&](int i) { return sbase + L::BAR_OFF + 8 * i; };
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::BAR_OFF + 8 * B_COUNT);
-  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::BAR_OFF + 8 * B_COUNT + 4);
-  float* zvec = reinterpret_cast<float*>(smem + L::ZVEC_OFF);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::BAR_OFF + 8 * K_BARS);
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::BAR_OFF + 8 * K_BARS + 4);
+  volatile uint32_t* skip = reinterpret_cast<volatile uint32_t*>(smem + L::BAR_OFF + 8 * K_BARS + 8);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bh = blockIdx.y, chunk = blockIdx.x, h = bh % p.H;
   const int tok_begin = chunk * p.chunk_tokens;
   const int tok_end = min(p.N, tok_begin + p.chunk_tokens);
-  const int nt = (tok_end - tok_begin + 127) / 128;
+  const int nt = (tok_end - tok_begin + 63) / 64;
 
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
-    mbar_init(bar(B_WFULL), 1); mbar_init(bar(B_FULL), 1); mbar_init(bar(B_FULL1), 1); mbar_init(bar(B_ARDY), 1);
-    mbar_init(bar(B_PRDY), BT_COMPUTE); mbar_init(bar(B_DONE), 1);
+    mbar_init(bar(K_WFULL), 1); mbar_init(bar(K_END), 1);
+    for (int i = 0; i < L::SLOTS; ++i) { mbar_init(bar(K_FULL + i), 1); mbar_init(bar(K_DONE + i), 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(bar(K_AT + i), 1); mbar_init(bar(K_PRDY + i), 256); }
     fence_barrier_init();
     fence_proxy_async();
   }
@@ -448,109 +443,109 @@ btk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
   griddep_launch();
   griddep_wait();                                    // the set-up above ran beside the kernel before this one
   // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
-  __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (threadIdx.x == 0) *skip = *reinterpret_cast<volatile uint32_t*>(p.status);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (s_skip != 0u) {
+  if (*skip != 0u) {
     if (warp == 16) tmem_dealloc(*tmem_slot, 512);
     return;
   }
   const uint32_t tmem = *tmem_slot;
-  const uint32_t tA = tmem, tT = tmem + 128, tdW = tmem + 256;
   const WaitCtx wc{p.status, abort_flag};
+  auto slot_off = [&](int t) { return L::KV_OFF + (t % L::SLOTS) * 2 * L::QTILE; };
+  bool ok = true;
 
-  if (warp == 16) {
+  if (warp == 17) {
     if (lane == 0) {
-      tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
-      mbar_expect_tx(bar(B_WFULL), 2 * TILE);
-      load_tile<128>(sbase + L::W_OFF, &tmW, bar(B_WFULL), 0, h);
-      load_tile<128>(sbase + L::S_OFF, &tmS, bar(B_WFULL), 0, bh);
-      // K and V tiles are double-buffered: tile t lives in set t & 1 (its own "full" barrier), and the tile after the
-      // next is requested as soon as the last product that reads the set has completed
-      auto sK = [&](int t) { return sbase + ((t & 1) ? L::H_OFF : L::X_OFF); };
-      auto sVt = [&](int t) { return sbase + ((t & 1) ? L::A_OFF : L::Y_OFF); };
-      auto full = [&](int t) { return bar((t & 1) ? B_FULL1 : B_FULL); };
-      auto request = [&](int t) {
-        mbar_expect_tx(full(t), 2 * TILE);
-        load_tile<128>(sK(t), &tmK, full(t), tok_begin + t * 128, bh);
-        load_tile<128>(sVt(t), &tmV, full(t), tok_begin + t * 128, bh);
+      auto load = [&](uint32_t dst, const CUtensorMap* m, uint32_t fb, int t) {
+        tma_load_3d(dst, m, fb, 0, tok_begin + t * 64, bh);
+        tma_load_3d(dst + BtqLayout::QBOX, m, fb, 64, tok_begin + t * 64, bh);
       };
-      auto first_products = [&](int t) {           // A = K W_k^T and T = V dS^T of tile t
-        tc_fence_after();
-        issue_kmajor<128>(tA, kmajor_desc(sK(t)), kmajor_desc(sbase + L::W_OFF), ID_KK, false);
-        issue_kmajor<128>(tT, kmajor_desc(sVt(t)), kmajor_desc(sbase + L::S_OFF), ID_KK, false);
-        tc_commit(bar(B_ARDY));
-      };
-      bool ok = nt > 0;
-      if (ok) {
-        request(0);
-        if (nt > 1) request(1);
-        ok = mbar_wait(bar(B_WFULL), 0, wc) && mbar_wait(full(0), 0, wc);
-        if (ok) first_products(0);
-      }
-      for (int t = 0; t < nt && ok; ++t) {
-        if (!mbar_wait(bar(B_PRDY), t & 1, wc)) break;                   // dL/da_k of tile t is in shared memory (over V)
-        tc_fence_after();
-        const uint64_t aD = mnmajor_desc(sVt(t)), bK = mnmajor_desc(sK(t));
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) mma_ss(tdW, aD + kstep_mnmajor(kk), bK + kstep_mnmajor(kk), ID_MM, (t > 0 || kk > 0) ? 1u : 0u);
-        tc_commit(bar(B_DONE));
-        // the threads have read A and T of tile t (they arrived on the barrier above): the next tile's may land
-        if (t + 1 < nt) {
-          if (!mbar_wait(full(t + 1), ((t + 1) >> 1) & 1, wc)) break;
-          first_products(t + 1);
-        }
-        if (t + 2 < nt) {
-          if (!mbar_wait(bar(B_DONE), t & 1, wc)) break;                 // the set of tile t is free
-          request(t + 2);
-        }
+      mbar_expect_tx(bar(K_WFULL), 2 * TILE);
+      load_tile<128>(sbase + L::W_OFF, &tmW, bar(K_WFULL), 0, h);
+      load_tile<128>(sbase + L::S_OFF, &tmS, bar(K_WFULL), 0, bh);
+      for (int t = 0; t < nt; ++t) {
+        const uint32_t fb = bar(K_FULL + t % L::SLOTS), dst = sbase + slot_off(t);
+        // (the product of the tile that had the slot has read it)
+        if (t >= L::SLOTS && !mbar_wait(bar(K_DONE + t % L::SLOTS), (t / L::SLOTS - 1) & 1, wc)) break;
+        mbar_expect_tx(fb, 2 * L::QTILE);
+        load(dst, &tmK, fb, t);
+        load(dst + L::QTILE, &tmV, fb, t);
       }
     }
     __syncwarp();
+  } else if (warp == 16) {
+    const uint32_t sb = __shfl_sync(0xffffffffu, sbase, 0), tm = __shfl_sync(0xffffffffu, tmem, 0);
+    // A^T and T^T of tile t over columns whose features the product of tile t - 2 reads: that was issued before (one
+    // thread's products complete in order), and the threads had read the A^T and T^T of that tile
+    auto first_products = [&](int t) -> bool {
+      const uint32_t sK = sb + slot_off(t), tAT = tm + (t & 1) * 128u;
+      if (!mbar_wait_warp(bar(K_FULL + t % L::SLOTS), (t / L::SLOTS) & 1, wc)) return false;
+      tc_fence_after();
+      if (elect_one()) {
+        btq_issue_tokens(tAT, sb + L::W_OFF, sK);
+        btq_issue_tokens(tAT + 64, sb + L::S_OFF, sK + L::QTILE);
+        tc_commit(bar(K_AT + (t & 1)));
+      }
+      return true;
+    };
+    ok = mbar_wait_warp(bar(K_WFULL), 0, wc) && first_products(0) && (nt < 2 || first_products(1));
+    for (int t = 0; t < nt && ok; ++t) {
+      if (!mbar_wait_warp(bar(K_PRDY + (t & 1)), (t >> 1) & 1, wc)) break;
+      tc_fence_after();
+      if (elect_one()) {
+        btq_issue_grad(tm + 256, tm + (t & 1) * 128u, sb + slot_off(t), t > 0);   // dW_k += (dL/da_k)^T K
+        tc_commit(bar(K_DONE + t % L::SLOTS));
+        if (t == nt - 1) tc_commit(bar(K_END));
+      }
+      if (t + 2 < nt && !first_products(t + 2)) break;
+    }
   } else {
-    const int r = threadIdx.x & 127, qt = threadIdx.x >> 7;
+    const int r = threadIdx.x & 127, cg = threadIdx.x >> 7;    // feature (= TMEM lane); tile group and token group: cg = 2 * group + tokens
+    const int grp = cg >> 1, tg = cg & 1;
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
-    const int part = 128 / p.P;
-    if (qt == 0) zvec[r] = p.dz[(size_t)bh * 128 + r];
-    named_barrier_sync(1, BT_COMPUTE);
-    bool ok = true;
-    auto is_linear = [&](int t) { const int n = tok_begin + t * 128 + r; return t < nt && n < tok_end && p.sm_rank[n] < 0; };
-    bool lin_next = is_linear(0);                    // fetched one tile ahead
-    for (int t = 0; t < nt; ++t) {
-      uint8_t* sV = smem + ((t & 1) ? L::A_OFF : L::Y_OFF);      // the V tile of the set tile t lives in
-      const bool lin_c = lin_next;
-      lin_next = is_linear(t + 1);
-      if (ok) ok = mbar_wait_warp(bar(B_ARDY), t & 1, wc);
-      const bool lin = ok && lin_c;
+    const int pw = min(((warp & 3) * 32) / (128 / p.P), p.P - 1) + 1;    // power of this warp's features
+    const uint32_t tA = tmem + grp * 128u, tT = tA + 64;
+    const float dz = p.dz[(size_t)bh * 128 + r];
+    // which of the tile's 32 tokens are linear tokens, fetched a turn ahead
+    auto linear_tokens = [&](int t) {
+      const int n = tok_begin + t * 64 + tg * 32 + lane;
+      return __ballot_sync(0xffffffffu, t < nt && n < tok_end && p.sm_rank[n] < 0);
+    };
+    uint32_t lin_next = linear_tokens(grp);
+    for (int t = grp; t < nt; t += 2) {
+      const uint32_t lin = lin_next;
+      lin_next = linear_tokens(t + 2);
+      if (ok) ok = mbar_wait_warp(bar(K_AT + grp), (t >> 1) & 1, wc);
+      uint32_t wa[16];
       if (ok) {
         tc_fence_after();
         uint32_t xa[32], xt[32];
-        const int cc = qt;                           // this thread's 32 features
-        tmem_ld32(tA + lane_off + cc * 32, xa);
-        tmem_ld32(tT + lane_off + cc * 32, xt);
+        tmem_ld32(tA + lane_off + tg * 32, xa);
+        tmem_ld32(tT + lane_off + tg * 32, xt);
         tmem_ld_wait(xa);
         tmem_ld_wait(xt);
-        const int pw = min((cc * 32) / part, p.P - 1) + 1;
-        uint32_t wa[16];
         switch (pw) {
-          case 1: bt_k_features<1>(xa, xt, zvec + cc * 32, lin, wa); break;
-          case 2: bt_k_features<2>(xa, xt, zvec + cc * 32, lin, wa); break;
-          case 3: bt_k_features<3>(xa, xt, zvec + cc * 32, lin, wa); break;
-          default: bt_k_features<4>(xa, xt, zvec + cc * 32, lin, wa); break;
+          case 1: btk_features<1>(xa, xt, dz, lin, wa); break;
+          case 2: btk_features<2>(xa, xt, dz, lin, wa); break;
+          case 3: btk_features<3>(xa, xt, dz, lin, wa); break;
+          default: btk_features<4>(xa, xt, dz, lin, wa); break;
         }
-        store_row_chunk(sV, r, cc * 32, wa);         // dL/da_k over v (the product that read v has completed)
+      }
+      named_barrier_sync(2 + (warp & 3) + 4 * grp, 64);        // both token groups of these lanes have read A^T
+      if (ok) {
+        tmem_st16(tA + lane_off + tg * 16, wa);
+        tmem_st_wait();
         tc_fence_before();
       }
-      fence_proxy_async();
-      mbar_arrive(bar(B_PRDY));
+      mbar_arrive(bar(K_PRDY + grp));
     }
-    if (ok && nt > 0) ok = mbar_wait_warp(bar(B_DONE), (nt - 1) & 1, wc);
+    if (ok && nt > 0) ok = mbar_wait_warp(bar(K_END), 0, wc);
     if (ok && nt > 0) {
       tc_fence_after();
       const size_t slot = (size_t)bh * p.chunks + chunk;
-      bt_store_acc(tdW + lane_off + qt * 32, p.part_dW + (slot * 128 + r) * 128 + qt * 32);
+      bt_store_acc(tmem + 256 + lane_off + cg * 32, p.part_dW + (slot * 128 + r) * 128 + cg * 32);
       tc_fence_before();
     }
   }
@@ -568,7 +563,7 @@ btk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
 cudaError_t as_bw_tensor_init() {
   cudaError_t e;
   if ((e = opt_in_smem(btq_kernel, BtqLayout::TOTAL)) != cudaSuccess) return e;
-  return opt_in_smem(btk_kernel, BtLayout::TOTAL);
+  return opt_in_smem(btk_kernel, BtkLayout::TOTAL);
 }
 
 cudaError_t as_bw_tensor_query(const BwParams& p, cudaStream_t st) {
@@ -584,8 +579,8 @@ cudaError_t as_bw_tensor_query(const BwParams& p, cudaStream_t st) {
 cudaError_t as_bw_tensor_key(const BwParams& p, cudaStream_t st) {
   const int BH = p.B * p.H;
   CUtensorMap tmK, tmV, tmW, tmS;
-  if (!make_map(&tmK, p.k, 128, p.N, BH, 128) || !make_map(&tmV, p.v, 128, p.N, BH, 128) ||
+  if (!make_map(&tmK, p.k, 128, p.N, BH, 64) || !make_map(&tmV, p.v, 128, p.N, BH, 64) ||
       !make_map(&tmW, p.wk, 128, 128, p.H, 128) || !make_map(&tmS, p.dSb, 128, 128, BH, 128))
     return cudaErrorInvalidValue;
-  return as_launch_dependent(btk_kernel, dim3(p.chunks, BH), dim3(BT_THREADS), BtLayout::TOTAL, st, tmK, tmV, tmW, tmS, p);
+  return as_launch_dependent(btk_kernel, dim3(p.chunks, BH), dim3(BTK_THREADS), BtkLayout::TOTAL, st, tmK, tmV, tmW, tmS, p);
 }
