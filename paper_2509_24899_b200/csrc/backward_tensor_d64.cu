@@ -368,7 +368,12 @@ struct BskLayout {
   static constexpr int Z_OFF = BAR_OFF + 128;               // 64 floats: dz
   static constexpr int TOTAL = Z_OFF + 256 + 1024;
 };
-enum { K_WFULL = 0, K_SRDY = 1, K_FULL = 2, K_AT = 5, K_XRDY = 7, K_DONE = 8, K_BARS = 10 };
+// Who has passed what before a barrier can complete again (a wait that looks after two more phases would not see its own).  The
+// compute threads can be a tile ahead of the issuing lane: for tile t + 1 they need AT(t + 1) and DONE(t - 1), both from before
+// the lane looks at XRDY(t).  So XRDY is one barrier per tile parity: arriving for tile t + 2 needs AT(t + 2), which the lane
+// issues only after it has passed XRDY(t).  AT(t + 2) and DONE(t + 2) come after XRDY(t + 1) and XRDY(t + 2), where every thread
+// has passed AT(t) and DONE(t); FULL(t + 3) is requested after DONE(t), whose products the lane issued after FULL(t).
+enum { K_WFULL = 0, K_SRDY = 1, K_FULL = 2, K_AT = 5, K_XRDY = 7, K_DONE = 9, K_BARS = 11 };
 
 __global__ void __launch_bounds__(BS_THREADS, 1)
 bsk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmW,
@@ -391,8 +396,7 @@ bsk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
     *abort_flag = 0u;
     mbar_init(bar(K_WFULL), 1); mbar_init(bar(K_SRDY), BS_COMPUTE);
     for (int s = 0; s < L::STAGES; ++s) mbar_init(bar(K_FULL + s), 1);
-    for (int b = 0; b < 2; ++b) { mbar_init(bar(K_AT + b), 1); mbar_init(bar(K_DONE + b), 1); }
-    mbar_init(bar(K_XRDY), BS_COMPUTE);
+    for (int b = 0; b < 2; ++b) { mbar_init(bar(K_AT + b), 1); mbar_init(bar(K_XRDY + b), BS_COMPUTE); mbar_init(bar(K_DONE + b), 1); }
     fence_barrier_init();
     fence_proxy_async();
   }
@@ -446,7 +450,7 @@ bsk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
           if (!mbar_wait(bar(K_DONE + ((t - 1) & 1)), ((t - 1) >> 1) & 1, wc)) break;      // the stage of tile t - 1 is free
           request(t + 2);
         }
-        if (!mbar_wait(bar(K_XRDY), t & 1, wc)) break;
+        if (!mbar_wait(bar(K_XRDY + (t & 1)), (t >> 1) & 1, wc)) break;
         tc_fence_after();
         const uint32_t x0 = sbase + L::X_OFF + (t & 1) * 3 * BOX;
         const uint64_t hm = mnmajor_desc(x0), ml = mnmajor_desc(x0 + BOX), bK = mnmajor_desc(sK(t));
@@ -502,7 +506,7 @@ bsk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
         if (ok) store_split16(sbase + L::X_OFF + (t & 1) * 3 * BOX, BOX, r, cg * 16, da);
       }
       fence_proxy_async();
-      mbar_arrive(bar(K_XRDY));
+      mbar_arrive(bar(K_XRDY + (t & 1)));
     }
     for (int t = nt > 1 ? nt - 2 : 0; t < nt; ++t) {
       if (ok) ok = mbar_wait_warp(bar(K_DONE + (t & 1)), (t >> 1) & 1, wc);
