@@ -160,8 +160,7 @@ btq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
-  griddep_launch();
+  if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   griddep_wait();                                    // the set-up above ran beside the kernel before this one
   // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
   if (threadIdx.x == 0) *skip = *reinterpret_cast<volatile uint32_t*>(p.status);
@@ -439,8 +438,7 @@ btk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
-  griddep_launch();
+  if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   griddep_wait();                                    // the set-up above ran beside the kernel before this one
   // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
   if (threadIdx.x == 0) *skip = *reinterpret_cast<volatile uint32_t*>(p.status);

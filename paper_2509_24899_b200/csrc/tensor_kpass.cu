@@ -103,11 +103,15 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   const WaitCtx wc{p.status, abort_flag};
   const bool gathers = (p.ks_w != nullptr) && fc == 0;       // this CTA copies the softmax rows out
 
-  griddep_launch();                                          // the query stage's CTAs may set up as these ones end
+  // the query stage's CTAs may set up as these ones end
+  if (warp == 9) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   __shared__ uint32_t s_skip;
   if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
   __syncthreads();
-  if (s_skip != 0u) return;
+  if (s_skip != 0u) {
+    if (warp == 9) tmem_dealloc(*tmem_slot, 512);
+    return;
+  }
 
   auto sW = [&](int j) { return sbase + L::W_OFF + j * L::TILE; };
   auto sSlot = [&](int it) { return sbase + L::RING_OFF + (it % SLOTS) * L::TILE; };
@@ -129,8 +133,8 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   }
   if (threadIdx.x == 8 * 32) {
     // The producer sets up the barriers of the ring itself and requests the weights and the first tiles at
-    // once: the first bytes of a CTA take several microseconds to arrive, and the allocation of tensor memory
-    // and the CTA-wide barrier below need not be waited for.
+    // once: the first bytes of a CTA take several microseconds to arrive, and the CTA-wide barrier below need
+    // not be waited for.
     mbar_init(bar(B_W), 1);
     // a slot is free again when the MMA that read it has completed and, where rows are gathered, when both
     // gather warps are through with it
@@ -142,7 +146,6 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     for (int j = 0; j < NH; ++j) load_boxes(sW(j), &tmW, bar(B_W), j * D, fc * 128, h, D / 64);
     for (int it = 0; it < FIRST && it < nt * IPT; ++it) load_item(it);
   }
-  if (warp == 9) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();

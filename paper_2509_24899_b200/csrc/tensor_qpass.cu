@@ -939,8 +939,7 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (warp == 17) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
-  griddep_launch();
+  if (warp == 17) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   griddep_wait();                                    // the set-up above ran beside the kernel before this one
   // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
   __shared__ uint32_t s_skip;
@@ -1010,8 +1009,7 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (warp == 9) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
-  griddep_launch();
+  if (warp == 9) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   griddep_wait();                                    // the set-up above ran beside the kernel before this one
   // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
   __shared__ uint32_t s_skip;

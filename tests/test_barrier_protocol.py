@@ -83,3 +83,21 @@ def test_key_side_gradient_at_d64_finishes_in_every_order(tiles):
         thread.append(("wait", "done%d" % (t & 1), (t >> 1) & 1))
     counts = {"at0": 1, "at1": 1, "done0": 1, "done1": 1, **{"x%d" % i: 2 for i in range(slots)}}
     assert _stuck_state([thread, thread, lane], counts) is None
+
+
+def test_dependents_are_let_in_only_by_ctas_that_own_their_tensor_memory():
+    """In every kernel that allocates tensor memory the allocating warp alone calls griddep_launch, behind the allocation (a dependent
+    CTA that took the columns first would wait for this kernel while this one waits for the columns, without a limit)."""
+    checked = 0
+    for name in sorted(os.listdir(CSRC)):
+        if not name.endswith(".cu"):
+            continue
+        with open(os.path.join(CSRC, name)) as f:
+            kernels = re.split(r"\b__global__\b", re.sub(r"//[^\n]*", "", f.read()))[1:]
+        for body in kernels:
+            if "griddep_launch()" not in body or "tmem_alloc(" not in body:
+                continue
+            assert body.count("griddep_launch()") == 1 and body.count("tmem_alloc(") == 1, (name, body[:120])
+            assert re.search(r"if \(warp == \d+\) \{ tmem_alloc\([^;]*\); tmem_relinquish\(\); griddep_launch\(\); \}", body), (name, body[:120])
+            checked += 1
+    assert checked >= 8
