@@ -27,7 +27,7 @@ cudaError_t as_bw_tensor_init();
 cudaError_t as_bw_tensor_query(const BwParams& p, cudaStream_t st);
 cudaError_t as_bw_tensor_key(const BwParams& p, cudaStream_t st);
 // The same for d = F = 64 (polynomial degree <= 2: a part is at least 32 wide), at the precision of the CUDA-core kernels (fp32 operands in three
-// bf16 pieces).  q, k, v, y, y_hat and the weights 16-byte aligned (TMA).
+// bf16 pieces).  q, k, v, y, y_hat and the weights 16-byte aligned (TMA), S as well (read 16 bytes at a time).
 cudaError_t as_bw_tensor_d64_init();
 cudaError_t as_bw_tensor_d64_query(const BwParams& p, cudaStream_t st);
 cudaError_t as_bw_tensor_d64_key(const BwParams& p, cudaStream_t st);

@@ -394,9 +394,10 @@ as_status_t as_hybrid_attn_backward_phi(as_hybrid_attn_t h, const void* q, const
 
   const int BH = d.B * d.H, D = d.d;
   const dim3 grid(L.chunks, BH), rgrid(D * D / (4 * BW_RED) + 1, std::max(BH, d.H), 2);
-  // TMA wants 16-byte aligned tensors; at d = 64 the CUDA-core kernels (eleven times slower) take what is not
+  // TMA wants 16-byte aligned tensors, and S is read 16 bytes at a time; at d = 64 the CUDA-core kernels (eleven times slower) take
+  // what is not (the forward pass had its workspace aligned, but the caller may hand over a copy)
   const bool aligned = (((uintptr_t)q | (uintptr_t)k | (uintptr_t)v | (uintptr_t)w->wq1 | (uintptr_t)w->wk1 | (uintptr_t)y_teacher |
-                         (uintptr_t)y_hat) & 15) == 0;
+                         (uintptr_t)y_hat | (uintptr_t)forward_workspace) & 15) == 0;
   auto reduce = [&](int stage) { return as_launch_dependent(bw_reduce_kernel, rgrid, dim3(BW_RED), 0, st, p, D, stage); };
   cudaError_t e = cudaSuccess;
   if (D == 128 && d.phi_dim == 128 && d.kernel_path == AS_PATH_TENSOR) {

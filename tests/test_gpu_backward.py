@@ -150,6 +150,28 @@ def test_narrow_head_gradient_has_the_precision_of_the_cuda_core_kernels(shape, 
         assert abs(loss.item() - diff.abs().sum().item()) <= 1e-5 * diff.abs().sum().item()
 
 
+def test_narrow_head_gradient_takes_a_copy_of_the_state_at_any_float_boundary():
+    """d = 64, the forward workspace copied to an address 4 bytes past a 16-byte boundary: the CUDA-core kernels' results, bit for bit."""
+    import torch
+    from paper_2509_24899_b200 import HybridAttention, binding
+    wl = W.Workload("bw_d64_copy", B=1, H=2, d=64, F=64, grid=(1, 9, 31), block=(1, 4, 4), rate=4, seed=69)
+    dev = {k: to_cuda_bf16(v) for k, v in W.generate(wl, wq_gain=2e-3).items()}
+    y = to_cuda_bf16(W.teacher_output(wl))
+    ops = [HybridAttention.from_workload(wl, kernel_path=k) for k in (binding.AS_PATH_TENSOR, binding.AS_PATH_SIMT)]
+    aux = torch.empty((wl.B, wl.H, wl.N, 3), dtype=torch.float32, device="cuda")
+    args = [dev[n] for n in ("q", "k", "v", "wq", "wk")]
+    y_hat = ops[0].forward(*args, aux=aux)
+    ws = ops[0].workspace()
+    copy = torch.empty(ws.numel() + 16, dtype=torch.uint8, device="cuda")[4:4 + ws.numel()]
+    assert copy.data_ptr() % 16 == 4
+    copy.copy_(ws)
+    ops[0]._ws, ops[1]._ws = copy, ws
+    got = [op.backward_phi(*args, y, y_hat, aux) for op in ops]
+    assert ops[0].last_status() == 0
+    for a, b in zip(*got):
+        assert torch.equal(a, b) and bool(torch.isfinite(a).all())
+
+
 # less than a tile of 64, whole tiles, one row more, an odd number of tiles, more tiles a chunk than the ring has slots; every power
 @pytest.mark.parametrize("B,H,N,rate,degree,mode", [(1, 1, 40, 2, 2, O.STAB_PAPER), (1, 2, 64, 0, 1, O.STAB_PAPER), (1, 2, 65, 4, 4, O.STAB_EXACT),
                                                     (1, 3, 192, 3, 2, O.STAB_EXACT), (2, 75, 700, 4, 4, O.STAB_PAPER), (1, 150, 321, 0, 2, O.STAB_PAPER)])
