@@ -29,6 +29,17 @@ AS_DEV uint32_t sub_bf16x2(uint32_t a, uint32_t b) {
   asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
   return r;
 }
+// the two halves of a, read as bf16, minus b in fp32 (mixed-precision subtraction of sm_100)
+AS_DEV float2 sub_bf16x2_f32(uint32_t a, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b16 lo, hi;\n\t"
+      "mov.b32 {lo, hi}, %2;\n\t"
+      "sub.rn.f32.bf16 %0, lo, %3;\n\t"
+      "sub.rn.f32.bf16 %1, hi, %4;\n\t}"
+      : "=f"(r.x), "=f"(r.y)
+      : "r"(a), "f"(b.x), "f"(b.y));
+  return r;
+}
 // all ones in the halves that differ (or are unordered)
 AS_DEV uint32_t ne_bf16x2(uint32_t a, uint32_t b) {
   uint32_t r;
@@ -282,7 +293,7 @@ btq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
           }
           const float inv_den = 1.f / den;
           const uint32_t inv2 = pack_bf16(inv_den, inv_den);
-          float h0 = 0.f, h1 = 0.f, y0 = 0.f, y1 = 0.f;      // sums of G y_hat and of G y
+          float2 hs = make_float2(0.f, 0.f), ls = make_float2(0.f, 0.f);      // sums of G y_hat and of -|y_hat - y|
 #pragma unroll
           for (int c4 = 0; c4 < 4; ++c4) {
             const uint32_t off = (gq >> 1) * L::QBOX + swz128_chunk_offset(gr, (gq & 1) * 4 + (c4 ^ ((gq >> 1) << 1)));
@@ -295,13 +306,17 @@ btq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
               // none where the two are equal - and rows past the end of the sequence arrive as zeros
               const uint32_t sign = sub_bf16x2(hw[i], yw[i]) & 0x80008000u, differ = ne_bf16x2(hw[i], yw[i]);
               gw[i] = (inv2 ^ sign) & differ;
-              add_bf16x2(h0, h1, (hw[i] ^ sign) & differ);
-              add_bf16x2(y0, y1, (yw[i] ^ sign) & differ);
+              const uint32_t Gh = (hw[i] ^ sign) & differ, Gy = (yw[i] ^ sign) & differ;
+              const float2 h2 = make_float2(bf_lo(Gh), bf_hi(Gh));
+              hs = __fadd2_rn(hs, h2);
+              // the differences in fp32 one by one: a difference of two sums would cancel where y_hat is close to y (y_hat one bf16 unit
+              // from y, values spread over several decades: 2e-6 to 9e-6 off)
+              ls = __fadd2_rn(ls, sub_bf16x2_f32(Gy, h2));
             }
             *reinterpret_cast<uint4*>(sY + off) = make_uint4(gw[0], gw[1], gw[2], gw[3]);
           }
-          float sdot = h0 + h1;
-          loss += sdot - (y0 + y1);                    // sum of |y_hat - y|
+          float sdot = hs.x + hs.y;
+          loss -= ls.x + ls.y;                         // sum of |y_hat - y|
           sdot += __shfl_xor_sync(0xffffffffu, sdot, 1);
           sdot += __shfl_xor_sync(0xffffffffu, sdot, 2);
           if (gq == 0) {

@@ -212,6 +212,30 @@ def test_gradient_at_the_edges_of_tiles(B, H, N, rate, degree, mode):
     assert abs(got[2].item() - diff.abs().sum().item()) <= 1e-5 * diff.abs().sum().item()
 
 
+@pytest.mark.parametrize("d", [64, 128])
+def test_loss_keeps_its_precision_near_the_teacher(d):
+    """y_hat one bf16 unit from y on half of the elements and equal on the rest, values spread over several decades.  The loss is a sum
+    of positive fp32 terms, each exact; a term goes through some 16 + 3 + 5 + 8 + 12 + 5 additions of 2^-24 each at most: 1e-6 with their
+    roundings at random (square root of 49 times 2^-24: 4e-7), 3e-6 at worst."""
+    import torch
+    from paper_2509_24899_b200 import HybridAttention
+    wl = W.Workload("bw_near", B=1, H=2, d=d, F=d, grid=(1, 1, 500), block=(1, 1, 500), rate=4, seed=70)
+    dev = {k: to_cuda_bf16(v) for k, v in W.generate(wl, wq_gain=2e-3).items()}
+    op = HybridAttention.from_workload(wl)
+    aux = torch.empty((wl.B, wl.H, wl.N, 3), dtype=torch.float32, device="cuda")
+    args = [dev[n] for n in ("q", "k", "v", "wq", "wk")]
+    op.forward(*args, aux=aux)
+    g = torch.Generator(device="cuda").manual_seed(70)
+    r = [torch.randn(aux.shape[:3] + (d,), device="cuda", generator=g) for _ in range(3)]
+    y = ((4.0 * r[0]).exp() * r[1].sign()).bfloat16()
+    bits = y.view(torch.int16)
+    y_hat = torch.where(r[2] > 0.5, bits + 1, torch.where(r[2] < -0.8, bits - 1, bits)).view(torch.bfloat16)
+    _, _, loss = op.backward_phi(*args, y, y_hat, aux)
+    assert op.last_status() == 0
+    want = (y_hat.double() - y.double()).abs().sum().item()
+    assert abs(loss.item() - want) <= 1e-6 * want
+
+
 def test_backward_argument_errors_and_zero_gradient_without_linear_tokens():
     import torch
     from paper_2509_24899_b200 import HybridAttention, binding, AsError
