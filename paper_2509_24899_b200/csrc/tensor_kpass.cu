@@ -103,14 +103,14 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   const WaitCtx wc{p.status, abort_flag};
   const bool gathers = (p.ks_w != nullptr) && fc == 0;       // this CTA copies the softmax rows out
 
-  // the query stage's CTAs may set up as these ones end
-  if (warp == 9) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
+  // an earlier CTA of this or a previous launch timed out: nothing is requested (decided once per CTA)
   __shared__ uint32_t s_skip;
   if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
-  __syncthreads();
-  if (s_skip != 0u) {
-    if (warp == 9) tmem_dealloc(*tmem_slot, 512);
-    return;
+  if (warp != 9) {
+    named_barrier_sync(3, K_THREADS - 32);
+  } else {
+    // first of all, and the others need not wait for it: the query stage's CTAs may then set up as these ones end
+    tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch();
   }
 
   auto sW = [&](int j) { return sbase + L::W_OFF + j * L::TILE; };
@@ -131,7 +131,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     mbar_init(bar(B_DONE), 1);
     fence_barrier_init();
   }
-  if (threadIdx.x == 8 * 32) {
+  if (threadIdx.x == 8 * 32 && s_skip == 0u) {
     // The producer sets up the barriers of the ring itself and requests the weights and the first tiles at
     // once: the first bytes of a CTA take several microseconds to arrive, and the CTA-wide barrier below need
     // not be waited for.
@@ -149,6 +149,10 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (s_skip != 0u) {
+    if (warp == 9) tmem_dealloc(*tmem_slot, 512);
+    return;
+  }
   const uint32_t tmem = *tmem_slot;
   const uint32_t tD1[2] = {tmem + 0u, tmem + 128u};          // Phi^T of a tile, fp32
   const uint32_t tAcc = tmem + 256u;                         // S of this feature chunk
