@@ -303,8 +303,9 @@ btq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               // on pairs of bf16: the sign of y_hat - y (rounding a difference changes neither its sign nor whether it is zero),
-              // none where the two are equal - and rows past the end of the sequence arrive as zeros
-              const uint32_t sign = sub_bf16x2(hw[i], yw[i]) & 0x80008000u, differ = ne_bf16x2(hw[i], yw[i]);
+              // none where it is zero - and rows past the end of the sequence arrive as zeros.  (Infinity less infinity is not zero: such
+              // an element makes the loss and the row's gradient NaN.)
+              const uint32_t diff = sub_bf16x2(hw[i], yw[i]), sign = diff & 0x80008000u, differ = ne_bf16x2(diff, 0u);
               gw[i] = (inv2 ^ sign) & differ;
               const uint32_t Gh = (hw[i] ^ sign) & differ, Gy = (yw[i] ^ sign) & differ;
               const float2 h2 = make_float2(bf_lo(Gh), bf_hi(Gh));

@@ -212,6 +212,39 @@ def test_gradient_at_the_edges_of_tiles(B, H, N, rate, degree, mode):
     assert abs(got[2].item() - diff.abs().sum().item()) <= 1e-5 * diff.abs().sum().item()
 
 
+def _small_step(d, degree=2, seed=74):
+    """A layer of 200 tokens after its forward: (handle, arguments of the gradient, y_hat, aux)."""
+    import torch
+    from paper_2509_24899_b200 import HybridAttention
+    wl = W.Workload("bw_small", B=1, H=2, d=d, F=d, grid=(1, 1, 200), block=(1, 1, 200), rate=4, seed=seed, degree=degree)
+    dev = {k: to_cuda_bf16(v) for k, v in W.generate(wl, wq_gain=2e-3).items()}
+    op = HybridAttention.from_workload(wl)
+    aux = torch.empty((wl.B, wl.H, wl.N, 3), dtype=torch.float32, device="cuda")
+    args = [dev[n] for n in ("q", "k", "v", "wq", "wk")]
+    return op, args, op.forward(*args, aux=aux), aux
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_signs_at_the_edges_of_bf16(d):
+    """sign(y_hat - y) where the difference is the smallest bf16 number, and where it is infinity less infinity: that is no number, and
+    neither is the loss, nor the gradient (which y_hat enters)."""
+    import torch
+    op, args, y_hat, aux = _small_step(d)
+    g = torch.Generator(device="cuda").manual_seed(75)
+    negative = torch.rand(y_hat.shape, device="cuda", generator=g) < 0.5
+    least = (negative.to(torch.int16) * -32768 + 1).to(torch.int16).view(torch.bfloat16)
+    zero, far = torch.zeros_like(y_hat), torch.where(negative, 1.0, -1.0).bfloat16()
+    got = [op.backward_phi(*args, y, least, aux)[:2] for y in (zero, far)]
+    for a, b in zip(*got):
+        assert torch.equal(a, b) and bool(a.any())
+    y = zero.clone()
+    y[0, 1, 77, 5] = y_hat[0, 1, 77, 5] = float("inf")
+    dwq, dwk, loss = op.backward_phi(*args, y, y_hat, aux)
+    assert op.last_status() == 0
+    assert bool(loss.isnan().all()) and not bool(dwq[1].isfinite().all()) and not bool(dwk[1].isfinite().all())
+    assert bool(dwq[0].isfinite().all()) and bool(dwk[0].isfinite().all())
+
+
 @pytest.mark.parametrize("d", [64, 128])
 def test_loss_keeps_its_precision_near_the_teacher(d):
     """y_hat one bf16 unit from y on half of the elements and equal on the rest, values spread over several decades.  The loss is a sum
