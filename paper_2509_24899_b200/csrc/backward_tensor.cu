@@ -120,7 +120,7 @@ AS_DEV void btq_features(const uint32_t (&xa)[32], const uint32_t (&xu)[32], con
       const float2 t = __ffma2_rn(z2, s2, make_float2(__uint_as_float(xu[k]), __uint_as_float(xu[k + 1])));
       float2 ph = r, da;
       if (PW == 1) {
-        da = make_float2(a0 > 0.f ? t.x : 0.f, a1 > 0.f ? t.y : 0.f);
+        da = __fmul2_rn(t, make_float2(a0 > 0.f ? 1.f : 0.f, a1 > 0.f ? 1.f : 0.f));      // (a product: a NaN reaches every feature)
       } else {
         float2 rp = r;                               // r^(p-1)
 #pragma unroll
@@ -417,7 +417,7 @@ AS_DEV void btk_features(const uint32_t (&xa)[32], const uint32_t (&xt)[32], flo
     const float a0 = __uint_as_float(xa[2 * i]), a1 = __uint_as_float(xa[2 * i + 1]);
     float2 t = __fadd2_rn(make_float2(__uint_as_float(xt[2 * i]), __uint_as_float(xt[2 * i + 1])), make_float2(dz, dz));
     if (PW == 1) {
-      t = make_float2(a0 > 0.f ? t.x : 0.f, a1 > 0.f ? t.y : 0.f);
+      t = __fmul2_rn(t, make_float2(a0 > 0.f ? 1.f : 0.f, a1 > 0.f ? 1.f : 0.f));
     } else {
       const float2 r = make_float2(fmaxf(a0, 0.f), fmaxf(a1, 0.f));
       float2 rp = r;                                 // r^(p-1)

@@ -245,6 +245,18 @@ def test_signs_at_the_edges_of_bf16(d):
     assert bool(dwq[0].isfinite().all()) and bool(dwk[0].isfinite().all())
 
 
+@pytest.mark.parametrize("d,degree", [(64, 1), (64, 2), (128, 1), (128, 2), (128, 4)])
+def test_a_student_output_that_is_no_number_reaches_every_feature(d, degree):
+    """One NaN in y_hat: dL/dphi of that token is NaN, and its product with a slope of zero as well, whatever the feature's power."""
+    op, args, y_hat, aux = _small_step(d, degree)
+    y = y_hat.clone()
+    y_hat[0, 1, 77, 5] = float("nan")
+    dwq, dwk, loss = op.backward_phi(*args, y, y_hat, aux)
+    assert op.last_status() == 0
+    assert bool(loss.isnan().all()) and bool(dwq[1].isnan().all()) and bool(dwk[1].isnan().all())
+    assert not bool(dwq[0].any()) and not bool(dwk[0].any())
+
+
 @pytest.mark.parametrize("d", [64, 128])
 def test_loss_keeps_its_precision_near_the_teacher(d):
     """y_hat one bf16 unit from y on half of the elements and equal on the rest, values spread over several decades.  The loss is a sum
