@@ -1,0 +1,117 @@
+"""Kernels that set up while the kernel before them in the stream drains: nothing of theirs may be read or written before that one has
+ended, whatever it is - one of the library's or the caller's - and a captured sequence has to keep that."""
+import numpy as np
+import pytest
+
+from paper_2509_24899_b200 import workloads as W
+from _util import to_cuda_bf16
+
+pytestmark = pytest.mark.gpu
+
+LAYERS = {
+    "softmax_d128": dict(d=128, rate=1), "softmax_d64": dict(d=64, rate=1), "hybrid_d128": dict(d=128, rate=4), "hybrid_d64": dict(d=64, rate=4),
+    "linear_d128": dict(d=128, rate=0), "linear_d64": dict(d=64, rate=0), "two_layers": dict(d=128, rate=4, F=256, hidden=256),
+}
+
+
+def _layer(d, rate, F=None, hidden=0):
+    from paper_2509_24899_b200 import HybridAttention
+    wl = W.Workload("order", B=1, H=4, d=d, F=F or d, grid=(1, 20, 26), block=(1, 4, 4), rate=rate, seed=81, layers=2 if hidden else 1,
+                    hidden=hidden)
+    dev = {k: to_cuda_bf16(v) for k, v in W.generate(wl, wq_gain=2e-3 if rate else 1.0).items()}
+    return wl, dev, HybridAttention.from_workload(wl), {n: dev[n] for n in ("wq2", "wk2") if n in dev}
+
+
+def _late(dst, src):
+    """Writes src into dst by a kernel on the current stream, a millisecond from now."""
+    import torch
+    torch.cuda._sleep(2_000_000)
+    torch.mul(src, 1.0, out=dst)
+
+
+@pytest.mark.parametrize("name", sorted(LAYERS))
+def test_a_forward_right_behind_the_kernel_that_writes_its_input(name):
+    import torch
+    wl, dev, op, second = _layer(**LAYERS[name])
+    want = op.forward(dev["q"], dev["k"], dev["v"], dev["wq"], dev["wk"], **second).clone()
+    for n in ("q", "k", "v"):
+        x = dict(dev, **{n: torch.full_like(dev[n], 3.0)})
+        torch.cuda.synchronize()
+        _late(x[n], dev[n])
+        got = op.forward(x["q"], x["k"], x["v"], x["wq"], x["wk"], **second)
+        assert op.last_status() == 0
+        assert torch.equal(got, want), n
+
+
+@pytest.mark.parametrize("with_state", [False, True])
+@pytest.mark.parametrize("d", [64, 128])
+def test_a_query_pass_right_behind_the_kernel_that_writes_its_input(d, with_state):
+    import torch
+    wl, dev, op, _ = _layer(d, 4)
+    ks, vs, S, z = (x.clone() for x in op.key_pass(dev["k"], dev["v"], dev["wq"], dev["wk"]))
+    state = (S, z) if with_state else (None, None)
+    want = op.query_pass(dev["q"], dev["wq"], dev["wk"], ks, vs, *state).clone()
+    inputs = {"q": dev["q"], "ks": ks, "S": S} if with_state else {"q": dev["q"], "ks": ks}
+    for n, src in inputs.items():
+        x = dict(q=dev["q"], ks=ks, S=state[0])
+        x[n] = torch.full_like(src, 3.0)
+        torch.cuda.synchronize()
+        _late(x[n], src)
+        got = op.query_pass(x["q"], dev["wq"], dev["wk"], x["ks"], vs, x["S"], state[1])
+        assert op.last_status() == 0
+        assert torch.equal(got, want), n
+
+
+@pytest.mark.parametrize("name", ["hybrid_d128", "hybrid_d64"])
+def test_a_gradient_right_behind_the_kernel_that_writes_the_teacher(name):
+    import torch
+    wl, dev, op, _ = _layer(**LAYERS[name])
+    args = [dev[n] for n in ("q", "k", "v", "wq", "wk")]
+    y = to_cuda_bf16(W.teacher_output(wl))
+    aux = torch.empty((wl.B, wl.H, wl.N, 3), dtype=torch.float32, device="cuda")
+    y_hat = op.forward(*args, aux=aux)
+    want = op.backward_phi(*args, y, y_hat, aux)
+    late = torch.full_like(y, 3.0)
+    torch.cuda.synchronize()
+    _late(late, y)
+    got = op.backward_phi(*args, late, y_hat, aux)
+    assert op.last_status() == 0
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("name", sorted(LAYERS))
+def test_a_captured_step_gives_the_results_of_the_calls(name):
+    """Forward (and gradient, where the layer has one) captured into a graph and replayed on other inputs in the same buffers."""
+    import torch
+    wl, dev, op, second = _layer(**LAYERS[name])
+    args = [dev[n] for n in ("q", "k", "v", "wq", "wk")]
+    gradient = wl.rate != 1 and not second
+    y = to_cuda_bf16(W.teacher_output(wl))
+    aux = torch.empty((wl.B, wl.H, wl.N, 3), dtype=torch.float32, device="cuda")
+    out = torch.empty_like(dev["q"])
+
+    def step():
+        op.forward(*args, out=out, aux=aux, **second)
+        return op.backward_phi(*args, y, out, aux) if gradient else ()
+
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        step()                                           # workspaces are there before the capture
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            captured = step()
+    torch.cuda.synchronize()
+    dev["q"].copy_(dev["q"].flip(2))
+    dev["v"].copy_(dev["v"].flip(1))
+    want = [x.clone() for x in step()] + [out.clone(), aux.clone()]
+    out.zero_()
+    for _ in range(2):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert op.last_status() == 0
+    got = list(captured) + [out, aux]
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
+    del graph
