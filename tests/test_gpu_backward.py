@@ -176,18 +176,22 @@ def test_narrow_head_gradient_takes_a_copy_of_the_state_at_any_float_boundary():
 @pytest.mark.parametrize("B,H,N,rate,degree,mode", [(1, 1, 40, 2, 2, O.STAB_PAPER), (1, 2, 64, 0, 1, O.STAB_PAPER), (1, 2, 65, 4, 4, O.STAB_EXACT),
                                                     (1, 3, 192, 3, 2, O.STAB_EXACT), (2, 75, 700, 4, 4, O.STAB_PAPER), (1, 150, 321, 0, 2, O.STAB_PAPER)])
 def test_gradient_at_the_edges_of_tiles(B, H, N, rate, degree, mode):
-    """d = 128: the tensor-core kernels next to the fp32 ones on the same y_hat, row statistics and state.  Their operands g, lambda phi_q,
-    dL/da, S, dS are rounded to bf16 (2^-9 each, at random): 2e-3 to 4e-3 in relative L2; 6e-3 asserted."""
+    """d = 128: the tensor-core kernels and (up to degree 2, which they take) the fp32 ones against the chain rule in 64 bits on the same
+    y_hat, row statistics and state.  The operands g, lambda phi_q, dL/da, S, dS of the first are rounded to bf16 (2^-9 each, at random):
+    2e-3 to 4e-3 in relative L2; 6e-3 asserted.  The fp32 kernels as at d = 64: 1e-6 for the median feature."""
     import torch
     from paper_2509_24899_b200 import HybridAttention, binding
     wl = W.Workload("bw_edges", B=B, H=H, d=128, F=128, grid=(1, 1, N), block=(1, 1, N), rate=rate, seed=68, degree=degree)
     dev = {k: to_cuda_bf16(v) for k, v in W.generate(wl, wq_gain=2e-3 if rate else 1.0).items()}
     y = to_cuda_bf16(W.teacher_output(wl))
-    ops = [HybridAttention.from_workload(wl, stab_mode=mode) for _ in range(2)]
+    paths = [binding.AS_PATH_TENSOR] + ([binding.AS_PATH_SIMT] if degree <= 2 else [])
+    ops = [HybridAttention.from_workload(wl, stab_mode=mode, kernel_path=k) for k in paths]
     aux = torch.empty((B, H, N, 3), dtype=torch.float32, device="cuda")
     args = [dev[n] for n in ("q", "k", "v", "wq", "wk")]
     y_hat = ops[0].forward(*args, aux=aux)
-    got = ops[0].backward_phi(*args, y, y_hat, aux)
+    for op in ops[1:]:
+        op._ws = ops[0].workspace()                     # S and z of the tensor path's forward
+    got, *got_fp32 = [op.backward_phi(*args, y, y_hat, aux) for op in ops]
     S, z = (x.double() for x in ops[0].linear_state())
     assert ops[0].last_status() == 0
     q, k, v, wq, wk = (x.double() for x in args)
@@ -210,6 +214,11 @@ def test_gradient_at_the_edges_of_tiles(B, H, N, rate, degree, mode):
     for a, r in ((got[0], dwq), (got[1], dwk)):
         assert float((a.double() - r).norm() / r.norm()) <= 6e-3
     assert abs(got[2].item() - diff.abs().sum().item()) <= 1e-5 * diff.abs().sum().item()
+    for dq, dk, loss in got_fp32:
+        for a, r in ((dq, dwq), (dk, dwk)):
+            err = (a.double() - r).norm(dim=-1) / r.norm(dim=-1)
+            assert err.median() <= 1e-6 and (err > 1e-5).sum() <= 2, err.max()
+        assert abs(loss.item() - diff.abs().sum().item()) <= 1e-5 * diff.abs().sum().item()
 
 
 def _small_step(d, degree=2, seed=74):
