@@ -216,9 +216,11 @@ AS_API as_status_t as_hybrid_attn_query_pass(as_hybrid_attn_t h, const void* q, 
  *   workspace  device scratch, 256-byte aligned, >= backward_workspace_bytes
  * L = sum |y - y_hat|; q, k, v and y are constants of the step.  lambda_i (AS_STAB_EXACT: exp(-c_i)) and the softmax
  * branch do not depend on the weights.  One-layer feature maps with F == d and no bias; anything else returns
- * AS_ERR_UNSUPPORTED.  With d = F = 128 on AS_PATH_TENSOR the products run on the tensor cores (bf16 operands, fp32
- * accumulation); every other supported shape, and AS_PATH_SIMT, in fp32 on CUDA cores.  Asynchronous on the stream;
- * sums in a fixed order (no float atomics), so results are run-to-run identical. */
+ * AS_ERR_UNSUPPORTED.  On AS_PATH_TENSOR the products run on the tensor cores: with d = F = 128 on bf16 operands, with
+ * d = F = 64 on fp32 operands in three bf16 pieces (fp32 precision), accumulated in fp32.  AS_PATH_SIMT runs in fp32 on
+ * CUDA cores, and so does, eleven times slower, d = F = 64 when one of q, k, v, wq1, wk1, y_teacher, y_hat or
+ * forward_workspace is not 16-byte aligned (with d = F = 128 they have to be).  Asynchronous on the stream; sums in a
+ * fixed order (no float atomics), so results are run-to-run identical. */
 AS_API as_status_t as_hybrid_attn_backward_workspace_bytes(as_hybrid_attn_t h, size_t* bytes);
 AS_API as_status_t as_hybrid_attn_backward_phi(as_hybrid_attn_t h, const void* q, const void* k, const void* v,
                                                const as_phi_weights_t* w, const void* y_teacher, const void* y_hat,

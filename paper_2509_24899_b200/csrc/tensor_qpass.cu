@@ -1,12 +1,12 @@
 // Q pass of the hybrid attention forward on the tensor cores of sm_100a: softmax branch, phi_q
 // projection, linear apply and merge, fused in one persistent kernel.
 //
-//   persistent, one CTA per SM (units left over after the full rounds are split into 128-row halves
-//   over twice as many CTAs); per unit of 2 x 128 query rows a flash-style loop over 128-key tiles
+//   persistent, one CTA per SM (what is left over after the full rounds is dealt out in one last round, in
+//   units of two 128-row tiles or of one, see plan_units); per unit a flash-style loop over 128-key tiles
 //   of K_S / V_S:        S = Q K_S^T -> TMEM; the softmax threads (one per row) read their row and
 //                        release the score columns at once, so the next tile's Q K_S^T runs under the
 //                        exponentials; running max / sum per row; P = exp2(.) as bf16 -> shared memory,
-//                        O += P V_S (smem x smem -> TMEM).  Two issuing threads: one for what writes
+//                        O += P V_S (smem x smem -> TMEM).  Two issuing warps: one for what writes
 //                        the score columns, one for what accumulates into O.
 //   tail, per chunk c of 128 features:
 //                        Phi_c = Q W_q[c]^T -> TMEM (in the place of a next tile's scores), phi_q scaled per
@@ -57,8 +57,9 @@ struct QLayout {
   static constexpr int TOTAL = BAR_OFF + 256 + 1024;       // + slack for the 1024-byte alignment
 };
 
-// Persistent: one CTA per SM walks over 256-row units (unit w = blockIdx.x + u * gridDim.x; the units of
-// one (batch, head) are consecutive, so the CTAs that run at the same time share K_S / V_S in L2).
+// Persistent: one CTA per SM walks over units of two 128-row tiles (unit w = blockIdx.x + u * gridDim.x, the last one
+// as plan_units deals it out; the units of one (batch, head) are consecutive, so the CTAs that run at the same time
+// share K_S / V_S in L2).
 // Barrier phases and the K/V ring run on across units.
 //
 // Scores and probabilities live in different memories: S = Q K^T lands in TMEM, the softmax threads read
@@ -68,7 +69,7 @@ struct QLayout {
 // and group, one Q K^T block as soon as S is free and one P V block as soon as P is there.
 //
 // The work of one unit is a function per role, kept out of line: each role then gets a register
-// allocation of its own (the softmax rows need nearly the whole budget, and the issuing thread must
+// allocation of its own (the softmax rows need nearly the whole budget, and the issuing warps must
 // not spill).  Everything about a unit is derived from its index u inside the function.
 struct QCtx {
   uint32_t sbase;            // shared-memory window address of the 1024-aligned base
@@ -797,7 +798,7 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
 // With no key loop a unit is: Phi = Q W^T, phi_q, O = phi_q S, y = O / (phi_q . z), store.  The tensor pipe has
 // little to do and the kernel is bound by how fast the threads turn rows around, so this variant of the kernel runs
 // SIXTEEN compute warps: each 128-row group is worked on by two warps per TMEM lane quadrant, each taking one half of
-// the columns of a row (features on the way in, output columns on the way out).  Producer and issuing threads are the
+// the columns of a row (features on the way in, output columns on the way out).  Producer and issuing warps are the
 // ones of the general kernel; a row's two threads add their shares of phi_q . z through shared memory.
 constexpr int QL_THREADS = 608;          // warps 0-15: compute (group = bit 2, quadrant = bits 0-1, column half = bit 3);
                                          // warp 16: TMA; warps 17, 18: MMA issuers
