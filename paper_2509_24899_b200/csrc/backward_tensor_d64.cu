@@ -38,25 +38,6 @@ constexpr uint32_t ID_TOK = make_idesc(128, 64, 0, 0);      // [tokens x 64] = [
 constexpr uint32_t ID_Q2 = make_idesc(128, 128, 1, 1);      // X^T [G | Q]
 constexpr uint32_t ID_K2 = make_idesc(128, 64, 1, 1);       // [two pieces of X]^T K
 
-// 16 columns of one TMEM lane per thread, not waited for
-AS_DEV void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
-AS_DEV void tmem_ld16_wait(uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.wait::ld.sync.aligned;"
-      : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-        "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-      :
-      : "memory");
-}
-
 // x = hi + mid + lo with eight significant bits each, by truncation: exact, and nothing overflows.  A value that is
 // not finite is all in hi (the pieces of an infinity would add up to NaN).
 AS_DEV void split3(float x0, float x1, uint32_t& hi, uint32_t& mid, uint32_t& lo) {

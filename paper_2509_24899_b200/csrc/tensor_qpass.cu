@@ -3,17 +3,17 @@
 //
 //   persistent, one CTA per SM (what is left over after the full rounds is dealt out in one last round, in
 //   units of two 128-row tiles or of one, see plan_units); per unit a flash-style loop over 128-key tiles
-//   of K_S / V_S:        S = Q K_S^T -> TMEM; the softmax threads (one per row) read their row and
-//                        release the score columns at once, so the next tile's Q K_S^T runs under the
-//                        exponentials; running max / sum per row; P = exp2(.) as bf16 -> shared memory,
-//                        O += P V_S (smem x smem -> TMEM).  Two issuing warps: one for what writes
+//   of K_S / V_S:        S = Q K_S^T -> TMEM; the softmax threads (one or two per row) read their row and
+//                        release the score columns at once, so the next product into them runs under the
+//                        exponentials; running max / sum per row; P = exp2(.) as bf16 -> TMEM,
+//                        O += P V_S (TMEM x smem -> TMEM).  Two issuing warps: one for what writes
 //                        the score columns, one for what accumulates into O.
 //   tail, per chunk c of 128 features:
 //                        Phi_c = Q W_q[c]^T -> TMEM (in the place of a next tile's scores), phi_q scaled per
-//                        row as bf16 where P sat, O += phi_q,c S_c (S in bf16 read like a V tile),
-//                        den = l + phi_q.z, y = O / den -> bf16 -> staged in the P tile -> TMA store.
+//                        row as bf16 into shared memory, O += phi_q,c S_c (S in bf16 read like a V tile),
+//                        den = l + phi_q.z, y = O / den -> bf16 -> staged where phi_q sat -> TMA store.
 //   two-layer feature map: the hidden activations relu(Q W_q1^T + b1) are formed in the same way first
-//                        (128 hidden units at a time) and kept as bf16 in the P tile and, once nothing reads
+//                        (128 hidden units at a time) and kept as bf16 in the group's phi_q tile and, once nothing reads
 //                        Q any more, in the Q tile; Phi_c = sum over the hidden slices of h1_j W_q2[c, j]^T.
 // All tiles are staged by TMA with the 128-byte swizzle; every mbarrier wait is bounded.
 #include "tensor_common.cuh"
@@ -42,16 +42,61 @@ struct QParams {
   uint32_t* status;
 };
 
-constexpr int Q_THREADS = 352;           // warps 0-3 / 4-7: softmax groups 0 / 1; warp 8: TMA; warps 9, 10: MMA issuers
+// How the compute threads share a 128-row tile: T = 1, one thread per row (eight warps), or T = 2, threads t and t + 16 of a warp, each
+// with half of the row's columns (sixteen warps; the two share their maxima and sums by one shuffle).  cf. q_threads_per_row.
+template <int D, int T>
+struct QShape {
+  static constexpr int TPR = T;                            // threads per row
+  static constexpr int COLS = 128 / TPR;                   // score columns of a thread
+  static constexpr int W_TMA = 8 * TPR, W_SCORE = W_TMA + 1, W_ACCUM = W_TMA + 2;
+  // warps 0 .. 8 * TPR - 1: compute (quadrant = bits 0-1, group = bit 2, T = 2: half of the quadrant's rows = bit 3)
+  static constexpr int THREADS = (W_TMA + 3) * 32, GROUP = 128 * TPR;
+};
 constexpr int KV_STAGES = 3;
 constexpr float RESCALE_THRESHOLD = 8.f; // log2 units: rescale O only when the row max grew by > 2^8
+
+// A thread's share of a row (of 32 columns in TMEM; SPLIT: distance of the two threads' shares where two share a row)
+template <int TPR, int SPLIT>
+AS_DEV void q_ld32(uint32_t t, uint32_t (&x)[32]) {
+  if constexpr (TPR == 1) tmem_ld32(t, x); else tmem_ldh32<SPLIT>(t, x);
+}
+template <int TPR, int SPLIT>
+AS_DEV void q_ld16(uint32_t t, uint32_t (&x)[16]) {
+  if constexpr (TPR == 1) tmem_ld16(t, x); else tmem_ldh16<SPLIT>(t, x);
+}
+template <int TPR, int SPLIT>
+AS_DEV void q_st16(uint32_t t, const uint32_t (&x)[16]) {
+  if constexpr (TPR == 1) tmem_st16(t, x); else tmem_sth16<SPLIT>(t, x);
+}
+
+// Of every EX2_FMA_EVERY-th group of four exponentials two are taken on the FMA pipe (0: none).  Sixteen warps: one in eight of all (the
+// special-function unit, 16 a clock, is what four warps per sub-partition wait for): d = 64, N 8505, 2142 keys 293 -> 279 us; one in
+// sixteen 284, one in four 304.  Eight warps: no gain (81 frames of full softmax 4637 us; one in sixteen 4650, one in eight 4709).
+template <int T> constexpr int EX2_FMA_EVERY = T == 2 ? 4 : 0;
+// Two exponentials 2^x, x <= 8, on the FMA pipe: x = n + f with n the nearest integer (added into the last bits of 1.5 * 2^23), 2^f by
+// the polynomial of degree 5 with constant term 1 that is closest to it on [-1/2, 1/2] in relative error (9.1e-8, found by
+// reweighted least squares), times 2^n put together from its exponent.  Within 1.7e-7 of 2^x for all x in [-126, 8] (ex2.approx: 2.4e-7);
+// smaller ones come out as 2^-126 instead of 0, and what is no number stays none.
+AS_DEV float2 ex2_fma(float2 x) {
+  auto both = [](float v) { return make_float2(v, v); };
+  x = make_float2(fmax_nan(x.x, -126.f), fmax_nan(x.y, -126.f));
+  const float2 t = __fadd2_rn(x, both(12582912.f));
+  const float2 f = __ffma2_rn(__fadd2_rn(t, both(-12582912.f)), both(-1.f), x);
+  float2 y = __ffma2_rn(both(1.326472731307149e-3f), f, both(9.671512991189957e-3f));
+  y = __ffma2_rn(y, f, both(5.550733581185341e-2f));
+  y = __ffma2_rn(y, f, both(2.4022242426872253e-1f));
+  y = __ffma2_rn(y, f, both(6.931470036506653e-1f));
+  y = __ffma2_rn(y, f, both(1.f));
+  const float2 p = make_float2(__uint_as_float((__float_as_uint(t.x) << 23) + 0x3f800000u), __uint_as_float((__float_as_uint(t.y) << 23) + 0x3f800000u));
+  return __fmul2_rn(y, p);
+}
 
 template <int D>
 struct QLayout {
   static constexpr int TILE = 128 * D * 2;                 // bytes of a [128 x D] bf16 tile
-  static constexpr int PTILE = 128 * 128 * 2;              // bytes of a [128 rows x 128 keys] bf16 P tile
+  static constexpr int PTILE = 128 * 128 * 2;              // bytes of a [128 rows x 128 features] bf16 tile
   static constexpr int Q_OFF = 0;
-  static constexpr int P_OFF = 2 * TILE;                   // per group: P, then phi_q, then the output rows
+  static constexpr int P_OFF = 2 * TILE;                   // per group: phi_q, then the output rows
   static constexpr int KV_OFF = P_OFF + 2 * PTILE;
   static constexpr int BAR_OFF = KV_OFF + KV_STAGES * TILE;
   static constexpr int TOTAL = BAR_OFF + 256 + 1024;       // + slack for the 1024-byte alignment
@@ -62,11 +107,19 @@ struct QLayout {
 // share K_S / V_S in L2).
 // Barrier phases and the K/V ring run on across units.
 //
-// Scores and probabilities live in different memories: S = Q K^T lands in TMEM, the softmax threads read
-// their rows into registers and release the S columns at once, so the next tile's Q K^T is computed while
-// the exponentials run; P goes to shared memory as bf16 and is the A operand of O += P V.  A group's
-// softmax therefore never waits for the tensor pipe in the steady state, and the pipe sees, per key tile
-// and group, one Q K^T block as soon as S is free and one P V block as soon as P is there.
+// Scores and probabilities live in different columns of tensor memory: the softmax threads read their rows of S = Q K^T into
+// registers and release the S columns at once; P goes back into columns of its own as bf16 and is the A operand of O += P V.  A
+// group waits for the tensor pipe neither with its scores nor with P in the steady state, and V is all that the second product
+// reads from shared memory.  (P through shared memory, with score columns for each group at d = 128, before: every key tile cost the
+// threads 16-byte stores, a proxy fence and a tile to wait for.  Measured in turn: 81 frames of full softmax 4940 -> 4720 us in short
+// runs, 81 frames at rate 1/8 710 -> 690, N = 7800 84.4 -> 82.4.)
+//
+// d = 128: both groups use the same 128 score columns in the key loop, in turn: Q_1 K(j)^T follows once group 0 has read its tile j, Q_0 K(j+1)^T once
+// group 1 has read its tile j.  A product into them takes 512 clk, the groups' reads 150 each and their waits and commits as much, so a
+// round is 2100 - 2500 clk where the exponentials of both groups take 2048 at the least: the groups run half a period
+// apart and little waits for the columns.  In the tail, where a group has little else to do than to wait for its next columns, group 1 has
+// the columns of both P's instead (two-layer map with 32 key tiles 920 -> 890 us).  One warp that issues everything in that fixed order, the second product in halves around
+// the next scores, is slower (full softmax 4700 -> 5130 us): issuing blocks it.
 //
 // The work of one unit is a function per role, kept out of line: each role then gets a register
 // allocation of its own (the softmax rows need nearly the whole budget, and the issuing warps must
@@ -99,19 +152,21 @@ AS_DEV int q_units_of_cta(const QParams& p) {
   return p.n_rounds + ((int)blockIdx.x < (p.split_last ? 2 * left : left) + p.n_single ? 1 : 0);
 }
 
-template <int D>
+// Tensor memory, 512 columns: O takes 2 x D, P (bf16 pairs) 2 x 64.  At d = 64 that leaves score columns for each group, at d = 128
+// for one: there the groups take turns at them.
+template <int D, bool SH = (D == 128)>
 struct QRing {
   using L = QLayout<D>;
   // barrier indices; per group: S (scores, hidden activations or Phi landed in the score columns), SF (score
-  // columns read out), P (P or phi_q in shared memory), PF (the product that reads the P tile has completed),
+  // columns read out), P (P in tensor memory, phi_q in shared memory), PF (the product that reads it has completed),
   // O (output accumulator final), QF (nothing of the unit reads the Q tile any more), H (two layers: the
-  // hidden activations are in shared memory)
+  // hidden activations are in shared memory); for both: PL (nothing reads the unit's P in tensor memory any more)
   static constexpr int B_Q0 = 0, B_FULL = 2, B_EMPTY = B_FULL + KV_STAGES, B_S = B_EMPTY + KV_STAGES, B_SF = B_S + 2,
-                       B_P = B_SF + 2, B_PF = B_P + 2, B_O = B_PF + 2, B_QF = B_O + 2, B_H = B_QF + 2, B_COUNT = B_H + 2;
+                       B_P = B_SF + 2, B_PF = B_P + 2, B_O = B_PF + 2, B_QF = B_O + 2, B_H = B_QF + 2, B_PL = B_H + 2, B_COUNT = B_PL + 1;
   const QCtx c;              // by value: nothing here is re-read from memory after a barrier or an MMA
   int nkv, lin, two, fc, nh, vl;
   int n_stream, n_items;
-  int n_s, n_p, n_pf;        // per unit and group: uses of the score columns, P hand-overs, releases of the P tile
+  int n_s, n_p, n_pf;        // per unit and group: uses of the score columns, hand-overs of P or phi_q, products that have read one
   // Ring items of one unit, in the order they are consumed: K_0; then K_{j+1}, V_j for j = 0 .. nkv-2; then
   // the linear tail with V_{nkv-1} in second place:
   //   one layer:   W[0], V_last, then W[c], S[c-1] for c = 1 .. fc-1, then S[fc-1]
@@ -143,8 +198,20 @@ struct QRing {
   AS_DEV uint32_t sP(int g) const { return c.sbase + L::P_OFF + g * L::PTILE; }
   // The K/V ring is indexed by a running item number that does not restart with a unit.
   AS_DEV uint32_t sKV(int item) const { return c.sbase + L::KV_OFF + (item % KV_STAGES) * L::TILE; }
-  AS_DEV uint32_t tS(int g) const { return c.tmem + 128u * g; }
-  AS_DEV uint32_t tO(int g) const { return c.tmem + 256u + 128u * g; }
+  AS_DEV uint32_t tS(int g) const { return SH ? c.tmem : c.tmem + 128u * g; }
+  AS_DEV uint32_t tP(int g) const { return c.tmem + (SH ? 128u : 384u) + 64u * g; }
+  AS_DEV uint32_t tO(int g) const { return c.tmem + 256u + (uint32_t)D * g; }
+  AS_DEV uint32_t tTail(int g) const { return c.tmem + 128u * g; }   // where the products of the linear tail land
+  // Before product i of the unit into group g's score columns, the ph-th of all: what lay there has been read.  With columns of its own
+  // (and in the tail, where group 1 has the columns of both P's) by the group itself; else by the groups in turn.
+  // (A unit of one group, the CTA's last one, follows a unit of two.)
+  AS_DEV bool s_free(int g, int ph, int ng, int i, int u) const {
+    if (!SH || i > nkv || nkv == 0) return ph == 0 ? true : wait(B_SF + g, ph - 1);
+    if (g == 1) return i < nkv ? wait(B_SF, ph) : wait(B_PL, u);
+    if (ph == 0) return true;
+    if (i == 0 && !wait(B_SF, ph - 1)) return false;   // the unit before: group 0's rows lay here, group 1's where P_0 will go
+    return wait(B_SF + (ng == 2 || i == 0 ? 1 : 0), ph - 1);
+  }
   AS_DEV bool wait(int b, int phase) const { return mbar_wait_warp(bar(b), phase & 1, c.wc); }
   AS_DEV void release(int item) const { tc_commit(bar(B_EMPTY + item % KV_STAGES)); }
   AS_DEV bool wait_full(int item) const { return wait(B_FULL + item % KV_STAGES, item / KV_STAGES); }
@@ -208,17 +275,17 @@ __device__ __noinline__ bool q_produce_unit(const QParams& p, const QCtx& c, con
 }
 
 // ---------------------------------------------------------------- MMA issuers, one unit
-// Two issuing warps (9 and 10): one issues what writes the score columns (Q K^T per tile, Phi at the end) as soon as
+// Two issuing warps: one issues what writes the score columns (Q K^T per tile, Phi at the end) as soon as
 // the softmax threads have read them out, the other what accumulates into O (P V per tile, phi_q S at the end) as soon as
-// P is in shared memory.  The two streams touch different TMEM columns and release different ring items, so they
+// P is there.  The two streams touch different TMEM columns and release different ring items, so they
 // need no ordering between them; each warp's commits cover its own MMAs.  The whole warp walks the loop and one elected
 // lane issues: from converged code the operands of an MMA sit in uniform registers.  With a single thread in a branch of
 // its own, eight MMAs took 630 - 700 clk to issue beside the softmax warps (N = 64, d = 64: as long, though they execute in
 // 380); now 320 - 380 (130 for the four of Q K^T at d = 64).  N = 7800: 96.3 -> 93.7 us, headline layer 838 -> 830 us
 // (sustained), two-layer map 1203 -> 1176 us.
-template <int D, bool TWO, bool GEN>
+template <int D, bool TWO, bool GEN, bool SH>
 __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u) {
-  using R = QRing<D>;
+  using R = QRing<D, SH>;
   constexpr uint32_t ID_QK = make_idesc(128, 128, 0, 0);      // S = Q K^T      (N = 128 keys)
   const int nkv = p.nkv, lin = p.lin;
   const R q(p, c, true);
@@ -233,9 +300,7 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
 #pragma unroll
     for (int kk = 0; kk < 8; ++kk) dq[g][kk] = q0 + kstep_kmajor(kk);
   }
-  // The i-th product of the unit into a group's score columns overwrites what the threads read last: the
-  // (i-1)-th use, or the previous unit's last one.
-  auto s_free = [&](int g, int i) -> bool { return (u == 0 && i == 0) ? true : q.wait(R::B_SF + g, ps + i - 1); };
+  auto s_free = [&](int g, int i) -> bool { return q.s_free(g, ps + i, ng, i, u); };
 
   // ---- first key tile (its product opens the unit)
   if (nkv > 0) {
@@ -262,7 +327,7 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
     for (int g = 0; g < 2; ++g) {
       if (g >= ng) break;
       if (g == 0 && !q.wait_full(ik)) return false;
-      if (!q.wait(R::B_SF + g, ps + j)) return false;
+      if (!s_free(g, j + 1)) return false;
       tc_fence_after();
       if (elect_one()) {
 #pragma unroll
@@ -288,7 +353,7 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
         tc_fence_after();
         if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tS(g), dq[g][kk], w0 + kstep_kmajor(kk), id_phi, kk > 0 ? 1u : 0u);
+          for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tTail(g), dq[g][kk], w0 + kstep_kmajor(kk), id_phi, kk > 0 ? 1u : 0u);
           tc_commit(q.bar(R::B_S + g));
           if (ch == q.fc - 1) tc_commit(q.bar(R::B_QF + g));     // nothing of this unit reads the group's Q tile any more
         }
@@ -298,7 +363,7 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
     return true;
   } else {
   // two layers: hidden slices first (A = Q), then Phi_c = sum_j h1_j W2[c, j]^T with the hidden slices read from
-  // where the threads put them: slice 0 in the group's P tile, slice 1 in its Q tile
+  // where the threads put them: slice 0 in the group's phi_q tile, slice 1 in its Q tile
   for (int j = 0; j < q.nh; ++j) {
     const int iw = base + q.it_w(j);
     const uint64_t w0 = kmajor_desc(q.sKV(iw));
@@ -309,7 +374,7 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
       tc_fence_after();
       if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tS(g), dq[g][kk], w0 + kstep_kmajor(kk), ID_HID, kk > 0 ? 1u : 0u);
+        for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tTail(g), dq[g][kk], w0 + kstep_kmajor(kk), ID_HID, kk > 0 ? 1u : 0u);
         tc_commit(q.bar(R::B_S + g));
         if (q.nh == 1 && q.fc == 1) tc_commit(q.bar(R::B_QF + g));   // the Q tile is not reused as a buffer in this shape
       }
@@ -317,53 +382,44 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
     if (elect_one()) q.release(iw);
   }
   for (int ch = 0; ch < q.fc; ++ch) {
-    for (int j = 0; j < q.nh; ++j) {
-      const int iw = base + q.it_w2(ch, j);
-      const uint64_t w0 = kmajor_desc(q.sKV(iw));
-      if (!q.wait_full(iw)) return false;
-      for (int g = 0; g < ng; ++g) {
-        if (j == 0) {
-          if (!s_free(g, nkv + q.nh + ch)) return false;
-          if (ch == 0 && !q.wait(R::B_H + g, u)) return false;   // the group's hidden activations are in shared memory
-        }
+    for (int g = 0; g < ng; ++g) {
+      if (!s_free(g, nkv + q.nh + ch)) return false;
+      if (ch == 0 && !q.wait(R::B_H + g, u)) return false;       // the group's hidden activations are in shared memory
+      for (int j = 0; j < q.nh; ++j) {
+        const int iw = base + q.it_w2(ch, j);
+        const uint64_t w0 = kmajor_desc(q.sKV(iw));
+        if (g == 0 && !q.wait_full(iw)) return false;
         tc_fence_after();
         const uint64_t a0 = kmajor_desc(j == 0 ? q.sP(g) : q.sQ(g));
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < D / 16; ++kk)
-            mma_ss(q.tS(g), a0 + kstep_kmajor(kk), w0 + kstep_kmajor(kk), id_phi, (j > 0 || kk > 0) ? 1u : 0u);
+            mma_ss(q.tTail(g), a0 + kstep_kmajor(kk), w0 + kstep_kmajor(kk), id_phi, (j > 0 || kk > 0) ? 1u : 0u);
           if (j == q.nh - 1) {
             tc_commit(q.bar(R::B_S + g));
             // two hidden slices, one feature chunk: this was the last read of the Q tile (as a buffer)
             if (q.nh == 2 && q.fc == 1) tc_commit(q.bar(R::B_QF + g));
           }
+          if (g == ng - 1) q.release(iw);
         }
       }
-      if (elect_one()) q.release(iw);
     }
   }
   return true;
   }
 }
 
-template <int D, bool TWO, bool GEN>
+template <int D, bool TWO, bool GEN, bool SH>
 __device__ __noinline__ bool q_accum_unit(const QParams& p, const QCtx& c, int u) {
-  using R = QRing<D>;
+  using R = QRing<D, SH>;
   constexpr uint32_t ID_PV = make_idesc(128, D, 0, 1);        // O += P V and O += phi_q S  (V, S are MN-major)
   const int nkv = p.nkv, lin = p.lin;
   const R q(p, c, true);
   const int base = u * q.n_items, pp = u * q.n_p;             // first ring item / first P hand-over phase of the unit
   const int ng = q_unit(p, u).ng;
-  uint64_t dp[2][8];                                          // the P tiles never move
-#pragma unroll
-  for (int g = 0; g < 2; ++g) {
-    const uint64_t p0 = kmajor_desc(q.sP(g));
-#pragma unroll
-    for (int kk = 0; kk < 8; ++kk) dp[g][kk] = p0 + kstep_kmajor(kk);
-  }
   for (int j = 0; j < nkv; ++j) {
     const bool last = (j + 1 == nkv);
-    // as soon as P is in shared memory: O += P V
+    // as soon as P is there: O += P V
     const int iv = base + q.item_v(j);
     const uint64_t v0 = mnmajor_desc(q.sKV(iv));
 #pragma unroll
@@ -374,15 +430,16 @@ __device__ __noinline__ bool q_accum_unit(const QParams& p, const QCtx& c, int u
       tc_fence_after();
       if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) mma_ss(q.tO(g), dp[g][kk], v0 + kstep_mnmajor(kk), ID_PV, (j > 0 || kk > 0) ? 1u : 0u);
+        for (int kk = 0; kk < 8; ++kk) mma_ts(q.tO(g), q.tP(g) + kk * 8, v0 + kstep_mnmajor(kk), ID_PV, (j > 0 || kk > 0) ? 1u : 0u);
         tc_commit(q.bar(R::B_PF + g));
         if (last && !lin) tc_commit(q.bar(R::B_O + g));
+        if (SH && last && lin && g == 1) tc_commit(q.bar(R::B_PL));    // (the other group's product was issued before)
       }
     }
     if (elect_one()) q.release(iv);
   }
   if (!lin) return true;
-  // O += phi_q,c S_c per feature chunk: phi_q sits where P sits (two layers, second chunk: in the Q tile),
+  // O += phi_q,c S_c per feature chunk: phi_q sits in its tile (two layers, second chunk: in the Q tile),
   // S plays the part of a V tile
   const int ksteps = (D == 128 ? 128 : p.fcw) / 16;           // a constant at d = 128: the chains below unroll
   for (int ch = 0; ch < q.fc; ++ch) {
@@ -393,12 +450,12 @@ __device__ __noinline__ bool q_accum_unit(const QParams& p, const QCtx& c, int u
       if (g == 0 && !q.wait_full(is)) return false;
       if (!q.wait(R::B_P + g, pp + nkv + ch)) return false;
       tc_fence_after();
-      const uint64_t a0 = in_q_tile ? kmajor_desc(q.sQ(g)) : dp[g][0];
+      const uint64_t a0 = kmajor_desc(in_q_tile ? q.sQ(g) : q.sP(g));
       if (elect_one()) {
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)
           if (kk < ksteps) mma_ss(q.tO(g), a0 + kstep_kmajor(kk), s0 + kstep_mnmajor(kk), ID_PV, (nkv > 0 || ch > 0 || kk > 0) ? 1u : 0u);
-        if (!in_q_tile) tc_commit(q.bar(R::B_PF + g));           // a reader of the P tile has completed
+        if (!in_q_tile) tc_commit(q.bar(R::B_PF + g));           // a reader of the phi_q tile has completed
         if (ch == q.fc - 1) {
           tc_commit(q.bar(R::B_O + g));
           if (in_q_tile) tc_commit(q.bar(R::B_QF + g));          // ... and the last reader of the Q tile
@@ -411,77 +468,38 @@ __device__ __noinline__ bool q_accum_unit(const QParams& p, const QCtx& c, int u
 }
 
 // ---------------------------------------------------------------- feature rows of the linear tail
-// One row of Phi (feature chunk ch), already read out of the score columns into ph -> bf16(lam * poly(relu(Phi + b)))
-// -> row r of `tile` (the A operand of the apply product).  Returns the row's share of phi_q.z, formed with the very
-// bf16 values the MMA multiplies with S.  GEN = false is the common case (no bias, polynomial degree <= 2).
-template <int D, bool GEN>
-AS_DEV float q_features_to_tile(const QParams& p, const uint32_t (&ph)[128], uint8_t* tile, int r, int bh, int ch, float lam) {
-  const int fcw = D == 128 ? 128 : p.fcw;            // a chunk is narrower than 128 only at d = F = 64
+// A thread's share of a row of Phi (feature chunk ch) from the score columns -> bf16(lam * poly(relu(Phi + b))) -> row r of `tile` (the A operand
+// of the apply product), 32 columns at a time (the loop is not unrolled: the tail runs once per unit, and on a CTA's first
+// unit its instructions come from L2 line by line, so its size is its cost).  Arrives on `sf_bar` once the last columns
+// are in registers.  Returns the share's part of phi_q.z, formed with the very bf16 values the MMA multiplies with S.
+// GEN = false is the common case (no bias, polynomial degree <= 2).
+template <int D, int T, bool GEN>
+AS_DEV float q_features_from_tmem(const QParams& p, uint32_t tSg, uint32_t sf_bar, uint8_t* tile, int r, int hc, int bh, int ch, float lam) {
+  constexpr int TPR = T;
+  const int fcw = D == 128 ? 128 : p.fcw, half = fcw / TPR;
   const int part = p.F / p.P;
-  const float2* zrow = reinterpret_cast<const float2*>(p.z + (size_t)bh * p.F + ch * 128);
+  const float2* zrow = reinterpret_cast<const float2*>(p.z + (size_t)bh * p.F + ch * 128 + hc * half);
   const uint32_t* brow = nullptr;
-  if (GEN && p.b2 != nullptr) brow = reinterpret_cast<const uint32_t*>(p.b2 + (size_t)(bh % p.H) * p.F + ch * 128);
-  float dl0 = 0.f, dl1 = 0.f;
-#pragma unroll
-  for (int cc = 0; cc < 4; ++cc) {
-    if (cc * 32 < fcw) {
-      const int pw = min((ch * 128 + cc * 32) / part, p.P - 1);     // 0-based part of these 32 features
-      uint32_t wd[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        float a0 = __uint_as_float(ph[cc * 32 + 2 * i]), a1 = __uint_as_float(ph[cc * 32 + 2 * i + 1]);
-        if (GEN && brow != nullptr) {
-          const uint32_t bb = __ldg(brow + cc * 16 + i);            // same address in every lane: one broadcast load
-          a0 += __uint_as_float(bb << 16);
-          a1 += __uint_as_float(bb & 0xffff0000u);
-        }
-        a0 = fmaxf(a0, 0.f); a1 = fmaxf(a1, 0.f);
-        float r0 = a0, r1 = a1;
-        if (pw >= 1) { r0 *= a0; r1 *= a1; }
-        if (GEN) {
-          if (pw >= 2) { r0 *= a0; r1 *= a1; }
-          if (pw >= 3) { r0 *= a0; r1 *= a1; }
-        }
-        wd[i] = pack_bf16(r0 * lam, r1 * lam);
-        const float2 zz = __ldg(zrow + cc * 16 + i);
-        dl0 = fmaf(__uint_as_float(wd[i] << 16), zz.x, dl0);
-        dl1 = fmaf(__uint_as_float(wd[i] & 0xffff0000u), zz.y, dl1);
-      }
-      store_row_chunk(tile, r, cc * 32, wd);
-    }
-  }
-  fence_proxy_async();
-  return dl0 + dl1;
-}
-
-// The same for the one-layer tail, 32 columns at a time straight from the score columns (the loop is not unrolled:
-// the tail runs once per unit, and on a CTA's first unit its instructions come from L2 line by line, so its
-// size is its cost).  Arrives on `sf_bar` once the last columns are in registers.
-template <int D, bool GEN>
-AS_DEV float q_features_from_tmem(const QParams& p, uint32_t tSg, uint32_t sf_bar, uint8_t* tile, int r, int bh, int ch, float lam) {
-  const int fcw = D == 128 ? 128 : p.fcw;
-  const int part = p.F / p.P;
-  const float2* zrow = reinterpret_cast<const float2*>(p.z + (size_t)bh * p.F + ch * 128);
-  const uint32_t* brow = nullptr;
-  if (GEN && p.b2 != nullptr) brow = reinterpret_cast<const uint32_t*>(p.b2 + (size_t)(bh % p.H) * p.F + ch * 128);
+  if (GEN && p.b2 != nullptr) brow = reinterpret_cast<const uint32_t*>(p.b2 + (size_t)(bh % p.H) * p.F + ch * 128 + hc * half);
   const float2 lam2 = make_float2(lam, lam);
   float2 dl2 = make_float2(0.f, 0.f);
   uint32_t x[32];
 #pragma unroll 1
-  for (int cc = 0; cc * 32 < fcw; ++cc) {
-    tmem_ld32(tSg + cc * 32, x);
+  for (int cc = 0; cc * 32 < half; ++cc) {
+    if (D == 128 || fcw == 128) q_ld32<TPR, 64>(tSg + cc * 32, x);
+    else q_ld32<TPR, 32>(tSg + cc * 32, x);
     tmem_ld_wait(x);
-    if (cc * 32 + 32 >= fcw) {
+    if (cc * 32 + 32 >= half) {
       tc_fence_before();
       mbar_arrive(sf_bar);                             // the next product into the score columns may follow
     }
-    const int pw = min((ch * 128 + cc * 32) / part, p.P - 1);     // 0-based part of these 32 features
+    const int pw = min((ch * 128 + hc * half + cc * 32) / part, p.P - 1);     // 0-based part of these 32 features
     uint32_t wd[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       float a0 = __uint_as_float(x[2 * i]), a1 = __uint_as_float(x[2 * i + 1]);
       if (GEN && brow != nullptr) {
-        const uint32_t bb = __ldg(brow + cc * 16 + i);            // same address in every lane: one broadcast load
+        const uint32_t bb = __ldg(brow + cc * 16 + i);            // same address in all lanes, or in half of them: broadcast loads
         a0 += __uint_as_float(bb << 16);
         a1 += __uint_as_float(bb & 0xffff0000u);
       }
@@ -497,53 +515,69 @@ AS_DEV float q_features_from_tmem(const QParams& p, uint32_t tSg, uint32_t sf_ba
       const float2 zz = __ldg(zrow + cc * 16 + i);
       dl2 = __ffma2_rn(make_float2(__uint_as_float(wd[i] << 16), __uint_as_float(wd[i] & 0xffff0000u)), zz, dl2);
     }
-    store_row_chunk(tile, r, cc * 32, wd);
+    store_row_chunk(tile, r, hc * half + cc * 32, wd);
   }
   fence_proxy_async();
   return dl2.x + dl2.y;
 }
 
-// Reads one row of the score columns (ncols of them) at once and releases the columns.
-template <int D>
-AS_DEV void q_read_row(const QRing<D>& q, int g, uint32_t tSg, int ncols, uint32_t (&ph)[128]) {
+// One-layer feature map, one unit and group: the feature chunks, one after the other.  Adds this thread's part of phi_q.z to dl;
+// false: a wait ran out.
+template <int D, int T, bool GEN>
+AS_DEV bool q_one_layer_tail(const QParams& p, const QRing<D>& q, int g, uint32_t tSg, uint8_t* sPg, int r, int hc, int bh, int ps, int ppf, float lam,
+                             float& dl) {
   using R = QRing<D>;
-  uint32_t x[32];
-#pragma unroll
-  for (int cc = 0; cc < 4; ++cc) {
-    if (cc * 32 < ncols) {
-      tmem_ld32(tSg + cc * 32, x);
-      tmem_ld_wait(x);
-#pragma unroll
-      for (int i = 0; i < 32; ++i) ph[cc * 32 + i] = x[i];
-    }
+  const int nkv = p.nkv;
+  for (int ch = 0; ch < q.fc; ++ch) {
+    if (!q.wait(R::B_S + g, ps + nkv + ch)) return false;
+    tc_fence_after();
+    // the tile may be written once this warp's previous output store has been read out and the previous chunk's product has read it
+    if ((threadIdx.x & 31) == 0) tma_store_wait_read();
+    if (ch == 0) __syncwarp();
+    else if (!q.wait(R::B_PF + g, ppf + nkv + ch - 1)) return false;
+    dl += q_features_from_tmem<D, T, GEN>(p, tSg, q.bar(R::B_SF + g), sPg, r, hc, bh, ch, lam);   // the A operand of the apply product
+    // not before every thread of the group has arrived for the last key tile
+    if (ch == 0 && ppf + nkv > 0 && !q.wait(R::B_PF + g, ppf + nkv - 1)) return false;
+    mbar_arrive(q.bar(R::B_P + g));
   }
-  tc_fence_before();
-  mbar_arrive(q.bar(R::B_SF + g));                   // the next product into the score columns may follow
+  return true;
 }
 
-// Two-layer feature map, one unit and group: hidden slices relu(Q W_1[j]^T + b_1) as bf16 (slice 0 into the P tile,
+// The same out of line.  With a score row in a thread's registers the key loop spills some of what it needs in every tile when the tail stands
+// beside it (81 frames at rate 1/8 717 us, full softmax 4840; with this 697 and 4675); with half a row it does not, and the call
+// costs more (d = 64, 2142 keys 279 -> 290).
+template <int D, int T, bool GEN>
+__device__ __noinline__ bool q_one_layer_tail_apart(const QParams& p, const QCtx& c, int g, uint32_t tSg, uint8_t* sPg, int r, int hc, int bh, int ps, int ppf,
+                                                    float lam, float& dl) {
+  float sum = 0.f;
+  const bool ok = q_one_layer_tail<D, T, GEN>(p, QRing<D>(p, c), g, tSg, sPg, r, hc, bh, ps, ppf, lam, sum);
+  dl = sum;
+  return ok;
+}
+
+// Two-layer feature map, one unit and group: hidden slices relu(Q W_1[j]^T + b_1) as bf16 (slice 0 into the phi_q tile,
 // slice 1 into the Q tile, free once the product that made slice 1, the last reader of Q, has completed), then the
 // feature chunks.  Returns phi_q.z, or -1 when a wait ran out.
-template <int D, bool GEN>
-__device__ __noinline__ float q_two_layer_tail(const QParams& p, const QRing<D>& q, int g, uint32_t tSg, uint8_t* sPg, uint8_t* sQg,
-                                               int r, int bh, int ps, int ppf, float lam) {
+template <int D, int T, bool GEN>
+__device__ __noinline__ float q_two_layer_tail(const QParams& p, const QRing<D>& q, int g, uint32_t tSg, uint8_t* sPg, uint8_t* sQg, int r, int hc,
+                                               int bh, int ps, int ppf, float lam) {
   using R = QRing<D>;
+  constexpr int TPR = T, DC = D / TPR, FC = 128 / TPR;   // hidden units / features of a slice / chunk per thread
   const int nkv = p.nkv, h = bh % p.H, lane = threadIdx.x & 31;
   const __nv_bfloat16* b1 = (GEN && p.b1) ? p.b1 + (size_t)h * (q.nh * D) : nullptr;
   uint32_t x[32];
   for (int j = 0; j < q.nh; ++j) {
     if (!q.wait(R::B_S + g, ps + nkv + j)) return -1.f;
     tc_fence_after();
-    if (j == 0) {                                    // the last tile's P V has read the P tile (cf. the key loop)
+    if (j == 0) {                                    // this warp's output store of the previous unit has read its rows
       if (lane == 0) tma_store_wait_read();
-      if (ppf + nkv == 0) __syncwarp();
-      else if (!q.wait(R::B_PF + g, ppf + nkv - 1)) return -1.f;
+      __syncwarp();
     }
-    const uint32_t* brow = b1 ? reinterpret_cast<const uint32_t*>(b1 + j * D) : nullptr;
+    const uint32_t* brow = b1 ? reinterpret_cast<const uint32_t*>(b1 + j * D + hc * DC) : nullptr;
     uint8_t* tile = j == 0 ? sPg : sQg;
 #pragma unroll
-    for (int cc = 0; cc < D / 32; ++cc) {
-      tmem_ld32(tSg + cc * 32, x);
+    for (int cc = 0; cc < DC / 32; ++cc) {
+      q_ld32<TPR, D / 2>(tSg + cc * 32, x);
       tmem_ld_wait(x);
       uint32_t wd[16];
 #pragma unroll
@@ -556,37 +590,35 @@ __device__ __noinline__ float q_two_layer_tail(const QParams& p, const QRing<D>&
         }
         wd[i] = pack_bf16(fmaxf(a0, 0.f), fmaxf(a1, 0.f));
       }
-      store_row_chunk(tile, r, cc * 32, wd);
+      store_row_chunk(tile, r, hc * DC + cc * 32, wd);
     }
     tc_fence_before();
     mbar_arrive(q.bar(R::B_SF + g));
     fence_proxy_async();
     mbar_arrive(q.bar(R::B_H + g));
   }
-  // Feature chunks.  The hidden slices stay in their buffers until the last chunk's product has completed, so with
-  // two chunks the first one's features wait in shared memory nobody else uses at that time: the rows of the group's
-  // P tile are still the hidden slice, but ... (see below)
+  // (waits by parity look at every phase in turn)
+  if (ppf + nkv > 0 && !q.wait(R::B_PF + g, ppf + nkv - 1)) return -1.f;
+  // Feature chunks.  The hidden slices stay in their buffers until the last chunk's product has completed.
   if (!q.wait(R::B_S + g, ps + nkv + q.nh)) return -1.f;
   tc_fence_after();
-  if (q.fc == 1) {
-    uint32_t ph[128];
-    q_read_row<D>(q, g, tSg, D == 128 ? 128 : p.fcw, ph);
-    const float dl = q_features_to_tile<D, GEN>(p, ph, sPg, r, bh, 0, lam);   // Phi_0 is complete: nothing reads the slices any more
+  if (q.fc == 1) {                                   // Phi_0 is complete: nothing reads the slices any more
+    const float dl = q_features_from_tmem<D, T, GEN>(p, tSg, q.bar(R::B_SF + g), sPg, r, hc, bh, 0, lam);
     mbar_arrive(q.bar(R::B_P + g));
     return dl;
   }
   // two chunks: chunk 0 is kept as bf16 pairs in registers until Phi_1 has landed (then the slices are free)
   float dl0 = 0.f, dl1 = 0.f;
-  uint32_t pk[64];
+  uint32_t pk[FC / 32][16];
   {
     const int part = p.F / p.P;
-    const float2* zrow = reinterpret_cast<const float2*>(p.z + (size_t)bh * p.F);
-    const uint32_t* brow = (GEN && p.b2) ? reinterpret_cast<const uint32_t*>(p.b2 + (size_t)h * p.F) : nullptr;
+    const float2* zrow = reinterpret_cast<const float2*>(p.z + (size_t)bh * p.F + hc * FC);
+    const uint32_t* brow = (GEN && p.b2) ? reinterpret_cast<const uint32_t*>(p.b2 + (size_t)h * p.F + hc * FC) : nullptr;
 #pragma unroll
-    for (int cc = 0; cc < 4; ++cc) {
-      tmem_ld32(tSg + cc * 32, x);
+    for (int cc = 0; cc < FC / 32; ++cc) {
+      q_ld32<TPR, 64>(tSg + cc * 32, x);
       tmem_ld_wait(x);
-      const int pw = min((cc * 32) / part, p.P - 1);
+      const int pw = min((hc * FC + cc * 32) / part, p.P - 1);
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
         float a0 = __uint_as_float(x[2 * i]), a1 = __uint_as_float(x[2 * i + 1]);
@@ -601,7 +633,7 @@ __device__ __noinline__ float q_two_layer_tail(const QParams& p, const QRing<D>&
         if (pw >= 2) { r0 *= a0; r1 *= a1; }
         if (pw >= 3) { r0 *= a0; r1 *= a1; }
         const uint32_t wv = pack_bf16(r0 * lam, r1 * lam);
-        pk[cc * 16 + i] = wv;
+        pk[cc][i] = wv;
         const float2 zz = __ldg(zrow + cc * 16 + i);
         dl0 = fmaf(__uint_as_float(wv << 16), zz.x, dl0);
         dl1 = fmaf(__uint_as_float(wv & 0xffff0000u), zz.y, dl1);
@@ -613,67 +645,56 @@ __device__ __noinline__ float q_two_layer_tail(const QParams& p, const QRing<D>&
   if (!q.wait(R::B_S + g, ps + nkv + q.nh + 1)) return -1.f;     // Phi_1 is there: nothing reads the hidden slices any more
   tc_fence_after();
 #pragma unroll
-  for (int cc = 0; cc < 4; ++cc) {
-    uint32_t wd[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) wd[i] = pk[cc * 16 + i];
-    store_row_chunk(sPg, r, cc * 32, wd);
-  }
+  for (int cc = 0; cc < FC / 32; ++cc) store_row_chunk(sPg, r, hc * FC + cc * 32, pk[cc]);
   fence_proxy_async();
   mbar_arrive(q.bar(R::B_P + g));
-  uint32_t ph[128];
-  q_read_row<D>(q, g, tSg, 128, ph);
-  const float dlb = q_features_to_tile<D, GEN>(p, ph, sQg, r, bh, 1, lam);
+  const float dlb = q_features_from_tmem<D, T, GEN>(p, tSg, q.bar(R::B_SF + g), sQg, r, hc, bh, 1, lam);
+  // not before every thread of the group has arrived for the first chunk
+  if (!q.wait(R::B_PF + g, ppf + nkv)) return -1.f;
   mbar_arrive(q.bar(R::B_P + g));
   return (dl0 + dl1) + dlb;
 }
 
 // ---------------------------------------------------------------- softmax / merge group, one unit
-template <int D, bool TWO, bool GEN>
+template <int D, int T, bool TWO, bool GEN>
 __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, const CUtensorMap* tmO, uint8_t* smem, int u) {
   using R = QRing<D>;
   using L = QLayout<D>;
+  using X = QShape<D, T>;
   const int nkv = p.nkv, n_s = p.n_s;
   const float scale_log2 = p.scale_log2;
   const R q(p, c);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = warp >> 2;                          // group 0 or 1
-  const int r = (warp & 3) * 32 + lane;             // row inside the group's 128-row tile
-  const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
-  const uint32_t tSg = q.tS(g) + lane_off, tOg = q.tO(g) + lane_off;
-  uint8_t* sPg = smem + L::P_OFF + g * L::PTILE;    // this group's P / phi_q / output staging tile
+  const int g = (warp >> 2) & 1;                    // group 0 or 1
+  const int r0 = (warp & 3) * 32 + (X::TPR == 2 ? (warp >> 3) * 16 : 0);   // this warp's rows of the group's 128-row tile
+  const int r = r0 + (X::TPR == 2 ? lane & 15 : lane), hc = X::TPR == 2 ? lane >> 4 : 0;   // this thread's row, its share of the columns
+  const uint32_t lane_off = (uint32_t)r0 << 16;
+  const uint32_t tSg = q.tS(g) + lane_off, tOg = q.tO(g) + lane_off, tPg = q.tP(g) + lane_off;
+  uint8_t* sPg = smem + L::P_OFF + g * L::PTILE;    // this group's phi_q / output staging tile
   const int ps = u * q.n_s, ppf = u * q.n_pf;       // first phases of the unit (cf. QRing)
   float m_ref = 0.f, m_true = -INFINITY, l = 0.f;
-  uint32_t x[32];
-
-  // The P buffer may be written once the product that read its previous contents has completed; the very
-  // first use only has to wait for this warp's output store of the previous unit to have been read out.
-  auto p_buffer_free = [&](int use) -> bool {       // use: running index of the buffer's uses
-    if (lane == 0) tma_store_wait_read();
-    if (use == 0) { __syncwarp(); return true; }
-    return q.wait(R::B_PF + g, use - 1);
-  };
 
   for (int j = 0; j < nkv; ++j) {
     if (!q.wait(R::B_S + g, ps + j)) return false;
     tc_fence_after();
-    uint32_t sv[128];                               // this thread's row of the 128 x 128 score tile
-    tmem_ld128_sync(tSg, sv);
+    uint32_t sv[X::COLS];                           // this thread's share of its row of the 128 x 128 score tile
+    if constexpr (X::TPR == 1) tmem_ld128_sync(tSg, sv); else tmem_ldh64_sync<64>(tSg, sv);
     tc_fence_before();
     mbar_arrive(q.bar(R::B_SF + g));                // the score columns may be overwritten
-    const int valid = n_s - j * 128;                // keys of this tile that exist (>= 128: all)
-    if (valid < 128) {
+    if (n_s - j * 128 < 128) {
+      const int valid = n_s - j * 128 - hc * X::COLS;   // this thread's keys of the tile that exist
 #pragma unroll
-      for (int i = 0; i < 128; ++i) sv[i] = (i < valid) ? sv[i] : 0xff800000u;   // -inf: exp2 gives 0
+      for (int i = 0; i < X::COLS; ++i) sv[i] = (i < valid) ? sv[i] : 0xff800000u;   // -inf: exp2 gives 0
     }
     float mx0 = fmax3(__uint_as_float(sv[0]), __uint_as_float(sv[1]), __uint_as_float(sv[2]));
     float mx1 = fmax3(__uint_as_float(sv[3]), __uint_as_float(sv[4]), __uint_as_float(sv[5]));
 #pragma unroll
-    for (int i = 6; i + 3 < 128; i += 4) {
+    for (int i = 6; i + 3 < X::COLS; i += 4) {
       mx0 = fmax3(mx0, __uint_as_float(sv[i]), __uint_as_float(sv[i + 1]));
       mx1 = fmax3(mx1, __uint_as_float(sv[i + 2]), __uint_as_float(sv[i + 3]));
     }
-    float mx = fmax3(mx0, mx1, fmaxf(__uint_as_float(sv[126]), __uint_as_float(sv[127])));
+    float mx = fmax3(mx0, mx1, fmaxf(__uint_as_float(sv[X::COLS - 2]), __uint_as_float(sv[X::COLS - 1])));
+    if (X::TPR == 2) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));   // the other half of the row
     mx *= scale_log2;
     m_true = fmaxf(m_true, mx);
     // The reference maximum only moves when the row maximum grew by more than 2^8; then O and l
@@ -681,27 +702,46 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
     const bool need = (j > 0) && (mx > m_ref + RESCALE_THRESHOLD);
     const float resc = need ? ex2(m_ref - mx) : 1.f;
     if (j == 0 || need) m_ref = mx;
-    // P = exp2(s * scale_log2 - m_ref) as bf16 into the group's P tile in shared memory
+    // P = exp2(s * scale_log2 - m_ref) as bf16 into the group's columns of tensor memory
     const float neg_m = -m_ref;
     // packed fp32x2 arithmetic halves the instruction count of the scaling and of the row sum
     const float2 scale2 = make_float2(scale_log2, scale_log2), negm2 = make_float2(neg_m, neg_m);
     float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
+    // Whether the previous tile's P V has completed is asked here and looked at behind the first exponentials (d = 128: a wait for
+    // something that is already there costs a round trip; at d = 64 the other warps cover it)
+    bool p_free = false;
+    if (X::TPR == 1 && ppf + j > 0) p_free = mbar_try_wait(q.bar(R::B_PF + g), (ppf + j - 1) & 1);
 #pragma unroll
-    for (int cc = 0; cc < 4; ++cc) {
+    for (int cc = 0; cc < X::COLS / 32; ++cc) {
       uint32_t pw[16];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int k = cc * 32 + 4 * i;
         const float2 xa = __ffma2_rn(make_float2(__uint_as_float(sv[k]), __uint_as_float(sv[k + 1])), scale2, negm2);
         const float2 xb = __ffma2_rn(make_float2(__uint_as_float(sv[k + 2]), __uint_as_float(sv[k + 3])), scale2, negm2);
-        const float2 pa = make_float2(ex2(xa.x), ex2(xa.y)), pc = make_float2(ex2(xb.x), ex2(xb.y));
+        const float2 pa = make_float2(ex2(xa.x), ex2(xa.y));
+        const float2 pc = EX2_FMA_EVERY<T> > 0 && i % (EX2_FMA_EVERY<T> + (EX2_FMA_EVERY<T> == 0)) == EX2_FMA_EVERY<T> - 1 ? ex2_fma(xb) : make_float2(ex2(xb.x), ex2(xb.y));
         la = __fadd2_rn(la, pa);
         lb = __fadd2_rn(lb, pc);
         pw[2 * i] = pack_bf16(pa.x, pa.y);
         pw[2 * i + 1] = pack_bf16(pc.x, pc.y);
       }
-      if (cc == 0 && !p_buffer_free(ppf + j)) return false;  // the previous tile's P V has read the buffer
-      store_row_chunk(sPg, r, cc * 32, pw);
+      if (cc == 0) {                                // the previous tile's P V has read the columns of P
+        if (ppf + j > 0 && (X::TPR == 2 || !__all_sync(0xffffffffu, p_free)) && !q.wait(R::B_PF + g, ppf + j - 1)) return false;
+        tc_fence_after();
+        if (__any_sync(0xffffffffu, need)) {        // ... and left its sum in O, which no product touches until this tile's P is handed over
+#pragma unroll 1
+          for (int o = 0; o < D / X::TPR; o += 16) {
+            uint32_t y[16];
+            q_ld16<X::TPR, D / 2>(tOg + o, y);
+            tmem_ld16_wait(y);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) y[i] = __float_as_uint(__uint_as_float(y[i]) * resc);
+            q_st16<X::TPR, D / 2>(tOg + o, y);
+          }
+        }
+      }
+      q_st16<X::TPR, 32>(tPg + cc * 16, pw);
     }
     // The sum above adds the unrounded probabilities while the MMA multiplies their bf16 roundings with V.
     // Over many keys the rounding errors average out, but the error of a probability that dominates its
@@ -709,27 +749,15 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
     // sum takes over the rounding error of the tile's largest probability.
     const float p_top = ex2(mx - m_ref);
     const float p_top_err = __uint_as_float(pack_bf16(0.f, p_top) & 0xffff0000u) - p_top;
-    l = l * resc + (((la.x + la.y) + (lb.x + lb.y)) + p_top_err);
-    if (__any_sync(0xffffffffu, need)) {
-      // the previous tile's P V has completed (waited for above) and this tile's has not been released yet
-      tc_fence_after();
-#pragma unroll
-      for (int cc = 0; cc < D / 32; ++cc) {
-        tmem_ld32(tOg + cc * 32, x);
-        tmem_ld_wait(x);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) x[i] = __float_as_uint(__uint_as_float(x[i]) * resc);
-        tmem_st32(tOg + cc * 32, x);
-      }
-      tmem_st_wait();
-      tc_fence_before();
-    }
-    fence_proxy_async();
+    l = l * resc + (((la.x + la.y) + (lb.x + lb.y)) + (X::TPR == 1 || hc == 0 ? p_top_err : 0.f));
+    tmem_st_wait();
+    tc_fence_before();
     mbar_arrive(q.bar(R::B_P + g));
   }
 
   const QUnit un = q_unit(p, u);
   const int bh = un.bh;
+  if (X::TPR == 2) l += __shfl_xor_sync(0xffffffffu, l, 16);
   const int row = un.row0 + g * 128 + r;
   float den = l, den_l_out = 0.f;
   if (p.lin) {
@@ -738,50 +766,50 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
     if (nkv > 0) e = (p.stab_mode == AS_STAB_EXACT) ? -m_ref : (m_true - m_ref);
     e = fminf(fmaxf(e, -100.f), 100.f);
     const float lam = ex2(e);
-    float dl;
-    dl = 0.f;
+    float dl = 0.f;
     if constexpr (!TWO) {
-      for (int ch = 0; ch < q.fc; ++ch) {
-        if (!q.wait(R::B_S + g, ps + nkv + ch)) return false;
-        tc_fence_after();
-        if (!p_buffer_free(ppf + nkv + ch)) return false;   // the last tile's P V / the previous chunk's product has read the P tile
-        dl += q_features_from_tmem<D, GEN>(p, tSg, q.bar(R::B_SF + g), sPg, r, bh, ch, lam);   // phi_q takes P's place as the A operand
-        mbar_arrive(q.bar(R::B_P + g));
-      }
-    }
-    if constexpr (TWO) {
+      const bool ok = T == 1 ? q_one_layer_tail_apart<D, T, GEN>(p, c, g, q.tTail(g) + lane_off, sPg, r, hc, bh, ps, ppf, lam, dl)
+                             : q_one_layer_tail<D, T, GEN>(p, q, g, q.tTail(g) + lane_off, sPg, r, hc, bh, ps, ppf, lam, dl);
+      if (!ok) return false;
+    } else {
       uint8_t* sQg = smem + L::Q_OFF + g * L::TILE;    // the group's Q tile: a second buffer once Q is done with
-      dl = q_two_layer_tail<D, GEN>(p, q, g, tSg, sPg, sQg, r, bh, ps, ppf, lam);
+      dl = q_two_layer_tail<D, T, GEN>(p, q, g, q.tTail(g) + lane_off, sPg, sQg, r, hc, bh, ps, ppf, lam);
       if (dl < 0.f) return false;                      // a wait ran out (the sum itself is never negative)
     }
+    if (X::TPR == 2) dl += __shfl_xor_sync(0xffffffffu, dl, 16);
     den = l + dl;
     den_l_out = dl / lam;
   }
   if (!q.wait(R::B_O + g, u)) return false;
   tc_fence_after();
   const float inv = 1.f / den;
-  // The output rows are staged in the group's P tile (the product that read it has completed with the O
-  // barrier); each warp stores its own 32 rows (rows past N are clipped by the tensor map).
-  const int wrow0 = row - lane;
+  // The output rows are staged in the group's phi_q tile (the product that read it has completed with the O
+  // barrier; a layer without linear tokens: this warp's previous output store has been read out); each warp stores its own rows (rows past N are clipped by the tensor map).
+  const int wrow0 = un.row0 + g * 128 + r0;
+  if (!p.lin) {
+    if (lane == 0) tma_store_wait_read();
+    __syncwarp();
+  }
+  uint32_t x[32];
 #pragma unroll 1
-  for (int cc = 0; cc < D / 32; ++cc) {
-    tmem_ld32(tOg + cc * 32, x);
+  for (int cc = 0; cc < D / X::TPR / 32; ++cc) {
+    q_ld32<X::TPR, D / 2>(tOg + cc * 32, x);
     tmem_ld_wait(x);
     uint32_t wd[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i)
       wd[i] = pack_bf16(__uint_as_float(x[2 * i]) * inv, __uint_as_float(x[2 * i + 1]) * inv);
-    store_row_chunk(sPg, r, cc * 32, wd);
+    store_row_chunk(sPg, r, hc * (D / X::TPR) + cc * 32, wd);
   }
   fence_proxy_async();
   __syncwarp();
   if (lane == 0 && wrow0 < p.N) {
 #pragma unroll
     for (int b = 0; b < D / 64; ++b)
-      tma_store_3d(tmO, smem_u32(sPg) + b * BOX_BYTES + (warp & 3) * 32 * 128, b * 64, wrow0, bh);
+      tma_store_3d(tmO, smem_u32(sPg) + b * BOX_BYTES + r0 * 128, b * 64, wrow0, bh);
     tma_store_commit();
   }
-  if (p.aux != nullptr && row < p.N) {
+  if (p.aux != nullptr && row < p.N && hc == 0) {
     const float ln2 = 0.6931471805599453f;
     float* ap = p.aux + ((size_t)bh * p.N + row) * 3;
     ap[0] = nkv > 0 ? m_true * ln2 : 0.f;
@@ -805,7 +833,7 @@ constexpr int QL_THREADS = 608;          // warps 0-15: compute (group = bit 2, 
 
 template <int D, bool GEN>
 __device__ __noinline__ bool q_linear_unit(const QParams& p, const QCtx& c, const CUtensorMap* tmO, uint8_t* smem, float* sDl, int u) {
-  using R = QRing<D>;
+  using R = QRing<D, false>;
   using L = QLayout<D>;
   const R q(p, c);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -826,7 +854,7 @@ __device__ __noinline__ bool q_linear_unit(const QParams& p, const QCtx& c, cons
   for (int ch = 0; ch < q.fc; ++ch) {
     if (!q.wait(R::B_S + g, ps + ch)) return false;
     tc_fence_after();
-    // the P tile may be written once the product that read it has completed and the previous unit's output store
+    // the phi_q tile may be written once the product that read it has completed and the previous unit's output store
     // has been read out (the stores are issued by the warps of column half 0)
     if (hf == 0 && lane == 0) tma_store_wait_read();
     if (ppf + ch > 0 && !q.wait(R::B_PF + g, ppf + ch - 1)) return false;
@@ -961,10 +989,10 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       if (!q_produce_unit<D, false, GEN>(p, c, &tmQ, &tmQ, &tmQ, &tmW, &tmSt, &tmW, u)) break;
   } else if (warp == 17) {
     for (int u = 0; u < n_mine; ++u)
-      if (!q_score_unit<D, false, GEN>(p, c, u)) break;
+      if (!q_score_unit<D, false, GEN, false>(p, c, u)) break;
   } else if (warp == 18) {
     for (int u = 0; u < n_mine; ++u)
-      if (!q_accum_unit<D, false, GEN>(p, c, u)) break;
+      if (!q_accum_unit<D, false, GEN, false>(p, c, u)) break;
   } else {
     const int g = (warp >> 2) & 1;
     // a unit worked on by one group only is the CTA's last one: group 1 stops before it
@@ -982,14 +1010,15 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   }
 }
 
-template <int D, bool TWO, bool GEN>
-__global__ void __launch_bounds__(Q_THREADS, 1)
+template <int D, int T, bool TWO, bool GEN>
+__global__ void __launch_bounds__(QShape<D, T>::THREADS, 1)
 qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
              const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmW,
              const __grid_constant__ CUtensorMap tmSt, const __grid_constant__ CUtensorMap tmW1,
              const __grid_constant__ CUtensorMap tmO, const __grid_constant__ QParams p) {
   using L = QLayout<D>;
   using R = QRing<D>;
+  using X = QShape<D, T>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
@@ -1003,14 +1032,15 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     mbar_init(bar(R::B_Q0), 1); mbar_init(bar(R::B_Q0 + 1), 1);
     for (int s = 0; s < KV_STAGES; ++s) { mbar_init(bar(R::B_FULL + s), 1); mbar_init(bar(R::B_EMPTY + s), 1); }
     for (int g = 0; g < 2; ++g) {
-      mbar_init(bar(R::B_S + g), 1); mbar_init(bar(R::B_SF + g), 128); mbar_init(bar(R::B_P + g), 128);
+      mbar_init(bar(R::B_S + g), 1); mbar_init(bar(R::B_SF + g), X::GROUP); mbar_init(bar(R::B_P + g), X::GROUP);
       mbar_init(bar(R::B_PF + g), 1); mbar_init(bar(R::B_O + g), 1); mbar_init(bar(R::B_QF + g), 1);
-      mbar_init(bar(R::B_H + g), 128 * (p.nh > 0 ? p.nh : 1));   // one arrival per thread and hidden slice
+      mbar_init(bar(R::B_H + g), X::GROUP * (p.nh > 0 ? p.nh : 1));   // one arrival per thread and hidden slice
     }
+    mbar_init(bar(R::B_PL), 1);
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (warp == 9) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
+  if (warp == X::W_SCORE) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   griddep_wait();                                    // the set-up above ran beside the kernel before this one
   // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
   __shared__ uint32_t s_skip;
@@ -1019,34 +1049,34 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   __syncthreads();
   tc_fence_after();
   if (s_skip != 0u) {
-    if (warp == 9) tmem_dealloc(*tmem_slot, 512);
+    if (warp == X::W_SCORE) tmem_dealloc(*tmem_slot, 512);
     return;
   }
   const QCtx c{sbase, *tmem_slot, WaitCtx{p.status, abort_flag}};
   const int n_mine = q_units_of_cta(p);               // units of this CTA
 
-  if (warp == 8) {
+  if (warp == X::W_TMA) {
     if ((threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); tma_prefetch_desc(&tmO); }
     for (int u = 0; u < n_mine; ++u)
       if (!q_produce_unit<D, TWO, GEN>(p, c, &tmQ, &tmK, &tmV, &tmW, &tmSt, &tmW1, u)) break;
-  } else if (warp == 9) {
+  } else if (warp == X::W_SCORE) {
     for (int u = 0; u < n_mine; ++u)
-      if (!q_score_unit<D, TWO, GEN>(p, c, u)) break;
-  } else if (warp == 10) {
+      if (!q_score_unit<D, TWO, GEN, D == 128>(p, c, u)) break;
+  } else if (warp == X::W_ACCUM) {
     for (int u = 0; u < n_mine; ++u)
-      if (!q_accum_unit<D, TWO, GEN>(p, c, u)) break;
+      if (!q_accum_unit<D, TWO, GEN, D == 128>(p, c, u)) break;
   } else {
     // a unit worked on by one group only is the CTA's last one: group 1 stops before it
-    const int n_grp = (n_mine > p.n_rounds && warp >= 4 && q_unit(p, p.n_rounds).ng == 1) ? p.n_rounds : n_mine;
+    const int n_grp = (n_mine > p.n_rounds && ((warp >> 2) & 1) == 1 && q_unit(p, p.n_rounds).ng == 1) ? p.n_rounds : n_mine;
     for (int u = 0; u < n_grp; ++u)
-      if (!q_softmax_unit<D, TWO, GEN>(p, c, &tmO, smem, u)) break;
+      if (!q_softmax_unit<D, T, TWO, GEN>(p, c, &tmO, smem, u)) break;
     if ((threadIdx.x & 31) == 0) tma_store_wait_read();  // this warp's output stores have read their rows (the writes land by the end of the kernel)
   }
 
   // ------------------------------------------------------------ teardown
   tc_fence_before();
   __syncthreads();
-  if (warp == 9) {
+  if (warp == X::W_SCORE) {
     tc_fence_after();
     tmem_dealloc(c.tmem, 512);
   }
@@ -1056,14 +1086,18 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 
 cudaError_t as_tensor_init_qpass() {
   cudaError_t e;
-  if ((e = opt_in_smem(qpass_kernel<128, false, false>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<128, false, true>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<128, true, false>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<128, true, true>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<64, false, false>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<64, false, true>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<64, true, false>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<64, true, true>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(qpass_kernel<128, 1, false, false>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(qpass_kernel<128, 2, false, false>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(qpass_kernel<128, 1, false, true>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(qpass_kernel<128, 2, false, true>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(qpass_kernel<128, 1, true, false>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(qpass_kernel<128, 2, true, false>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(qpass_kernel<128, 1, true, true>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(qpass_kernel<128, 2, true, true>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(qpass_kernel<64, 2, false, false>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(qpass_kernel<64, 2, false, true>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(qpass_kernel<64, 2, true, false>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(qpass_kernel<64, 2, true, true>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
   if ((e = opt_in_smem(qlin_kernel<128, false>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
   if ((e = opt_in_smem(qlin_kernel<128, true>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
   if ((e = opt_in_smem(qlin_kernel<64, false>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
@@ -1078,6 +1112,11 @@ cudaError_t as_tensor_init_qpass() {
 // us; N = 1024 with 2 heads on 16 CTAs instead of 8: 22.5 -> 21.4).  Returns the
 // number of CTAs.
 namespace {
+// Threads per row of the kernel with a key loop.  Two (sixteen compute warps) keep the special-function unit busier and turn the rows of
+// the tail around faster; but at d = 128, where the groups take turns at the score columns, a long key loop goes better with one.
+// Layers with 12 heads, against P through shared memory, two / one: 2 key tiles 1.035 / 1.00, 8 1.085 / 1.01, 16 1.06 / 1.01 - 1.03, 20 1.03 /
+// 1.03, 32 1.02 / 1.03, 64 1.016 / 1.035, 128 1.013 / 1.04; two-layer map, 8 tiles 1.07 / 1.045, 17 1.01 / 1.014.
+int q_threads_per_row(int d, int nkv) { return d == 64 || nkv <= 16 ? 2 : 1; }
 int plan_units(QParams& p, int BH, int sms) {
   const int tiles = (p.N + 127) / 128;
   double best = 0.;
@@ -1103,14 +1142,16 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   const int BH = a.B * a.H;
   const bool lin = a.n_l > 0;
   CUtensorMap tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO;
-  // the output is stored warp by warp: boxes of 32 rows
-  if (!make_map(&tmQ, a.q, a.d, a.N, BH, 128) || !make_map(&tmO, a.out, a.d, a.N, BH, 32)) return cudaErrorInvalidValue;
+  const bool two = lin && a.layers == 2;
+  const bool qlin = a.n_s == 0 && lin && !two;         // no softmax tokens, one-layer map: the variant without a key loop
+  const int tpr = q_threads_per_row(a.d, (a.n_s + 127) / 128);
+  // the output is stored warp by warp: boxes of a warp's rows
+  if (!make_map(&tmQ, a.q, a.d, a.N, BH, 128) || !make_map(&tmO, a.out, a.d, a.N, BH, qlin ? 32 : 32 / tpr)) return cudaErrorInvalidValue;
   if (a.n_s > 0) {
     if (!make_map(&tmK, a.ks, a.d, a.n_s, BH, 128) || !make_map(&tmV, a.vs, a.d, a.n_s, BH, 128)) return cudaErrorInvalidValue;
   } else {
     tmK = tmQ; tmV = tmQ;       // never used: the key loop is empty
   }
-  const bool two = lin && a.layers == 2;
   if (lin) {
     // boxes are always 128 rows: rows past F (or the hidden width) are out of bounds and arrive as zeros.
     // tmW: last-layer weights [H][F][width of their input]; tmW1: first-layer weights of a two-layer map.
@@ -1138,22 +1179,22 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   const dim3 grid(plan_units(p, BH, sms), 1, 1);
   // the general kernels carry the bias and the powers beyond 2; the common case does without them
   const bool gen = lin && (a.P > 2 || p.b1 != nullptr || p.b2 != nullptr);
-  if (p.nkv == 0 && lin && !two) {
-    // no softmax tokens, one-layer map: the variant with sixteen compute warps
+  if (qlin) {
 #define AS_LAUNCH_QL(D_, GEN_) \
   return as_launch_dependent(qlin_kernel<D_, GEN_>, grid, dim3(QL_THREADS), QLayout<D_>::TOTAL, st, tmQ, tmW, tmSt, tmO, p)
     if (a.d == 128) { if (gen) AS_LAUNCH_QL(128, true); else AS_LAUNCH_QL(128, false); }
     if (gen) AS_LAUNCH_QL(64, true); else AS_LAUNCH_QL(64, false);
 #undef AS_LAUNCH_QL
   }
-#define AS_LAUNCH_Q(D_, TWO_, GEN_) \
-  return as_launch_dependent(qpass_kernel<D_, TWO_, GEN_>, grid, dim3(Q_THREADS), QLayout<D_>::TOTAL, st, tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO, p)
-  if (a.d == 128) {
-    if (two) { if (gen) AS_LAUNCH_Q(128, true, true); else AS_LAUNCH_Q(128, true, false); }
-    else { if (gen) AS_LAUNCH_Q(128, false, true); else AS_LAUNCH_Q(128, false, false); }
-  } else {
-    if (two) { if (gen) AS_LAUNCH_Q(64, true, true); else AS_LAUNCH_Q(64, true, false); }
-    else { if (gen) AS_LAUNCH_Q(64, false, true); else AS_LAUNCH_Q(64, false, false); }
-  }
+#define AS_LAUNCH_Q(D_, T_, TWO_, GEN_) \
+  return as_launch_dependent(qpass_kernel<D_, T_, TWO_, GEN_>, grid, dim3(QShape<D_, T_>::THREADS), QLayout<D_>::TOTAL, st, tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO, p)
+#define AS_LAUNCH_QT(D_, T_) \
+  do { \
+    if (two) { if (gen) AS_LAUNCH_Q(D_, T_, true, true); else AS_LAUNCH_Q(D_, T_, true, false); } \
+    else { if (gen) AS_LAUNCH_Q(D_, T_, false, true); else AS_LAUNCH_Q(D_, T_, false, false); } \
+  } while (0)
+  if (a.d == 128) { if (tpr == 2) AS_LAUNCH_QT(128, 2); else AS_LAUNCH_QT(128, 1); }
+  AS_LAUNCH_QT(64, 2);
+#undef AS_LAUNCH_QT
 #undef AS_LAUNCH_Q
 }

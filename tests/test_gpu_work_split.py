@@ -94,3 +94,40 @@ def test_softmax_rows_of_a_two_layer_map_are_gathered_bit_for_bit(N, rate, d, F,
     assert op.last_status() == 0
     for got, x in ((ks, dev["k"]), (vs, dev["v"])):
         assert torch.equal(got.view(torch.int16), x[:, :, at].reshape(6, len(at), d).view(torch.int16))
+
+
+# keys at the edges of what a thread holds of a score row (32-column pieces, half rows, whole rows), of a key tile, and of the rule that gives
+# a row one thread or two (16 key tiles)
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("N", [1, 31, 33, 63, 64, 65, 97, 127, 128, 129, 193, 2048, 2049])
+def test_key_counts_at_the_edges_of_a_thread_s_share(N, d):
+    """Full softmax, the tensor path next to the fp32 check path (bounds as above); rows whose largest score lies in either half."""
+    import torch
+    from paper_2509_24899_b200 import HybridAttention, binding
+    wl, dev = _inputs(1, 3, N, d, 1, 73)
+    q = dev["q"].clone()
+    q[:, :, ::3] *= 6.0                                       # some rows dominated by a key, others near uniform
+    out = [HybridAttention.from_workload(wl, kernel_path=path).forward(q, dev["k"], dev["v"], dev["wq"], dev["wk"]).double()
+           for path in (binding.AS_PATH_TENSOR, binding.AS_PATH_SIMT)]
+    assert float((out[0] - out[1]).norm() / out[1].norm()) <= 5e-3
+    assert float(((out[0] - out[1]).norm(dim=-1) / out[1].norm(dim=-1)).max()) <= 5e-2
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_a_key_that_is_no_number_reaches_every_row(bad, d):
+    """Whichever column of a tile the key's scores land in, and so whichever unit takes their exponentials."""
+    import torch
+    from paper_2509_24899_b200 import HybridAttention
+    wl, dev = _inputs(1, 1, 128, d, 1, 74)
+    op = HybridAttention.from_workload(wl)
+    for col in list(range(0, 40)) + [63, 64, 95, 110, 127]:
+        k = dev["k"].clone()
+        k[0, 0, col, 0] = bad
+        out = op.forward(dev["q"], k, dev["v"], dev["wq"], dev["wk"])
+        hit = torch.isnan(out[0, 0]).any(dim=-1)
+        if bad != bad:
+            assert bool(hit.all()), col
+        else:                                                 # infinite scores where q_0 > 0: infinity less infinity; where q_0 < 0 a weight of 0
+            assert bool(hit[dev["q"][0, 0, :, 0] > 0].all()), col
+            assert not bool(hit[dev["q"][0, 0, :, 0] < 0].any()), col
