@@ -117,8 +117,9 @@ struct QLayout {
 // d = 128: both groups use the same 128 score columns in the key loop, in turn: Q_1 K(j)^T follows once group 0 has read its tile j, Q_0 K(j+1)^T once
 // group 1 has read its tile j.  A product into them takes 512 clk, the groups' reads 150 each and their waits and commits as much, so a
 // round is 2100 - 2500 clk where the exponentials of both groups take 2048 at the least: the groups run half a period
-// apart and little waits for the columns.  In the tail, where a group has little else to do than to wait for its next columns, group 1 has
-// the columns of both P's instead (two-layer map with 32 key tiles 920 -> 890 us).  One warp that issues everything in that fixed order, the second product in halves around
+// apart and little waits for the columns.  In the long tail of a two-layer map, where a group has little else to do than to wait for its
+// next columns, group 1 has the columns of both P's instead (32 key tiles 920 -> 890 us; the one-layer tail has as many products as feature
+// chunks, and the last P V to wait for costs more: N = 7800 79.4 -> 82.2 us).  One warp that issues everything in that fixed order, the second product in halves around
 // the next scores, is slower (full softmax 4700 -> 5130 us): issuing blocks it.
 //
 // The work of one unit is a function per role, kept out of line: each role then gets a register
@@ -160,7 +161,7 @@ struct QRing {
   // barrier indices; per group: S (scores, hidden activations or Phi landed in the score columns), SF (score
   // columns read out), P (P in tensor memory, phi_q in shared memory), PF (the product that reads it has completed),
   // O (output accumulator final), QF (nothing of the unit reads the Q tile any more), H (two layers: the
-  // hidden activations are in shared memory); for both: PL (nothing reads the unit's P in tensor memory any more)
+  // hidden activations are in shared memory); for both, two layers: PL (nothing reads the unit's P in tensor memory any more)
   static constexpr int B_Q0 = 0, B_FULL = 2, B_EMPTY = B_FULL + KV_STAGES, B_S = B_EMPTY + KV_STAGES, B_SF = B_S + 2,
                        B_P = B_SF + 2, B_PF = B_P + 2, B_O = B_PF + 2, B_QF = B_O + 2, B_H = B_QF + 2, B_PL = B_H + 2, B_COUNT = B_PL + 1;
   const QCtx c;              // by value: nothing here is re-read from memory after a barrier or an MMA
@@ -201,15 +202,17 @@ struct QRing {
   AS_DEV uint32_t tS(int g) const { return SH ? c.tmem : c.tmem + 128u * g; }
   AS_DEV uint32_t tP(int g) const { return c.tmem + (SH ? 128u : 384u) + 64u * g; }
   AS_DEV uint32_t tO(int g) const { return c.tmem + 256u + (uint32_t)D * g; }
-  AS_DEV uint32_t tTail(int g) const { return c.tmem + 128u * g; }   // where the products of the linear tail land
+  // Two layers: where the products of the linear tail land
+  AS_DEV uint32_t tTail(int g) const { return c.tmem + 128u * g; }
   // Before product i of the unit into group g's score columns, the ph-th of all: what lay there has been read.  With columns of its own
-  // (and in the tail, where group 1 has the columns of both P's) by the group itself; else by the groups in turn.
+  // (at d = 64; in a two-layer map's tail, where group 1 has the columns of both P's) by the group itself; else by the groups in turn.
   // (A unit of one group, the CTA's last one, follows a unit of two.)
+  template <bool TWO>
   AS_DEV bool s_free(int g, int ph, int ng, int i, int u) const {
-    if (!SH || i > nkv || nkv == 0) return ph == 0 ? true : wait(B_SF + g, ph - 1);
-    if (g == 1) return i < nkv ? wait(B_SF, ph) : wait(B_PL, u);
+    if (!SH || (TWO && (i > nkv || nkv == 0))) return ph == 0 ? true : wait(B_SF + g, ph - 1);
+    if (g == 1) return !TWO || i < nkv ? wait(B_SF, ph) : wait(B_PL, u);
     if (ph == 0) return true;
-    if (i == 0 && !wait(B_SF, ph - 1)) return false;   // the unit before: group 0's rows lay here, group 1's where P_0 will go
+    if (TWO && i == 0 && !wait(B_SF, ph - 1)) return false;   // the unit before: group 0's rows lay here, group 1's where P_0 will go
     return wait(B_SF + (ng == 2 || i == 0 ? 1 : 0), ph - 1);
   }
   AS_DEV bool wait(int b, int phase) const { return mbar_wait_warp(bar(b), phase & 1, c.wc); }
@@ -300,7 +303,7 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
 #pragma unroll
     for (int kk = 0; kk < 8; ++kk) dq[g][kk] = q0 + kstep_kmajor(kk);
   }
-  auto s_free = [&](int g, int i) -> bool { return q.s_free(g, ps + i, ng, i, u); };
+  auto s_free = [&](int g, int i) -> bool { return q.template s_free<TWO>(g, ps + i, ng, i, u); };
 
   // ---- first key tile (its product opens the unit)
   if (nkv > 0) {
@@ -353,7 +356,7 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
         tc_fence_after();
         if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tTail(g), dq[g][kk], w0 + kstep_kmajor(kk), id_phi, kk > 0 ? 1u : 0u);
+          for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tS(g), dq[g][kk], w0 + kstep_kmajor(kk), id_phi, kk > 0 ? 1u : 0u);
           tc_commit(q.bar(R::B_S + g));
           if (ch == q.fc - 1) tc_commit(q.bar(R::B_QF + g));     // nothing of this unit reads the group's Q tile any more
         }
@@ -433,7 +436,7 @@ __device__ __noinline__ bool q_accum_unit(const QParams& p, const QCtx& c, int u
         for (int kk = 0; kk < 8; ++kk) mma_ts(q.tO(g), q.tP(g) + kk * 8, v0 + kstep_mnmajor(kk), ID_PV, (j > 0 || kk > 0) ? 1u : 0u);
         tc_commit(q.bar(R::B_PF + g));
         if (last && !lin) tc_commit(q.bar(R::B_O + g));
-        if (SH && last && lin && g == 1) tc_commit(q.bar(R::B_PL));    // (the other group's product was issued before)
+        if (SH && TWO && last && lin && g == 1) tc_commit(q.bar(R::B_PL));    // (the other group's product was issued before)
       }
     }
     if (elect_one()) q.release(iv);
@@ -768,8 +771,8 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
     const float lam = ex2(e);
     float dl = 0.f;
     if constexpr (!TWO) {
-      const bool ok = T == 1 ? q_one_layer_tail_apart<D, T, GEN>(p, c, g, q.tTail(g) + lane_off, sPg, r, hc, bh, ps, ppf, lam, dl)
-                             : q_one_layer_tail<D, T, GEN>(p, q, g, q.tTail(g) + lane_off, sPg, r, hc, bh, ps, ppf, lam, dl);
+      const bool ok = T == 1 ? q_one_layer_tail_apart<D, T, GEN>(p, c, g, tSg, sPg, r, hc, bh, ps, ppf, lam, dl)
+                             : q_one_layer_tail<D, T, GEN>(p, q, g, tSg, sPg, r, hc, bh, ps, ppf, lam, dl);
       if (!ok) return false;
     } else {
       uint8_t* sQg = smem + L::Q_OFF + g * L::TILE;    // the group's Q tile: a second buffer once Q is done with
@@ -1114,9 +1117,9 @@ cudaError_t as_tensor_init_qpass() {
 namespace {
 // Threads per row of the kernel with a key loop.  Two (sixteen compute warps) keep the special-function unit busier and turn the rows of
 // the tail around faster; but at d = 128, where the groups take turns at the score columns, a long key loop goes better with one.
-// Layers with 12 heads, against P through shared memory, two / one: 2 key tiles 1.035 / 1.00, 8 1.085 / 1.01, 16 1.06 / 1.01 - 1.03, 20 1.03 /
-// 1.03, 32 1.02 / 1.03, 64 1.016 / 1.035, 128 1.013 / 1.04; two-layer map, 8 tiles 1.07 / 1.045, 17 1.01 / 1.014.
-int q_threads_per_row(int d, int nkv) { return d == 64 || nkv <= 16 ? 2 : 1; }
+// Layers with 12 heads, against P through shared memory, two / one: 3 key tiles 1.09 / 1.01, 8 1.07 / 1.01, 16 1.07 / 1.03, 20 1.035 / 1.01, 31
+// 1.06 / 1.02, 32 1.016 / 1.018, 64 1.016 / 1.03, 128 1.013 / 1.035; two-layer maps, 32 tiles 1.045 / 1.06.
+int q_threads_per_row(int d, int nkv, bool two) { return d == 64 || nkv <= (two ? 16 : 31) ? 2 : 1; }
 int plan_units(QParams& p, int BH, int sms) {
   const int tiles = (p.N + 127) / 128;
   double best = 0.;
@@ -1144,7 +1147,7 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   CUtensorMap tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO;
   const bool two = lin && a.layers == 2;
   const bool qlin = a.n_s == 0 && lin && !two;         // no softmax tokens, one-layer map: the variant without a key loop
-  const int tpr = q_threads_per_row(a.d, (a.n_s + 127) / 128);
+  const int tpr = q_threads_per_row(a.d, (a.n_s + 127) / 128, two);
   // the output is stored warp by warp: boxes of a warp's rows
   if (!make_map(&tmQ, a.q, a.d, a.N, BH, 128) || !make_map(&tmO, a.out, a.d, a.N, BH, qlin ? 32 : 32 / tpr)) return cudaErrorInvalidValue;
   if (a.n_s > 0) {

@@ -106,9 +106,10 @@ def test_dependents_are_let_in_only_by_ctas_that_own_their_tensor_memory():
     assert checked >= 8
 
 
-def _query_stage(tiles, chunks, groups, shared, threads, ring, units=1):
+def _query_stage(tiles, chunks, groups, shared, threads, ring, units=1, own_tail=True):
     """The query stage with a one-layer map, unit after unit (the last one of `groups` groups, the others of two): compute threads (one or
-    two stand for a group's), the warp that issues what writes the score columns (shared by the groups at d = 128, but for the feature rows),
+    two stand for a group's), the warp that issues what writes the score columns (shared by the groups at d = 128, with `own_tail` only
+    in the key loop),
     the warp that issues what accumulates into O and, with `ring`, the loads."""
     n, counts = tiles + chunks, {}
     compute, score, accum, load = [[], []], [], [], []
@@ -148,18 +149,18 @@ def _query_stage(tiles, chunks, groups, shared, threads, ring, units=1):
                     steps += wait("o", g, u)
                 # what writes the score columns
                 score += full("k", i) if g == 0 else []
-                if not shared or i > tiles or tiles == 0:
+                if not shared or (own_tail and (i > tiles or tiles == 0)):
                     score += wait("sf", g, ph - 1)
                 elif g == 1:
-                    score += wait("sf", 0, ph) if i < tiles else wait("pl", 0, u)
+                    score += wait("sf", 0, ph) if i < tiles or not own_tail else wait("pl", 0, u)
                 else:
-                    score += wait("sf", 0, ph - 1) if i == 0 else []
+                    score += wait("sf", 0, ph - 1) if i == 0 and own_tail else []
                     score += wait("sf", 1 if ng == 2 or i == 0 else 0, ph - 1)
                 score.append(("commit", "s%d" % g))
                 # what accumulates
                 accum += full("v", i) if g == 0 else []
                 accum += wait("p", g, ph) + [("commit", "pf%d" % g)] + ([("commit", "o%d" % g)] if i + 1 == n else [])
-                accum += [("commit", "pl0")] if shared and chunks and g == 1 and i + 1 == tiles else []
+                accum += [("commit", "pl0")] if shared and own_tail and chunks and g == 1 and i + 1 == tiles else []
             score += release("k", i)
             accum += release("v", i)
     for g in range(2 if units > 1 else groups):
@@ -175,10 +176,10 @@ def _query_stage(tiles, chunks, groups, shared, threads, ring, units=1):
 @pytest.mark.parametrize("tiles,chunks,units", [(1, 0, 1), (3, 0, 1), (0, 1, 1), (0, 3, 1), (1, 1, 1), (2, 1, 1), (3, 2, 1), (1, 0, 3), (2, 0, 2), (0, 1, 3),
                                                 (1, 1, 3), (2, 1, 2), (1, 2, 2)])
 @pytest.mark.parametrize("groups", [1, 2])
-@pytest.mark.parametrize("shared", [False, True])
+@pytest.mark.parametrize("shared,own_tail", [(False, True), (True, True), (True, False)])
 @pytest.mark.parametrize("threads,ring", [(2, False), (1, True)])
-def test_query_stage_finishes_in_every_order(tiles, chunks, units, groups, shared, threads, ring):
-    assert _stuck_state(*_query_stage(tiles, chunks, groups, shared, threads, ring, units)) is None
+def test_query_stage_finishes_in_every_order(tiles, chunks, units, groups, shared, own_tail, threads, ring):
+    assert _stuck_state(*_query_stage(tiles, chunks, groups, shared, threads, ring, units, own_tail)) is None
 
 
 def test_the_model_finds_what_it_is_there_for():

@@ -97,9 +97,9 @@ def test_softmax_rows_of_a_two_layer_map_are_gathered_bit_for_bit(N, rate, d, F,
 
 
 # keys at the edges of what a thread holds of a score row (32-column pieces, half rows, whole rows), of a key tile, and of the rule that gives
-# a row one thread or two (16 key tiles)
+# a row one thread or two (31 key tiles)
 @pytest.mark.parametrize("d", [64, 128])
-@pytest.mark.parametrize("N", [1, 31, 33, 63, 64, 65, 97, 127, 128, 129, 193, 2048, 2049])
+@pytest.mark.parametrize("N", [1, 31, 33, 63, 64, 65, 97, 127, 128, 129, 193, 3968, 3969])
 def test_key_counts_at_the_edges_of_a_thread_s_share(N, d):
     """Full softmax, the tensor path next to the fp32 check path (bounds as above); rows whose largest score lies in either half."""
     import torch
