@@ -453,9 +453,13 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
 // for the product.  (The K pass, which has h1 tiles in its ring instead, fetched them from global memory one row after
 // the other and held its slots of the ring meanwhile: the whole key side 338 us against 181 at N = 32760, rate 1/8, hidden =
 // F = 256, the layer 1182 against 1071.)
+// Two CTAs share an SM, and what bounds the kernel is the chain of one (set-up, 96 KB of loads, products, rows, stores): so each slice goes
+// its own way, rows by eight warps under the next slice's product, staged over its own weights and stored at once, and the CTA ends
+// when its stores have been read.  With four warps, both slices' rows behind both products, and an end that waited for the stores to
+// land: the same layer 906 us against 897, N = 7800 152.0 against 150.7 (74 us of this kernel; floor 47).
 // ======================================================================================
 struct P1Params { int H, hid, N, n_s; const __nv_bfloat16* bias; const int32_t* sm_rank; __nv_bfloat16* ks_w; uint32_t* status; };
-constexpr int P1_THREADS = 160;          // warps 0-3: epilogue (one thread per token row); warp 4: TMA + MMA
+constexpr int P1_THREADS = 288;          // warps 0-7: epilogue (two threads per token row, each half of a slice's columns); warp 8: TMA + MMA
 
 template <int D, int NH>
 struct P1Layout {
@@ -474,13 +478,14 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::BAR_OFF);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::BAR_OFF + 16);
-  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::BAR_OFF + 20);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::BAR_OFF + 32);
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::BAR_OFF + 36);
   float* sBias = reinterpret_cast<float*>(smem + L::BIAS_OFF);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bh = blockIdx.y, h = bh % p.H, row0 = blockIdx.x * 128;
   const WaitCtx wc{p.status, abort_flag};
-  const uint32_t bar_full = smem_u32(bars), bar_done = smem_u32(bars + 1);
+  const uint32_t bar_full = smem_u32(bars);
+  auto bar_done = [&](int j) { return smem_u32(bars + 1 + j); };   // slice j's product has completed
   constexpr int TM_COLS = NH * 128;                             // 128 or 256: a power of two
 
   __shared__ uint32_t s_skip;
@@ -489,23 +494,25 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
   if (s_skip != 0u) return;
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
-    mbar_init(bar_full, 1); mbar_init(bar_done, 1);
+    mbar_init(bar_full, 1);
+    for (int j = 0; j < NH; ++j) mbar_init(bar_done(j), 1);
     fence_barrier_init();
     fence_proxy_async();
   }
   for (int i = threadIdx.x; i < NH * D; i += P1_THREADS)
     sBias[i] = (p.bias != nullptr && i < p.hid) ? __bfloat162float(p.bias[(size_t)h * p.hid + i]) : 0.f;
-  if (warp == 4) { tmem_alloc(smem_u32(tmem_slot), TM_COLS); tmem_relinquish(); }
+  if (warp == 8) { tmem_alloc(smem_u32(tmem_slot), TM_COLS); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const uint32_t sX = sbase + L::X_OFF;
   auto sW = [&](int j) { return sbase + L::W_OFF + j * L::TILE; };
-  // hidden slice j is staged for its store where an operand sat: slice 0 over the X tile, slice j over W tile j - 1
-  auto stage_off = [&](int j) { return j == 0 ? L::X_OFF : L::W_OFF + (j - 1) * L::TILE; };
+  // Hidden slice j is staged for its store over W tile j, which nothing reads once its product has completed: slice 0 leaves while slice 1
+  // is still being formed.
+  auto stage_off = [&](int j) { return L::W_OFF + j * L::TILE; };
 
-  if (warp == 4) {
+  if (warp == 8) {
     if (lane == 0) {
       mbar_expect_tx(bar_full, (1 + NH) * L::TILE);
       load_tile<D>(sX, &tmX, bar_full, row0, bh);
@@ -515,20 +522,21 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
     if (mbar_wait_warp(bar_full, 0, wc)) {
       tc_fence_after();
       if (lane == 0) {
-        for (int j = 0; j < NH; ++j)      // X W_1^T, N = 128 hidden units of slice j (N = D when the hidden width is 64)
+        for (int j = 0; j < NH; ++j) {    // X W_1^T, N = 128 hidden units of slice j (N = D when the hidden width is 64)
           issue_kmajor<D>(tmem + j * 128, kmajor_desc(sX), kmajor_desc(sW(j)), make_idesc(128, NH == 1 ? D : 128, 0, 0), false);
-        tc_commit(bar_done);
+          tc_commit(bar_done(j));
+        }
       }
       __syncwarp();
     }
   } else {
-    const int r = warp * 32 + lane;
-    const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
+    const int quad = warp & 3, hf = warp >> 2, r = quad * 32 + lane;
+    const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
     bool ok = true;
     if (p.ks_w != nullptr) {
-      // this warp's 32 rows of the K tile (which its threads overwrite below, each its own row); D / 8 lanes a row
+      // sixteen rows of the K tile; D / 8 lanes a row
       constexpr int CH = D / 8, RPI = 32 / CH;
-      const int rank = row0 + r < p.N ? p.sm_rank[row0 + r] : -1;
+      const int rank = lane / 16 == hf && row0 + r < p.N ? p.sm_rank[row0 + r] : -1;
       uint32_t bits = __ballot_sync(0xffffffffu, rank >= 0);
       if (bits) ok = mbar_wait_warp(bar_full, 0, wc);
       while (ok && bits) {
@@ -543,44 +551,44 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
         const int to = __shfl_sync(0xffffffffu, rank, src < 0 ? 0 : src);
         if (src >= 0) {
           const int c = lane % CH;
-          const uint4 val = *reinterpret_cast<const uint4*>(smem + L::X_OFF + (c / 8) * BOX_BYTES + swz128_chunk_offset(warp * 32 + src, c % 8));
+          const uint4 val = *reinterpret_cast<const uint4*>(smem + L::X_OFF + (c / 8) * BOX_BYTES + swz128_chunk_offset(quad * 32 + src, c % 8));
           *reinterpret_cast<uint4*>(p.ks_w + ((size_t)bh * p.n_s + to) * D + c * 8) = val;
         }
       }
       __syncwarp();
     }
-    if (ok) ok = mbar_wait_warp(bar_done, 0, wc);
-    if (ok) {
-      tc_fence_after();
-      uint32_t x[32];
+    uint32_t x[32];
 #pragma unroll
-      for (int j = 0; j < NH; ++j) {
+    for (int j = 0; j < NH; ++j) {
+      if (ok) ok = mbar_wait_warp(bar_done(j), 0, wc);
+      if (ok) {
+        tc_fence_after();
 #pragma unroll
-        for (int c = 0; c < D / 32; ++c) {
-          tmem_ld32(tmem + lane_off + j * 128 + c * 32, x);
+        for (int c = 0; c < D / 64; ++c) {
+          const int col = hf * (D / 2) + c * 32;
+          tmem_ld32(tmem + lane_off + j * 128 + col, x);
           tmem_ld_wait(x);
-          const float* bb = sBias + j * D + c * 32;
+          const float* bb = sBias + j * D + col;
           uint32_t w[16];
 #pragma unroll
           for (int i = 0; i < 16; ++i)
             w[i] = pack_bf16(fmaxf(__uint_as_float(x[2 * i]) + bb[2 * i], 0.f), fmaxf(__uint_as_float(x[2 * i + 1]) + bb[2 * i + 1], 0.f));
-          store_row_chunk(smem + stage_off(j), r, c * 32, w);   // every MMA has completed: the operand tiles are free
+          store_row_chunk(smem + stage_off(j), r, col, w);
         }
+        fence_proxy_async();
       }
-      fence_proxy_async();
-    }
-    named_barrier_sync(1, 128);                               // reached by every epilogue thread, also after a failed wait
-    if (ok && r == 0) {
-      for (int j = 0; j < NH; ++j)
+      named_barrier_sync(1, 256);                             // reached by every epilogue thread, also after a failed wait
+      if (ok && threadIdx.x == 0) {
 #pragma unroll
         for (int b = 0; b < D / 64; ++b) tma_store_3d(&tmH, sbase + stage_off(j) + b * BOX_BYTES, j * D + b * 64, row0, bh);
-      tma_store_commit();
-      tma_store_wait_all();
+        tma_store_commit();
+      }
     }
+    if (threadIdx.x == 0) tma_store_wait_read();              // (the writes land by the end of the kernel)
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 4) {
+  if (warp == 8) {
     tc_fence_after();
     tmem_dealloc(tmem, TM_COLS);
   }
