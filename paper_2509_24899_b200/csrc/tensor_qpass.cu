@@ -74,12 +74,14 @@ AS_DEV void q_st16(uint32_t t, const uint32_t (&x)[16]) {
 // sixteen 284, one in four 304.  Eight warps: no gain (81 frames of full softmax 4637 us; one in sixteen 4650, one in eight 4709).
 template <int T> constexpr int EX2_FMA_EVERY = T == 2 ? 4 : 0;
 // Two exponentials 2^x, x <= 8, on the FMA pipe: x = n + f with n the nearest integer (added into the last bits of 1.5 * 2^23), 2^f by
-// the polynomial of degree 5 with constant term 1 that is closest to it on [-1/2, 1/2] in relative error (9.1e-8, found by
-// reweighted least squares), times 2^n put together from its exponent.  Within 1.7e-7 of 2^x for all x in [-126, 8] (ex2.approx: 2.4e-7);
-// smaller ones come out as 2^-126 instead of 0, and what is no number stays none.
+// the polynomial of degree 5 with constant term 1 that is closest to it on [-1/2, 1/2] in relative error (1.08e-7 with the coefficients
+// rounded, found by reweighted least squares), times 2^n put together from its exponent.  Within 1.72e-7 of 2^x for all x in [-126, 8]
+// (ex2.approx: 2.4e-7).  Below that 0, as ex2.approx.ftz gives it: 2^-127 comes out of the exponent as 0, and the product flushes what lies
+// between (a key far below its row's maximum weighs nothing in every column, also with a value near the end of the range).  What is no
+// number stays none.
 AS_DEV float2 ex2_fma(float2 x) {
   auto both = [](float v) { return make_float2(v, v); };
-  x = make_float2(fmax_nan(x.x, -126.f), fmax_nan(x.y, -126.f));
+  x = make_float2(fmax_nan(x.x, -127.f), fmax_nan(x.y, -127.f));
   const float2 t = __fadd2_rn(x, both(12582912.f));
   const float2 f = __ffma2_rn(__fadd2_rn(t, both(-12582912.f)), both(-1.f), x);
   float2 y = __ffma2_rn(both(1.326472731307149e-3f), f, both(9.671512991189957e-3f));
@@ -88,7 +90,7 @@ AS_DEV float2 ex2_fma(float2 x) {
   y = __ffma2_rn(y, f, both(6.931470036506653e-1f));
   y = __ffma2_rn(y, f, both(1.f));
   const float2 p = make_float2(__uint_as_float((__float_as_uint(t.x) << 23) + 0x3f800000u), __uint_as_float((__float_as_uint(t.y) << 23) + 0x3f800000u));
-  return __fmul2_rn(y, p);
+  return fmul2_ftz(y, p);
 }
 
 template <int D>

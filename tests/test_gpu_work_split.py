@@ -131,3 +131,24 @@ def test_a_key_that_is_no_number_reaches_every_row(bad, d):
         else:                                                 # infinite scores where q_0 > 0: infinity less infinity; where q_0 < 0 a weight of 0
             assert bool(hit[dev["q"][0, 0, :, 0] > 0].all()), col
             assert not bool(hit[dev["q"][0, 0, :, 0] < 0].any()), col
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("N", [128, 300, 3969])
+def test_a_key_far_below_the_maximum_weighs_nothing(N, d):
+    """One key 2^260 above all others, whose values are near the end of the range: the rows are that key's value, in whichever column it is (a
+    weight of 2^-126 for one other key would add 1)."""
+    import torch
+    from paper_2509_24899_b200 import HybridAttention
+    wl, dev = _inputs(1, 1, N, d, 1, 75)
+    op = HybridAttention.from_workload(wl)
+    q, k, v = (torch.zeros_like(dev["q"]) for _ in range(3))
+    a = (130.0 / 1.4426950408889634 * d ** 0.5) ** 0.5
+    q[..., 0] = a
+    for col in [0, 1, 14, 15, 31, 47, 63, 64, 79, 126, 127]:
+        k[..., 0] = -a
+        k[0, 0, col, 0] = a
+        v.fill_(2.0 ** 126)
+        v[0, 0, col] = torch.arange(1, d + 1, device="cuda").to(v.dtype)
+        out = op.forward(q, k, v, dev["wq"], dev["wk"])
+        assert bool((out == v[0, 0, col]).all()), col
