@@ -473,6 +473,21 @@ __device__ __noinline__ bool q_accum_unit(const QParams& p, const QCtx& c, int u
 }
 
 // ---------------------------------------------------------------- feature rows of the linear tail
+// Biases of 2 * M columns as bf16 pairs, zeros without a bias: the loads (the same address in all lanes, or in half of them) go out together,
+// the first of a piece of 32 columns ahead of the columns' own load (nothing stands between that and its wait).  Each behind the test of its
+// pointer, one after the other, in a loop that is not unrolled, before; query stage with biases at N = 32760, 12 heads, one thread per row / two:
+// two layers 128 / 128, no softmax tokens 132 -> 115 / 134 -> 129 us, 8 key tiles 291 -> 277 / 299 -> 296; 256 / 256, 4 key tiles 306 -> 302 /
+// 283 -> 273; one layer, F = 256, 8 key tiles 383 -> 338 / 305 -> 303.
+template <int M>
+AS_DEV void q_bias(const uint32_t* row, int at, uint32_t (&w)[M]) {
+#pragma unroll
+  for (int i = 0; i < M; ++i) w[i] = 0u;
+  if (row != nullptr) {
+#pragma unroll
+    for (int i = 0; i < M; ++i) w[i] = __ldg(row + at + i);
+  }
+}
+
 // A thread's share of a row of Phi (feature chunk ch) from the score columns -> bf16(lam * poly(relu(Phi + b))) -> row r of `tile` (the A operand
 // of the apply product), 32 columns at a time (the loop is not unrolled: the tail runs once per unit, and on a CTA's first
 // unit its instructions come from L2 line by line, so its size is its cost).  Arrives on `sf_bar` once the last columns
@@ -488,9 +503,11 @@ AS_DEV float q_features_from_tmem(const QParams& p, uint32_t tSg, uint32_t sf_ba
   if (GEN && p.b2 != nullptr) brow = reinterpret_cast<const uint32_t*>(p.b2 + (size_t)(bh % p.H) * p.F + ch * 128 + hc * half);
   const float2 lam2 = make_float2(lam, lam);
   float2 dl2 = make_float2(0.f, 0.f);
-  uint32_t x[32];
+  constexpr int BW = 16 / T;                             // bias words at a time
+  uint32_t x[32], bw[BW];
 #pragma unroll 1
   for (int cc = 0; cc * 32 < half; ++cc) {
+    if (GEN) q_bias(brow, cc * 16, bw);
     if (D == 128 || fcw == 128) q_ld32<TPR, 64>(tSg + cc * 32, x);
     else q_ld32<TPR, 32>(tSg + cc * 32, x);
     tmem_ld_wait(x);
@@ -503,10 +520,10 @@ AS_DEV float q_features_from_tmem(const QParams& p, uint32_t tSg, uint32_t sf_ba
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       float a0 = __uint_as_float(x[2 * i]), a1 = __uint_as_float(x[2 * i + 1]);
-      if (GEN && brow != nullptr) {
-        const uint32_t bb = __ldg(brow + cc * 16 + i);            // same address in all lanes, or in half of them: broadcast loads
-        a0 += __uint_as_float(bb << 16);
-        a1 += __uint_as_float(bb & 0xffff0000u);
+      if (GEN) {
+        if (i > 0 && i % BW == 0) q_bias(brow, cc * 16 + i, bw);
+        a0 += __uint_as_float(bw[i % BW] << 16);
+        a1 += __uint_as_float(bw[i % BW] & 0xffff0000u);
       }
       const float2 a = make_float2(fmaxf(a0, 0.f), fmaxf(a1, 0.f));
       float2 rr = a;
@@ -570,7 +587,8 @@ __device__ __noinline__ float q_two_layer_tail(const QParams& p, const QRing<D>&
   constexpr int TPR = T, DC = D / TPR, FC = 128 / TPR;   // hidden units / features of a slice / chunk per thread
   const int nkv = p.nkv, h = bh % p.H, lane = threadIdx.x & 31;
   const __nv_bfloat16* b1 = (GEN && p.b1) ? p.b1 + (size_t)h * (q.nh * D) : nullptr;
-  uint32_t x[32];
+  constexpr int BW = 16 / T;                             // bias words at a time
+  uint32_t x[32], bw[BW];
   for (int j = 0; j < q.nh; ++j) {
     if (!q.wait(R::B_S + g, ps + nkv + j)) return -1.f;
     tc_fence_after();
@@ -582,16 +600,17 @@ __device__ __noinline__ float q_two_layer_tail(const QParams& p, const QRing<D>&
     uint8_t* tile = j == 0 ? sPg : sQg;
 #pragma unroll
     for (int cc = 0; cc < DC / 32; ++cc) {
+      if (GEN) q_bias(brow, cc * 16, bw);
       q_ld32<TPR, D / 2>(tSg + cc * 32, x);
       tmem_ld_wait(x);
       uint32_t wd[16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
         float a0 = __uint_as_float(x[2 * i]), a1 = __uint_as_float(x[2 * i + 1]);
-        if (brow != nullptr) {
-          const uint32_t bb = __ldg(brow + cc * 16 + i);
-          a0 += __uint_as_float(bb << 16);
-          a1 += __uint_as_float(bb & 0xffff0000u);
+        if (GEN) {
+          if (i > 0 && i % BW == 0) q_bias(brow, cc * 16 + i, bw);
+          a0 += __uint_as_float(bw[i % BW] << 16);
+          a1 += __uint_as_float(bw[i % BW] & 0xffff0000u);
         }
         wd[i] = pack_bf16(fmaxf(a0, 0.f), fmaxf(a1, 0.f));
       }
@@ -621,16 +640,17 @@ __device__ __noinline__ float q_two_layer_tail(const QParams& p, const QRing<D>&
     const uint32_t* brow = (GEN && p.b2) ? reinterpret_cast<const uint32_t*>(p.b2 + (size_t)h * p.F + hc * FC) : nullptr;
 #pragma unroll
     for (int cc = 0; cc < FC / 32; ++cc) {
+      if (GEN) q_bias(brow, cc * 16, bw);
       q_ld32<TPR, 64>(tSg + cc * 32, x);
       tmem_ld_wait(x);
       const int pw = min((hc * FC + cc * 32) / part, p.P - 1);
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
         float a0 = __uint_as_float(x[2 * i]), a1 = __uint_as_float(x[2 * i + 1]);
-        if (brow != nullptr) {
-          const uint32_t bb = __ldg(brow + cc * 16 + i);
-          a0 += __uint_as_float(bb << 16);
-          a1 += __uint_as_float(bb & 0xffff0000u);
+        if (GEN) {
+          if (i > 0 && i % BW == 0) q_bias(brow, cc * 16 + i, bw);
+          a0 += __uint_as_float(bw[i % BW] << 16);
+          a1 += __uint_as_float(bw[i % BW] & 0xffff0000u);
         }
         a0 = fmaxf(a0, 0.f); a1 = fmaxf(a1, 0.f);
         float r0 = a0, r1 = a1;
