@@ -164,7 +164,11 @@ struct QRing {
   // columns read out), P (P in tensor memory, phi_q in shared memory), PF (the product that reads it has completed),
   // O (output accumulator final), QF (nothing of the unit reads the Q tile any more), H (two layers: the
   // hidden activations are in shared memory); for both, two layers: PL (nothing reads the unit's P in tensor memory any more)
-  static constexpr int B_Q0 = 0, B_FULL = 2, B_EMPTY = B_FULL + KV_STAGES, B_S = B_EMPTY + KV_STAGES, B_SF = B_S + 2,
+  // Whether a ring slot is full is told on a barrier of the warp that will use the item: KFULL for what is multiplied into the score columns (K,
+  // weights), VFULL for what is added to O (V, S).  Each warp looks at every phase of its own barriers, in order.  (With one barrier for both a
+  // warp would look at some of its phases only, and a wait by parity for a phase two ahead of the last one looked at passes while
+  // the one between - a copy still under way for the other warp - is not over.)
+  static constexpr int B_Q0 = 0, B_KFULL = 2, B_VFULL = B_KFULL + KV_STAGES, B_EMPTY = B_VFULL + KV_STAGES, B_S = B_EMPTY + KV_STAGES, B_SF = B_S + 2,
                        B_P = B_SF + 2, B_PF = B_P + 2, B_O = B_PF + 2, B_QF = B_O + 2, B_H = B_QF + 2, B_PL = B_H + 2, B_COUNT = B_PL + 1;
   const QCtx c;              // by value: nothing here is re-read from memory after a barrier or an MMA
   int nkv, lin, two, fc, nh, vl;
@@ -219,7 +223,12 @@ struct QRing {
   }
   AS_DEV bool wait(int b, int phase) const { return mbar_wait_warp(bar(b), phase & 1, c.wc); }
   AS_DEV void release(int item) const { tc_commit(bar(B_EMPTY + item % KV_STAGES)); }
-  AS_DEV bool wait_full(int item) const { return wait(B_FULL + item % KV_STAGES, item / KV_STAGES); }
+  // `looks`: bit s is the parity of the next phase of the warp's barrier of slot s; it runs on across units
+  AS_DEV bool wait_full(int b, int item, uint32_t& looks) const {
+    const int slot = item % KV_STAGES, parity = (int)(looks >> slot) & 1;
+    looks ^= 1u << slot;
+    return wait(b + slot, parity);
+  }
 };
 
 // ---------------------------------------------------------------- TMA producer, one unit
@@ -251,27 +260,27 @@ __device__ __noinline__ bool q_produce_unit(const QParams& p, const QCtx& c, con
     const int gi = base + it, st = gi % KV_STAGES;
     if (!q.wait(R::B_EMPTY + st, gi / KV_STAGES + 1)) return false;
     if (lane == 0) {
-      mbar_expect_tx(q.bar(R::B_FULL + st), L::TILE);
-      const uint32_t fb = q.bar(R::B_FULL + st), dst = q.sKV(gi);
+      const uint32_t dst = q.sKV(gi);
+      auto to = [&](int b) { mbar_expect_tx(q.bar(b + st), L::TILE); return q.bar(b + st); };   // the barrier that the item arrives at
       if (it < q.n_stream) {
-        if (it == 0 || (it & 1)) load_tile<D>(dst, tmK, fb, ((it + 1) >> 1) * 128, bh);   // K_0 at 0, K_j at 2j-1
-        else load_tile<D>(dst, tmV, fb, ((it >> 1) - 1) * 128, bh);                        // V_j at 2j+2
+        if (it == 0 || (it & 1)) load_tile<D>(dst, tmK, to(R::B_KFULL), ((it + 1) >> 1) * 128, bh);   // K_0 at 0, K_j at 2j-1
+        else load_tile<D>(dst, tmV, to(R::B_VFULL), ((it >> 1) - 1) * 128, bh);                        // V_j at 2j+2
       } else if (q.vl && it == q.it_vlast()) {
-        load_tile<D>(dst, tmV, fb, (nkv - 1) * 128, bh);
+        load_tile<D>(dst, tmV, to(R::B_VFULL), (nkv - 1) * 128, bh);
       } else if (!TWO) {
         // W[ch] / S[ch] in bf16: [128 feature rows][D]; rows past F arrive as zeros
         const int r = it - q.n_stream - (it > q.n_stream ? q.vl : 0);     // 0: W[0]; 2ch-1: W[ch]; 2ch+2 (and the last): S[ch]
-        if (r == 0) load_tile<D>(dst, tmW, fb, 0, h);
-        else if (r == 2 * q.fc - 1) load_tile<D>(dst, tmSt, fb, (q.fc - 1) * 128, bh);
-        else if (r & 1) load_tile<D>(dst, tmW, fb, ((r + 1) >> 1) * 128, h);
-        else load_tile<D>(dst, tmSt, fb, ((r >> 1) - 1) * 128, bh);
+        if (r == 0) load_tile<D>(dst, tmW, to(R::B_KFULL), 0, h);
+        else if (r == 2 * q.fc - 1) load_tile<D>(dst, tmSt, to(R::B_VFULL), (q.fc - 1) * 128, bh);
+        else if (r & 1) load_tile<D>(dst, tmW, to(R::B_KFULL), ((r + 1) >> 1) * 128, h);
+        else load_tile<D>(dst, tmSt, to(R::B_VFULL), ((r >> 1) - 1) * 128, bh);
       } else {
         const int r = it - q.n_stream - (it > q.n_stream ? q.vl : 0);     // W1[0 .. nh-1], W2[c, j], S[c]
-        if (r < q.nh) load_tile<D>(dst, tmW1, fb, r * 128, h);                                  // hidden rows of slice r
+        if (r < q.nh) load_tile<D>(dst, tmW1, to(R::B_KFULL), r * 128, h);                                  // hidden rows of slice r
         else if (r < q.nh + q.fc * q.nh) {
           const int e = r - q.nh;
-          load_boxes(dst, tmW, fb, (e % q.nh) * D, (e / q.nh) * 128, h, D / 64);                // W2[feature chunk, hidden slice]
-        } else load_tile<D>(dst, tmSt, fb, (r - q.nh - q.fc * q.nh) * 128, bh);
+          load_boxes(dst, tmW, to(R::B_KFULL), (e % q.nh) * D, (e / q.nh) * 128, h, D / 64);                // W2[feature chunk, hidden slice]
+        } else load_tile<D>(dst, tmSt, to(R::B_VFULL), (r - q.nh - q.fc * q.nh) * 128, bh);
       }
     }
     __syncwarp();
@@ -279,7 +288,8 @@ __device__ __noinline__ bool q_produce_unit(const QParams& p, const QCtx& c, con
   return true;
 }
 
-// ---------------------------------------------------------------- MMA issuers, one unit
+// ---------------------------------------------------------------- MMA issuers, one unit: what to look for next (see wait_full), or Q_FAILED
+constexpr uint32_t Q_FAILED = ~0u;
 // Two issuing warps: one issues what writes the score columns (Q K^T per tile, Phi at the end) as soon as
 // the softmax threads have read them out, the other what accumulates into O (P V per tile, phi_q S at the end) as soon as
 // P is there.  The two streams touch different TMEM columns and release different ring items, so they
@@ -289,7 +299,7 @@ __device__ __noinline__ bool q_produce_unit(const QParams& p, const QCtx& c, con
 // 380); now 320 - 380 (130 for the four of Q K^T at d = 64).  N = 7800: 96.3 -> 93.7 us, headline layer 838 -> 830 us
 // (sustained), two-layer map 1203 -> 1176 us.
 template <int D, bool TWO, bool GEN, bool SH>
-__device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u) {
+__device__ __noinline__ uint32_t q_score_unit(const QParams& p, const QCtx& c, int u, uint32_t looks) {
   using R = QRing<D, SH>;
   constexpr uint32_t ID_QK = make_idesc(128, 128, 0, 0);      // S = Q K^T      (N = 128 keys)
   const int nkv = p.nkv, lin = p.lin;
@@ -310,9 +320,9 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
   // ---- first key tile (its product opens the unit)
   if (nkv > 0) {
     for (int g = 0; g < ng; ++g) {
-      if (!s_free(g, 0)) return false;
-      if (g == 0 && !q.wait_full(base)) return false;
-      if (!q.wait(R::B_Q0 + g, u)) return false;
+      if (!s_free(g, 0)) return Q_FAILED;
+      if (g == 0 && !q.wait_full(R::B_KFULL, base, looks)) return Q_FAILED;
+      if (!q.wait(R::B_Q0 + g, u)) return Q_FAILED;
       tc_fence_after();
       const uint64_t k0 = kmajor_desc(q.sKV(base));
       if (elect_one()) {
@@ -331,8 +341,8 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
 #pragma unroll
     for (int g = 0; g < 2; ++g) {
       if (g >= ng) break;
-      if (g == 0 && !q.wait_full(ik)) return false;
-      if (!s_free(g, j + 1)) return false;
+      if (g == 0 && !q.wait_full(R::B_KFULL, ik, looks)) return Q_FAILED;
+      if (!s_free(g, j + 1)) return Q_FAILED;
       tc_fence_after();
       if (elect_one()) {
 #pragma unroll
@@ -343,7 +353,7 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
     }
     if (elect_one()) q.release(ik);
   }
-  if (!lin) return true;
+  if (!lin) return looks;
 
   // ---- linear tail: what lands in the score columns after the last key tile
   if constexpr (!TWO) {
@@ -352,9 +362,9 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
       const int iw = base + q.it_w(ch);
       const uint64_t w0 = kmajor_desc(q.sKV(iw));
       for (int g = 0; g < ng; ++g) {
-        if (!s_free(g, nkv + ch)) return false;
-        if (nkv == 0 && ch == 0 && !q.wait(R::B_Q0 + g, u)) return false;
-        if (g == 0 && !q.wait_full(iw)) return false;
+        if (!s_free(g, nkv + ch)) return Q_FAILED;
+        if (nkv == 0 && ch == 0 && !q.wait(R::B_Q0 + g, u)) return Q_FAILED;
+        if (g == 0 && !q.wait_full(R::B_KFULL, iw, looks)) return Q_FAILED;
         tc_fence_after();
         if (elect_one()) {
 #pragma unroll
@@ -365,7 +375,7 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
       }
       if (elect_one()) q.release(iw);
     }
-    return true;
+    return looks;
   } else {
   // two layers: hidden slices first (A = Q), then Phi_c = sum_j h1_j W2[c, j]^T with the hidden slices read from
   // where the threads put them: slice 0 in the group's phi_q tile, slice 1 in its Q tile
@@ -373,9 +383,9 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
     const int iw = base + q.it_w(j);
     const uint64_t w0 = kmajor_desc(q.sKV(iw));
     for (int g = 0; g < ng; ++g) {
-      if (!s_free(g, nkv + j)) return false;
-      if (nkv == 0 && j == 0 && !q.wait(R::B_Q0 + g, u)) return false;
-      if (g == 0 && !q.wait_full(iw)) return false;
+      if (!s_free(g, nkv + j)) return Q_FAILED;
+      if (nkv == 0 && j == 0 && !q.wait(R::B_Q0 + g, u)) return Q_FAILED;
+      if (g == 0 && !q.wait_full(R::B_KFULL, iw, looks)) return Q_FAILED;
       tc_fence_after();
       if (elect_one()) {
 #pragma unroll
@@ -388,12 +398,12 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
   }
   for (int ch = 0; ch < q.fc; ++ch) {
     for (int g = 0; g < ng; ++g) {
-      if (!s_free(g, nkv + q.nh + ch)) return false;
-      if (ch == 0 && !q.wait(R::B_H + g, u)) return false;       // the group's hidden activations are in shared memory
+      if (!s_free(g, nkv + q.nh + ch)) return Q_FAILED;
+      if (ch == 0 && !q.wait(R::B_H + g, u)) return Q_FAILED;       // the group's hidden activations are in shared memory
       for (int j = 0; j < q.nh; ++j) {
         const int iw = base + q.it_w2(ch, j);
         const uint64_t w0 = kmajor_desc(q.sKV(iw));
-        if (g == 0 && !q.wait_full(iw)) return false;
+        if (g == 0 && !q.wait_full(R::B_KFULL, iw, looks)) return Q_FAILED;
         tc_fence_after();
         const uint64_t a0 = kmajor_desc(j == 0 ? q.sP(g) : q.sQ(g));
         if (elect_one()) {
@@ -410,12 +420,12 @@ __device__ __noinline__ bool q_score_unit(const QParams& p, const QCtx& c, int u
       }
     }
   }
-  return true;
+  return looks;
   }
 }
 
 template <int D, bool TWO, bool GEN, bool SH>
-__device__ __noinline__ bool q_accum_unit(const QParams& p, const QCtx& c, int u) {
+__device__ __noinline__ uint32_t q_accum_unit(const QParams& p, const QCtx& c, int u, uint32_t looks) {
   using R = QRing<D, SH>;
   constexpr uint32_t ID_PV = make_idesc(128, D, 0, 1);        // O += P V and O += phi_q S  (V, S are MN-major)
   const int nkv = p.nkv, lin = p.lin;
@@ -430,8 +440,8 @@ __device__ __noinline__ bool q_accum_unit(const QParams& p, const QCtx& c, int u
 #pragma unroll
     for (int g = 0; g < 2; ++g) {
       if (g >= ng) break;
-      if (g == 0 && !q.wait_full(iv)) return false;
-      if (!q.wait(R::B_P + g, pp + j)) return false;
+      if (g == 0 && !q.wait_full(R::B_VFULL, iv, looks)) return Q_FAILED;
+      if (!q.wait(R::B_P + g, pp + j)) return Q_FAILED;
       tc_fence_after();
       if (elect_one()) {
 #pragma unroll
@@ -443,7 +453,7 @@ __device__ __noinline__ bool q_accum_unit(const QParams& p, const QCtx& c, int u
     }
     if (elect_one()) q.release(iv);
   }
-  if (!lin) return true;
+  if (!lin) return looks;
   // O += phi_q,c S_c per feature chunk: phi_q sits in its tile (two layers, second chunk: in the Q tile),
   // S plays the part of a V tile
   const int ksteps = (D == 128 ? 128 : p.fcw) / 16;           // a constant at d = 128: the chains below unroll
@@ -452,8 +462,8 @@ __device__ __noinline__ bool q_accum_unit(const QParams& p, const QCtx& c, int u
     const uint64_t s0 = mnmajor_desc(q.sKV(is));
     const bool in_q_tile = TWO && ch == 1;
     for (int g = 0; g < ng; ++g) {
-      if (g == 0 && !q.wait_full(is)) return false;
-      if (!q.wait(R::B_P + g, pp + nkv + ch)) return false;
+      if (g == 0 && !q.wait_full(R::B_VFULL, is, looks)) return Q_FAILED;
+      if (!q.wait(R::B_P + g, pp + nkv + ch)) return Q_FAILED;
       tc_fence_after();
       const uint64_t a0 = kmajor_desc(in_q_tile ? q.sQ(g) : q.sP(g));
       if (elect_one()) {
@@ -469,7 +479,7 @@ __device__ __noinline__ bool q_accum_unit(const QParams& p, const QCtx& c, int u
     }
     if (elect_one()) q.release(is);
   }
-  return true;
+  return looks;
 }
 
 // ---------------------------------------------------------------- feature rows of the linear tail
@@ -984,7 +994,7 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
     mbar_init(bar(R::B_Q0), 1); mbar_init(bar(R::B_Q0 + 1), 1);
-    for (int s = 0; s < KV_STAGES; ++s) { mbar_init(bar(R::B_FULL + s), 1); mbar_init(bar(R::B_EMPTY + s), 1); }
+    for (int s = 0; s < KV_STAGES; ++s) { mbar_init(bar(R::B_KFULL + s), 1); mbar_init(bar(R::B_VFULL + s), 1); mbar_init(bar(R::B_EMPTY + s), 1); }
     for (int g = 0; g < 2; ++g) {
       mbar_init(bar(R::B_S + g), 1); mbar_init(bar(R::B_SF + g), 256); mbar_init(bar(R::B_P + g), 256);
       mbar_init(bar(R::B_PF + g), 1); mbar_init(bar(R::B_O + g), 1); mbar_init(bar(R::B_QF + g), 1);
@@ -1013,11 +1023,11 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     for (int u = 0; u < n_mine; ++u)
       if (!q_produce_unit<D, false, GEN>(p, c, &tmQ, &tmQ, &tmQ, &tmW, &tmSt, &tmW, u)) break;
   } else if (warp == 17) {
-    for (int u = 0; u < n_mine; ++u)
-      if (!q_score_unit<D, false, GEN, false>(p, c, u)) break;
+    uint32_t looks = 0u;
+    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_score_unit<D, false, GEN, false>(p, c, u, looks);
   } else if (warp == 18) {
-    for (int u = 0; u < n_mine; ++u)
-      if (!q_accum_unit<D, false, GEN, false>(p, c, u)) break;
+    uint32_t looks = 0u;
+    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_accum_unit<D, false, GEN, false>(p, c, u, looks);
   } else {
     const int g = (warp >> 2) & 1;
     // a unit worked on by one group only is the CTA's last one: group 1 stops before it
@@ -1055,7 +1065,7 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
     mbar_init(bar(R::B_Q0), 1); mbar_init(bar(R::B_Q0 + 1), 1);
-    for (int s = 0; s < KV_STAGES; ++s) { mbar_init(bar(R::B_FULL + s), 1); mbar_init(bar(R::B_EMPTY + s), 1); }
+    for (int s = 0; s < KV_STAGES; ++s) { mbar_init(bar(R::B_KFULL + s), 1); mbar_init(bar(R::B_VFULL + s), 1); mbar_init(bar(R::B_EMPTY + s), 1); }
     for (int g = 0; g < 2; ++g) {
       mbar_init(bar(R::B_S + g), 1); mbar_init(bar(R::B_SF + g), X::GROUP); mbar_init(bar(R::B_P + g), X::GROUP);
       mbar_init(bar(R::B_PF + g), 1); mbar_init(bar(R::B_O + g), 1); mbar_init(bar(R::B_QF + g), 1);
@@ -1085,11 +1095,11 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     for (int u = 0; u < n_mine; ++u)
       if (!q_produce_unit<D, TWO, GEN>(p, c, &tmQ, &tmK, &tmV, &tmW, &tmSt, &tmW1, u)) break;
   } else if (warp == X::W_SCORE) {
-    for (int u = 0; u < n_mine; ++u)
-      if (!q_score_unit<D, TWO, GEN, D == 128>(p, c, u)) break;
+    uint32_t looks = 0u;
+    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_score_unit<D, TWO, GEN, D == 128>(p, c, u, looks);
   } else if (warp == X::W_ACCUM) {
-    for (int u = 0; u < n_mine; ++u)
-      if (!q_accum_unit<D, TWO, GEN, D == 128>(p, c, u)) break;
+    uint32_t looks = 0u;
+    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_accum_unit<D, TWO, GEN, D == 128>(p, c, u, looks);
   } else {
     // a unit worked on by one group only is the CTA's last one: group 1 stops before it
     const int n_grp = (n_mine > p.n_rounds && ((warp >> 2) & 1) == 1 && q_unit(p, p.n_rounds).ng == 1) ? p.n_rounds : n_mine;
