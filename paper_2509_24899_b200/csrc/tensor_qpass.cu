@@ -52,6 +52,9 @@ struct QShape {
   // warps 0 .. 8 * TPR - 1: compute (quadrant = bits 0-1, group = bit 2, T = 2: half of the quadrant's rows = bit 3)
   static constexpr int THREADS = (W_TMA + 3) * 32, GROUP = 128 * TPR;
 };
+// The feature maps that the kernel with a key loop is compiled for: one layer whose tail is one product at d = 128 (F = 128; of any width at
+// d = 64), one layer of several products at d = 128, two layers.
+constexpr int MAP_ONE = 0, MAP_WIDE = 1, MAP_TWO = 2;
 constexpr int KV_STAGES = 3;
 constexpr float RESCALE_THRESHOLD = 8.f; // log2 units: rescale O only when the row max grew by > 2^8
 
@@ -120,8 +123,8 @@ struct QLayout {
 // group 1 has read its tile j.  A product into them takes 512 clk, the groups' reads 150 each and their waits and commits as much, so a
 // round is 2100 - 2500 clk where the exponentials of both groups take 2048 at the least: the groups run half a period
 // apart and little waits for the columns.  In the long tail of a two-layer map, where a group has little else to do than to wait for its
-// next columns, group 1 has the columns of both P's instead (32 key tiles 920 -> 890 us; the one-layer tail has as many products as feature
-// chunks, and the last P V to wait for costs more: N = 7800 79.4 -> 82.2 us).  One warp that issues everything in that fixed order, the second product in halves around
+// next columns, group 1 has the columns of both P's instead (32 key tiles 920 -> 890 us), and in that of a one-layer map with several feature
+// chunks (see own_tail).  One warp that issues everything in that fixed order, the second product in halves around
 // the next scores, is slower (full softmax 4700 -> 5130 us): issuing blocks it.
 //
 // The work of one unit is a function per role, kept out of line: each role then gets a register
@@ -163,7 +166,7 @@ struct QRing {
   // barrier indices; per group: S (scores, hidden activations or Phi landed in the score columns), SF (score
   // columns read out), P (P in tensor memory, phi_q in shared memory), PF (the product that reads it has completed),
   // O (output accumulator final), QF (nothing of the unit reads the Q tile any more), H (two layers: the
-  // hidden activations are in shared memory); for both, two layers: PL (nothing reads the unit's P in tensor memory any more)
+  // hidden activations are in shared memory); for both, a tail in columns of their own: PL (nothing reads the unit's P in tensor memory any more)
   // Whether a ring slot is full is told on a barrier of the warp that will use the item: KFULL for what is multiplied into the score columns (K,
   // weights), VFULL for what is added to O (V, S).  Each warp looks at every phase of its own barriers, in order.  (With one barrier for both a
   // warp would look at some of its phases only, and a wait by parity for a phase two ahead of the last one looked at passes while
@@ -208,17 +211,24 @@ struct QRing {
   AS_DEV uint32_t tS(int g) const { return SH ? c.tmem : c.tmem + 128u * g; }
   AS_DEV uint32_t tP(int g) const { return c.tmem + (SH ? 128u : 384u) + 64u * g; }
   AS_DEV uint32_t tO(int g) const { return c.tmem + 256u + (uint32_t)D * g; }
-  // Two layers: where the products of the linear tail land
-  AS_DEV uint32_t tTail(int g) const { return c.tmem + 128u * g; }
+  // At d = 128 a tail of several products lands in columns of each group's own: group 1 has those of both P's for it.  One layer with 256 features,
+  // N = 32760, 12 heads, groups in turn -> own columns, two threads per row / one: 1 key tile 118 -> 114 / 134 -> 119 us, 8 tiles 271 -> 265 /
+  // 281 -> 268; 512 features, 8 tiles 335 -> 323 / 367 -> 325.  (A tail of one product isn't worth the wait for the last P V of both groups:
+  // N = 7800 79.4 -> 82.2 us.)
+  template <int MAP>
+  static constexpr bool own_tail = SH && MAP != MAP_ONE;
+  template <int MAP>
+  AS_DEV uint32_t tTail(int g) const { return own_tail<MAP> ? c.tmem + 128u * g : tS(g); }
   // Before product i of the unit into group g's score columns, the ph-th of all: what lay there has been read.  With columns of its own
-  // (at d = 64; in a two-layer map's tail, where group 1 has the columns of both P's) by the group itself; else by the groups in turn.
+  // (at d = 64; in a tail as above) by the group itself; else by the groups in turn.
   // (A unit of one group, the CTA's last one, follows a unit of two.)
-  template <bool TWO>
+  template <int MAP>
   AS_DEV bool s_free(int g, int ph, int ng, int i, int u) const {
-    if (!SH || (TWO && (i > nkv || nkv == 0))) return ph == 0 ? true : wait(B_SF + g, ph - 1);
-    if (g == 1) return !TWO || i < nkv ? wait(B_SF, ph) : wait(B_PL, u);
+    constexpr bool OWN = own_tail<MAP>;
+    if (!SH || (OWN && (i > nkv || nkv == 0))) return ph == 0 ? true : wait(B_SF + g, ph - 1);
+    if (g == 1) return !OWN || i < nkv ? wait(B_SF, ph) : wait(B_PL, u);
     if (ph == 0) return true;
-    if (TWO && i == 0 && !wait(B_SF, ph - 1)) return false;   // the unit before: group 0's rows lay here, group 1's where P_0 will go
+    if (OWN && i == 0 && !wait(B_SF, ph - 1)) return false;   // the unit before: group 0's rows lay here, group 1's where P_0 will go
     return wait(B_SF + (ng == 2 || i == 0 ? 1 : 0), ph - 1);
   }
   AS_DEV bool wait(int b, int phase) const { return mbar_wait_warp(bar(b), phase & 1, c.wc); }
@@ -232,7 +242,7 @@ struct QRing {
 };
 
 // ---------------------------------------------------------------- TMA producer, one unit
-template <int D, bool TWO, bool GEN>
+template <int D, int MAP, bool GEN>
 __device__ __noinline__ bool q_produce_unit(const QParams& p, const QCtx& c, const CUtensorMap* tmQ, const CUtensorMap* tmK,
                                             const CUtensorMap* tmV, const CUtensorMap* tmW, const CUtensorMap* tmSt,
                                             const CUtensorMap* tmW1, int u) {
@@ -267,7 +277,7 @@ __device__ __noinline__ bool q_produce_unit(const QParams& p, const QCtx& c, con
         else load_tile<D>(dst, tmV, to(R::B_VFULL), ((it >> 1) - 1) * 128, bh);                        // V_j at 2j+2
       } else if (q.vl && it == q.it_vlast()) {
         load_tile<D>(dst, tmV, to(R::B_VFULL), (nkv - 1) * 128, bh);
-      } else if (!TWO) {
+      } else if (MAP != MAP_TWO) {
         // W[ch] / S[ch] in bf16: [128 feature rows][D]; rows past F arrive as zeros
         const int r = it - q.n_stream - (it > q.n_stream ? q.vl : 0);     // 0: W[0]; 2ch-1: W[ch]; 2ch+2 (and the last): S[ch]
         if (r == 0) load_tile<D>(dst, tmW, to(R::B_KFULL), 0, h);
@@ -298,7 +308,7 @@ constexpr uint32_t Q_FAILED = ~0u;
 // its own, eight MMAs took 630 - 700 clk to issue beside the softmax warps (N = 64, d = 64: as long, though they execute in
 // 380); now 320 - 380 (130 for the four of Q K^T at d = 64).  N = 7800: 96.3 -> 93.7 us, headline layer 838 -> 830 us
 // (sustained), two-layer map 1203 -> 1176 us.
-template <int D, bool TWO, bool GEN, bool SH>
+template <int D, int MAP, bool GEN, bool SH>
 __device__ __noinline__ uint32_t q_score_unit(const QParams& p, const QCtx& c, int u, uint32_t looks) {
   using R = QRing<D, SH>;
   constexpr uint32_t ID_QK = make_idesc(128, 128, 0, 0);      // S = Q K^T      (N = 128 keys)
@@ -315,7 +325,7 @@ __device__ __noinline__ uint32_t q_score_unit(const QParams& p, const QCtx& c, i
 #pragma unroll
     for (int kk = 0; kk < 8; ++kk) dq[g][kk] = q0 + kstep_kmajor(kk);
   }
-  auto s_free = [&](int g, int i) -> bool { return q.template s_free<TWO>(g, ps + i, ng, i, u); };
+  auto s_free = [&](int g, int i) -> bool { return q.template s_free<MAP>(g, ps + i, ng, i, u); };
 
   // ---- first key tile (its product opens the unit)
   if (nkv > 0) {
@@ -356,7 +366,7 @@ __device__ __noinline__ uint32_t q_score_unit(const QParams& p, const QCtx& c, i
   if (!lin) return looks;
 
   // ---- linear tail: what lands in the score columns after the last key tile
-  if constexpr (!TWO) {
+  if constexpr (MAP != MAP_TWO) {
     // Phi_c = Q W[c]^T, one chunk of features after the other
     for (int ch = 0; ch < q.fc; ++ch) {
       const int iw = base + q.it_w(ch);
@@ -368,7 +378,7 @@ __device__ __noinline__ uint32_t q_score_unit(const QParams& p, const QCtx& c, i
         tc_fence_after();
         if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tS(g), dq[g][kk], w0 + kstep_kmajor(kk), id_phi, kk > 0 ? 1u : 0u);
+          for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.template tTail<MAP>(g), dq[g][kk], w0 + kstep_kmajor(kk), id_phi, kk > 0 ? 1u : 0u);
           tc_commit(q.bar(R::B_S + g));
           if (ch == q.fc - 1) tc_commit(q.bar(R::B_QF + g));     // nothing of this unit reads the group's Q tile any more
         }
@@ -389,7 +399,7 @@ __device__ __noinline__ uint32_t q_score_unit(const QParams& p, const QCtx& c, i
       tc_fence_after();
       if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.tTail(g), dq[g][kk], w0 + kstep_kmajor(kk), ID_HID, kk > 0 ? 1u : 0u);
+        for (int kk = 0; kk < D / 16; ++kk) mma_ss(q.template tTail<MAP>(g), dq[g][kk], w0 + kstep_kmajor(kk), ID_HID, kk > 0 ? 1u : 0u);
         tc_commit(q.bar(R::B_S + g));
         if (q.nh == 1 && q.fc == 1) tc_commit(q.bar(R::B_QF + g));   // the Q tile is not reused as a buffer in this shape
       }
@@ -409,7 +419,7 @@ __device__ __noinline__ uint32_t q_score_unit(const QParams& p, const QCtx& c, i
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < D / 16; ++kk)
-            mma_ss(q.tTail(g), a0 + kstep_kmajor(kk), w0 + kstep_kmajor(kk), id_phi, (j > 0 || kk > 0) ? 1u : 0u);
+            mma_ss(q.template tTail<MAP>(g), a0 + kstep_kmajor(kk), w0 + kstep_kmajor(kk), id_phi, (j > 0 || kk > 0) ? 1u : 0u);
           if (j == q.nh - 1) {
             tc_commit(q.bar(R::B_S + g));
             // two hidden slices, one feature chunk: this was the last read of the Q tile (as a buffer)
@@ -424,7 +434,7 @@ __device__ __noinline__ uint32_t q_score_unit(const QParams& p, const QCtx& c, i
   }
 }
 
-template <int D, bool TWO, bool GEN, bool SH>
+template <int D, int MAP, bool GEN, bool SH>
 __device__ __noinline__ uint32_t q_accum_unit(const QParams& p, const QCtx& c, int u, uint32_t looks) {
   using R = QRing<D, SH>;
   constexpr uint32_t ID_PV = make_idesc(128, D, 0, 1);        // O += P V and O += phi_q S  (V, S are MN-major)
@@ -448,7 +458,7 @@ __device__ __noinline__ uint32_t q_accum_unit(const QParams& p, const QCtx& c, i
         for (int kk = 0; kk < 8; ++kk) mma_ts(q.tO(g), q.tP(g) + kk * 8, v0 + kstep_mnmajor(kk), ID_PV, (j > 0 || kk > 0) ? 1u : 0u);
         tc_commit(q.bar(R::B_PF + g));
         if (last && !lin) tc_commit(q.bar(R::B_O + g));
-        if (SH && TWO && last && lin && g == 1) tc_commit(q.bar(R::B_PL));    // (the other group's product was issued before)
+        if (R::template own_tail<MAP> && last && lin && g == 1) tc_commit(q.bar(R::B_PL));    // (the other group's product was issued before)
       }
     }
     if (elect_one()) q.release(iv);
@@ -460,7 +470,7 @@ __device__ __noinline__ uint32_t q_accum_unit(const QParams& p, const QCtx& c, i
   for (int ch = 0; ch < q.fc; ++ch) {
     const int is = base + q.it_st(ch);
     const uint64_t s0 = mnmajor_desc(q.sKV(is));
-    const bool in_q_tile = TWO && ch == 1;
+    const bool in_q_tile = MAP == MAP_TWO && ch == 1;
     for (int g = 0; g < ng; ++g) {
       if (g == 0 && !q.wait_full(R::B_VFULL, is, looks)) return Q_FAILED;
       if (!q.wait(R::B_P + g, pp + nkv + ch)) return Q_FAILED;
@@ -691,7 +701,7 @@ __device__ __noinline__ float q_two_layer_tail(const QParams& p, const QRing<D>&
 }
 
 // ---------------------------------------------------------------- softmax / merge group, one unit
-template <int D, int T, bool TWO, bool GEN>
+template <int D, int T, int MAP, bool GEN>
 __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, const CUtensorMap* tmO, uint8_t* smem, int u) {
   using R = QRing<D>;
   using L = QLayout<D>;
@@ -802,13 +812,14 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
     e = fminf(fmaxf(e, -100.f), 100.f);
     const float lam = ex2(e);
     float dl = 0.f;
-    if constexpr (!TWO) {
-      const bool ok = T == 1 ? q_one_layer_tail_apart<D, T, GEN>(p, c, g, tSg, sPg, r, hc, bh, ps, ppf, lam, dl)
-                             : q_one_layer_tail<D, T, GEN>(p, q, g, tSg, sPg, r, hc, bh, ps, ppf, lam, dl);
+    const uint32_t tTail = q.template tTail<MAP>(g) + lane_off;
+    if constexpr (MAP != MAP_TWO) {
+      const bool ok = T == 1 ? q_one_layer_tail_apart<D, T, GEN>(p, c, g, tTail, sPg, r, hc, bh, ps, ppf, lam, dl)
+                             : q_one_layer_tail<D, T, GEN>(p, q, g, tTail, sPg, r, hc, bh, ps, ppf, lam, dl);
       if (!ok) return false;
     } else {
       uint8_t* sQg = smem + L::Q_OFF + g * L::TILE;    // the group's Q tile: a second buffer once Q is done with
-      dl = q_two_layer_tail<D, T, GEN>(p, q, g, q.tTail(g) + lane_off, sPg, sQg, r, hc, bh, ps, ppf, lam);
+      dl = q_two_layer_tail<D, T, GEN>(p, q, g, tTail, sPg, sQg, r, hc, bh, ps, ppf, lam);
       if (dl < 0.f) return false;                      // a wait ran out (the sum itself is never negative)
     }
     if (X::TPR == 2) dl += __shfl_xor_sync(0xffffffffu, dl, 16);
@@ -1021,13 +1032,13 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   if (warp == 16) {
     if ((threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmW); tma_prefetch_desc(&tmSt); tma_prefetch_desc(&tmO); }
     for (int u = 0; u < n_mine; ++u)
-      if (!q_produce_unit<D, false, GEN>(p, c, &tmQ, &tmQ, &tmQ, &tmW, &tmSt, &tmW, u)) break;
+      if (!q_produce_unit<D, MAP_ONE, GEN>(p, c, &tmQ, &tmQ, &tmQ, &tmW, &tmSt, &tmW, u)) break;
   } else if (warp == 17) {
     uint32_t looks = 0u;
-    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_score_unit<D, false, GEN, false>(p, c, u, looks);
+    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_score_unit<D, MAP_ONE, GEN, false>(p, c, u, looks);
   } else if (warp == 18) {
     uint32_t looks = 0u;
-    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_accum_unit<D, false, GEN, false>(p, c, u, looks);
+    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_accum_unit<D, MAP_ONE, GEN, false>(p, c, u, looks);
   } else {
     const int g = (warp >> 2) & 1;
     // a unit worked on by one group only is the CTA's last one: group 1 stops before it
@@ -1045,7 +1056,7 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   }
 }
 
-template <int D, int T, bool TWO, bool GEN>
+template <int D, int T, int MAP, bool GEN>
 __global__ void __launch_bounds__(QShape<D, T>::THREADS, 1)
 qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
              const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmW,
@@ -1093,18 +1104,18 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   if (warp == X::W_TMA) {
     if ((threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); tma_prefetch_desc(&tmO); }
     for (int u = 0; u < n_mine; ++u)
-      if (!q_produce_unit<D, TWO, GEN>(p, c, &tmQ, &tmK, &tmV, &tmW, &tmSt, &tmW1, u)) break;
+      if (!q_produce_unit<D, MAP, GEN>(p, c, &tmQ, &tmK, &tmV, &tmW, &tmSt, &tmW1, u)) break;
   } else if (warp == X::W_SCORE) {
     uint32_t looks = 0u;
-    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_score_unit<D, TWO, GEN, D == 128>(p, c, u, looks);
+    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_score_unit<D, MAP, GEN, D == 128>(p, c, u, looks);
   } else if (warp == X::W_ACCUM) {
     uint32_t looks = 0u;
-    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_accum_unit<D, TWO, GEN, D == 128>(p, c, u, looks);
+    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_accum_unit<D, MAP, GEN, D == 128>(p, c, u, looks);
   } else {
     // a unit worked on by one group only is the CTA's last one: group 1 stops before it
     const int n_grp = (n_mine > p.n_rounds && ((warp >> 2) & 1) == 1 && q_unit(p, p.n_rounds).ng == 1) ? p.n_rounds : n_mine;
     for (int u = 0; u < n_grp; ++u)
-      if (!q_softmax_unit<D, T, TWO, GEN>(p, c, &tmO, smem, u)) break;
+      if (!q_softmax_unit<D, T, MAP, GEN>(p, c, &tmO, smem, u)) break;
     if ((threadIdx.x & 31) == 0) tma_store_wait_read();  // this warp's output stores have read their rows (the writes land by the end of the kernel)
   }
 
@@ -1121,18 +1132,13 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 
 cudaError_t as_tensor_init_qpass() {
   cudaError_t e;
-  if ((e = opt_in_smem(qpass_kernel<128, 1, false, false>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<128, 2, false, false>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<128, 1, false, true>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<128, 2, false, true>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<128, 1, true, false>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<128, 2, true, false>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<128, 1, true, true>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<128, 2, true, true>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<64, 2, false, false>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<64, 2, false, true>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<64, 2, true, false>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(qpass_kernel<64, 2, true, true>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
+#define AS_OPT_IN_Q(D_, T_, MAP_) \
+  if ((e = opt_in_smem(qpass_kernel<D_, T_, MAP_, false>, QLayout<D_>::TOTAL)) != cudaSuccess) return e; \
+  if ((e = opt_in_smem(qpass_kernel<D_, T_, MAP_, true>, QLayout<D_>::TOTAL)) != cudaSuccess) return e
+  AS_OPT_IN_Q(128, 1, MAP_ONE); AS_OPT_IN_Q(128, 1, MAP_WIDE); AS_OPT_IN_Q(128, 1, MAP_TWO);
+  AS_OPT_IN_Q(128, 2, MAP_ONE); AS_OPT_IN_Q(128, 2, MAP_WIDE); AS_OPT_IN_Q(128, 2, MAP_TWO);
+  AS_OPT_IN_Q(64, 2, MAP_ONE); AS_OPT_IN_Q(64, 2, MAP_TWO);
+#undef AS_OPT_IN_Q
   if ((e = opt_in_smem(qlin_kernel<128, false>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
   if ((e = opt_in_smem(qlin_kernel<128, true>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
   if ((e = opt_in_smem(qlin_kernel<64, false>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
@@ -1221,15 +1227,17 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
     if (gen) AS_LAUNCH_QL(64, true); else AS_LAUNCH_QL(64, false);
 #undef AS_LAUNCH_QL
   }
-#define AS_LAUNCH_Q(D_, T_, TWO_, GEN_) \
-  return as_launch_dependent(qpass_kernel<D_, T_, TWO_, GEN_>, grid, dim3(QShape<D_, T_>::THREADS), QLayout<D_>::TOTAL, st, tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO, p)
-#define AS_LAUNCH_QT(D_, T_) \
+#define AS_LAUNCH_Q(D_, T_, MAP_) \
   do { \
-    if (two) { if (gen) AS_LAUNCH_Q(D_, T_, true, true); else AS_LAUNCH_Q(D_, T_, true, false); } \
-    else { if (gen) AS_LAUNCH_Q(D_, T_, false, true); else AS_LAUNCH_Q(D_, T_, false, false); } \
+    if (gen) return as_launch_dependent(qpass_kernel<D_, T_, MAP_, true>, grid, dim3(QShape<D_, T_>::THREADS), QLayout<D_>::TOTAL, st, tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO, p); \
+    return as_launch_dependent(qpass_kernel<D_, T_, MAP_, false>, grid, dim3(QShape<D_, T_>::THREADS), QLayout<D_>::TOTAL, st, tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO, p); \
   } while (0)
-  if (a.d == 128) { if (tpr == 2) AS_LAUNCH_QT(128, 2); else AS_LAUNCH_QT(128, 1); }
-  AS_LAUNCH_QT(64, 2);
+#define AS_LAUNCH_QT(T_) \
+  do { \
+    if (two) AS_LAUNCH_Q(128, T_, MAP_TWO); else if (lin && p.fc > 1) AS_LAUNCH_Q(128, T_, MAP_WIDE); else AS_LAUNCH_Q(128, T_, MAP_ONE); \
+  } while (0)
+  if (a.d == 128) { if (tpr == 2) AS_LAUNCH_QT(2); else AS_LAUNCH_QT(1); }
+  if (two) AS_LAUNCH_Q(64, 2, MAP_TWO); else AS_LAUNCH_Q(64, 2, MAP_ONE);
 #undef AS_LAUNCH_QT
 #undef AS_LAUNCH_Q
 }
