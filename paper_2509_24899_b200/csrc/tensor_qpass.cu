@@ -1153,11 +1153,6 @@ cudaError_t as_tensor_init_qpass() {
 // us; N = 1024 with 2 heads on 16 CTAs instead of 8: 22.5 -> 21.4).  Returns the
 // number of CTAs.
 namespace {
-// Threads per row of the kernel with a key loop.  Two (sixteen compute warps) keep the special-function unit busier and turn the rows of
-// the tail around faster; but at d = 128, where the groups take turns at the score columns, a long key loop goes better with one.
-// Layers with 12 heads, against P through shared memory, two / one: 3 key tiles 1.09 / 1.01, 8 1.07 / 1.01, 16 1.07 / 1.03, 20 1.035 / 1.01, 31
-// 1.06 / 1.02, 32 1.016 / 1.018, 64 1.016 / 1.03, 128 1.013 / 1.035; two-layer maps, 32 tiles 1.045 / 1.06.
-int q_threads_per_row(int d, int nkv, bool two) { return d == 64 || nkv <= (two ? 16 : 31) ? 2 : 1; }
 int plan_units(QParams& p, int BH, int sms) {
   const int tiles = (p.N + 127) / 128;
   double best = 0.;
@@ -1176,6 +1171,21 @@ int plan_units(QParams& p, int BH, int sms) {
   }
   return grid;
 }
+// Threads per row of the kernel with a key loop (after plan_units).  Two (sixteen compute warps) hide more of the latencies, one draws less power per
+// exponential and has 168 registers where two have 96.  At d = 64 always two.  At d = 128 the gain of two over one in the query stage, on layers that differ in
+// the number of key tiles only (12 heads, N = 32760, 16384, 7800 and 24 heads, N = 2430; bursts of 3 ms / runs of 0.12 s, which the power cap
+// slows down):
+//   a CTA has one tile at most (2 heads, N = 4096), so that one group has the SM to itself: 4 - 10 % at any length with one layer, 0 - 5 % with two;
+//   one layer without biases: 4 tiles 3 - 8 % / 1 - 6 %, 8 0 - 2 / 0 - 3, 16 0 - 3 / -1 - +1, 24 1 / -1, 48 0 / -1, 96 0 / -1 - -3 (F = 256 alike);
+//   one layer with biases or powers beyond 2: 8 tiles 6 - 12 / 5 - 7, 16 3 - 5 / 2, 31 3 - 5 / 0 - 2, 48 1 - 4 / -2 - +1, 96 1 - 3 / -1 - 0;
+//   two layers: -2 - -4 / -3 - -5 at almost any length, without softmax tokens -3 - -14 / -3 - -11; with biases and two
+//   feature chunks, which one thread has to keep in its registers, 16 tiles +3 - +8 / +3 - +5, 32 +3 - +5 / 0 - 2, 48 1 - 7 / -1 - +3.
+int q_threads_per_row(const QParams& p, int d, bool two, bool gen) {
+  const bool one_tile_each = p.n_rounds == 0 && p.split_last;
+  if (d == 64 || one_tile_each) return 2;
+  if (two) return gen && p.fc > 1 && p.nkv <= 32 ? 2 : 1;
+  return p.nkv <= (gen ? 40 : 16) ? 2 : 1;
+}
 }  // namespace
 
 cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
@@ -1185,24 +1195,6 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   CUtensorMap tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO;
   const bool two = lin && a.layers == 2;
   const bool qlin = a.n_s == 0 && lin && !two;         // no softmax tokens, one-layer map: the variant without a key loop
-  const int tpr = q_threads_per_row(a.d, (a.n_s + 127) / 128, two);
-  // the output is stored warp by warp: boxes of a warp's rows
-  if (!make_map(&tmQ, a.q, a.d, a.N, BH, 128) || !make_map(&tmO, a.out, a.d, a.N, BH, qlin ? 32 : 32 / tpr)) return cudaErrorInvalidValue;
-  if (a.n_s > 0) {
-    if (!make_map(&tmK, a.ks, a.d, a.n_s, BH, 128) || !make_map(&tmV, a.vs, a.d, a.n_s, BH, 128)) return cudaErrorInvalidValue;
-  } else {
-    tmK = tmQ; tmV = tmQ;       // never used: the key loop is empty
-  }
-  if (lin) {
-    // boxes are always 128 rows: rows past F (or the hidden width) are out of bounds and arrive as zeros.
-    // tmW: last-layer weights [H][F][width of their input]; tmW1: first-layer weights of a two-layer map.
-    if (!make_map(&tmW, two ? a.wq2 : a.wq, two ? a.hid : a.d, a.F, a.H, 128) || !make_map(&tmSt, a.Sb, a.d, a.F, BH, 128))
-      return cudaErrorInvalidValue;
-  } else {
-    tmW = tmQ; tmSt = tmQ;      // never used: no linear branch at rate 1
-  }
-  if (two) { if (!make_map(&tmW1, a.wq, a.d, a.hid, a.H, 128)) return cudaErrorInvalidValue; }
-  else tmW1 = tmQ;            // never used with a one-layer map
   QParams p{};
   p.layers = lin ? a.layers : 1;
   p.N = a.N; p.n_s = a.n_s; p.nkv = (a.n_s + 127) / 128; p.lin = lin ? 1 : 0; p.stab_mode = a.stab_mode; p.P = a.P;
@@ -1220,6 +1212,24 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   const dim3 grid(plan_units(p, BH, sms), 1, 1);
   // the general kernels carry the bias and the powers beyond 2; the common case does without them
   const bool gen = lin && (a.P > 2 || p.b1 != nullptr || p.b2 != nullptr);
+  const int tpr = q_threads_per_row(p, a.d, two, gen);
+  // the output is stored warp by warp: boxes of a warp's rows
+  if (!make_map(&tmQ, a.q, a.d, a.N, BH, 128) || !make_map(&tmO, a.out, a.d, a.N, BH, qlin ? 32 : 32 / tpr)) return cudaErrorInvalidValue;
+  if (a.n_s > 0) {
+    if (!make_map(&tmK, a.ks, a.d, a.n_s, BH, 128) || !make_map(&tmV, a.vs, a.d, a.n_s, BH, 128)) return cudaErrorInvalidValue;
+  } else {
+    tmK = tmQ; tmV = tmQ;       // never used: the key loop is empty
+  }
+  if (lin) {
+    // boxes are always 128 rows: rows past F (or the hidden width) are out of bounds and arrive as zeros.
+    // tmW: last-layer weights [H][F][width of their input]; tmW1: first-layer weights of a two-layer map.
+    if (!make_map(&tmW, two ? a.wq2 : a.wq, two ? a.hid : a.d, a.F, a.H, 128) || !make_map(&tmSt, a.Sb, a.d, a.F, BH, 128))
+      return cudaErrorInvalidValue;
+  } else {
+    tmW = tmQ; tmSt = tmQ;      // never used: no linear branch at rate 1
+  }
+  if (two) { if (!make_map(&tmW1, a.wq, a.d, a.hid, a.H, 128)) return cudaErrorInvalidValue; }
+  else tmW1 = tmQ;            // never used with a one-layer map
   if (qlin) {
 #define AS_LAUNCH_QL(D_, GEN_) \
   return as_launch_dependent(qlin_kernel<D_, GEN_>, grid, dim3(QL_THREADS), QLayout<D_>::TOTAL, st, tmQ, tmW, tmSt, tmO, p)
