@@ -44,13 +44,12 @@ struct QParams {
 
 // How the compute threads share a 128-row tile: T = 1, one thread per row (eight warps), or T = 2, threads t and t + 16 of a warp, each
 // with half of the row's columns (sixteen warps; the two share their maxima and sums by one shuffle).  cf. q_threads_per_row.
-template <int D, int T>
+template <int T>
 struct QShape {
-  static constexpr int TPR = T;                            // threads per row
-  static constexpr int COLS = 128 / TPR;                   // score columns of a thread
-  static constexpr int W_TMA = 8 * TPR, W_SCORE = W_TMA + 1, W_ACCUM = W_TMA + 2;
-  // warps 0 .. 8 * TPR - 1: compute (quadrant = bits 0-1, group = bit 2, T = 2: half of the quadrant's rows = bit 3)
-  static constexpr int THREADS = (W_TMA + 3) * 32, GROUP = 128 * TPR;
+  static constexpr int COLS = 128 / T;                     // score columns of a thread
+  static constexpr int W_TMA = 8 * T, W_SCORE = W_TMA + 1, W_ACCUM = W_TMA + 2;
+  // warps 0 .. 8 * T - 1: compute (quadrant = bits 0-1, group = bit 2, T = 2: half of the quadrant's rows = bit 3)
+  static constexpr int THREADS = (W_TMA + 3) * 32, GROUP = 128 * T;
 };
 // The feature maps that the kernel with a key loop is compiled for: one layer whose tail is one product at d = 128 (F = 128; of any width at
 // d = 64), one layer of several products at d = 128, two layers.
@@ -59,23 +58,19 @@ constexpr int KV_STAGES = 3;
 constexpr float RESCALE_THRESHOLD = 8.f; // log2 units: rescale O only when the row max grew by > 2^8
 
 // A thread's share of a row (of 32 columns in TMEM; SPLIT: distance of the two threads' shares where two share a row)
-template <int TPR, int SPLIT>
+template <int T, int SPLIT>
 AS_DEV void q_ld32(uint32_t t, uint32_t (&x)[32]) {
-  if constexpr (TPR == 1) tmem_ld32(t, x); else tmem_ldh32<SPLIT>(t, x);
+  if constexpr (T == 1) tmem_ld32(t, x); else tmem_ldh32<SPLIT>(t, x);
 }
-template <int TPR, int SPLIT>
+template <int T, int SPLIT>
 AS_DEV void q_ld16(uint32_t t, uint32_t (&x)[16]) {
-  if constexpr (TPR == 1) tmem_ld16(t, x); else tmem_ldh16<SPLIT>(t, x);
+  if constexpr (T == 1) tmem_ld16(t, x); else tmem_ldh16<SPLIT>(t, x);
 }
-template <int TPR, int SPLIT>
+template <int T, int SPLIT>
 AS_DEV void q_st16(uint32_t t, const uint32_t (&x)[16]) {
-  if constexpr (TPR == 1) tmem_st16(t, x); else tmem_sth16<SPLIT>(t, x);
+  if constexpr (T == 1) tmem_st16(t, x); else tmem_sth16<SPLIT>(t, x);
 }
 
-// Of every EX2_FMA_EVERY-th group of four exponentials two are taken on the FMA pipe (0: none).  Sixteen warps: one in eight of all (the
-// special-function unit, 16 a clock, is what four warps per sub-partition wait for): d = 64, N 8505, 2142 keys 293 -> 279 us; one in
-// sixteen 284, one in four 304.  Eight warps: no gain (81 frames of full softmax 4637 us; one in sixteen 4650, one in eight 4709).
-template <int T> constexpr int EX2_FMA_EVERY = T == 2 ? 4 : 0;
 // Two exponentials 2^x, x <= 8, on the FMA pipe: x = n + f with n the nearest integer (added into the last bits of 1.5 * 2^23), 2^f by
 // the polynomial of degree 5 with constant term 1 that is closest to it on [-1/2, 1/2] in relative error (1.08e-7 with the coefficients
 // rounded, found by reweighted least squares), times 2^n put together from its exponent.  Within 1.72e-7 of 2^x for all x in [-126, 8]
@@ -95,6 +90,12 @@ AS_DEV float2 ex2_fma(float2 x) {
   const float2 p = make_float2(__uint_as_float((__float_as_uint(t.x) << 23) + 0x3f800000u), __uint_as_float((__float_as_uint(t.y) << 23) + 0x3f800000u));
   return fmul2_ftz(y, p);
 }
+
+// The second two of the i-th group of four exponentials.  Sixteen warps: every fourth such pair on the FMA pipe, one exponential in eight of all (the
+// special-function unit, 16 a clock, is what four warps per sub-partition wait for): d = 64, N 8505, 2142 keys 293 -> 279 us; one in
+// sixteen 284, one in four 304.  Eight warps: none (81 frames of full softmax 4637 us; one in sixteen 4650, one in eight 4709).
+template <int T>
+AS_DEV float2 ex2_second_pair(int i, float2 x) { return T == 2 && i % 4 == 3 ? ex2_fma(x) : make_float2(ex2(x.x), ex2(x.y)); }
 
 template <int D>
 struct QLayout {
@@ -493,19 +494,38 @@ __device__ __noinline__ uint32_t q_accum_unit(const QParams& p, const QCtx& c, i
 }
 
 // ---------------------------------------------------------------- feature rows of the linear tail
-// Biases of 2 * M columns as bf16 pairs, zeros without a bias: the loads (the same address in all lanes, or in half of them) go out together,
-// the first of a piece of 32 columns ahead of the columns' own load (nothing stands between that and its wait).  Each behind the test of its
-// pointer, one after the other, in a loop that is not unrolled, before; query stage with biases at N = 32760, 12 heads, one thread per row / two:
-// two layers 128 / 128, no softmax tokens 132 -> 115 / 134 -> 129 us, 8 key tiles 291 -> 277 / 299 -> 296; 256 / 256, 4 key tiles 306 -> 302 /
-// 283 -> 273; one layer, F = 256, 8 key tiles 383 -> 338 / 305 -> 303.
-template <int M>
-AS_DEV void q_bias(const uint32_t* row, int at, uint32_t (&w)[M]) {
+// The biases of 32 columns as bf16 pairs, zeros without a bias; their loads (the same address in all lanes, or in half of them) go out together.
+AS_DEV void q_ask_bias(const uint32_t* row, uint32_t (&w)[16]) {
 #pragma unroll
-  for (int i = 0; i < M; ++i) w[i] = 0u;
-  if (row != nullptr) {
+  for (int i = 0; i < 16; ++i) w[i] = 0u;
+  if (row == nullptr) return;
 #pragma unroll
-    for (int i = 0; i < M; ++i) w[i] = __ldg(row + at + i);
+  for (int i = 0; i < 16; ++i) w[i] = __ldg(row + i);
+}
+AS_DEV void q_add_bias(const uint32_t (&w)[16], uint32_t (&x)[32]) {
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const float2 y = __fadd2_rn(make_float2(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])),
+                                make_float2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u)));
+    x[2 * i] = __float_as_uint(y.x);
+    x[2 * i + 1] = __float_as_uint(y.y);
   }
+}
+// 32 columns of a thread's row (of its share, SPLIT as in q_ld32) with their biases added.  One thread per row has the registers to ask for the
+// biases ahead of the columns (nothing stands between the columns' load and its wait); with two the other warps cover that latency, and the
+// sums are left out where there is no bias.  Each bias behind the test of its pointer, one after the other, before; query stage with biases at
+// N = 32760, 12 heads: two layers 128 / 128, no softmax tokens, one thread per row 132 -> 115 us, 8 key tiles 291 -> 277; whole layers at N = 7800,
+// rate 1/8, two threads: 256 / 256 162 -> 158, one layer with F = 256 105.0 -> 104.6, with F = 128 and degree 4 87.6 -> 86.4.  (Asked for ahead with
+// two threads per row, 8 at a time: the features' registers spill, degree 4 without a bias 1 % slower.)
+template <int T, int SPLIT, bool GEN>
+AS_DEV void q_ld32_biased(uint32_t t, const uint32_t* row, uint32_t (&x)[32], bool half_split = false) {
+  uint32_t w[16];
+  if (GEN && T == 1) q_ask_bias(row, w);
+  if (half_split) q_ld32<T, SPLIT / 2>(t, x);
+  else q_ld32<T, SPLIT>(t, x);
+  tmem_ld_wait(x);
+  if (GEN && T == 1) q_add_bias(w, x);
+  if (GEN && T == 2 && row != nullptr) { q_ask_bias(row, w); q_add_bias(w, x); }
 }
 
 // A thread's share of a row of Phi (feature chunk ch) from the score columns -> bf16(lam * poly(relu(Phi + b))) -> row r of `tile` (the A operand
@@ -515,22 +535,17 @@ AS_DEV void q_bias(const uint32_t* row, int at, uint32_t (&w)[M]) {
 // GEN = false is the common case (no bias, polynomial degree <= 2).
 template <int D, int T, bool GEN>
 AS_DEV float q_features_from_tmem(const QParams& p, uint32_t tSg, uint32_t sf_bar, uint8_t* tile, int r, int hc, int bh, int ch, float lam) {
-  constexpr int TPR = T;
-  const int fcw = D == 128 ? 128 : p.fcw, half = fcw / TPR;
+  const int fcw = D == 128 ? 128 : p.fcw, half = fcw / T;
   const int part = p.F / p.P;
   const float2* zrow = reinterpret_cast<const float2*>(p.z + (size_t)bh * p.F + ch * 128 + hc * half);
   const uint32_t* brow = nullptr;
   if (GEN && p.b2 != nullptr) brow = reinterpret_cast<const uint32_t*>(p.b2 + (size_t)(bh % p.H) * p.F + ch * 128 + hc * half);
   const float2 lam2 = make_float2(lam, lam);
   float2 dl2 = make_float2(0.f, 0.f);
-  constexpr int BW = 16 / T;                             // bias words at a time
-  uint32_t x[32], bw[BW];
+  uint32_t x[32];
 #pragma unroll 1
   for (int cc = 0; cc * 32 < half; ++cc) {
-    if (GEN) q_bias(brow, cc * 16, bw);
-    if (D == 128 || fcw == 128) q_ld32<TPR, 64>(tSg + cc * 32, x);
-    else q_ld32<TPR, 32>(tSg + cc * 32, x);
-    tmem_ld_wait(x);
+    q_ld32_biased<T, 64, GEN>(tSg + cc * 32, brow == nullptr ? nullptr : brow + cc * 16, x, D == 64 && fcw == 64);
     if (cc * 32 + 32 >= half) {
       tc_fence_before();
       mbar_arrive(sf_bar);                             // the next product into the score columns may follow
@@ -539,13 +554,7 @@ AS_DEV float q_features_from_tmem(const QParams& p, uint32_t tSg, uint32_t sf_ba
     uint32_t wd[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-      float a0 = __uint_as_float(x[2 * i]), a1 = __uint_as_float(x[2 * i + 1]);
-      if (GEN) {
-        if (i > 0 && i % BW == 0) q_bias(brow, cc * 16 + i, bw);
-        a0 += __uint_as_float(bw[i % BW] << 16);
-        a1 += __uint_as_float(bw[i % BW] & 0xffff0000u);
-      }
-      const float2 a = make_float2(fmaxf(a0, 0.f), fmaxf(a1, 0.f));
+      const float2 a = make_float2(fmaxf(__uint_as_float(x[2 * i]), 0.f), fmaxf(__uint_as_float(x[2 * i + 1]), 0.f));
       float2 rr = a;
       if (pw >= 1) rr = __fmul2_rn(rr, a);
       if (GEN) {
@@ -585,9 +594,10 @@ AS_DEV bool q_one_layer_tail(const QParams& p, const QRing<D>& q, int g, uint32_
   return true;
 }
 
-// The same out of line.  With a score row in a thread's registers the key loop spills some of what it needs in every tile when the tail stands
-// beside it (81 frames at rate 1/8 717 us, full softmax 4840; with this 697 and 4675); with half a row it does not, and the call
-// costs more (d = 64, 2142 keys 279 -> 290).
+// The same out of line.  With a score row in a thread's registers, and the tail beside it, the key loop spills some of what it needs in every
+// tile (81 frames at rate 1/8 717 us, full softmax 4840; with this 697 and 4675).  That is not all of it: q_softmax_unit<128, 1, ., .> still
+// reloads 76 bytes (44 with biases) and stores 0 (8), as -Xptxas -v counts them.  With half a row (0 and 20) the call costs more than it gains (d = 64,
+// 2142 keys 279 -> 290).
 template <int D, int T, bool GEN>
 __device__ __noinline__ bool q_one_layer_tail_apart(const QParams& p, const QCtx& c, int g, uint32_t tSg, uint8_t* sPg, int r, int hc, int bh, int ps, int ppf,
                                                     float lam, float& dl) {
@@ -604,11 +614,10 @@ template <int D, int T, bool GEN>
 __device__ __noinline__ float q_two_layer_tail(const QParams& p, const QRing<D>& q, int g, uint32_t tSg, uint8_t* sPg, uint8_t* sQg, int r, int hc,
                                                int bh, int ps, int ppf, float lam) {
   using R = QRing<D>;
-  constexpr int TPR = T, DC = D / TPR, FC = 128 / TPR;   // hidden units / features of a slice / chunk per thread
+  constexpr int DC = D / T, FC = 128 / T;   // hidden units / features of a slice / chunk per thread
   const int nkv = p.nkv, h = bh % p.H, lane = threadIdx.x & 31;
   const __nv_bfloat16* b1 = (GEN && p.b1) ? p.b1 + (size_t)h * (q.nh * D) : nullptr;
-  constexpr int BW = 16 / T;                             // bias words at a time
-  uint32_t x[32], bw[BW];
+  uint32_t x[32];
   for (int j = 0; j < q.nh; ++j) {
     if (!q.wait(R::B_S + g, ps + nkv + j)) return -1.f;
     tc_fence_after();
@@ -620,19 +629,11 @@ __device__ __noinline__ float q_two_layer_tail(const QParams& p, const QRing<D>&
     uint8_t* tile = j == 0 ? sPg : sQg;
 #pragma unroll
     for (int cc = 0; cc < DC / 32; ++cc) {
-      if (GEN) q_bias(brow, cc * 16, bw);
-      q_ld32<TPR, D / 2>(tSg + cc * 32, x);
-      tmem_ld_wait(x);
+      q_ld32_biased<T, D / 2, GEN>(tSg + cc * 32, brow == nullptr ? nullptr : brow + cc * 16, x);
       uint32_t wd[16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
-        float a0 = __uint_as_float(x[2 * i]), a1 = __uint_as_float(x[2 * i + 1]);
-        if (GEN) {
-          if (i > 0 && i % BW == 0) q_bias(brow, cc * 16 + i, bw);
-          a0 += __uint_as_float(bw[i % BW] << 16);
-          a1 += __uint_as_float(bw[i % BW] & 0xffff0000u);
-        }
-        wd[i] = pack_bf16(fmaxf(a0, 0.f), fmaxf(a1, 0.f));
+        wd[i] = pack_bf16(fmaxf(__uint_as_float(x[2 * i]), 0.f), fmaxf(__uint_as_float(x[2 * i + 1]), 0.f));
       }
       store_row_chunk(tile, r, hc * DC + cc * 32, wd);
     }
@@ -660,19 +661,11 @@ __device__ __noinline__ float q_two_layer_tail(const QParams& p, const QRing<D>&
     const uint32_t* brow = (GEN && p.b2) ? reinterpret_cast<const uint32_t*>(p.b2 + (size_t)h * p.F + hc * FC) : nullptr;
 #pragma unroll
     for (int cc = 0; cc < FC / 32; ++cc) {
-      if (GEN) q_bias(brow, cc * 16, bw);
-      q_ld32<TPR, 64>(tSg + cc * 32, x);
-      tmem_ld_wait(x);
+      q_ld32_biased<T, 64, GEN>(tSg + cc * 32, brow == nullptr ? nullptr : brow + cc * 16, x);
       const int pw = min((hc * FC + cc * 32) / part, p.P - 1);
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
-        float a0 = __uint_as_float(x[2 * i]), a1 = __uint_as_float(x[2 * i + 1]);
-        if (GEN) {
-          if (i > 0 && i % BW == 0) q_bias(brow, cc * 16 + i, bw);
-          a0 += __uint_as_float(bw[i % BW] << 16);
-          a1 += __uint_as_float(bw[i % BW] & 0xffff0000u);
-        }
-        a0 = fmaxf(a0, 0.f); a1 = fmaxf(a1, 0.f);
+        const float a0 = fmaxf(__uint_as_float(x[2 * i]), 0.f), a1 = fmaxf(__uint_as_float(x[2 * i + 1]), 0.f);
         float r0 = a0, r1 = a1;
         if (pw >= 1) { r0 *= a0; r1 *= a1; }
         if (pw >= 2) { r0 *= a0; r1 *= a1; }
@@ -705,14 +698,14 @@ template <int D, int T, int MAP, bool GEN>
 __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, const CUtensorMap* tmO, uint8_t* smem, int u) {
   using R = QRing<D>;
   using L = QLayout<D>;
-  using X = QShape<D, T>;
+  using X = QShape<T>;
   const int nkv = p.nkv, n_s = p.n_s;
   const float scale_log2 = p.scale_log2;
   const R q(p, c);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = (warp >> 2) & 1;                    // group 0 or 1
-  const int r0 = (warp & 3) * 32 + (X::TPR == 2 ? (warp >> 3) * 16 : 0);   // this warp's rows of the group's 128-row tile
-  const int r = r0 + (X::TPR == 2 ? lane & 15 : lane), hc = X::TPR == 2 ? lane >> 4 : 0;   // this thread's row, its share of the columns
+  const int r0 = (warp & 3) * 32 + (T == 2 ? (warp >> 3) * 16 : 0);   // this warp's rows of the group's 128-row tile
+  const int r = r0 + (T == 2 ? lane & 15 : lane), hc = T == 2 ? lane >> 4 : 0;   // this thread's row, its share of the columns
   const uint32_t lane_off = (uint32_t)r0 << 16;
   const uint32_t tSg = q.tS(g) + lane_off, tOg = q.tO(g) + lane_off, tPg = q.tP(g) + lane_off;
   uint8_t* sPg = smem + L::P_OFF + g * L::PTILE;    // this group's phi_q / output staging tile
@@ -723,7 +716,7 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
     if (!q.wait(R::B_S + g, ps + j)) return false;
     tc_fence_after();
     uint32_t sv[X::COLS];                           // this thread's share of its row of the 128 x 128 score tile
-    if constexpr (X::TPR == 1) tmem_ld128_sync(tSg, sv); else tmem_ldh64_sync<64>(tSg, sv);
+    if constexpr (T == 1) tmem_ld128_sync(tSg, sv); else tmem_ldh64_sync<64>(tSg, sv);
     tc_fence_before();
     mbar_arrive(q.bar(R::B_SF + g));                // the score columns may be overwritten
     if (n_s - j * 128 < 128) {
@@ -739,7 +732,7 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
       mx1 = fmax3(mx1, __uint_as_float(sv[i + 2]), __uint_as_float(sv[i + 3]));
     }
     float mx = fmax3(mx0, mx1, fmaxf(__uint_as_float(sv[X::COLS - 2]), __uint_as_float(sv[X::COLS - 1])));
-    if (X::TPR == 2) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));   // the other half of the row
+    if (T == 2) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));   // the other half of the row
     mx *= scale_log2;
     m_true = fmaxf(m_true, mx);
     // The reference maximum only moves when the row maximum grew by more than 2^8; then O and l
@@ -755,7 +748,7 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
     // Whether the previous tile's P V has completed is asked here and looked at behind the first exponentials (d = 128: a wait for
     // something that is already there costs a round trip; at d = 64 the other warps cover it)
     bool p_free = false;
-    if (X::TPR == 1 && ppf + j > 0) p_free = mbar_try_wait(q.bar(R::B_PF + g), (ppf + j - 1) & 1);
+    if (T == 1 && ppf + j > 0) p_free = mbar_try_wait(q.bar(R::B_PF + g), (ppf + j - 1) & 1);
 #pragma unroll
     for (int cc = 0; cc < X::COLS / 32; ++cc) {
       uint32_t pw[16];
@@ -765,28 +758,28 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
         const float2 xa = __ffma2_rn(make_float2(__uint_as_float(sv[k]), __uint_as_float(sv[k + 1])), scale2, negm2);
         const float2 xb = __ffma2_rn(make_float2(__uint_as_float(sv[k + 2]), __uint_as_float(sv[k + 3])), scale2, negm2);
         const float2 pa = make_float2(ex2(xa.x), ex2(xa.y));
-        const float2 pc = EX2_FMA_EVERY<T> > 0 && i % (EX2_FMA_EVERY<T> + (EX2_FMA_EVERY<T> == 0)) == EX2_FMA_EVERY<T> - 1 ? ex2_fma(xb) : make_float2(ex2(xb.x), ex2(xb.y));
+        const float2 pc = ex2_second_pair<T>(i, xb);
         la = __fadd2_rn(la, pa);
         lb = __fadd2_rn(lb, pc);
         pw[2 * i] = pack_bf16(pa.x, pa.y);
         pw[2 * i + 1] = pack_bf16(pc.x, pc.y);
       }
       if (cc == 0) {                                // the previous tile's P V has read the columns of P
-        if (ppf + j > 0 && (X::TPR == 2 || !__all_sync(0xffffffffu, p_free)) && !q.wait(R::B_PF + g, ppf + j - 1)) return false;
+        if (ppf + j > 0 && (T == 2 || !__all_sync(0xffffffffu, p_free)) && !q.wait(R::B_PF + g, ppf + j - 1)) return false;
         tc_fence_after();
         if (__any_sync(0xffffffffu, need)) {        // ... and left its sum in O, which no product touches until this tile's P is handed over
 #pragma unroll 1
-          for (int o = 0; o < D / X::TPR; o += 16) {
+          for (int o = 0; o < D / T; o += 16) {
             uint32_t y[16];
-            q_ld16<X::TPR, D / 2>(tOg + o, y);
+            q_ld16<T, D / 2>(tOg + o, y);
             tmem_ld16_wait(y);
 #pragma unroll
             for (int i = 0; i < 16; ++i) y[i] = __float_as_uint(__uint_as_float(y[i]) * resc);
-            q_st16<X::TPR, D / 2>(tOg + o, y);
+            q_st16<T, D / 2>(tOg + o, y);
           }
         }
       }
-      q_st16<X::TPR, 32>(tPg + cc * 16, pw);
+      q_st16<T, 32>(tPg + cc * 16, pw);
     }
     // The sum above adds the unrounded probabilities while the MMA multiplies their bf16 roundings with V.
     // Over many keys the rounding errors average out, but the error of a probability that dominates its
@@ -794,7 +787,7 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
     // sum takes over the rounding error of the tile's largest probability.
     const float p_top = ex2(mx - m_ref);
     const float p_top_err = __uint_as_float(pack_bf16(0.f, p_top) & 0xffff0000u) - p_top;
-    l = l * resc + (((la.x + la.y) + (lb.x + lb.y)) + (X::TPR == 1 || hc == 0 ? p_top_err : 0.f));
+    l = l * resc + (((la.x + la.y) + (lb.x + lb.y)) + (T == 1 || hc == 0 ? p_top_err : 0.f));
     tmem_st_wait();
     tc_fence_before();
     mbar_arrive(q.bar(R::B_P + g));
@@ -802,7 +795,7 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
 
   const QUnit un = q_unit(p, u);
   const int bh = un.bh;
-  if (X::TPR == 2) l += __shfl_xor_sync(0xffffffffu, l, 16);
+  if (T == 2) l += __shfl_xor_sync(0xffffffffu, l, 16);
   const int row = un.row0 + g * 128 + r;
   float den = l, den_l_out = 0.f;
   if (p.lin) {
@@ -822,7 +815,7 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
       dl = q_two_layer_tail<D, T, GEN>(p, q, g, tTail, sPg, sQg, r, hc, bh, ps, ppf, lam);
       if (dl < 0.f) return false;                      // a wait ran out (the sum itself is never negative)
     }
-    if (X::TPR == 2) dl += __shfl_xor_sync(0xffffffffu, dl, 16);
+    if (T == 2) dl += __shfl_xor_sync(0xffffffffu, dl, 16);
     den = l + dl;
     den_l_out = dl / lam;
   }
@@ -838,14 +831,14 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
   }
   uint32_t x[32];
 #pragma unroll 1
-  for (int cc = 0; cc < D / X::TPR / 32; ++cc) {
-    q_ld32<X::TPR, D / 2>(tOg + cc * 32, x);
+  for (int cc = 0; cc < D / T / 32; ++cc) {
+    q_ld32<T, D / 2>(tOg + cc * 32, x);
     tmem_ld_wait(x);
     uint32_t wd[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i)
       wd[i] = pack_bf16(__uint_as_float(x[2 * i]) * inv, __uint_as_float(x[2 * i + 1]) * inv);
-    store_row_chunk(sPg, r, hc * (D / X::TPR) + cc * 32, wd);
+    store_row_chunk(sPg, r, hc * (D / T) + cc * 32, wd);
   }
   fence_proxy_async();
   __syncwarp();
@@ -1057,14 +1050,14 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 }
 
 template <int D, int T, int MAP, bool GEN>
-__global__ void __launch_bounds__(QShape<D, T>::THREADS, 1)
+__global__ void __launch_bounds__(QShape<T>::THREADS, 1)
 qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
              const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmW,
              const __grid_constant__ CUtensorMap tmSt, const __grid_constant__ CUtensorMap tmW1,
              const __grid_constant__ CUtensorMap tmO, const __grid_constant__ QParams p) {
   using L = QLayout<D>;
   using R = QRing<D>;
-  using X = QShape<D, T>;
+  using X = QShape<T>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
@@ -1239,8 +1232,8 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   }
 #define AS_LAUNCH_Q(D_, T_, MAP_) \
   do { \
-    if (gen) return as_launch_dependent(qpass_kernel<D_, T_, MAP_, true>, grid, dim3(QShape<D_, T_>::THREADS), QLayout<D_>::TOTAL, st, tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO, p); \
-    return as_launch_dependent(qpass_kernel<D_, T_, MAP_, false>, grid, dim3(QShape<D_, T_>::THREADS), QLayout<D_>::TOTAL, st, tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO, p); \
+    if (gen) return as_launch_dependent(qpass_kernel<D_, T_, MAP_, true>, grid, dim3(QShape<T_>::THREADS), QLayout<D_>::TOTAL, st, tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO, p); \
+    return as_launch_dependent(qpass_kernel<D_, T_, MAP_, false>, grid, dim3(QShape<T_>::THREADS), QLayout<D_>::TOTAL, st, tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO, p); \
   } while (0)
 #define AS_LAUNCH_QT(T_) \
   do { \
