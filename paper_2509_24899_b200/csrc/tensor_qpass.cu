@@ -51,8 +51,8 @@ struct QShape {
   // warps 0 .. 8 * T - 1: compute (quadrant = bits 0-1, group = bit 2, T = 2: half of the quadrant's rows = bit 3)
   static constexpr int THREADS = (W_TMA + 3) * 32, GROUP = 128 * T;
 };
-// The feature maps that the kernel with a key loop is compiled for: one layer whose tail is one product at d = 128 (F = 128; of any width at
-// d = 64), one layer of several products at d = 128, two layers.
+// The feature maps that the kernel with a key loop is compiled for: one layer, one layer whose tail is several products at d = 128 (more than 128
+// features; not where a CTA has one tile only and there are no groups to take turns), two layers.
 constexpr int MAP_ONE = 0, MAP_WIDE = 1, MAP_TWO = 2;
 constexpr int KV_STAGES = 3;
 constexpr float RESCALE_THRESHOLD = 8.f; // log2 units: rescale O only when the row max grew by > 2^8
@@ -1164,20 +1164,25 @@ int plan_units(QParams& p, int BH, int sms) {
   }
   return grid;
 }
-// Threads per row of the kernel with a key loop (after plan_units).  Two (sixteen compute warps) hide more of the latencies, one draws less power per
-// exponential and has 168 registers where two have 96.  At d = 64 always two.  At d = 128 the gain of two over one in the query stage, on layers that differ in
-// the number of key tiles only (12 heads, N = 32760, 16384, 7800 and 24 heads, N = 2430; bursts of 3 ms / runs of 0.12 s, which the power cap
-// slows down):
+// no CTA has more than one tile: one group works, the other one has nothing to do
+bool one_tile_each(const QParams& p) { return p.n_rounds == 0 && p.split_last; }
+// Threads per row of the kernel with a key loop (after plan_units).  Two (sixteen compute warps) hide more of the latencies; one draws less power per
+// exponential and has 168 registers where two have 96.  At d = 64 always two.  At d = 128 the gain of two over one in the query stage, on layers that differ
+// in the number of key tiles only (12 heads, N = 32760, 16384, 7800, 1560; 2 - 46 heads of 20140 - 442 rows; in bursts of 3 ms / in runs of 0.06 - 0.12 s,
+// which the power cap slows down where a CTA has several units):
 //   a CTA has one tile at most (2 heads, N = 4096), so that one group has the SM to itself: 4 - 10 % at any length with one layer, 0 - 5 % with two;
-//   one layer without biases: 4 tiles 3 - 8 % / 1 - 6 %, 8 0 - 2 / 0 - 3, 16 0 - 3 / -1 - +1, 24 1 / -1, 48 0 / -1, 96 0 / -1 - -3 (F = 256 alike);
-//   one layer with biases or powers beyond 2: 8 tiles 6 - 12 / 5 - 7, 16 3 - 5 / 2, 31 3 - 5 / 0 - 2, 48 1 - 4 / -2 - +1, 96 1 - 3 / -1 - 0;
-//   two layers: -2 - -4 / -3 - -5 at almost any length, without softmax tokens -3 - -14 / -3 - -11; with biases and two
-//   feature chunks, which one thread has to keep in its registers, 16 tiles +3 - +8 / +3 - +5, 32 +3 - +5 / 0 - 2, 48 1 - 7 / -1 - +3.
+//   one layer without biases: 4 tiles 0 - 8 % / 0 - 8 %, 16 0 - 3 / -1 - +3, 31 0 - 2 / -2 - +3, 40 -1 - +2 / -2 - +3, 96 -1 - +1 / -3 - -1; F = 256 alike;
+//   one layer with biases or powers beyond 2: 8 tiles 4 - 12 / 2 - 13, 16 2 - 7 / 2 - 6, 31 2 - 5 / -3 - +3, 48 1 - 4 / 0 - 2, 64 0 - 4 / -1 - +2;
+//   two layers with one feature chunk: 0 tiles -14 - 0 / -11 - 0, 4 and more -7 - 0 / -8 - 0, biased or not; with two, which one thread has
+//   to keep in its registers: 0 tiles -5 - 0 / -6 - 0, else -3 - +1 / -4 - +3, with biases or powers beyond 2 4 - 30 at few tiles, 16 4 - 16 / 2 - 12, 48 1 - 10 / -1 - +5.
+// That is the query stage over and over.  In a whole layer its instructions arrive cold, which costs one thread's longer code more: of two-layer
+// maps of few rounds 256 / 256 are 2 - 7 % faster with two (N = 1560 ... 9360, 0 to 10 tiles), 128 / 128 0 - 3 %.
 int q_threads_per_row(const QParams& p, int d, bool two, bool gen) {
-  const bool one_tile_each = p.n_rounds == 0 && p.split_last;
-  if (d == 64 || one_tile_each) return 2;
-  if (two) return gen && p.fc > 1 && p.nkv <= 32 ? 2 : 1;
-  return p.nkv <= (gen ? 40 : 16) ? 2 : 1;
+  if (d == 64 || one_tile_each(p)) return 2;
+  if (!two) return p.nkv <= (gen ? 48 : 31) ? 2 : 1;
+  if (gen && p.fc > 1) return p.nkv <= 48 ? 2 : 1;
+  if (p.fc == 1 && p.nkv == 0) return 1;
+  return p.nkv <= 16 && p.n_rounds < 4 ? 2 : 1;
 }
 }  // namespace
 
@@ -1237,7 +1242,7 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   } while (0)
 #define AS_LAUNCH_QT(T_) \
   do { \
-    if (two) AS_LAUNCH_Q(128, T_, MAP_TWO); else if (lin && p.fc > 1) AS_LAUNCH_Q(128, T_, MAP_WIDE); else AS_LAUNCH_Q(128, T_, MAP_ONE); \
+    if (two) AS_LAUNCH_Q(128, T_, MAP_TWO); else if (lin && p.fc > 1 && !one_tile_each(p)) AS_LAUNCH_Q(128, T_, MAP_WIDE); else AS_LAUNCH_Q(128, T_, MAP_ONE); \
   } while (0)
   if (a.d == 128) { if (tpr == 2) AS_LAUNCH_QT(2); else AS_LAUNCH_QT(1); }
   if (two) AS_LAUNCH_Q(64, 2, MAP_TWO); else AS_LAUNCH_Q(64, 2, MAP_ONE);
