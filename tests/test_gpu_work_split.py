@@ -154,20 +154,20 @@ def test_a_key_far_below_the_maximum_weighs_nothing(N, d):
         assert bool((out == v[0, 0, col]).all()), col
 
 
-# every feature map with a key loop and a tail, at key tiles on both sides of where a row has one thread or two, and at one; heads enough for several
-# units a CTA and a last one of a single tile
-@pytest.mark.parametrize("n_keys", [100, 1024, 1025, 2048, 2049, 4097, 5200])
+# every feature map with a tail: no softmax tokens, one key tile, and key tiles on both sides of where a row has one thread or two (16, 31 and 48 tiles);
+# heads enough for several units a CTA and a last one of a single tile
+@pytest.mark.parametrize("n_keys", [0, 100, 1025, 2048, 2049, 3968, 3969, 6144, 6145])
 @pytest.mark.parametrize("F,hidden,degree,bias", [(128, 0, 2, False), (128, 0, 4, True), (256, 0, 2, False), (512, 0, 4, True), (128, 128, 2, False),
                                                   (128, 256, 2, True), (256, 128, 2, True), (256, 256, 2, False), (256, 256, 4, True)])
 def test_key_loop_and_tail_of_every_feature_map(F, hidden, degree, bias, n_keys):
     """Some rows of every head against the oracle: relative L2 as everywhere, per row 5e-2 as above, row statistics as above."""
     import torch
     from paper_2509_24899_b200 import HybridAttention
-    N = 2 * n_keys - 1
+    N = 2 * n_keys - 1 if n_keys else 2600
     tiles = (N + 127) // 128
-    wl = W.Workload("tails", B=1, H=max(3, -(-330 // tiles)), d=128, F=F, grid=(1, 1, N), block=(1, 1, N), rate=2, seed=76, degree=degree,
-                    layers=2 if hidden else 1, hidden=hidden, bias=bias)
-    data = W.generate(wl, wq_gain=2e-3)
+    wl = W.Workload("tails", B=1, H=max(3, -(-330 // tiles)), d=128, F=F, grid=(1, 1, N), block=(1, 1, N), rate=2 if n_keys else 0, seed=76,
+                    degree=degree, layers=2 if hidden else 1, hidden=hidden, bias=bias)
+    data = W.generate(wl, wq_gain=2e-3 if n_keys else 1.0)
     dev = {n: to_cuda_bf16(x) for n, x in data.items()}
     op = HybridAttention.from_workload(wl)
     assert op.n_softmax == n_keys
@@ -182,5 +182,7 @@ def test_key_loop_and_tail_of_every_feature_map(F, hidden, degree, bias, n_keys)
     assert errors(got, ref)[0] <= 5e-3
     row_err = np.sqrt(((got - ref) ** 2).sum(-1) / (ref ** 2).sum(-1))
     assert row_err.max() <= 5e-2, row_err.max()
-    np.testing.assert_allclose(got_aux[..., 0], ref_aux[..., 0], atol=2e-3, rtol=0)
-    assert errors(got_aux[..., 1], ref_aux[..., 1])[0] <= 5e-3 and errors(got_aux[..., 2], ref_aux[..., 2])[0] <= 5e-3
+    if n_keys:
+        np.testing.assert_allclose(got_aux[..., 0], ref_aux[..., 0], atol=2e-3, rtol=0)
+        assert errors(got_aux[..., 1], ref_aux[..., 1])[0] <= 5e-3
+    assert errors(got_aux[..., 2], ref_aux[..., 2])[0] <= 5e-3
