@@ -96,8 +96,7 @@ def test_softmax_rows_of_a_two_layer_map_are_gathered_bit_for_bit(N, rate, d, F,
         assert torch.equal(got.view(torch.int16), x[:, :, at].reshape(6, len(at), d).view(torch.int16))
 
 
-# keys at the edges of what a thread holds of a score row (32-column pieces, half rows, whole rows), of a key tile, and of the rule that gives
-# a row one thread or two (31 key tiles)
+# keys at the edges of what a thread holds of a score row (32-column pieces, half rows), of a key tile, and of a key loop of 31 tiles
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("N", [1, 31, 33, 63, 64, 65, 97, 127, 128, 129, 193, 3968, 3969])
 def test_key_counts_at_the_edges_of_a_thread_s_share(N, d):
@@ -186,3 +185,18 @@ def test_key_loop_and_tail_of_every_feature_map(F, hidden, degree, bias, n_keys)
         np.testing.assert_allclose(got_aux[..., 0], ref_aux[..., 0], atol=2e-3, rtol=0)
         assert errors(got_aux[..., 1], ref_aux[..., 1])[0] <= 5e-3
     assert errors(got_aux[..., 2], ref_aux[..., 2])[0] <= 5e-3
+
+
+# rows of one thread: heads enough that CTAs have two tiles, and more key tiles than rows of two threads take
+@pytest.mark.parametrize("N", [3968, 3969, 4032, 4065, 4096, 4097])
+def test_long_key_loops_where_a_row_has_one_thread(N):
+    """As in test_key_counts_at_the_edges_of_a_thread_s_share, whose three heads are one tile a CTA."""
+    import torch
+    from paper_2509_24899_b200 import HybridAttention, binding
+    wl, dev = _inputs(1, 6, N, 128, 1, 77)
+    q = dev["q"].clone()
+    q[:, :, ::3] *= 6.0
+    out = [HybridAttention.from_workload(wl, kernel_path=path).forward(q, dev["k"], dev["v"], dev["wq"], dev["wk"]).double()
+           for path in (binding.AS_PATH_TENSOR, binding.AS_PATH_SIMT)]
+    assert float((out[0] - out[1]).norm() / out[1].norm()) <= 5e-3
+    assert float(((out[0] - out[1]).norm(dim=-1) / out[1].norm(dim=-1)).max()) <= 5e-2
