@@ -46,8 +46,8 @@ struct KLayout {
   static constexpr int RING_OFF = NH * TILE;
   static constexpr int BAR_OFF = RING_OFF + SLOTS * TILE;
   static constexpr int N_BARS = 1 + 2 * SLOTS + 5;
-  static constexpr int PAIR_OFF = BAR_OFF + 8 * N_BARS + 16;    // 2 x 64 words: per token pair, which halves are linear tokens
-  static constexpr int Z_OFF = PAIR_OFF + 2 * 64 * 4;           // 128 floats: z of the upper column half
+  static constexpr int PAIR_OFF = BAR_OFF + 8 * N_BARS + 16;    // 32 words a feature warp: per token pair, which halves are linear tokens
+  static constexpr int Z_OFF = PAIR_OFF + 8 * 32 * 4;           // 128 floats: z of the upper column half
   static constexpr int TOTAL = Z_OFF + 128 * 4 + 1024;          // + slack for the 1024-byte alignment
   // the chunk's partial S leaves through the ring (idle by then): 128 rows of D floats, each row padded by 16
   // bytes so that the 32 lanes of a warp, one row each, write to different banks
@@ -255,22 +255,35 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
         if (!ok) break;
         const uint8_t* kt = LAYERS == 1 ? smem + L::RING_OFF + ((t * IPT) % SLOTS) * L::TILE : nullptr;
         const uint8_t* vt = smem + L::RING_OFF + ((t * IPT + NX) % SLOTS) * L::TILE;
-        constexpr int CH = D / 8;                          // 16-byte chunks per row
+        // CH 16-byte pieces a row; a row is LPR lanes wide: its K and its V pieces (two layers: V's alone, phi1_kernel has copied K).
+        // AHEAD loads per lane before the first of their stores: one row after the other, each a chain of bit search, shuffle, load and store, the two
+        // warps took 3000 - 4000 clk for the 32 rows of a tile at rate 1/4, and held its ring slots meanwhile (N = 8505, 32 heads, d = 64: this
+        // kernel 44.7 us against 33.9; rate 1/2 67.6 against 44.8; d = 128, N = 32760, 12 heads, rate 1/2: 73.7 against 59.3).
+        constexpr int CH = D / 8, LPR = LAYERS == 1 ? 2 * CH : CH, RPI = 32 / LPR, AHEAD = 4;
+        const int c = lane % CH;
+        const bool is_v = LAYERS == 2 || lane % LPR >= CH;
+        const uint8_t* from = (is_v ? vt : kt) + (c / 8) * BOX_BYTES;
+        __nv_bfloat16* to = (is_v ? p.vs_w : p.ks_w) + (size_t)bh * p.n_s * D + c * 8;
         for (int e = 0; e < 2; ++e) {
-          uint32_t bits = __ballot_sync(0xffffffffu, rk[e] >= 0);
+          const int mine = e == 0 ? rk[0] : rk[1];
+          uint32_t bits = __ballot_sync(0xffffffffu, mine >= 0);
           while (bits) {
-            const int src = __ffs(bits) - 1;
-            bits &= bits - 1;
-            const int rank = __shfl_sync(0xffffffffu, rk[e], src);
-            const uint32_t rrow = gw * 64 + e * 32 + src;
-            // lanes [0, CH) move the K row (two layers: phi1_kernel has done that), lanes [16, 16 + CH) the V row
-            const int c = lane & 15;
-            if (c < CH && (LAYERS == 1 || lane >= 16)) {
-              const uint8_t* tile = (lane < 16) ? kt : vt;
-              const uint4 val = *reinterpret_cast<const uint4*>(tile + (c / 8) * BOX_BYTES + swz128_chunk_offset(rrow, c % 8));
-              __nv_bfloat16* dst = ((lane < 16) ? p.ks_w : p.vs_w) + ((size_t)bh * p.n_s + rank) * D + c * 8;
-              *reinterpret_cast<uint4*>(dst) = val;
+            int src[AHEAD], rank[AHEAD];
+            uint4 val[AHEAD];
+#pragma unroll
+            for (int a = 0; a < AHEAD; ++a) {
+              src[a] = -1;
+#pragma unroll
+              for (int i = 0; i < RPI; ++i) {
+                if (lane / LPR == i && bits) src[a] = __ffs(bits) - 1;
+                bits &= bits - 1;                          // (0 stays 0)
+              }
+              rank[a] = __shfl_sync(0xffffffffu, mine, src[a] < 0 ? 0 : src[a]);
+              if (src[a] >= 0) val[a] = *reinterpret_cast<const uint4*>(from + swz128_chunk_offset(gw * 64 + e * 32 + src[a], c % 8));
             }
+#pragma unroll
+            for (int a = 0; a < AHEAD; ++a)
+              if (src[a] >= 0) *reinterpret_cast<uint4*>(to + (size_t)rank[a] * D) = val[a];
           }
         }
         __syncwarp();
@@ -282,7 +295,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   } else {
     // ------------------------------------------------------------ feature warps: lane of TMEM = feature
     // warp w works on TMEM lanes 32 * (w % 4) .. + 31 and on token columns 64 * (w / 4) .. + 63
-    const int quad = warp & 3, hf = warp >> 2, tid = threadIdx.x;
+    const int quad = warp & 3, hf = warp >> 2;
     const int f_local = quad * 32 + lane, f = fc * 128 + f_local;
     const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
     const int part = p.F / p.P;
@@ -293,32 +306,32 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     bool ok = true;
     uint32_t x[32];
     // Which tokens of a tile are linear tokens (inside the sequence, not softmax tokens), as one word per
-    // token pair that masks the packed bf16 features; the first 64 threads each prepare one pair, one tile ahead.
-    auto pair_mask = [&](int t) -> uint32_t {
-      if (tid >= 64 || t >= nt) return 0u;
-      const int n0 = (t_begin + t) * 128 + 2 * tid;
-      uint32_t m = 0u;
-      if (n0 < p.N && p.sm_rank[n0] < 0) m |= 0x0000ffffu;
-      if (n0 + 1 < p.N && p.sm_rank[n0 + 1] < 0) m |= 0xffff0000u;
-      return m;
+    // token pair that masks the packed bf16 features.  A lane makes the word of one pair of its warp's 64 tokens; the ranks are asked for a tile ahead
+    // and not looked at before (a comparison at the load made two warps wait for L2 in every tile and, with masks shared by
+    // all eight, the others for these two: 700 - 1900 clk of the 3000 - 3800 that a tile took.  N = 7800, 12 heads, no softmax tokens:
+    // 21.4 us before, 19.7 with this).
+    const int pair_n0 = t_begin * 128 + hf * 64 + 2 * lane;
+    auto ranks = [&](int t) -> int2 {                          // (the table is N + 8 long)
+      const int n0 = pair_n0 + t * 128;
+      return t < nt && n0 < p.N ? *reinterpret_cast<const int2*>(p.sm_rank + n0) : make_int2(0, 0);
     };
-    uint32_t m_next = pair_mask(0);
+    uint32_t* pairs = sPair + warp * 32;
+    int2 rk_next = ranks(0);
     for (int t = 0; t < nt; ++t) {
       const int b = t & 1;
-      if (tid < 64) sPair[b * 64 + tid] = m_next;
-      m_next = pair_mask(t + 1);
-      // every feature thread reaches this barrier in every iteration, also after a failed wait: a warp
-      // that left the loop early would leave the others waiting here for good
-      named_barrier_sync(1, K_FEATURE_THREADS);
+      __syncwarp();                                            // the tile before: every lane has read the words
+      pairs[lane] = (rk_next.x < 0 ? 0x0000ffffu : 0u) | (rk_next.y < 0 && pair_n0 + t * 128 + 1 < p.N ? 0xffff0000u : 0u);
+      rk_next = ranks(t + 1);
+      __syncwarp();
       if (ok) ok = mbar_wait_warp(bar(B_D1 + b), (t >> 1) & 1, wc);
-      if (!ok) continue;
+      if (!ok) break;
       tc_fence_after();
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const int col = hf * 64 + c * 32;
         tmem_ld32(tD1[b] + lane_off + col, x);
         tmem_ld_wait(x);
-        const uint4* mask4 = reinterpret_cast<const uint4*>(sPair + b * 64 + col / 2);
+        const uint4* mask4 = reinterpret_cast<const uint4*>(pairs + c * 16);
         uint32_t w[16];
         switch (pw) {
           case 1: k_features<1>(x, mask4, bias, w, z0, z1); break;
