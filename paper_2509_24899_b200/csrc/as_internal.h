@@ -40,7 +40,7 @@ struct as_launch_args {
   const int32_t* sm_rank;               // [N]: position in T_S, or -1 for a linear token
   uint32_t* status;                     // device status word
   uint32_t* counters;                   // [B*H*4][2], zero between launches: K-pass CTAs of a (batch, head, feature chunk)
-                                        // that have stored their partial state / that have added their slice up
+                                        // that have stored their partial state (and given up) / that have left
   int B, H, N, d, F, P;
   int n_s, n_l;
   int n_chunks, chunk_tiles;            // K-pass split of the token axis

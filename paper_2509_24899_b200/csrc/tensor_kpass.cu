@@ -23,15 +23,17 @@ struct KParams {
   const int32_t* sm_rank;              // [N (+ padding)]: position in T_S, or -1 for a linear token
   __nv_bfloat16 *ks_w, *vs_w;          // compact softmax K / V (nullptr when nothing is gathered)
   const __nv_bfloat16* bias;           // last-layer bias [H][F], or nullptr
-  float *part_s, *part_z;
+  float *part_s, *part_z;              // the chunk's state
   float *S, *z;                        // [B*H][F][D], [B*H][F]: the chunks' partials added up ...
   __nv_bfloat16* Sb;                   // ... and S once more rounded to bf16 (the query stage's MMA operand)
-  uint32_t* counters;                  // [B*H][feature chunks][2]: CTAs that have stored / that have added; zero between launches
+  uint32_t* counters;                  // [B*H][feature chunks][2]: CTAs that have stored (and, times 2^16, that have given up) / that have left; zero
+                                       // between launches
   uint32_t* status;
 };
 
-constexpr int K_THREADS = 384;           // warps 0-7: feature warps; 8: TMA; 9: MMA issuer; 10-11: gather
+constexpr int K_THREADS = 416;           // warps 0-7: feature warps; 8: TMA; 9: issues Phi^T; 10: issues S; 11-12: gather
 constexpr int K_FEATURE_THREADS = 256;
+constexpr long long kSumPatience = 400ll * 1000ll;   // clocks, 0.2 ms: the chunks of a head differ by a few us where all CTAs run
 
 // LAYERS == 1: ring items per token tile are (K, V), one resident weight tile.
 // LAYERS == 2: ring items are (h1 slice 0 .. NH-1, V), NH resident weight tiles W_2[feature chunk, hidden slice].
@@ -45,14 +47,16 @@ struct KLayout {
   static constexpr int W_OFF = 0;
   static constexpr int RING_OFF = NH * TILE;
   static constexpr int BAR_OFF = RING_OFF + SLOTS * TILE;
-  static constexpr int N_BARS = 1 + 2 * SLOTS + 5;
-  static constexpr int PAIR_OFF = BAR_OFF + 8 * N_BARS + 16;    // 32 words a feature warp: per token pair, which halves are linear tokens
+  static constexpr int N_BARS = 1 + 3 * SLOTS + 7;
+  static constexpr int PAIR_OFF = (BAR_OFF + 8 * N_BARS + 8 + 15) / 16 * 16;   // (behind two words) 32 words a feature warp: per token pair, which halves are linear tokens
   static constexpr int Z_OFF = PAIR_OFF + 8 * 32 * 4;           // 128 floats: z of the upper column half
   static constexpr int TOTAL = Z_OFF + 128 * 4 + 1024;          // + slack for the 1024-byte alignment
   // the chunk's partial S leaves through the ring (idle by then): 128 rows of D floats, each row padded by 16
   // bytes so that the 32 lanes of a warp, one row each, write to different banks
   static constexpr int OUT_PITCH = D * 4 + 16;
   static_assert(128 * OUT_PITCH <= SLOTS * TILE, "staging area");
+  static_assert(RING_OFF % 1024 == 0 && PAIR_OFF % 16 == 0 && Z_OFF % 16 == 0 && OUT_PITCH % 16 == 0, "tiles, and what is read 16 bytes at a time");
+  static_assert(TOTAL <= 232448, "shared memory of a CTA");
 };
 
 // Features of 32 token columns of one TMEM lane: bias, ReLU, power, linear-token mask, bf16.
@@ -86,8 +90,10 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::BAR_OFF);
-  enum { B_W = 0, B_FULL = 1, B_EMPTY = B_FULL + SLOTS, B_D1 = B_EMPTY + SLOTS, B_PK = B_D1 + 2, B_DONE = B_PK + 2,
-         B_COUNT = B_DONE + 1 };
+  // Whether a ring slot is full is told on a barrier of its item's kind, XFULL (K, hidden slices) or VFULL: whoever waits looks at every phase of a
+  // barrier, in order.  D1: Phi^T has landed; PK: it has been read and the features are packed; SD: the product that reads these has completed.
+  enum { B_W = 0, B_XFULL = 1, B_VFULL = B_XFULL + SLOTS, B_EMPTY = B_VFULL + SLOTS, B_D1 = B_EMPTY + SLOTS, B_PK = B_D1 + 2, B_SD = B_PK + 2,
+         B_DONE = B_SD + 2, B_COUNT = B_DONE + 1 };
   static_assert(B_COUNT == L::N_BARS, "barrier count");
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::BAR_OFF + 8 * B_COUNT);
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::BAR_OFF + 8 * B_COUNT + 4);
@@ -103,56 +109,75 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   const WaitCtx wc{p.status, abort_flag};
   const bool gathers = (p.ks_w != nullptr) && fc == 0;       // this CTA copies the softmax rows out
 
-  // an earlier CTA of this or a previous launch timed out: nothing is requested (decided once per CTA)
-  __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
-  if (warp != 9) {
-    named_barrier_sync(3, K_THREADS - 32);
-  } else {
-    // first of all, and the others need not wait for it: the query stage's CTAs may then set up as these ones end
-    tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch();
-  }
-
   auto sW = [&](int j) { return sbase + L::W_OFF + j * L::TILE; };
   auto sSlot = [&](int it) { return sbase + L::RING_OFF + (it % SLOTS) * L::TILE; };
   // one ring item: tile t's K (one layer) or hidden slice i (two layers), or its V tile
   auto load_item = [&](int it) {
     const int st = it % SLOTS, t = it / IPT, i = it % IPT, row = (t_begin + t) * 128;
-    mbar_expect_tx(bar(B_FULL + st), L::TILE);
-    if (i == NX) load_tile<D>(sSlot(it), &tmV, bar(B_FULL + st), row, bh);
-    else if (LAYERS == 1) load_tile<D>(sSlot(it), &tmK, bar(B_FULL + st), row, bh);
-    else load_boxes(sSlot(it), &tmH, bar(B_FULL + st), i * D, row, bh, D / 64);
+    const uint32_t full = bar((i == NX ? B_VFULL : B_XFULL) + st);
+    mbar_expect_tx(full, L::TILE);
+    if (i == NX) load_tile<D>(sSlot(it), &tmV, full, row, bh);
+    else if (LAYERS == 1) load_tile<D>(sSlot(it), &tmK, full, row, bh);
+    else load_boxes(sSlot(it), &tmH, full, i * D, row, bh, D / 64);
   };
-  constexpr int FIRST = SLOTS;                               // items requested before the CTA has finished setting up: the whole ring
+  // `looks`: bit s is the parity of the next phase of the barrier of slot s that the warp has not looked at
+  auto wait_full = [&](int first_bar, int it, uint32_t& looks) -> bool {
+    const int st = it % SLOTS;
+    const uint32_t parity = (looks >> st) & 1u;
+    looks ^= 1u << st;
+    return mbar_wait_warp(bar(first_bar + st), parity, wc);
+  };
+  constexpr int FIRST = IPT;                                 // items requested at once, the first tile's
 
-  if (threadIdx.x == 0) {
+  // ---- Set-up that runs beside the kernel before this one.  The table of softmax ranks is the handle's and does not change; and the status word is asked
+  // for here because small loads that come behind the first tiles' wait as long as these do (4 us at N = 7800, 12 heads).
+  __shared__ uint32_t s_skip;
+  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (warp == 9) {
+    // the query stage's CTAs may then set up as these ones end
+    tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch();
+  } else if (threadIdx.x == 0) {
     *abort_flag = 0u;
-    for (int b = 0; b < 2; ++b) { mbar_init(bar(B_D1 + b), 1); mbar_init(bar(B_PK + b), K_FEATURE_THREADS); }
+    mbar_init(bar(B_W), 1);
+    // a slot is free again when the MMA that read it has completed and, where rows are gathered, when both gather warps are through with it
+    for (int s = 0; s < SLOTS; ++s) { mbar_init(bar(B_XFULL + s), 1); mbar_init(bar(B_VFULL + s), 1); mbar_init(bar(B_EMPTY + s), gathers ? 3 : 1); }
+    for (int b = 0; b < 2; ++b) { mbar_init(bar(B_D1 + b), 1); mbar_init(bar(B_PK + b), K_FEATURE_THREADS); mbar_init(bar(B_SD + b), 1); }
     mbar_init(bar(B_DONE), 1);
     fence_barrier_init();
-  }
-  if (threadIdx.x == 8 * 32 && s_skip == 0u) {
-    // The producer sets up the barriers of the ring itself and requests the weights and the first tiles at
-    // once: the first bytes of a CTA take several microseconds to arrive, and the CTA-wide barrier below need
-    // not be waited for.
-    mbar_init(bar(B_W), 1);
-    // a slot is free again when the MMA that read it has completed and, where rows are gathered, when both
-    // gather warps are through with it
-    for (int s = 0; s < SLOTS; ++s) { mbar_init(bar(B_FULL + s), 1); mbar_init(bar(B_EMPTY + s), gathers ? 3 : 1); }
-    fence_barrier_init();
     fence_proxy_async();
-    mbar_expect_tx(bar(B_W), NH * L::TILE);
-    // rows past F are out of bounds and arrive as zeros
-    for (int j = 0; j < NH; ++j) load_boxes(sW(j), &tmW, bar(B_W), j * D, fc * 128, h, D / 64);
-    for (int it = 0; it < FIRST && it < nt * IPT; ++it) load_item(it);
   }
+  // Feature warps: the ranks of a pair of their 64 tokens of a tile, the first tile's.  Gather warps: those of two of their 64 rows.
+  const int my_n0 = t_begin * 128 + (warp < 8 ? (warp >> 2) * 64 + 2 * lane : (warp & 1 ? 0 : 64) + lane);
+  auto pair_ranks = [&](int t) -> int2 {                       // (the table is N + 8 long)
+    const int n0 = my_n0 + t * 128;
+    return t < nt && n0 < p.N ? *reinterpret_cast<const int2*>(p.sm_rank + n0) : make_int2(0, 0);
+  };
+  auto row_ranks = [&](int t) -> int2 {
+    const int n0 = my_n0 + t * 128;
+    return make_int2(t < nt && n0 < p.N ? p.sm_rank[n0] : -1, t < nt && n0 + 32 < p.N ? p.sm_rank[n0 + 32] : -1);
+  };
+  // Four tiles ahead: under the load of the tiles' copies these take longer than a tile.  (A register that waits for its load cannot be moved to another
+  // without waiting, hence a branch by t % 4 where they are used.)
+  int2 rk0 = make_int2(-1, -1), rk1 = rk0, rk2 = rk0, rk3 = rk0;
+  if (warp < 8) { rk0 = pair_ranks(0); rk1 = pair_ranks(1); rk2 = pair_ranks(2); rk3 = pair_ranks(3); }
+  else if (warp >= 11 && gathers) { rk0 = row_ranks(0); rk1 = row_ranks(1); rk2 = row_ranks(2); rk3 = row_ranks(3); }
+  auto by_turns = [&](int t, auto use) {
+    switch (t & 3) {
+      case 0: use(rk0); break;
+      case 1: use(rk1); break;
+      case 2: use(rk2); break;
+      default: use(rk3); break;
+    }
+  };
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (s_skip != 0u) {
+  if (s_skip != 0u) {                                        // an earlier launch timed out: nothing is requested
+    griddep_wait();
     if (warp == 9) tmem_dealloc(*tmem_slot, 512);
     return;
   }
+  if (warp >= 8) griddep_wait();                             // (the feature warps: see their loop)
   const uint32_t tmem = *tmem_slot;
   const uint32_t tD1[2] = {tmem + 0u, tmem + 128u};          // Phi^T of a tile, fp32
   const uint32_t tAcc = tmem + 256u;                         // S of this feature chunk
@@ -160,96 +185,78 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
 
   if (warp == 8) {
     // ------------------------------------------------------------ TMA producer
-    for (int it = FIRST; it < nt * IPT; ++it) {              // the first items were requested during set-up
+    if (lane == 0) {
+      mbar_expect_tx(bar(B_W), NH * L::TILE);
+      // rows past F are out of bounds and arrive as zeros
+      for (int j = 0; j < NH; ++j) load_boxes(sW(j), &tmW, bar(B_W), j * D, fc * 128, h, D / 64);
+      for (int it = 0; it < FIRST; ++it) load_item(it);
+    }
+    __syncwarp();
+    for (int it = FIRST; it < nt * IPT; ++it) {
+      // (the first tile has the memory system to itself: with the whole ring asked for at once its latency is that of the ring)
+      if (it == FIRST && !mbar_wait_warp(bar(B_XFULL), 0, wc)) break;
       const int st = it % SLOTS;
       if (!mbar_wait_warp(bar(B_EMPTY + st), ((it / SLOTS) & 1) ^ 1, wc)) break;
       if (lane == 0) load_item(it);
       __syncwarp();
     }
   } else if (warp == 9) {
-    // ------------------------------------------------------------ MMA issuer (one thread)
-    // Two kinds of product per tile: Phi^T(t) as soon as the tile's X items have landed, and S += phi^T V (t) as
-    // soon as the feature warps have packed the tile.  The thread issues whichever is ready, so that neither a
-    // late tile holds up the accumulation of an earlier one (and with it the release of its V slot) nor the
-    // other way round.  Phi^T(t) reuses the columns the feature warps read for tile t - 2 and its features will
-    // overwrite the packed operand of S(t - 2): it is only issued once S(t - 2) has been (products of one thread
-    // complete in order).
-    if (lane == 0) {
-      constexpr uint32_t ID_PHI = make_idesc(128, 128, 0, 0);    // Phi^T = W X^T : M = features, N = 128 tokens
-      constexpr uint32_t ID_ACC = make_idesc(128, D, 0, 1);      // S += phi^T V  : V is MN-major
-      bool ok = mbar_wait(bar(B_W), 0, wc);
-      int tp = 0, ts = 0;                                        // next tile for Phi^T / for the accumulation
-      long long t0 = 0;
-      uint32_t polls = 0;
-      while (ok && ts < nt) {
-        bool did = false;
-        if (ts < tp) {                                           // S(ts): packed features and the V tile
-          const int it = ts * IPT + NX;
-          if (mbar_try_wait(bar(B_PK + (ts & 1)), (ts >> 1) & 1) && mbar_try_wait(bar(B_FULL + it % SLOTS), (it / SLOTS) & 1)) {
-            tc_fence_after();
-            issue_tmemA_mnB(tAcc, tPA[ts & 1], mnmajor_desc(sSlot(it)), ID_ACC, ts > 0);
-            tc_commit(bar(B_EMPTY + it % SLOTS));
-            if (ts == nt - 1) tc_commit(bar(B_DONE));
-            ++ts;
-            did = true;
-          }
-        }
-        if (tp < nt && tp - ts < 2) {                            // Phi^T(tp): its X items
-          bool ready = true;
+    // ------------------------------------------------------------ issues Phi^T(t) as soon as the tile's X items have landed and the features of tile
+    // t - 2, which lay in the same columns, have been read.  Two issuing warps, a lane of each elected from converged code: one thread that took whichever of
+    // the two products was ready, by turns of non-blocking looks, needed 1700 - 2000 clk a tile (XX).
+    constexpr uint32_t ID_PHI = make_idesc(128, 128, 0, 0);    // Phi^T = W X^T : M = features, N = 128 tokens
+    uint32_t looks = 0u;
+    bool ok = mbar_wait_warp(bar(B_W), 0, wc);
+    for (int t = 0; ok && t < nt; ++t) {
+      const int b = t & 1;
+      if (t >= 2) ok = mbar_wait_warp(bar(B_PK + b), ((t - 2) >> 1) & 1, wc);
 #pragma unroll
-          for (int j = 0; j < NX; ++j) {
-            const int it = tp * IPT + j;
-            ready = ready && mbar_try_wait(bar(B_FULL + it % SLOTS), (it / SLOTS) & 1);
-          }
-          if (ready) {
-            tc_fence_after();
-#pragma unroll
-            for (int j = 0; j < NX; ++j) {
-              const int it = tp * IPT + j;
-              issue_kmajor<D>(tD1[tp & 1], kmajor_desc(sW(j)), kmajor_desc(sSlot(it)), ID_PHI, j > 0);
-              tc_commit(bar(B_EMPTY + it % SLOTS));
-            }
-            tc_commit(bar(B_D1 + (tp & 1)));
-            ++tp;
-            did = true;
-          }
+      for (int j = 0; j < NX; ++j) {
+        const int it = t * IPT + j;
+        ok = ok && wait_full(B_XFULL, it, looks);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t w0 = kmajor_desc(sW(j)), x0 = kmajor_desc(sSlot(it));
+        if (elect_one()) {
+          issue_kmajor<D>(tD1[b], w0, x0, ID_PHI, j > 0);
+          tc_commit(bar(B_EMPTY + it % SLOTS));
+          if (j == NX - 1) tc_commit(bar(B_D1 + b));
         }
-        if (did) { polls = 0; t0 = 0; continue; }
-        // nothing was ready: the same bound as every other wait (the clock is looked at every 64 idle rounds)
-        if ((++polls & 63u) == 0u) {
-          const long long now = clock64();
-          if (t0 == 0) t0 = now;
-          if (*wc.abort != 0u || now - t0 > kWaitLimitCycles) {
-            *wc.abort = 1u;
-            atomicOr(wc.status, 1u);
-            ok = false;
-          }
-        }
+        __syncwarp();
       }
     }
-    __syncwarp();
-  } else if (warp >= 10) {
+  } else if (warp == 10) {
+    // ------------------------------------------------------------ issues S += phi^T V (t) as soon as the features are packed
+    constexpr uint32_t ID_ACC = make_idesc(128, D, 0, 1);      // S += phi^T V  : V is MN-major
+    uint32_t looks = 0u;
+    bool ok = true;
+    for (int t = 0; ok && t < nt; ++t) {
+      const int b = t & 1, it = t * IPT + NX;
+      ok = wait_full(B_VFULL, it, looks) && mbar_wait_warp(bar(B_PK + b), (t >> 1) & 1, wc);
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t v0 = mnmajor_desc(sSlot(it));
+      if (elect_one()) {
+        issue_tmemA_mnB(tAcc, tPA[b], v0, ID_ACC, t > 0);
+        tc_commit(bar(B_EMPTY + it % SLOTS));
+        tc_commit(bar(B_SD + b));
+        if (t == nt - 1) tc_commit(bar(B_DONE));
+      }
+      __syncwarp();
+    }
+  } else if (warp >= 11) {
     // ------------------------------------------------------------ gather of softmax-token rows
     if (gathers) {
-      const int gw = warp - 10;
-      // rows handled by this warp: gw*64 .. gw*64+63; two ranks per lane.  The ranks of tile t + 1 are
-      // fetched while tile t is being copied, so that the global-load latency stays off the critical path.
-      auto load_ranks = [&](int t, int (&rk)[2]) {
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int n = (t_begin + t) * 128 + gw * 64 + e * 32 + lane;
-          rk[e] = (t < nt && n < p.N) ? p.sm_rank[n] : -1;
-        }
-      };
-      int rk_next[2];
-      load_ranks(0, rk_next);
+      const int gw = warp & 1 ? 0 : 1;
+      // rows handled by this warp: gw*64 .. gw*64+63; two ranks per lane
+      uint32_t looks_x = 0u, looks_v = 0u;
       for (int t = 0; t < nt; ++t) {
-        int rk[2] = {rk_next[0], rk_next[1]};
-        load_ranks(t + 1, rk_next);
+        int rk[2];
+        by_turns(t, [&](int2& r) { rk[0] = r.x; rk[1] = r.y; r = row_ranks(t + 4); });
         bool ok = true;
         for (int i = 0; i < IPT; ++i) {
           const int it = t * IPT + i;
-          ok = ok && mbar_wait_warp(bar(B_FULL + it % SLOTS), (it / SLOTS) & 1, wc);
+          ok = ok && (i == NX ? wait_full(B_VFULL, it, looks_v) : wait_full(B_XFULL, it, looks_x));
           if (LAYERS == 2 && i < NX && ok && lane == 0) mbar_arrive(bar(B_EMPTY + it % SLOTS));   // a hidden slice: not read here
         }
         if (!ok) break;
@@ -306,26 +313,27 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     bool ok = true;
     uint32_t x[32];
     // Which tokens of a tile are linear tokens (inside the sequence, not softmax tokens), as one word per
-    // token pair that masks the packed bf16 features.  A lane makes the word of one pair of its warp's 64 tokens; the ranks are asked for a tile ahead
+    // token pair that masks the packed bf16 features.  A lane makes the word of one pair of its warp's 64 tokens; the ranks are asked for tiles ahead
     // and not looked at before (a comparison at the load made two warps wait for L2 in every tile and, with masks shared by
     // all eight, the others for these two: 700 - 1900 clk of the 3000 - 3800 that a tile took.  N = 7800, 12 heads, no softmax tokens:
     // 21.4 us before, 19.7 with this).
-    const int pair_n0 = t_begin * 128 + hf * 64 + 2 * lane;
-    auto ranks = [&](int t) -> int2 {                          // (the table is N + 8 long)
-      const int n0 = pair_n0 + t * 128;
-      return t < nt && n0 < p.N ? *reinterpret_cast<const int2*>(p.sm_rank + n0) : make_int2(0, 0);
-    };
     uint32_t* pairs = sPair + warp * 32;
-    int2 rk_next = ranks(0);
-    for (int t = 0; t < nt; ++t) {
+    // The loop's first turn is none of a tile: it brings the loop's instructions into the SM beside the kernel before this one.  They come through the
+    // same memory system as the first tiles, and behind those they took 2 - 4 us to arrive (N = 7800, N = 32760, 12 heads: first features 1.9 and 4.2 us,
+    // each later tile's 0.6).  What it computes from whatever lies in tensor memory goes into operand columns that the tiles overwrite.
+    for (int t = -1; t < nt; ++t) {
       const int b = t & 1;
       __syncwarp();                                            // the tile before: every lane has read the words
-      pairs[lane] = (rk_next.x < 0 ? 0x0000ffffu : 0u) | (rk_next.y < 0 && pair_n0 + t * 128 + 1 < p.N ? 0xffff0000u : 0u);
-      rk_next = ranks(t + 1);
-      __syncwarp();
-      if (ok) ok = mbar_wait_warp(bar(B_D1 + b), (t >> 1) & 1, wc);
-      if (!ok) break;
-      tc_fence_after();
+      if (t >= 0) {
+        by_turns(t, [&](int2& r) {
+          pairs[lane] = (r.x < 0 ? 0x0000ffffu : 0u) | (r.y < 0 && my_n0 + t * 128 + 1 < p.N ? 0xffff0000u : 0u);
+          r = pair_ranks(t + 4);
+        });
+        __syncwarp();
+        ok = mbar_wait_warp(bar(B_D1 + b), (t >> 1) & 1, wc);
+        if (!ok) break;
+        tc_fence_after();
+      }
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const int col = hf * 64 + c * 32;
@@ -339,22 +347,33 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
           case 3: k_features<3>(x, mask4, bias, w, z0, z1); break;
           default: k_features<4>(x, mask4, bias, w, z0, z1); break;
         }
+        if (c == 0 && t >= 2) {                                // the product that read tile t - 2's features has completed
+          ok = mbar_wait_warp(bar(B_SD + b), ((t - 2) >> 1) & 1, wc);
+          if (!ok) break;
+          tc_fence_after();
+        }
         tmem_st16(tPA[b] + lane_off + col / 2, w);
       }
+      if (!ok) break;
       tmem_st_wait();
       tc_fence_before();
+      if (t < 0) {
+        z0 = 0.f; z1 = 0.f;
+        griddep_wait();
+        continue;
+      }
       mbar_arrive(bar(B_PK + b));
     }
     if (ok) ok = mbar_wait_warp(bar(B_DONE), 0, wc);
     // z of the two column halves is added through shared memory.  The partial S leaves through the ring: each
-    // thread puts its half row there (rows padded so that a warp's lanes hit different banks), then the row's
-    // owner hands the row to the copy engine as one contiguous piece - a row written straight from registers
-    // would cost one 32-byte sector per lane and instruction.  The ring is idle once the last product has
+    // thread puts its half row there (rows padded so that a warp's lanes hit different banks), and the warps store whole rows, 512 bytes an instruction - a
+    // row written straight from registers would cost one 32-byte sector per lane and instruction; row by row by the copy engine, the CTA waited 2400 clk
+    // for the rows to be read.  The ring is idle once the last product has
     // completed and the gather warps (barrier 2) have read their last tile.  Every feature thread takes part in
     // the barriers whatever its waits returned.
     if (hf == 1) sZ[f_local] = z0 + z1;
     named_barrier_sync(2, K_FEATURE_THREADS + 64);
-    uint8_t* stage = smem + L::RING_OFF + f_local * L::OUT_PITCH;
+    uint8_t* stage = smem + L::RING_OFF;
     if (ok) {
       tc_fence_after();
       constexpr int HALF = D / 2;                              // accumulator columns per warp
@@ -365,18 +384,19 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
         tmem_ld_wait(x);
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-          *reinterpret_cast<uint4*>(stage + (col + 4 * i) * 4) = make_uint4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
+          *reinterpret_cast<uint4*>(stage + f_local * L::OUT_PITCH + (col + 4 * i) * 4) = make_uint4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
       }
-      fence_proxy_async();
     }
     named_barrier_sync(1, K_FEATURE_THREADS);
-    if (ok && hf == 0 && f < p.F) {
-      const size_t slot = (size_t)bh * p.n_chunks + chunk;
-      bulk_store_1d(p.part_s + (slot * p.F + f) * D, smem_u32(stage), D * 4);
-      tma_store_commit();
-      p.part_z[slot * p.F + f] = (z0 + z1) + sZ[f_local];
-      tma_store_wait_all();                                    // the partial state is in global memory ...
-      fence_proxy_async_all();                                 // ... and ordered before what this CTA publishes below
+    if (ok) {
+      constexpr int LPR = D / 4, RPW = 32 / LPR;               // lanes a row, rows an instruction
+      const size_t slot = ((size_t)bh * p.n_chunks + chunk) * p.F + fc * 128;
+      const int nf = min(128, p.F - fc * 128);
+      float4* out = reinterpret_cast<float4*>(p.part_s + slot * D);
+#pragma unroll 4
+      for (int r = warp * RPW + lane / LPR; r < nf; r += 8 * RPW)
+        out[(size_t)r * LPR + lane % LPR] = *reinterpret_cast<const float4*>(stage + r * L::OUT_PITCH + lane % LPR * 16);
+      if (hf == 0 && f_local < nf) p.part_z[slot + f_local] = (z0 + z1) + sZ[f_local];
     }
   }
 
@@ -388,41 +408,46 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   }
   // ---- The chunks' partial states are added up here, in chunk order (fixed order, no float atomics): every CTA of
   // a (batch, head, feature chunk) takes a slice of the [F x (D + 1)] entries once all of them have stored theirs.
-  // The CTAs of one launch are resident together (one per SM, a cooperative launch when there is more than one
-  // chunk), so the wait ends; it is bounded like every other wait.  The second counter tells the last CTA to finish
-  // its slice that both counters can go back to zero for the next launch.  This is a chain of L2 round trips: the loads of all
+  // The CTAs of a launch are resident together where nothing else is on the GPU (one per SM at most).  A CTA that has waited for kSumPatience for
+  // one that has not even started gives its slice up and leaves its SM: the last to store adds all slices up then (the same sums once more where
+  // others do theirs).  So no CTA waits for good, and this is no cooperative launch, which the kernel before it in the stream would have to end for
+  // first (N = 1024, 2 heads, d = 64: a call 18.3 -> XX us).  The second counter tells the last CTA to leave that both
+  // counters can go back to zero for the next launch.  This is a chain of L2 round trips: the loads of all
   // chunks at once instead of four by four, and no sleep between two looks at the counter, took N = 7800 from 87.5 to 86.3 us
-  // and N = 1024 with 2 heads from 19.5 to 18.5 us.
-  __shared__ uint32_t s_go;
+  // and N = 1024 with 2 heads from 19.5 to 18.5 us.  (Added up in the query stage's kernel instead, by its compute warps ahead of their first scores: its loads
+  // come behind the first tiles' copies, 9.5 us where it takes 4 here, N = 32760 without softmax tokens 103.7 -> 108.9 us; by
+  // one warp beside the key loop: latency after latency, N = 7800 82.6 -> 103.)
+  __shared__ uint32_t s_go;                                    // 0: nothing, 1: this CTA's slice, 2: all slices
   uint32_t* cnt = p.counters + 2 * ((size_t)bh * gridDim.z + fc);
   const uint32_t n_ctas = gridDim.x;
   if (threadIdx.x == 0) {
     __threadfence();
-    atomicAdd(cnt, 1u);
-    uint32_t go = 1u, it = 0;
+    const uint32_t stored = atomicAdd(cnt, 1u);
+    uint32_t go = (stored & 0xffffu) + 1u == n_ctas && stored >> 16 != 0u ? 2u : 1u, it = 0;
     long long t0 = 0;
-    while (*reinterpret_cast<volatile uint32_t*>(cnt) < n_ctas) {
+    while ((*reinterpret_cast<volatile uint32_t*>(cnt) & 0xffffu) < n_ctas) {
       if ((++it & 15u) != 0u) continue;                        // a look at the counter is a round trip to L2: no need to sleep between
-      // a CTA that found the status word set never arrives: the others stop waiting when they see it too
-      if (*reinterpret_cast<volatile uint32_t*>(p.status) != 0u) { go = 0u; break; }
       const long long now = clock64();
       if (t0 == 0) t0 = now;
-      if (*abort_flag != 0u || now - t0 > kWaitLimitCycles) { atomicOr(p.status, 1u); go = 0u; break; }
+      if (now - t0 > kSumPatience) {
+        if ((atomicAdd(cnt, 0x10000u) & 0xffffu) < n_ctas) go = 0u;
+        break;
+      }
     }
     s_go = go;
   }
   __syncthreads();
-  if (s_go == 0u) return;
-  __threadfence();
-  {
+  const uint32_t go = s_go;
+  if (go != 0u) {
+    __threadfence();
     const int f0 = fc * 128, nf = min(128, p.F - f0);
     const size_t pitch = (size_t)p.F * D;                      // floats between two chunks' partials
     const float* src = p.part_s + ((size_t)bh * p.n_chunks * p.F + f0) * D;
     float* dS = p.S + ((size_t)bh * p.F + f0) * D;
     __nv_bfloat16* dSb = p.Sb + ((size_t)bh * p.F + f0) * D;
-    const int n4 = nf * D / 4, per = (n4 + (int)n_ctas - 1) / (int)n_ctas;       // float4 entries, this CTA's slice
-    const int i_end = min(n4, (chunk + 1) * per);
-    for (int i = chunk * per + (int)threadIdx.x; i < i_end; i += K_THREADS) {
+    const int n4 = nf * D / 4, per = (n4 + (int)n_ctas - 1) / (int)n_ctas;       // float4 entries, a CTA's slice
+    const int i_end = go == 2u ? n4 : min(n4, (chunk + 1) * per);
+    for (int i = (go == 2u ? 0 : chunk * per) + (int)threadIdx.x; i < i_end; i += K_THREADS) {
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
       int c = 0;
       for (; c < p.n_chunks; c += 12) {                        // up to twelve chunks' loads in flight, added in chunk order
@@ -437,7 +462,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       reinterpret_cast<float4*>(dS)[i] = acc;
       reinterpret_cast<uint2*>(dSb)[i] = make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
     }
-    if (chunk == 0) {
+    if (chunk == 0 || go == 2u) {
       for (int f = threadIdx.x; f < nf; f += K_THREADS) {
         float acc = 0.f;
         for (int c = 0; c < p.n_chunks; c += 12) {
@@ -454,8 +479,8 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    const uint32_t done = atomicAdd(cnt + 1, 1u);
-    if (done + 1u == n_ctas) { cnt[0] = 0u; cnt[1] = 0u; }     // everyone has read the first counter: ready for the next launch
+    const uint32_t left = atomicAdd(cnt + 1, 1u);
+    if (left + 1u == n_ctas) { cnt[0] = 0u; cnt[1] = 0u; }     // nobody looks at the first counter any more: ready for the next launch
   }
 }
 
@@ -610,14 +635,7 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
 template <int D, int LAYERS, int NH>
 cudaError_t launch_kpass(const CUtensorMap& tmK, const CUtensorMap& tmV, const CUtensorMap& tmW, const CUtensorMap& tmH,
                          const KParams& p, dim3 grid, cudaStream_t st) {
-  if (grid.x == 1) {                   // one chunk per head: no CTA waits for another
-    kpass_kernel<D, LAYERS, NH><<<grid, K_THREADS, KLayout<D, LAYERS, NH>::TOTAL, st>>>(tmK, tmV, tmW, tmH, p);
-    return cudaGetLastError();
-  }
-  // several chunks per head: the CTAs wait for one another at the end, so they must be resident together
-  void* args[] = {(void*)&tmK, (void*)&tmV, (void*)&tmW, (void*)&tmH, (void*)&p};
-  return cudaLaunchCooperativeKernel((const void*)kpass_kernel<D, LAYERS, NH>, grid, dim3(K_THREADS), args,
-                                     (size_t)KLayout<D, LAYERS, NH>::TOTAL, st);
+  return as_launch_dependent(kpass_kernel<D, LAYERS, NH>, grid, dim3(K_THREADS), KLayout<D, LAYERS, NH>::TOTAL, st, tmK, tmV, tmW, tmH, p);
 }
 
 }  // namespace
