@@ -242,7 +242,25 @@ struct QRing {
   }
 };
 
-// ---------------------------------------------------------------- TMA producer, one unit
+// ---------------------------------------------------------------- TMA producer
+// The first copies of a CTA, by one thread: ring item 0 (the first key tile, else the first weights) and the first unit's Q tiles.  In line, right behind the wait for
+// the kernel before: as a part of q_produce_unit they went out 2500 - 3500 clk later, which is what its
+// instructions and its parameters take to arrive in a CTA that has just started.
+template <int D, int MAP>
+__device__ __noinline__ void q_first_loads(const QParams& p, const QCtx& c, const QUnit& un, const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmW,
+                          const CUtensorMap* tmW1) {
+  using R = QRing<D>;
+  using L = QLayout<D>;
+  const R q(c);
+  const CUtensorMap* first = p.nkv > 0 ? tmK : MAP == MAP_TWO ? tmW1 : tmW;
+  mbar_expect_tx(q.bar(R::B_KFULL), L::TILE);
+  load_tile<D>(q.sKV(0), first, q.bar(R::B_KFULL), 0, p.nkv > 0 ? un.bh : un.bh % p.H);
+  for (int g = 0; g < un.ng; ++g) {
+    mbar_expect_tx(q.bar(R::B_Q0 + g), L::TILE);
+    load_tile<D>(q.sQ(g), tmQ, q.bar(R::B_Q0 + g), un.row0 + g * 128, un.bh);
+  }
+}
+// one unit
 template <int D, int MAP, bool GEN>
 __device__ __noinline__ bool q_produce_unit(const QParams& p, const QCtx& c, const CUtensorMap* tmQ, const CUtensorMap* tmK,
                                             const CUtensorMap* tmV, const CUtensorMap* tmW, const CUtensorMap* tmSt,
@@ -257,10 +275,10 @@ __device__ __noinline__ bool q_produce_unit(const QParams& p, const QCtx& c, con
   const int base = u * q.n_items;
   const int q_at = nkv > 0 ? 1 : 0;                   // the Q tiles are requested right after the unit's first K tile
   for (int it = 0; it < q.n_items; ++it) {
-    if (it == q_at) {
+    if (it == q_at && u > 0) {
       for (int g = 0; g < un.ng; ++g) {
         // the previous unit's last product that reads this Q buffer has completed
-        if (u > 0 && !q.wait(R::B_QF + g, u - 1)) return false;
+        if (!q.wait(R::B_QF + g, u - 1)) return false;
         if (lane == 0) {
           mbar_expect_tx(q.bar(R::B_Q0 + g), L::TILE);
           load_tile<D>(q.sQ(g), tmQ, q.bar(R::B_Q0 + g), row0 + g * 128, bh);
@@ -269,6 +287,7 @@ __device__ __noinline__ bool q_produce_unit(const QParams& p, const QCtx& c, con
       }
     }
     const int gi = base + it, st = gi % KV_STAGES;
+    if (u == 0 && it == 0) continue;                  // (requested with the Q tiles, see q_first_loads)
     if (!q.wait(R::B_EMPTY + st, gi / KV_STAGES + 1)) return false;
     if (lane == 0) {
       const uint32_t dst = q.sKV(gi);
@@ -1007,23 +1026,24 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (warp == 17) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
-  griddep_wait();                                    // the set-up above ran beside the kernel before this one
-  // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
   __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);    // (ahead of the wait: behind the first copies it would wait for these)
+  if (warp == 17) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
+  if (warp == 16 && (threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmW); tma_prefetch_desc(&tmSt); tma_prefetch_desc(&tmO); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (s_skip != 0u) {
-    if (warp == 17) tmem_dealloc(*tmem_slot, 512);
-    return;
-  }
   const QCtx c{sbase, *tmem_slot, WaitCtx{p.status, abort_flag}};
   const int n_mine = q_units_of_cta(p);
+  griddep_wait();                                    // the set-up above ran beside the kernel before this one
+  if (s_skip != 0u) {                                // an earlier launch timed out: do nothing (decided once per CTA)
+    if (warp == 17) tmem_dealloc(c.tmem, 512);
+    return;
+  }
 
   if (warp == 16) {
-    if ((threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmW); tma_prefetch_desc(&tmSt); tma_prefetch_desc(&tmO); }
+    if ((threadIdx.x & 31) == 0) q_first_loads<D, MAP_ONE>(p, c, q_unit(p, 0), &tmQ, &tmQ, &tmW, &tmW);
+    __syncwarp();
     for (int u = 0; u < n_mine; ++u)
       if (!q_produce_unit<D, MAP_ONE, GEN>(p, c, &tmQ, &tmQ, &tmQ, &tmW, &tmSt, &tmW, u)) break;
   } else if (warp == 17) {
@@ -1079,15 +1099,15 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (warp == X::W_SCORE) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
-  griddep_wait();                                    // the set-up above ran beside the kernel before this one
-  // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
   __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);    // (ahead of the wait: behind the first copies it would wait for these)
+  if (warp == X::W_SCORE) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
+  if (warp == X::W_TMA && (threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); tma_prefetch_desc(&tmO); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (s_skip != 0u) {
+  griddep_wait();                                    // the set-up above ran beside the kernel before this one
+  if (s_skip != 0u) {                                // an earlier launch timed out: do nothing (decided once per CTA)
     if (warp == X::W_SCORE) tmem_dealloc(*tmem_slot, 512);
     return;
   }
@@ -1095,7 +1115,8 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   const int n_mine = q_units_of_cta(p);               // units of this CTA
 
   if (warp == X::W_TMA) {
-    if ((threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); tma_prefetch_desc(&tmO); }
+    if ((threadIdx.x & 31) == 0) q_first_loads<D, MAP>(p, c, q_unit(p, 0), &tmQ, &tmK, &tmW, &tmW1);
+    __syncwarp();
     for (int u = 0; u < n_mine; ++u)
       if (!q_produce_unit<D, MAP, GEN>(p, c, &tmQ, &tmK, &tmV, &tmW, &tmSt, &tmW1, u)) break;
   } else if (warp == X::W_SCORE) {

@@ -61,30 +61,36 @@ struct QSCtx {
 AS_DEV int qs_bh(const QSParams& p, long long t) { return (int)(t / p.nt); }
 
 // ---------------------------------------------------------------- TMA producer
+AS_DEV void qs_load_q(const QSParams& p, const QSCtx& c, const CUtensorMap* tmQ, int i) {
+  const long long t = c.t0 + i;
+  const int slot = i % QS_SLOTS;
+  mbar_expect_tx(c.bar(B_QFULL + slot), TILE);
+  load_tile<128>(c.sbase + QSLayout::Q_OFF + slot * TILE, tmQ, c.bar(B_QFULL + slot), (int)(t % p.nt) * 128, qs_bh(p, t));
+}
+AS_DEV void qs_load_pair(const QSParams& p, const QSCtx& c, const CUtensorMap* tmW, const CUtensorMap* tmSt, int bh) {
+  mbar_expect_tx(c.bar(B_WFULL), 2 * TILE);
+  load_tile<128>(c.sbase + QSLayout::W_OFF, tmW, c.bar(B_WFULL), 0, bh % p.H);
+  load_tile<128>(c.sbase + QSLayout::ST_OFF, tmSt, c.bar(B_WFULL), 0, bh);
+}
+
 __device__ __noinline__ void qs_produce(const QSParams& p, const QSCtx& c, const CUtensorMap* tmQ, const CUtensorMap* tmW,
                                         const CUtensorMap* tmSt) {
   const int lane = threadIdx.x & 31;
   const int n = (int)(c.t1 - c.t0);
-  int seg = -1, bh_prev = -1;
+  int seg = 0, bh_prev = qs_bh(p, c.t0);
   for (int i = 0; i < n; ++i) {
-    const long long t = c.t0 + i;
-    const int bh = qs_bh(p, t), row0 = (int)(t % p.nt) * 128, slot = i % QS_SLOTS;
-    if (!c.wait_warp(B_QEMPTY + slot, i / QS_SLOTS + 1)) return;      // the product that read the slot has completed
-    if (lane == 0) {
-      mbar_expect_tx(c.bar(B_QFULL + slot), TILE);
-      load_tile<128>(c.sbase + QSLayout::Q_OFF + slot * TILE, tmQ, c.bar(B_QFULL + slot), row0, bh);
+    const int bh = qs_bh(p, c.t0 + i), slot = i % QS_SLOTS;
+    if (i >= QS_SLOTS) {
+      if (!c.wait_warp(B_QEMPTY + slot, i / QS_SLOTS + 1)) return;    // the product that read the slot has completed
+      if (lane == 0) qs_load_q(p, c, tmQ, i);
+      __syncwarp();
     }
-    __syncwarp();
     if (bh != bh_prev) {
       // a new (batch, head): its weights and state replace the previous pair's once every product that reads
       // those has completed
       ++seg;
-      if (seg > 0 && !c.wait_warp(B_WFREE, seg - 1)) return;
-      if (lane == 0) {
-        mbar_expect_tx(c.bar(B_WFULL), 2 * TILE);
-        load_tile<128>(c.sbase + QSLayout::W_OFF, tmW, c.bar(B_WFULL), 0, bh % p.H);
-        load_tile<128>(c.sbase + QSLayout::ST_OFF, tmSt, c.bar(B_WFULL), 0, bh);
-      }
+      if (!c.wait_warp(B_WFREE, seg - 1)) return;
+      if (lane == 0) qs_load_pair(p, c, tmW, tmSt, bh);
       __syncwarp();
       bh_prev = bh;
     }
@@ -230,18 +236,13 @@ qstream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (warp == 9) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
-  griddep_wait();                                    // the set-up above ran beside the kernel before this one
-  // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
   __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);    // (ahead of the wait: behind the first copies it would wait for these)
+  if (warp == 9) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
+  if (warp == 8 && (threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmW); tma_prefetch_desc(&tmSt); tma_prefetch_desc(&tmO); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (s_skip != 0u) {
-    if (warp == 9) tmem_dealloc(*tmem_slot, 512);
-    return;
-  }
   // Every CTA gets a contiguous run of tiles.  With at least as many CTAs as (batch, head) pairs no run crosses a
   // pair (a change of pair stalls the pipeline while W and S are replaced): the pairs get floor or ceil(G / pairs)
   // CTAs each, which share the pair's tiles evenly.  Otherwise the tiles of all pairs are cut into G near-equal runs.
@@ -259,9 +260,20 @@ qstream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     t1 = (cta + 1) * p.tiles / G;
   }
   const QSCtx c{sbase, *tmem_slot, WaitCtx{p.status, abort_flag}, t0, t1};
+  griddep_wait();                                    // the set-up above ran beside the kernel before this one
+  if (s_skip != 0u) {                                // an earlier launch timed out: do nothing (decided once per CTA)
+    if (warp == 9) tmem_dealloc(c.tmem, 512);
+    return;
+  }
 
   if (warp == 8) {
-    if ((threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmW); tma_prefetch_desc(&tmSt); tma_prefetch_desc(&tmO); }
+    // the first copies in line: as a part of qs_produce they go out 2500 clk later, which is what its instructions take to arrive
+    if ((threadIdx.x & 31) == 0) {
+      qs_load_q(p, c, &tmQ, 0);
+      qs_load_pair(p, c, &tmW, &tmSt, qs_bh(p, t0));
+      for (int i = 1; i < min((int)(t1 - t0), QS_SLOTS); ++i) qs_load_q(p, c, &tmQ, i);
+    }
+    __syncwarp();
     qs_produce(p, c, &tmQ, &tmW, &tmSt);
   } else if (warp == 9) {
     if ((threadIdx.x & 31) == 0) qs_issue_phi(p, c);
