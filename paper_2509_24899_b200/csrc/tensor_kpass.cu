@@ -203,7 +203,8 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   } else if (warp == 9) {
     // ------------------------------------------------------------ issues Phi^T(t) as soon as the tile's X items have landed and the features of tile
     // t - 2, which lay in the same columns, have been read.  Two issuing warps, a lane of each elected from converged code: one thread that took whichever of
-    // the two products was ready, by turns of non-blocking looks, needed 1700 - 2000 clk a tile (XX).
+    // the two products was ready, by turns of non-blocking looks, needed 1700 - 2000 clk a tile,
+    // more than the feature warps.
     constexpr uint32_t ID_PHI = make_idesc(128, 128, 0, 0);    // Phi^T = W X^T : M = features, N = 128 tokens
     uint32_t looks = 0u;
     bool ok = mbar_wait_warp(bar(B_W), 0, wc);
@@ -411,7 +412,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   // The CTAs of a launch are resident together where nothing else is on the GPU (one per SM at most).  A CTA that has waited for kSumPatience for
   // one that has not even started gives its slice up and leaves its SM: the last to store adds all slices up then (the same sums once more where
   // others do theirs).  So no CTA waits for good, and this is no cooperative launch, which the kernel before it in the stream would have to end for
-  // first (N = 1024, 2 heads, d = 64: a call 18.3 -> XX us).  The second counter tells the last CTA to leave that both
+  // first (N = 1024, 2 heads, d = 64: a call 18.3 -> 15.8 us).  The second counter tells the last CTA to leave that both
   // counters can go back to zero for the next launch.  This is a chain of L2 round trips: the loads of all
   // chunks at once instead of four by four, and no sleep between two looks at the counter, took N = 7800 from 87.5 to 86.3 us
   // and N = 1024 with 2 heads from 19.5 to 18.5 us.  (Added up in the query stage's kernel instead, by its compute warps ahead of their first scores: its loads
