@@ -151,14 +151,15 @@ bsq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 256); tmem_relinquish(); griddep_launch(); }
-  griddep_wait();                                    // the set-up above ran beside the kernel before this one
-  // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
   __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 256); tmem_relinquish(); griddep_launch(); }
+  if (threadIdx.x == 15 * 32) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmY); tma_prefetch_desc(&tmH); tma_prefetch_desc(&tmW); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  griddep_wait();                                    // the set-up above ran beside the kernel before this one
+  // an earlier launch timed out: do nothing (decided once per CTA)
   if (s_skip != 0u) {
     if (warp == 16) tmem_dealloc(*tmem_slot, 256);
     return;
@@ -380,14 +381,15 @@ bsk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
-  griddep_wait();                                    // the set-up above ran beside the kernel before this one
-  // an earlier CTA of this or a previous launch timed out: do nothing (decided once per CTA)
   __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
+  if (threadIdx.x == 15 * 32) { tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); tma_prefetch_desc(&tmW); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  griddep_wait();                                    // the set-up above ran beside the kernel before this one
+  // an earlier launch timed out: do nothing (decided once per CTA)
   if (s_skip != 0u) {
     if (warp == 16) tmem_dealloc(*tmem_slot, 512);
     return;
