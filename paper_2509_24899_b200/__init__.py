@@ -13,6 +13,14 @@ __all__ = ["binding", "HybridAttention", "AS_PATH_SIMT", "AS_PATH_TENSOR", "AS_S
            "AS_STAB_PAPER", "AsError", "select_block_rates"]
 
 
+def _stream_ptr(stream):
+    """Address of `stream`, or of the current device's current one (whose Stream object takes 3 us to make: a fifth of a small call)."""
+    if stream is not None:
+        return stream.cuda_stream
+    import torch
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
 class HybridAttention:
     """One layer geometry bound to the current CUDA device.
 
@@ -36,6 +44,7 @@ class HybridAttention:
         self.workspace_bytes = binding.as_hybrid_attn_workspace_bytes(self._h)
         self.workspace_bytes_host = binding.as_hybrid_attn_workspace_bytes_host(self._h)
         self.n_softmax, _ = binding.as_hybrid_attn_softmax_tokens(self._h, want_indices=False)
+        self._offsets = binding.as_hybrid_attn_workspace_offsets(self._h)
         self._ws = None
 
     @classmethod
@@ -67,24 +76,21 @@ class HybridAttention:
         if workspace is not None:
             self._ws = workspace
         ws = self.workspace()
-        st = torch.cuda.current_stream() if stream is None else stream
         binding.as_hybrid_attn_forward(
             self._h, q.data_ptr(), k.data_ptr(), v.data_ptr(),
             0 if wq is None else wq.data_ptr(), 0 if wk is None else wk.data_ptr(),
-            out.data_ptr(), 0 if aux is None else aux.data_ptr(), ws.data_ptr(), ws.numel(), st.cuda_stream,
+            out.data_ptr(), 0 if aux is None else aux.data_ptr(), ws.data_ptr(), ws.numel(), _stream_ptr(stream),
             0 if wq2 is None else wq2.data_ptr(), 0 if wk2 is None else wk2.data_ptr(),
             None if biases is None else {n: t.data_ptr() for n, t in biases.items()})
         return out
 
     def forward_host(self, q_host, k_host, v_host, wq, wk, out_host, stream=None, wq2=None, wk2=None, biases=None):
         """q_host, k_host, v_host, out_host: pinned CPU tensors; the weights are device tensors."""
-        import torch
         ws = self.workspace(host=True)
-        st = torch.cuda.current_stream() if stream is None else stream
         binding.as_hybrid_attn_forward_host(
             self._h, q_host.data_ptr(), k_host.data_ptr(), v_host.data_ptr(),
             0 if wq is None else wq.data_ptr(), 0 if wk is None else wk.data_ptr(),
-            out_host.data_ptr(), ws.data_ptr(), ws.numel(), st.cuda_stream,
+            out_host.data_ptr(), ws.data_ptr(), ws.numel(), _stream_ptr(stream),
             0 if wq2 is None else wq2.data_ptr(), 0 if wk2 is None else wk2.data_ptr(),
             None if biases is None else {n: t.data_ptr() for n, t in biases.items()})
         return out_host
@@ -102,17 +108,16 @@ class HybridAttention:
                     torch.zeros(BH, self.F, d, dtype=torch.float32, device=k.device),
                     torch.zeros(BH, self.F, dtype=torch.float32, device=k.device))
         ws = self.workspace()
-        st = torch.cuda.current_stream() if stream is None else stream
         binding.as_hybrid_attn_key_pass(
             self._h, k.data_ptr(), v.data_ptr(), 0 if wq is None else wq.data_ptr(), 0 if wk is None else wk.data_ptr(),
-            ws.data_ptr(), ws.numel(), st.cuda_stream, 0 if wq2 is None else wq2.data_ptr(),
+            ws.data_ptr(), ws.numel(), _stream_ptr(stream), 0 if wq2 is None else wq2.data_ptr(),
             0 if wk2 is None else wk2.data_ptr(), None if biases is None else {n: t.data_ptr() for n, t in biases.items()})
-        o_ks, o_vs, o_S, o_z = binding.as_hybrid_attn_workspace_offsets(self._h)
-        n_s = self.n_softmax
-        view = lambda off, count, dtype, shape: ws[off:off + count * dtype.itemsize].view(dtype).view(*shape)
-        ks = view(o_ks, BH * n_s * d, torch.bfloat16, (BH, n_s, d))
-        vs = view(o_vs, BH * n_s * d, torch.bfloat16, (BH, n_s, d))
-        return ks, vs, view(o_S, BH * self.F * d, torch.float32, (BH, self.F, d)), view(o_z, BH * self.F, torch.float32, (BH, self.F))
+        n_s, F, ws = self.n_softmax, self.F, ws[:self.workspace_bytes]
+        bf16, f32 = ws.view(torch.bfloat16), ws.view(torch.float32)
+        o_ks, o_vs = (o // 2 + bf16.storage_offset() for o in self._offsets[:2])
+        o_S, o_z = (o // 4 + f32.storage_offset() for o in self._offsets[2:])
+        return (bf16.as_strided((BH, n_s, d), (n_s * d, d, 1), o_ks), bf16.as_strided((BH, n_s, d), (n_s * d, d, 1), o_vs),
+                f32.as_strided((BH, F, d), (F * d, d, 1), o_S), f32.as_strided((BH, F), (F, 1), o_z))
 
     def query_pass(self, q, wq, wk, ks, vs, S, z, out=None, aux=None, stream=None, wq2=None, wk2=None, biases=None):
         """Second stage: this range's queries against the gathered softmax keys ks, vs [B*H, n_keys, d] and the summed
@@ -121,13 +126,12 @@ class HybridAttention:
         if out is None:
             out = torch.empty_like(q)
         ws = self.workspace()
-        st = torch.cuda.current_stream() if stream is None else stream
         n_keys = 0 if ks is None else ks.shape[1]
         binding.as_hybrid_attn_query_pass(
             self._h, q.data_ptr(), 0 if wq is None else wq.data_ptr(), 0 if wk is None else wk.data_ptr(),
             ks.data_ptr() if n_keys else 0, vs.data_ptr() if n_keys else 0, n_keys,
             0 if S is None else S.data_ptr(), 0 if z is None else z.data_ptr(), out.data_ptr(),
-            0 if aux is None else aux.data_ptr(), ws.data_ptr(), ws.numel(), st.cuda_stream,
+            0 if aux is None else aux.data_ptr(), ws.data_ptr(), ws.numel(), _stream_ptr(stream),
             0 if wq2 is None else wq2.data_ptr(), 0 if wk2 is None else wk2.data_ptr(),
             None if biases is None else {n: t.data_ptr() for n, t in biases.items()})
         return out
@@ -139,15 +143,14 @@ class HybridAttention:
         B, H, N, d = self.shape
         dwq = torch.empty(H, self.F, d, dtype=torch.float32, device="cuda")
         dwk = torch.empty_like(dwq)
-        loss = torch.zeros(1, dtype=torch.float32, device="cuda") if want_loss else None
+        loss = torch.empty(1, dtype=torch.float32, device="cuda") if want_loss else None
         need = binding.as_hybrid_attn_backward_workspace_bytes(self._h)
         if getattr(self, "_bws", None) is None or self._bws.numel() < need:
             self._bws = torch.empty(need, dtype=torch.uint8, device="cuda")
-        st = torch.cuda.current_stream() if stream is None else stream
         binding.as_hybrid_attn_backward_phi(
             self._h, q.data_ptr(), k.data_ptr(), v.data_ptr(), wq.data_ptr(), wk.data_ptr(), y_teacher.data_ptr(),
             y_hat.data_ptr(), aux.data_ptr(), self.workspace().data_ptr(), dwq.data_ptr(), dwk.data_ptr(),
-            0 if loss is None else loss.data_ptr(), self._bws.data_ptr(), self._bws.numel(), st.cuda_stream)
+            0 if loss is None else loss.data_ptr(), self._bws.data_ptr(), self._bws.numel(), _stream_ptr(stream))
         return dwq, dwk, loss
 
     def linear_state(self, stream=None):
@@ -156,15 +159,12 @@ class HybridAttention:
         B, H, N, d = self.shape
         S = torch.empty(B, H, self.F, d, dtype=torch.float32, device="cuda")
         z = torch.empty(B, H, self.F, dtype=torch.float32, device="cuda")
-        st = torch.cuda.current_stream() if stream is None else stream
         binding.as_hybrid_attn_linear_state(self._h, self.workspace().data_ptr(), S.data_ptr(), z.data_ptr(),
-                                            st.cuda_stream)
+                                            _stream_ptr(stream))
         return S, z
 
     def last_status(self, stream=None) -> int:
-        import torch
-        st = torch.cuda.current_stream() if stream is None else stream
-        return binding.as_hybrid_attn_last_status(self._h, st.cuda_stream)
+        return binding.as_hybrid_attn_last_status(self._h, _stream_ptr(stream))
 
     def close(self):
         if getattr(self, "_h", None) is not None:

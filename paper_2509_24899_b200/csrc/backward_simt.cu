@@ -402,12 +402,12 @@ as_status_t as_hybrid_attn_backward_phi(as_hybrid_attn_t h, const void* q, const
   cudaError_t e = cudaSuccess;
   if (D == 128 && d.phi_dim == 128 && d.kernel_path == AS_PATH_TENSOR) {
     // the products on the tensor cores; the same fixed-order reductions
-    if ((e = as_bw_tensor_init()) == cudaSuccess && (e = as_bw_tensor_query(p, st)) == cudaSuccess && (e = reduce(0)) == cudaSuccess &&
+    if ((e = as_bw_tensor_query(p, st)) == cudaSuccess && (e = reduce(0)) == cudaSuccess &&
         (e = as_bw_tensor_key(p, st)) == cudaSuccess)
       e = reduce(1);
   } else if (D == 64 && d.kernel_path == AS_PATH_TENSOR && aligned) {
     // the products on the tensor cores, fp32 operands in three bf16 pieces
-    if ((e = as_bw_tensor_d64_init()) == cudaSuccess && (e = as_bw_tensor_d64_query(p, st)) == cudaSuccess && (e = reduce(0)) == cudaSuccess &&
+    if ((e = as_bw_tensor_d64_query(p, st)) == cudaSuccess && (e = reduce(0)) == cudaSuccess &&
         (e = as_bw_tensor_d64_key(p, st)) == cudaSuccess)
       e = reduce(1);
   } else if (D == 128) {

@@ -2,6 +2,7 @@
 // per-device shared-memory opt-in of every kernel.
 #include <mutex>
 
+#include "backward_common.h"
 #include "tensor_common.cuh"
 
 namespace {
@@ -67,5 +68,7 @@ cudaError_t as_tensor_init() {
   cudaError_t e;
   if ((e = as_tensor_init_qpass()) != cudaSuccess) return e;
   if ((e = as_tensor_init_kpass()) != cudaSuccess) return e;
-  return as_tensor_init_qstream();
+  if ((e = as_tensor_init_qstream()) != cudaSuccess) return e;
+  if ((e = as_bw_tensor_init()) != cudaSuccess) return e;
+  return as_bw_tensor_d64_init();
 }
