@@ -335,7 +335,8 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
         if (!ok) break;
         tc_fence_after();
       }
-#pragma unroll
+      // (not unrolled: half the instructions to fetch in the first turn, N = 7800 77.9 -> 77.0 us a call)
+#pragma unroll 1
       for (int c = 0; c < 2; ++c) {
         const int col = hf * 64 + c * 32;
         tmem_ld32(tD1[b] + lane_off + col, x);
@@ -497,6 +498,8 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
 // when its stores have been read.  With four warps, both slices' rows behind both products, and an end that waited for the stores to
 // land: the same layer 906 us against 897, N = 7800 152.0 against 150.7 (74 us of this kernel; floor 47).
 // ======================================================================================
+// A dependent launch: its CTAs set up beside the kernel before it (N = 1144, 2 heads, 128 / 128: a call 28.9 -> 27.8 us; N = 1036, 5 heads, d = 64
+// 24.9 -> 22.9).
 struct P1Params { int H, hid, N, n_s; const __nv_bfloat16* bias; const int32_t* sm_rank; __nv_bfloat16* ks_w; uint32_t* status; };
 constexpr int P1_THREADS = 288;          // warps 0-7: epilogue (two threads per token row, each half of a slice's columns); warp 8: TMA + MMA
 
@@ -528,9 +531,7 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
   constexpr int TM_COLS = NH * 128;                             // 128 or 256: a power of two
 
   __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
-  __syncthreads();
-  if (s_skip != 0u) return;
+  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
     mbar_init(bar_full, 1);
@@ -538,12 +539,17 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
     fence_barrier_init();
     fence_proxy_async();
   }
+  if (warp == 8) { tmem_alloc(smem_u32(tmem_slot), TM_COLS); tmem_relinquish(); }
+  griddep_wait();                                    // the set-up above ran beside the kernel before this one
   for (int i = threadIdx.x; i < NH * D; i += P1_THREADS)
     sBias[i] = (p.bias != nullptr && i < p.hid) ? __bfloat162float(p.bias[(size_t)h * p.hid + i]) : 0.f;
-  if (warp == 8) { tmem_alloc(smem_u32(tmem_slot), TM_COLS); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (s_skip != 0u) {                                // an earlier launch timed out: do nothing
+    if (warp == 8) tmem_dealloc(*tmem_slot, TM_COLS);
+    return;
+  }
   const uint32_t tmem = *tmem_slot;
   const uint32_t sX = sbase + L::X_OFF;
   auto sW = [&](int j) { return sbase + L::W_OFF + j * L::TILE; };
@@ -663,10 +669,9 @@ cudaError_t as_tensor_phi1(const as_launch_args& a, cudaStream_t st) {
     return cudaErrorInvalidValue;
   P1Params p{a.H, a.hid, a.N, a.n_s, a.bk1, a.sm_rank, a.ks_w, a.status};
   dim3 grid((a.N + 127) / 128, BH, 1);
-  if (a.d == 128 && a.hid == 256) phi1_kernel<128, 2><<<grid, P1_THREADS, P1Layout<128, 2>::TOTAL, st>>>(tmX, tmW, tmH, p);
-  else if (a.d == 128) phi1_kernel<128, 1><<<grid, P1_THREADS, P1Layout<128, 1>::TOTAL, st>>>(tmX, tmW, tmH, p);
-  else phi1_kernel<64, 1><<<grid, P1_THREADS, P1Layout<64, 1>::TOTAL, st>>>(tmX, tmW, tmH, p);
-  return cudaGetLastError();
+  if (a.d == 128 && a.hid == 256) return as_launch_dependent(phi1_kernel<128, 2>, grid, dim3(P1_THREADS), P1Layout<128, 2>::TOTAL, st, tmX, tmW, tmH, p);
+  if (a.d == 128) return as_launch_dependent(phi1_kernel<128, 1>, grid, dim3(P1_THREADS), P1Layout<128, 1>::TOTAL, st, tmX, tmW, tmH, p);
+  return as_launch_dependent(phi1_kernel<64, 1>, grid, dim3(P1_THREADS), P1Layout<64, 1>::TOTAL, st, tmX, tmW, tmH, p);
 }
 
 cudaError_t as_tensor_kpass(const as_launch_args& a, cudaStream_t st) {
