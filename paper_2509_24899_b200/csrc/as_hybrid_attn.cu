@@ -85,12 +85,19 @@ void layout_workspace(as_hybrid_attn_s* h) {
   w.Sb = take(lin ? BH * d.phi_dim * d.d * 2 : 0);
   const bool two = lin && d.phi_layers == 2;
   w.h1k = take(two ? BH * (size_t)d.N * d.phi_hidden * 2 : 0);
+  // (a range of a sequence-sharded layer attends to the other ranges' softmax tokens as well; it comes with an index list)
+  const size_t parts = d.kernel_path == AS_PATH_TENSOR && (h->n_s > 0 || h->listed) ? as_qpass_parts_bytes(d.N, (int)BH, d.d, h->sms) : 0;
+  w.has_parts = parts > 0;
+  w.parts = take(parts);
   w.total = std::max<size_t>(off, 256);
   const size_t t = BH * d.N * d.d * 2;
   off = w.total;
   w.stage_q = take(t); w.stage_k = take(t); w.stage_v = take(t); w.stage_o = take(t);
   w.total_host = off;
 }
+
+// the K pass's arrival counters, then the flags of the query stage's unfinished units
+size_t n_counters(const as_hybrid_attn_s* h) { return 8 * (size_t)h->desc.B * h->desc.H + 2 * (size_t)h->sms; }
 
 struct ProfileScope {
   as_hybrid_attn_s* h; cudaStream_t st; int slot = -1;
@@ -187,6 +194,8 @@ as_status_t as_hybrid_attn_create(const as_hybrid_attn_desc_t* desc, as_hybrid_a
   const int tiles = (desc->N + AS_TILE - 1) / AS_TILE;
   int sms = 148;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  h->sms = sms;
+  h->listed = desc->softmax_idx != nullptr;
   const int BH = desc->B * desc->H;
   const int f_chunks = (desc->phi_dim + 127) / 128;       // the tensor K pass runs one CTA per 128 features as well
   int chunks = std::max(1, std::min(tiles, sms / (BH * f_chunks)));
@@ -198,12 +207,12 @@ as_status_t as_hybrid_attn_create(const as_hybrid_attn_desc_t* desc, as_hybrid_a
   for (int i = 0; i < h->n_s; ++i) rank[h->idx_host[i]] = i;
   if (cudaMalloc(&h->d_sm_rank, sizeof(int32_t) * ((size_t)desc->N + 8)) != cudaSuccess ||
       cudaMalloc(&h->d_status, 256) != cudaSuccess ||
-      cudaMalloc(&h->d_counters, sizeof(uint32_t) * 8 * (size_t)BH) != cudaSuccess) {
+      cudaMalloc(&h->d_counters, sizeof(uint32_t) * n_counters(h)) != cudaSuccess) {
     cudaGetLastError(); as_hybrid_attn_destroy(h); return AS_ERR_ALLOC;
   }
   if (cudaMemcpy(h->d_sm_rank, rank.data(), sizeof(int32_t) * desc->N, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(h->d_status, 0, 256) != cudaSuccess ||
-      cudaMemset(h->d_counters, 0, sizeof(uint32_t) * 8 * (size_t)BH) != cudaSuccess) {
+      cudaMemset(h->d_counters, 0, sizeof(uint32_t) * n_counters(h)) != cudaSuccess) {
     cudaGetLastError(); as_hybrid_attn_destroy(h); return AS_ERR_CUDA;
   }
   if (desc->kernel_path == AS_PATH_TENSOR && as_tensor_init() != cudaSuccess) {
@@ -309,6 +318,8 @@ static as_status_t launch_heads(as_hybrid_attn_t h, const void* q, const void* k
   a.S = (float*)(ws + h->ws.S) + (size_t)first * F * dd; a.z = (float*)(ws + h->ws.z) + (size_t)first * F;
   a.Sb = (__nv_bfloat16*)(ws + h->ws.Sb) + (size_t)first * F * dd;
   a.sm_rank = h->d_sm_rank; a.status = h->d_status; a.counters = h->d_counters;
+  a.parts = h->ws.has_parts ? (float*)(ws + h->ws.parts) : nullptr;
+  a.part_flags = h->d_counters + 8 * (size_t)d.B * d.H;
   a.B = nb; a.H = nh; a.N = d.N; a.d = d.d; a.F = d.phi_dim; a.P = d.poly_degree;
   a.n_s = h->n_s; a.n_l = h->n_l; a.n_chunks = h->n_chunks; a.chunk_tiles = h->chunk_tiles;
   a.scale = h->scale; a.stab_mode = d.stab_mode;
@@ -442,9 +453,9 @@ as_status_t as_hybrid_attn_last_status(as_hybrid_attn_t h, void* cuda_stream) {
       cudaMemcpy(&word, h->d_status, 4, cudaMemcpyDeviceToHost) != cudaSuccess) {
     cudaGetLastError(); return AS_ERR_CUDA;
   }
-  // after a time-out CTAs have left early: the K pass's arrival counters may stand anywhere
+  // after a time-out CTAs have left early: the K pass's arrival counters and the query stage's flags may stand anywhere
   if (word != 0 && (cudaMemset(h->d_status, 0, 4) != cudaSuccess ||
-                    cudaMemset(h->d_counters, 0, sizeof(uint32_t) * 8 * (size_t)h->desc.B * h->desc.H) != cudaSuccess)) {
+                    cudaMemset(h->d_counters, 0, sizeof(uint32_t) * n_counters(h)) != cudaSuccess)) {
     cudaGetLastError(); return AS_ERR_CUDA;
   }
   return (word & AS_DEV_TIMEOUT) ? AS_ERR_DEVICE_TIMEOUT : AS_OK;

@@ -18,6 +18,8 @@ struct as_ws_layout {
   size_t part_s = 0, part_z = 0;        // per-chunk partial state   [B*H, chunks, F, d] / [.., F] fp32
   size_t S = 0, z = 0;                  // final state               [B*H, F, d] / [B*H, F] fp32
   size_t Sb = 0;                        // S rounded to bf16         [B*H, F, d] (MMA operand of the Q pass)
+  size_t parts = 0;                     // the query stage's unfinished units, one per SM (layers with softmax tokens)
+  bool has_parts = false;
   size_t h1k = 0;                       // first-layer activations of the keys [B*H, N, hidden] bf16 (two-layer feature map only)
   size_t total = 0;
   size_t stage_q = 0, stage_k = 0, stage_v = 0, stage_o = 0, total_host = 0;
@@ -41,6 +43,8 @@ struct as_launch_args {
   uint32_t* status;                     // device status word
   uint32_t* counters;                   // [B*H*4][2], zero between launches: K-pass CTAs of a (batch, head, feature chunk)
                                         // that have stored their partial state (and given up) / that have left
+  float* parts;                         // where the query stage's CTAs leave unfinished units (NULL: they do not), and the flags that go with it
+  uint32_t* part_flags;                 // [SMs][2], zero between launches
   int B, H, N, d, F, P;
   int n_s, n_l;
   int n_chunks, chunk_tiles;            // K-pass split of the token axis
@@ -56,8 +60,10 @@ struct as_hybrid_attn_s {
   std::vector<int32_t> idx_host;        // sorted T_S
   int32_t* d_sm_rank = nullptr;
   uint32_t* d_status = nullptr;
-  uint32_t* d_counters = nullptr;       // arrival counters of the K pass (cf. as_launch_args::counters)
+  uint32_t* d_counters = nullptr;       // cf. as_launch_args::counters, then ::part_flags
   int n_chunks = 1, chunk_tiles = 1;
+  int sms = 0;
+  bool listed = false;                  // the softmax tokens came as a list
   as_ws_layout ws;
   uint64_t launches = 0;
   // profiling
@@ -80,6 +86,8 @@ cudaError_t as_reduce_state(const as_launch_args& a, cudaStream_t st);
 cudaError_t as_round_state(const as_launch_args& a, cudaStream_t st);
 cudaError_t as_tensor_kpass(const as_launch_args& a, cudaStream_t st);
 cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st);
+// Workspace of the query stage for unfinished units, 0 where its rule leaves them whole whatever the number of keys.
+size_t as_qpass_parts_bytes(int N, int BH, int d, int sms);
 // Query stage of layers without softmax tokens in its streaming form (one-layer map, F = d = 128, no bias, degree
 // <= 2): whether it covers the launch, and the launch itself.  as_tensor_qpass dispatches to it.
 bool as_tensor_qstream_handles(const as_launch_args& a);

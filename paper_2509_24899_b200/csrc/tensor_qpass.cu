@@ -2,7 +2,7 @@
 // projection, linear apply and merge, fused in one persistent kernel.
 //
 //   persistent, one CTA per SM (what is left over after the full rounds is dealt out in one last round, in
-//   units of two 128-row tiles or of one, see plan_units); per unit a flash-style loop over 128-key tiles
+//   units of two 128-row tiles or of one, see plan_units, or by key tiles, see plan_parts); per unit a flash-style loop over 128-key tiles
 //   of K_S / V_S:        S = Q K_S^T -> TMEM; the softmax threads (one or two per row) read their row and
 //                        release the score columns at once, so the next product into them runs under the
 //                        exponentials; running max / sum per row; P = exp2(.) as bf16 -> TMEM,
@@ -16,6 +16,8 @@
 //                        (128 hidden units at a time) and kept as bf16 in the group's phi_q tile and, once nothing reads
 //                        Q any more, in the Q tile; Phi_c = sum over the hidden slices of h1_j W_q2[c, j]^T.
 // All tiles are staged by TMA with the 128-byte swizzle; every mbarrier wait is bounded.
+#include <algorithm>
+
 #include "tensor_common.cuh"
 
 namespace {
@@ -40,6 +42,15 @@ struct QParams {
   const float* z;            // [B*H][F]
   float* aux;                // [B*H][N][3] or nullptr
   uint32_t* status;
+  // ---- key loops in parts (cf. plan_parts; only the kernels compiled for them look at these)
+  int share;                 // key tiles of a CTA in the last round; 0: units are whole
+  float* parts;              // [CTAs]: what a CTA leaves of a unit that another one finishes, see QPart
+  uint32_t* part_flags;      // [CTAs][2 groups]: it is there; zero between launches
+  // of one part (0 / unused in the launch's own parameters): in place of nkv, n_s and lin above those of the part, and
+  int part;                  // 1: a part
+  int bh, row0, key0;        // its unit; its first key
+  int at_items, at_s, at_p, at_pf, at_tail;   // ring items, phases and tails of the CTA before it
+  int leaves, merges;        // 1: leaves what it has to another CTA; number of CTAs right before this one that have left it theirs
 };
 
 // How the compute threads share a 128-row tile: T = 1, one thread per row (eight warps), or T = 2, threads t and t + 16 of a warp, each
@@ -143,7 +154,9 @@ struct QCtx {
 // an odd number of them (see plan_units).  A group that has the tensor and XU pipes to itself needs about two thirds of
 // the time that the two of a two-tile unit take.
 struct QUnit { int bh, row0, ng; };
+template <bool KS = false>
 AS_DEV QUnit q_unit(const QParams& p, int u) {
+  if (KS && p.part) return QUnit{p.bh, p.row0, 2};
   const int c = (int)blockIdx.x, n = (int)gridDim.x;
   int w = c + u * n, half = 0, ng = 2;
   if (u >= p.n_rounds) {
@@ -246,7 +259,7 @@ struct QRing {
 // The first copies of a CTA, by one thread: ring item 0 (the first key tile, else the first weights) and the first unit's Q tiles.  In line, right behind the wait for
 // the kernel before: as a part of q_produce_unit they went out 2500 - 3500 clk later, which is what its
 // instructions and its parameters take to arrive in a CTA that has just started.
-template <int D, int MAP>
+template <int D, int MAP, bool KS = false>
 __device__ __noinline__ void q_first_loads(const QParams& p, const QCtx& c, const QUnit& un, const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmW,
                           const CUtensorMap* tmW1) {
   using R = QRing<D>;
@@ -254,14 +267,14 @@ __device__ __noinline__ void q_first_loads(const QParams& p, const QCtx& c, cons
   const R q(c);
   const CUtensorMap* first = p.nkv > 0 ? tmK : MAP == MAP_TWO ? tmW1 : tmW;
   mbar_expect_tx(q.bar(R::B_KFULL), L::TILE);
-  load_tile<D>(q.sKV(0), first, q.bar(R::B_KFULL), 0, p.nkv > 0 ? un.bh : un.bh % p.H);
+  load_tile<D>(q.sKV(0), first, q.bar(R::B_KFULL), KS ? p.key0 : 0, p.nkv > 0 ? un.bh : un.bh % p.H);
   for (int g = 0; g < un.ng; ++g) {
     mbar_expect_tx(q.bar(R::B_Q0 + g), L::TILE);
     load_tile<D>(q.sQ(g), tmQ, q.bar(R::B_Q0 + g), un.row0 + g * 128, un.bh);
   }
 }
 // one unit
-template <int D, int MAP, bool GEN>
+template <int D, int MAP, bool GEN, bool KS = false>
 __device__ __noinline__ bool q_produce_unit(const QParams& p, const QCtx& c, const CUtensorMap* tmQ, const CUtensorMap* tmK,
                                             const CUtensorMap* tmV, const CUtensorMap* tmW, const CUtensorMap* tmSt,
                                             const CUtensorMap* tmW1, int u) {
@@ -270,9 +283,9 @@ __device__ __noinline__ bool q_produce_unit(const QParams& p, const QCtx& c, con
   const int nkv = p.nkv;
   const R q(p, c);
   const int lane = threadIdx.x & 31;
-  const QUnit un = q_unit(p, u);
+  const QUnit un = q_unit<KS>(p, u);
   const int bh = un.bh, h = bh % p.H, row0 = un.row0;
-  const int base = u * q.n_items;
+  const int base = KS && p.part ? p.at_items : u * q.n_items, key0 = KS ? p.key0 : 0;
   const int q_at = nkv > 0 ? 1 : 0;                   // the Q tiles are requested right after the unit's first K tile
   for (int it = 0; it < q.n_items; ++it) {
     if (it == q_at && u > 0) {
@@ -293,10 +306,10 @@ __device__ __noinline__ bool q_produce_unit(const QParams& p, const QCtx& c, con
       const uint32_t dst = q.sKV(gi);
       auto to = [&](int b) { mbar_expect_tx(q.bar(b + st), L::TILE); return q.bar(b + st); };   // the barrier that the item arrives at
       if (it < q.n_stream) {
-        if (it == 0 || (it & 1)) load_tile<D>(dst, tmK, to(R::B_KFULL), ((it + 1) >> 1) * 128, bh);   // K_0 at 0, K_j at 2j-1
-        else load_tile<D>(dst, tmV, to(R::B_VFULL), ((it >> 1) - 1) * 128, bh);                        // V_j at 2j+2
+        if (it == 0 || (it & 1)) load_tile<D>(dst, tmK, to(R::B_KFULL), key0 + ((it + 1) >> 1) * 128, bh);   // K_0 at 0, K_j at 2j-1
+        else load_tile<D>(dst, tmV, to(R::B_VFULL), key0 + ((it >> 1) - 1) * 128, bh);                 // V_j at 2j+2
       } else if (q.vl && it == q.it_vlast()) {
-        load_tile<D>(dst, tmV, to(R::B_VFULL), (nkv - 1) * 128, bh);
+        load_tile<D>(dst, tmV, to(R::B_VFULL), key0 + (nkv - 1) * 128, bh);
       } else if (MAP != MAP_TWO) {
         // W[ch] / S[ch] in bf16: [128 feature rows][D]; rows past F arrive as zeros
         const int r = it - q.n_stream - (it > q.n_stream ? q.vl : 0);     // 0: W[0]; 2ch-1: W[ch]; 2ch+2 (and the last): S[ch]
@@ -328,7 +341,7 @@ constexpr uint32_t Q_FAILED = ~0u;
 // its own, eight MMAs took 630 - 700 clk to issue beside the softmax warps (N = 64, d = 64: as long, though they execute in
 // 380); now 320 - 380 (130 for the four of Q K^T at d = 64).  N = 7800: 96.3 -> 93.7 us, headline layer 838 -> 830 us
 // (sustained), two-layer map 1203 -> 1176 us.
-template <int D, int MAP, bool GEN, bool SH>
+template <int D, int MAP, bool GEN, bool SH, bool KS = false>
 __device__ __noinline__ uint32_t q_score_unit(const QParams& p, const QCtx& c, int u, uint32_t looks) {
   using R = QRing<D, SH>;
   constexpr uint32_t ID_QK = make_idesc(128, 128, 0, 0);      // S = Q K^T      (N = 128 keys)
@@ -336,8 +349,9 @@ __device__ __noinline__ uint32_t q_score_unit(const QParams& p, const QCtx& c, i
   const R q(p, c, true);
   const uint32_t id_phi = make_idesc(128, D == 128 ? 128 : p.fcw, 0, 0);   // Phi_c = X W^T  (N = features of a chunk; 128 at d = 128)
   constexpr uint32_t ID_HID = make_idesc(128, D, 0, 0);       // hidden slice = Q W_1[j]^T (N = D hidden units)
-  const int base = u * q.n_items, ps = u * q.n_s;             // first ring item / first score-column phase of the unit
-  const int ng = q_unit(p, u).ng;                             // groups at work on this unit (the last one of a group: ng - 1)
+  const int base = KS && p.part ? p.at_items : u * q.n_items, ps = KS && p.part ? p.at_s : u * q.n_s;   // first ring item / first score-column phase of the unit
+  const int tail = KS && p.part ? p.at_tail : u;              // tails before the unit's
+  const int ng = q_unit<KS>(p, u).ng;                             // groups at work on this unit (the last one of a group: ng - 1)
   uint64_t dq[2][8];                                          // the Q tiles do not move within a unit
 #pragma unroll
   for (int g = 0; g < 2; ++g) {
@@ -345,7 +359,7 @@ __device__ __noinline__ uint32_t q_score_unit(const QParams& p, const QCtx& c, i
 #pragma unroll
     for (int kk = 0; kk < 8; ++kk) dq[g][kk] = q0 + kstep_kmajor(kk);
   }
-  auto s_free = [&](int g, int i) -> bool { return q.template s_free<MAP>(g, ps + i, ng, i, u); };
+  auto s_free = [&](int g, int i) -> bool { return q.template s_free<MAP>(g, ps + i, ng, i, tail); };
 
   // ---- first key tile (its product opens the unit)
   if (nkv > 0) {
@@ -429,7 +443,7 @@ __device__ __noinline__ uint32_t q_score_unit(const QParams& p, const QCtx& c, i
   for (int ch = 0; ch < q.fc; ++ch) {
     for (int g = 0; g < ng; ++g) {
       if (!s_free(g, nkv + q.nh + ch)) return Q_FAILED;
-      if (ch == 0 && !q.wait(R::B_H + g, u)) return Q_FAILED;       // the group's hidden activations are in shared memory
+      if (ch == 0 && !q.wait(R::B_H + g, tail)) return Q_FAILED;       // the group's hidden activations are in shared memory
       for (int j = 0; j < q.nh; ++j) {
         const int iw = base + q.it_w2(ch, j);
         const uint64_t w0 = kmajor_desc(q.sKV(iw));
@@ -454,14 +468,14 @@ __device__ __noinline__ uint32_t q_score_unit(const QParams& p, const QCtx& c, i
   }
 }
 
-template <int D, int MAP, bool GEN, bool SH>
+template <int D, int MAP, bool GEN, bool SH, bool KS = false>
 __device__ __noinline__ uint32_t q_accum_unit(const QParams& p, const QCtx& c, int u, uint32_t looks) {
   using R = QRing<D, SH>;
   constexpr uint32_t ID_PV = make_idesc(128, D, 0, 1);        // O += P V and O += phi_q S  (V, S are MN-major)
   const int nkv = p.nkv, lin = p.lin;
   const R q(p, c, true);
-  const int base = u * q.n_items, pp = u * q.n_p;             // first ring item / first P hand-over phase of the unit
-  const int ng = q_unit(p, u).ng;
+  const int base = KS && p.part ? p.at_items : u * q.n_items, pp = KS && p.part ? p.at_p : u * q.n_p;   // first ring item / first P hand-over phase of the unit
+  const int ng = q_unit<KS>(p, u).ng;
   for (int j = 0; j < nkv; ++j) {
     const bool last = (j + 1 == nkv);
     // as soon as P is there: O += P V
@@ -712,8 +726,105 @@ __device__ __noinline__ float q_two_layer_tail(const QParams& p, const QRing<D>&
   return (dl0 + dl1) + dlb;
 }
 
+// ---------------------------------------------------------------- key loops in parts
+// What a CTA leaves of a unit whose key loop another one finishes: per group O (fp32, unnormalised, [4 columns][row][4]: a warp's lanes are neighbours), then of
+// each row the reference maximum, the true one and the sum.
+template <int D>
+struct QPart {
+  static constexpr int O = 128 * D, GROUP = O + 128 * 4, TOTAL = 2 * GROUP;    // floats
+  AS_DEV static float4* of(const QParams& p, int cta, int g) { return reinterpret_cast<float4*>(p.parts + (size_t)cta * TOTAL + (size_t)g * GROUP); }
+};
+
+// By the threads of a group, whose last product into O has completed.
+template <int D, int T>
+__device__ __noinline__ void q_leave_part(const QParams& p, uint32_t tOg, int g, int r, int hc, float m_ref, float m_true, float l) {
+  float4* to = QPart<D>::of(p, (int)blockIdx.x, g);
+#pragma unroll 1
+  for (int o = 0; o < D / T; o += 16) {
+    uint32_t y[16];
+    q_ld16<T, D / 2>(tOg + o, y);
+    tmem_ld16_wait(y);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      to[((hc * (D / T) + o) / 4 + i) * 128 + r] = make_float4(__uint_as_float(y[4 * i]), __uint_as_float(y[4 * i + 1]), __uint_as_float(y[4 * i + 2]),
+                                                                __uint_as_float(y[4 * i + 3]));
+  }
+  if (hc == 0) to[QPart<D>::O / 4 + r] = make_float4(m_ref, m_true, l, 0.f);
+  named_barrier_sync(1 + g, 128 * T);
+  if ((threadIdx.x & 127) == 0 && threadIdx.x < 256)           // (one thread of either group; what the barrier has ordered before it goes with it)
+    asm volatile("st.release.gpu.global.u32 [%0], 1;" ::"l"(p.part_flags + 2 * blockIdx.x + g) : "memory");
+}
+
+// Adds to O, and to the row's maxima and sum, what the p.merges CTAs right before this one have left.  CTAs start in the order of their index, so
+// those are running or through, and their parts that are left come first in them and wait for nothing: the wait ends whatever else is on the GPU (and is bounded
+// like every other).  Returns (m_ref, m_true, l); the sum is negative when a wait ran out.
+template <int D, int T>
+__device__ __noinline__ float4 q_merge_parts(const QParams& p, const WaitCtx& wc, uint32_t tOg, int g, int r, int hc, float m_ref, float m_true, float l) {
+  constexpr int STEP = 32, N = STEP / 4;                       // columns and loads at once
+  for (int n = 1; n <= p.merges; ++n) {
+    const int cta = (int)blockIdx.x - n;
+    uint32_t* flag = p.part_flags + 2 * cta + g;
+    bool ok = true;
+    if ((threadIdx.x & 31) == 0) {
+      uint32_t there, it = 0;
+      long long t0 = 0;
+      while (true) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(there) : "l"(flag) : "memory");
+        if (there != 0u) break;
+        if ((++it & 15u) != 0u) continue;
+        const long long now = clock64();
+        if (t0 == 0) t0 = now;
+        if (*wc.abort != 0u || now - t0 > kWaitLimitCycles) { *wc.abort = 1u; atomicOr(wc.status, 1u); ok = false; break; }
+      }
+    }
+    if (!__all_sync(0xffffffffu, ok)) return make_float4(0.f, 0.f, -1.f, 0.f);
+    const float4* from = QPart<D>::of(p, cta, g);
+    const float4* mine_from = from + hc * (D / T / 4) * 128 + r;
+    const float4 st = __ldcg(from + QPart<D>::O / 4 + r);
+    float4 x[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) x[i] = __ldcg(mine_from + i * 128);
+    const float m = fmaxf(m_ref, st.x), mine = ex2(m_ref - m), theirs = ex2(st.x - m);
+#pragma unroll 1
+    for (int o = 0; o < D / T; o += STEP) {
+      uint32_t y[32];
+      q_ld32<T, D / 2>(tOg + o, y);
+      tmem_ld_wait(y);
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        const float part[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          // a sum that weighs nothing is left out, also where it is past the end of the range (many keys with values near it)
+          const float own = mine > 0.f ? __uint_as_float(y[4 * i + e]) * mine : 0.f;
+          y[4 * i + e] = __float_as_uint(theirs > 0.f ? fmaf(part[e], theirs, own) : own);
+        }
+      }
+      if (o + STEP < D / T) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) x[i] = __ldcg(mine_from + ((o + STEP) / 4 + i) * 128);
+      }
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        uint32_t z[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) z[i] = y[16 * half + i];
+        q_st16<T, D / 2>(tOg + o + 16 * half, z);
+      }
+    }
+    tmem_st_wait();
+    l = l * mine + st.z * theirs;
+    m_true = fmaxf(m_true, st.y);
+    m_ref = m;
+    named_barrier_sync(1 + g, 128 * T);                        // every warp has seen the flag: zero for the next launch
+    if ((threadIdx.x & 127) == 0 && threadIdx.x < 256) *reinterpret_cast<volatile uint32_t*>(flag) = 0u;
+  }
+  tc_fence_before();
+  return make_float4(m_ref, m_true, l, 0.f);
+}
+
 // ---------------------------------------------------------------- softmax / merge group, one unit
-template <int D, int T, int MAP, bool GEN>
+template <int D, int T, int MAP, bool GEN, bool KS = false>
 __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, const CUtensorMap* tmO, uint8_t* smem, int u) {
   using R = QRing<D>;
   using L = QLayout<D>;
@@ -728,7 +839,7 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
   const uint32_t lane_off = (uint32_t)r0 << 16;
   const uint32_t tSg = q.tS(g) + lane_off, tOg = q.tO(g) + lane_off, tPg = q.tP(g) + lane_off;
   uint8_t* sPg = smem + L::P_OFF + g * L::PTILE;    // this group's phi_q / output staging tile
-  const int ps = u * q.n_s, ppf = u * q.n_pf;       // first phases of the unit (cf. QRing)
+  const int ps = KS && p.part ? p.at_s : u * q.n_s, ppf = KS && p.part ? p.at_pf : u * q.n_pf;   // first phases of the unit (cf. QRing)
   float m_ref = 0.f, m_true = -INFINITY, l = 0.f;
 
   for (int j = 0; j < nkv; ++j) {
@@ -812,9 +923,25 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
     mbar_arrive(q.bar(R::B_P + g));
   }
 
-  const QUnit un = q_unit(p, u);
+  const QUnit un = q_unit<KS>(p, u);
   const int bh = un.bh;
   if (T == 2) l += __shfl_xor_sync(0xffffffffu, l, 16);
+  if constexpr (KS) {
+    if (p.leaves) {
+      if (!q.wait(R::B_O + g, u)) return false;
+      tc_fence_after();
+      q_leave_part<D, T>(p, tOg, g, r, hc, m_ref, m_true, l);
+      tc_fence_before();
+      return true;
+    }
+    if (p.merges > 0) {
+      if (!q.wait(R::B_PF + g, ppf + nkv - 1)) return false;   // the last P V has completed (looked at once more in the tail)
+      tc_fence_after();
+      const float4 sum = q_merge_parts<D, T>(p, c.wc, tOg, g, r, hc, m_ref, m_true, l);
+      if (sum.z < 0.f) return false;
+      m_ref = sum.x; m_true = sum.y; l = sum.z;
+    }
+  }
   const int row = un.row0 + g * 128 + r;
   float den = l, den_l_out = 0.f;
   if (p.lin) {
@@ -1069,7 +1196,36 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   }
 }
 
-template <int D, int T, int MAP, bool GEN>
+// The parts of CTA c in the last round (see plan_parts): at most two, the one that it leaves to the next CTA first.  Written by one thread.
+template <int D>
+AS_DEV int q_parts(const QParams& p, QParams* to) {
+  const int c = (int)blockIdx.x, n = (int)gridDim.x, left = p.n_pairs - p.n_rounds * n, all = left * p.nkv;
+  const int r0 = c * p.share, r1 = min(all, r0 + p.share);
+  if (r0 >= r1) return 0;
+  const bool tailed = p.lin != 0;
+  const int fc = tailed ? p.fc : 0, slices = tailed && p.layers == 2 ? p.nh : 0, tail_items = slices ? slices + fc * slices + fc : 2 * fc;
+  int at_items = p.n_rounds * (2 * p.nkv + tail_items), at_s = p.n_rounds * (p.nkv + slices + fc), at_p = p.n_rounds * (p.nkv + fc);
+  int at_pf = p.n_rounds * (p.nkv + (slices ? 1 : fc)), at_tail = p.n_rounds, np = 0;
+  auto add = [&](int unit, int k0, int k1) {
+    QParams& q = to[np++];
+    const int w = p.n_rounds * n + unit;
+    q = p;
+    q.part = 1;
+    q.bh = w / p.nx; q.row0 = (w % p.nx) * 256; q.key0 = k0 * 128;
+    q.nkv = k1 - k0; q.n_s = p.n_s - q.key0;
+    q.leaves = k1 < p.nkv ? 1 : 0;
+    q.lin = q.leaves ? 0 : p.lin;
+    q.merges = q.leaves || k0 == 0 ? 0 : c - unit * p.nkv / p.share;
+    q.at_items = at_items; q.at_s = at_s; q.at_p = at_p; q.at_pf = at_pf; q.at_tail = at_tail;
+    at_items += 2 * q.nkv; at_s += q.nkv; at_p += q.nkv; at_pf += q.nkv;       // (of one that is left; nothing comes behind another)
+  };
+  const int unit = r0 / p.nkv, k0 = r0 - unit * p.nkv, over = r1 - (unit + 1) * p.nkv;
+  if (over > 0) add(unit + 1, 0, over);
+  add(unit, k0, over > 0 ? p.nkv : r1 - unit * p.nkv);
+  return np;
+}
+
+template <int D, int T, int MAP, bool GEN, bool KS = false>
 __global__ void __launch_bounds__(QShape<T>::THREADS, 1)
 qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
              const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmW,
@@ -1100,6 +1256,9 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     fence_proxy_async();
   }
   __shared__ uint32_t s_skip;
+  __shared__ QParams s_part[KS ? 2 : 1];
+  __shared__ int s_parts;
+  if (KS && threadIdx.x == 64) s_parts = q_parts<D>(p, s_part);
   if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);    // (ahead of the wait: behind the first copies it would wait for these)
   if (warp == X::W_SCORE) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   if (warp == X::W_TMA && (threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); tma_prefetch_desc(&tmO); }
@@ -1112,24 +1271,25 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     return;
   }
   const QCtx c{sbase, *tmem_slot, WaitCtx{p.status, abort_flag}};
-  const int n_mine = q_units_of_cta(p);               // units of this CTA
+  const int n_mine = KS ? p.n_rounds + s_parts : q_units_of_cta(p);   // units of this CTA
+  auto of = [&](int u) -> const QParams& { return KS && u >= p.n_rounds ? s_part[KS ? u - p.n_rounds : 0] : p; };
 
   if (warp == X::W_TMA) {
-    if ((threadIdx.x & 31) == 0) q_first_loads<D, MAP>(p, c, q_unit(p, 0), &tmQ, &tmK, &tmW, &tmW1);
+    if ((threadIdx.x & 31) == 0) q_first_loads<D, MAP, KS>(of(0), c, q_unit<KS>(of(0), 0), &tmQ, &tmK, &tmW, &tmW1);
     __syncwarp();
     for (int u = 0; u < n_mine; ++u)
-      if (!q_produce_unit<D, MAP, GEN>(p, c, &tmQ, &tmK, &tmV, &tmW, &tmSt, &tmW1, u)) break;
+      if (!q_produce_unit<D, MAP, GEN, KS>(of(u), c, &tmQ, &tmK, &tmV, &tmW, &tmSt, &tmW1, u)) break;
   } else if (warp == X::W_SCORE) {
     uint32_t looks = 0u;
-    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_score_unit<D, MAP, GEN, D == 128>(p, c, u, looks);
+    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_score_unit<D, MAP, GEN, D == 128, KS>(of(u), c, u, looks);
   } else if (warp == X::W_ACCUM) {
     uint32_t looks = 0u;
-    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_accum_unit<D, MAP, GEN, D == 128>(p, c, u, looks);
+    for (int u = 0; u < n_mine && looks != Q_FAILED; ++u) looks = q_accum_unit<D, MAP, GEN, D == 128, KS>(of(u), c, u, looks);
   } else {
     // a unit worked on by one group only is the CTA's last one: group 1 stops before it
-    const int n_grp = (n_mine > p.n_rounds && ((warp >> 2) & 1) == 1 && q_unit(p, p.n_rounds).ng == 1) ? p.n_rounds : n_mine;
+    const int n_grp = (!KS && n_mine > p.n_rounds && ((warp >> 2) & 1) == 1 && q_unit(p, p.n_rounds).ng == 1) ? p.n_rounds : n_mine;
     for (int u = 0; u < n_grp; ++u)
-      if (!q_softmax_unit<D, T, MAP, GEN>(p, c, &tmO, smem, u)) break;
+      if (!q_softmax_unit<D, T, MAP, GEN, KS>(of(u), c, &tmO, smem, u)) break;
     if ((threadIdx.x & 31) == 0) tma_store_wait_read();  // this warp's output stores have read their rows (the writes land by the end of the kernel)
   }
 
@@ -1149,10 +1309,15 @@ cudaError_t as_tensor_init_qpass() {
 #define AS_OPT_IN_Q(D_, T_, MAP_) \
   if ((e = opt_in_smem(qpass_kernel<D_, T_, MAP_, false>, QLayout<D_>::TOTAL)) != cudaSuccess) return e; \
   if ((e = opt_in_smem(qpass_kernel<D_, T_, MAP_, true>, QLayout<D_>::TOTAL)) != cudaSuccess) return e
+#define AS_OPT_IN_QP(D_, T_, MAP_) \
+  if ((e = opt_in_smem(qpass_kernel<D_, T_, MAP_, false, true>, QLayout<D_>::TOTAL)) != cudaSuccess) return e; \
+  if ((e = opt_in_smem(qpass_kernel<D_, T_, MAP_, true, true>, QLayout<D_>::TOTAL)) != cudaSuccess) return e
   AS_OPT_IN_Q(128, 1, MAP_ONE); AS_OPT_IN_Q(128, 1, MAP_WIDE); AS_OPT_IN_Q(128, 1, MAP_TWO);
   AS_OPT_IN_Q(128, 2, MAP_ONE); AS_OPT_IN_Q(128, 2, MAP_WIDE); AS_OPT_IN_Q(128, 2, MAP_TWO);
   AS_OPT_IN_Q(64, 2, MAP_ONE); AS_OPT_IN_Q(64, 2, MAP_TWO);
+  AS_OPT_IN_QP(128, 1, MAP_ONE); AS_OPT_IN_QP(128, 1, MAP_WIDE); AS_OPT_IN_QP(128, 1, MAP_TWO); AS_OPT_IN_QP(64, 2, MAP_ONE); AS_OPT_IN_QP(64, 2, MAP_TWO);
 #undef AS_OPT_IN_Q
+#undef AS_OPT_IN_QP
   if ((e = opt_in_smem(qlin_kernel<128, false>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
   if ((e = opt_in_smem(qlin_kernel<128, true>, QLayout<128>::TOTAL)) != cudaSuccess) return e;
   if ((e = opt_in_smem(qlin_kernel<64, false>, QLayout<64>::TOTAL)) != cudaSuccess) return e;
@@ -1185,6 +1350,31 @@ int plan_units(QParams& p, int BH, int sms) {
   }
   return grid;
 }
+// The last round with the key loops of its units cut across CTAs: the key tiles of what is left after the full rounds, unit after unit, are dealt out in equal
+// shares, so that a CTA finishes one unit and leaves the beginning of the next one to the CTA after it (q_parts).  Whole units, or lone tiles, leave
+// much of the GPU idle where a little more than half of a round is left, or little work in long loops.  What it costs: O of a part through L2, the wait for it, a
+// unit's fixed work twice, 5 - 8 us in all (the 10000 or 14000 and 2500 clk below).  Taken where the rounds as plan_units deals them out take longer by more than
+// that, in the clocks that a key tile of a unit, one of a lone tile and a unit's tail were measured at.  Whole calls, units whole -> in parts (us): full softmax,
+// d = 128, 2 heads of N = 10000 135 -> 86, 1 of 15000 126 -> 96, 1 of 8000 72 -> 49, 4 of 5600 79 -> 61, 7 of 3999 59 -> 57; d = 64, 1 of 8000 70 -> 38, 4 of
+// 5600 76 -> 57; one key in two, 2 of 12288 102 -> 87, d = 64 94 -> 80; one rank of four of the 81-frame layer (two rounds and 88 units) 205 -> 202.  Below
+// the line: 5 heads of N = 5000, one key in two (0.96 by this rule with 10000) 56.5 -> 59.6.  Returns the number of CTAs, 0: units stay whole.
+int plan_parts(QParams& p, int BH, int sms, int slices) {
+  if (p.nkv < 2) return 0;
+  const int nx = ((p.N + 127) / 128 + 1) / 2, pairs = nx * BH, rounds = pairs / sms, left = pairs - rounds * sms;
+  if (left == 0) return 0;
+  const int all = left * p.nkv, share = std::max(2, (all + sms - 1) / sms);
+  if (share >= p.nkv) return 0;
+  const int merges = (p.nkv - 1) / share + 1;                 // the most that a CTA adds up
+  if (merges > 8) return 0;
+  const double tail = p.lin ? 9000. + 4500. * ((p.fc - 1) + (slices ? slices * (1 + p.fc) : 0)) : 4000.;
+  const double unit = p.nkv * 2900. + tail, lone = p.nkv * 1800. + 0.7 * tail;
+  const int last = p.split_last ? (p.n_pairs > p.n_rounds * sms || p.n_single > 0) : 2 * (p.n_pairs > p.n_rounds * sms);   // 0: none, 1: lone tiles, 2: units
+  const double now = p.n_rounds * unit + (last == 2 ? unit : last == 1 ? lone : 0.);
+  const double then = rounds * unit + share * 2900. + tail + (p.lin ? 14000. : 10000.) + 2500. * merges;
+  if (then > 0.96 * now) return 0;
+  p.nx = nx; p.n_pairs = pairs; p.n_single = 0; p.n_rounds = rounds; p.split_last = 0; p.share = share;
+  return rounds > 0 ? sms : (all + share - 1) / share;
+}
 // no CTA has more than one tile: one group works, the other one has nothing to do
 bool one_tile_each(const QParams& p) { return p.n_rounds == 0 && p.split_last; }
 // Threads per row of the kernel with a key loop (after plan_units).  Two (sixteen compute warps) hide more of the latencies; one draws less power per
@@ -1200,12 +1390,23 @@ bool one_tile_each(const QParams& p) { return p.n_rounds == 0 && p.split_last; }
 // maps of few rounds 256 / 256 are 2 - 7 % faster with two (N = 1560 ... 9360, 0 to 10 tiles), 128 / 128 0 - 3 %.
 int q_threads_per_row(const QParams& p, int d, bool two, bool gen) {
   if (d == 64 || one_tile_each(p)) return 2;
+  if (p.share > 0) return 1;                         // (with parts the key loop does not stay in 96 registers: full softmax, 4 heads of N = 5600 61 -> 67 us)
   if (!two) return p.nkv <= (gen ? 48 : 31) ? 2 : 1;
   if (gen && p.fc > 1) return p.nkv <= 48 ? 2 : 1;
   if (p.fc == 1 && p.nkv == 0) return 1;
   return p.nkv <= 16 && p.n_rounds < 4 ? 2 : 1;
 }
 }  // namespace
+
+size_t as_qpass_parts_bytes(int N, int BH, int d, int sms) {
+  QParams p{};
+  p.N = N;
+  plan_units(p, BH, sms);
+  const int pairs = ((N + 127) / 128 + 1) / 2 * BH, rounds = pairs / sms;
+  const double now = p.n_rounds + (p.split_last ? (p.n_pairs > p.n_rounds * sms || p.n_single > 0 ? 0.62 : 0.) : p.n_pairs > p.n_rounds * sms ? 1. : 0.);
+  if (pairs == rounds * sms || (double)pairs / sms > 0.96 * now) return 0;   // as plan_parts with a key loop without an end
+  return sizeof(float) * (size_t)(d == 128 ? QPart<128>::TOTAL : QPart<64>::TOTAL) * sms;
+}
 
 cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   if (as_tensor_qstream_handles(a)) return as_tensor_qstream(a, st);   // no softmax tokens, the common feature map
@@ -1228,7 +1429,11 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
     return cudaErrorInvalidValue;
-  const dim3 grid(plan_units(p, BH, sms), 1, 1);
+  dim3 grid(plan_units(p, BH, sms), 1, 1);
+  p.parts = a.parts; p.part_flags = a.part_flags;
+  const int ctas = a.parts != nullptr && !qlin ? plan_parts(p, BH, sms, p.nh) : 0;
+  const bool ks = ctas > 0;
+  if (ks) grid.x = ctas;
   // the general kernels carry the bias and the powers beyond 2; the common case does without them
   const bool gen = lin && (a.P > 2 || p.b1 != nullptr || p.b2 != nullptr);
   const int tpr = q_threads_per_row(p, a.d, two, gen);
@@ -1256,17 +1461,32 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
     if (gen) AS_LAUNCH_QL(64, true); else AS_LAUNCH_QL(64, false);
 #undef AS_LAUNCH_QL
   }
-#define AS_LAUNCH_Q(D_, T_, MAP_) \
+#define AS_LAUNCH_Q(...) \
+  return as_launch_dependent(qpass_kernel<__VA_ARGS__>, grid, dim3(threads), smem, st, tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO, p)
+#define AS_LAUNCH_QG(D_, T_, MAP_) \
   do { \
-    if (gen) return as_launch_dependent(qpass_kernel<D_, T_, MAP_, true>, grid, dim3(QShape<T_>::THREADS), QLayout<D_>::TOTAL, st, tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO, p); \
-    return as_launch_dependent(qpass_kernel<D_, T_, MAP_, false>, grid, dim3(QShape<T_>::THREADS), QLayout<D_>::TOTAL, st, tmQ, tmK, tmV, tmW, tmSt, tmW1, tmO, p); \
+    const int threads = QShape<T_>::THREADS, smem = QLayout<D_>::TOTAL; \
+    if (gen) AS_LAUNCH_Q(D_, T_, MAP_, true); else AS_LAUNCH_Q(D_, T_, MAP_, false); \
   } while (0)
+#define AS_LAUNCH_QP(D_, T_, MAP_) \
+  do { \
+    const int threads = QShape<T_>::THREADS, smem = QLayout<D_>::TOTAL; \
+    if (gen) AS_LAUNCH_Q(D_, T_, MAP_, true, true); else AS_LAUNCH_Q(D_, T_, MAP_, false, true); \
+  } while (0)
+  const int map = two ? MAP_TWO : lin && p.fc > 1 && !one_tile_each(p) ? MAP_WIDE : MAP_ONE;
+  if (ks) {
+    if (a.d == 64) { if (two) AS_LAUNCH_QP(64, 2, MAP_TWO); else AS_LAUNCH_QP(64, 2, MAP_ONE); }
+    if (map == MAP_TWO) AS_LAUNCH_QP(128, 1, MAP_TWO);
+    if (map == MAP_WIDE) AS_LAUNCH_QP(128, 1, MAP_WIDE); else AS_LAUNCH_QP(128, 1, MAP_ONE);
+  }
 #define AS_LAUNCH_QT(T_) \
   do { \
-    if (two) AS_LAUNCH_Q(128, T_, MAP_TWO); else if (lin && p.fc > 1 && !one_tile_each(p)) AS_LAUNCH_Q(128, T_, MAP_WIDE); else AS_LAUNCH_Q(128, T_, MAP_ONE); \
+    if (map == MAP_TWO) AS_LAUNCH_QG(128, T_, MAP_TWO); else if (map == MAP_WIDE) AS_LAUNCH_QG(128, T_, MAP_WIDE); else AS_LAUNCH_QG(128, T_, MAP_ONE); \
   } while (0)
   if (a.d == 128) { if (tpr == 2) AS_LAUNCH_QT(2); else AS_LAUNCH_QT(1); }
-  if (two) AS_LAUNCH_Q(64, 2, MAP_TWO); else AS_LAUNCH_Q(64, 2, MAP_ONE);
-#undef AS_LAUNCH_QT
+  if (two) AS_LAUNCH_QG(64, 2, MAP_TWO); else AS_LAUNCH_QG(64, 2, MAP_ONE);
 #undef AS_LAUNCH_Q
+#undef AS_LAUNCH_QG
+#undef AS_LAUNCH_QP
+#undef AS_LAUNCH_QT
 }
