@@ -130,6 +130,7 @@ __global__ void reduce_state_kernel(as_launch_args a) {
 
 __global__ void round_state_kernel(const float* S, __nv_bfloat16* Sb, size_t n) {
   sm100::griddep_launch();
+  sm100::griddep_wait();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) Sb[i] = __float2bfloat16_rn(S[i]);
 }
@@ -276,8 +277,7 @@ cudaError_t as_reduce_state(const as_launch_args& a, cudaStream_t st) {
 
 cudaError_t as_round_state(const as_launch_args& a, cudaStream_t st) {
   const size_t n = (size_t)a.B * a.H * a.F * a.d;
-  round_state_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a.S, a.Sb, n);
-  return cudaGetLastError();
+  return as_launch_dependent(round_state_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, (const float*)a.S, a.Sb, n);
 }
 
 cudaError_t as_simt_qpass(const as_launch_args& a, cudaStream_t st) {
