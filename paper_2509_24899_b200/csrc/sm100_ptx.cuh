@@ -108,6 +108,7 @@ AS_DEV void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: 
 AS_DEV void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // Only until the sources of all committed stores have been read: the shared memory can be reused.
 AS_DEV void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+AS_DEV void tma_store_wait_read_but_last() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 
 // ---------------------------------------------------------------- tensor memory
 AS_DEV void tmem_alloc(uint32_t smem_slot, uint32_t ncols) {

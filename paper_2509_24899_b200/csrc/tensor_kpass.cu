@@ -488,34 +488,32 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
 
 // ======================================================================================
 // First layer of a two-layer feature map for the keys ("Characterization of phi": the embedding
-// network): h1 = relu(k W_1^T + b_1), [B*H, N, hidden] bf16.  One 128-token tile per CTA, all hidden slices.
+// network): h1 = relu(k W_1^T + b_1), [B*H, N, hidden] bf16.  One 128-token tile per CTA.
 // The softmax rows of K are copied to K_S here, where the K tile is in shared memory, by the warps that otherwise only wait
 // for the product.  (The K pass, which has h1 tiles in its ring instead, fetched them from global memory one row after
 // the other and held its slots of the ring meanwhile: the whole key side 338 us against 181 at N = 32760, rate 1/8, hidden =
 // F = 256, the layer 1182 against 1071.)
-// Two CTAs share an SM, and what bounds the kernel is the chain of one (set-up, 96 KB of loads, products, rows, stores): so each slice goes
-// its own way, rows by eight warps under the next slice's product, staged over its own weights and stored at once, and the CTA ends
-// when its stores have been read.  With four warps, both slices' rows behind both products, and an end that waited for the stores to
-// land: the same layer 906 us against 897, N = 7800 152.0 against 150.7 (74 us of this kernel; floor 47).
+// This one: hidden widths of 64 and 128, several CTAs on an SM; what bounds it is the chain of one (set-up, loads, product, rows, stores), so the rows are
+// taken by eight warps, staged over the weights and stored at once, and the CTA ends when its stores have been read.
 // ======================================================================================
 // A dependent launch: its CTAs set up beside the kernel before it (N = 1144, 2 heads, 128 / 128: a call 28.9 -> 27.8 us; N = 1036, 5 heads, d = 64
 // 24.9 -> 22.9).
-struct P1Params { int H, hid, N, n_s; const __nv_bfloat16* bias; const int32_t* sm_rank; __nv_bfloat16* ks_w; uint32_t* status; };
+struct P1Params { int H, hid, N, n_s, tiles, total; const __nv_bfloat16* bias; const int32_t* sm_rank; __nv_bfloat16* ks_w; uint32_t* status; };
 constexpr int P1_THREADS = 288;          // warps 0-7: epilogue (two threads per token row, each half of a slice's columns); warp 8: TMA + MMA
 
-template <int D, int NH>
+template <int D>
 struct P1Layout {
   static constexpr int TILE = 128 * D * 2;
-  static constexpr int X_OFF = 0, W_OFF = TILE, BAR_OFF = (1 + NH) * TILE;
-  static constexpr int BIAS_OFF = BAR_OFF + 64;                 // NH * D floats
-  static constexpr int TOTAL = BIAS_OFF + NH * D * 4 + 1024;
+  static constexpr int X_OFF = 0, W_OFF = TILE, BAR_OFF = 2 * TILE;
+  static constexpr int BIAS_OFF = BAR_OFF + 64;                 // D floats
+  static constexpr int TOTAL = BIAS_OFF + D * 4 + 1024;
 };
 
-template <int D, int NH>
+template <int D>
 __global__ void __launch_bounds__(P1_THREADS)
 phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
             const __grid_constant__ CUtensorMap tmH, const P1Params p) {
-  using L = P1Layout<D, NH>;
+  using L = P1Layout<D>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
@@ -527,21 +525,21 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
   const int bh = blockIdx.y, h = bh % p.H, row0 = blockIdx.x * 128;
   const WaitCtx wc{p.status, abort_flag};
   const uint32_t bar_full = smem_u32(bars);
-  auto bar_done = [&](int j) { return smem_u32(bars + 1 + j); };   // slice j's product has completed
-  constexpr int TM_COLS = NH * 128;                             // 128 or 256: a power of two
+  const uint32_t bar_done = smem_u32(bars + 1);                  // the product has completed
+  constexpr int TM_COLS = 128;
 
   __shared__ uint32_t s_skip;
   if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
     mbar_init(bar_full, 1);
-    for (int j = 0; j < NH; ++j) mbar_init(bar_done(j), 1);
+    mbar_init(bar_done, 1);
     fence_barrier_init();
     fence_proxy_async();
   }
   if (warp == 8) { tmem_alloc(smem_u32(tmem_slot), TM_COLS); tmem_relinquish(); }
   griddep_wait();                                    // the set-up above ran beside the kernel before this one
-  for (int i = threadIdx.x; i < NH * D; i += P1_THREADS)
+  for (int i = threadIdx.x; i < D; i += P1_THREADS)
     sBias[i] = (p.bias != nullptr && i < p.hid) ? __bfloat162float(p.bias[(size_t)h * p.hid + i]) : 0.f;
   tc_fence_before();
   __syncthreads();
@@ -552,25 +550,20 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
   }
   const uint32_t tmem = *tmem_slot;
   const uint32_t sX = sbase + L::X_OFF;
-  auto sW = [&](int j) { return sbase + L::W_OFF + j * L::TILE; };
-  // Hidden slice j is staged for its store over W tile j, which nothing reads once its product has completed: slice 0 leaves while slice 1
-  // is still being formed.
-  auto stage_off = [&](int j) { return L::W_OFF + j * L::TILE; };
+  const uint32_t sW = sbase + L::W_OFF;             // h1 is staged for its store over the weights, which nothing reads once the product has completed
 
   if (warp == 8) {
     if (lane == 0) {
-      mbar_expect_tx(bar_full, (1 + NH) * L::TILE);
+      mbar_expect_tx(bar_full, 2 * L::TILE);
       load_tile<D>(sX, &tmX, bar_full, row0, bh);
-      for (int j = 0; j < NH; ++j) load_tile<D>(sW(j), &tmW, bar_full, j * 128, h);   // W_1[h] rows of slice j (past hid: zeros)
+      load_tile<D>(sW, &tmW, bar_full, 0, h);          // W_1[h] (rows past hid: zeros)
     }
     __syncwarp();
     if (mbar_wait_warp(bar_full, 0, wc)) {
       tc_fence_after();
       if (lane == 0) {
-        for (int j = 0; j < NH; ++j) {    // X W_1^T, N = 128 hidden units of slice j (N = D when the hidden width is 64)
-          issue_kmajor<D>(tmem + j * 128, kmajor_desc(sX), kmajor_desc(sW(j)), make_idesc(128, NH == 1 ? D : 128, 0, 0), false);
-          tc_commit(bar_done(j));
-        }
+        issue_kmajor<D>(tmem, kmajor_desc(sX), kmajor_desc(sW), make_idesc(128, D, 0, 0), false);   // X W_1^T
+        tc_commit(bar_done);
       }
       __syncwarp();
     }
@@ -603,31 +596,28 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
       __syncwarp();
     }
     uint32_t x[32];
+    if (ok) ok = mbar_wait_warp(bar_done, 0, wc);
+    if (ok) {
+      tc_fence_after();
 #pragma unroll
-    for (int j = 0; j < NH; ++j) {
-      if (ok) ok = mbar_wait_warp(bar_done(j), 0, wc);
-      if (ok) {
-        tc_fence_after();
+      for (int c = 0; c < D / 64; ++c) {
+        const int col = hf * (D / 2) + c * 32;
+        tmem_ld32(tmem + lane_off + col, x);
+        tmem_ld_wait(x);
+        const float* bb = sBias + col;
+        uint32_t w[16];
 #pragma unroll
-        for (int c = 0; c < D / 64; ++c) {
-          const int col = hf * (D / 2) + c * 32;
-          tmem_ld32(tmem + lane_off + j * 128 + col, x);
-          tmem_ld_wait(x);
-          const float* bb = sBias + j * D + col;
-          uint32_t w[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i)
-            w[i] = pack_bf16(fmaxf(__uint_as_float(x[2 * i]) + bb[2 * i], 0.f), fmaxf(__uint_as_float(x[2 * i + 1]) + bb[2 * i + 1], 0.f));
-          store_row_chunk(smem + stage_off(j), r, col, w);
-        }
-        fence_proxy_async();
+        for (int i = 0; i < 16; ++i)
+          w[i] = pack_bf16(fmaxf(__uint_as_float(x[2 * i]) + bb[2 * i], 0.f), fmaxf(__uint_as_float(x[2 * i + 1]) + bb[2 * i + 1], 0.f));
+        store_row_chunk(smem + L::W_OFF, r, col, w);
       }
-      named_barrier_sync(1, 256);                             // reached by every epilogue thread, also after a failed wait
-      if (ok && threadIdx.x == 0) {
+      fence_proxy_async();
+    }
+    named_barrier_sync(1, 256);                               // reached by every epilogue thread, also after a failed wait
+    if (ok && threadIdx.x == 0) {
 #pragma unroll
-        for (int b = 0; b < D / 64; ++b) tma_store_3d(&tmH, sbase + stage_off(j) + b * BOX_BYTES, j * D + b * 64, row0, bh);
-        tma_store_commit();
-      }
+      for (int b = 0; b < D / 64; ++b) tma_store_3d(&tmH, sW + b * BOX_BYTES, b * 64, row0, bh);
+      tma_store_commit();
     }
     if (threadIdx.x == 0) tma_store_wait_read();              // (the writes land by the end of the kernel)
   }
@@ -636,6 +626,210 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
   if (warp == 8) {
     tc_fence_after();
     tmem_dealloc(tmem, TM_COLS);
+  }
+}
+
+// The same for a hidden width of 256 at d = 128, bound by HBM (k in, h1 out twice as wide): a CTA per SM takes a run of tiles, one after the other.  The
+// head's weights stay in shared memory, three tiles of K are in flight, the products of a tile run under the rows of the one before (two sets of
+// accumulators), and a slice of h1 is stored while the next one is formed.  Where a run goes on into the next head, its weights come when the last
+// product with the old ones has completed; its first tile of K is asked for before that.  N = 32760, 12 heads, no softmax tokens: this stage 65 -> 56 us (floor
+// 46), the call 310 -> 300; rate 1/8 990 -> 980, N = 7800 140.5 -> 138.1, 8 heads of N = 1560 38.4 -> 37.7.  Narrower maps keep the kernel above, which has
+// several CTAs on an SM there: in runs of tiles, 128 / 128 with 2 heads of N = 1560 27.4 -> 28.2 us, d = 64 with 12 of 7800 78.4 -> 79.5 (24 of 15600 without
+// softmax tokens 110.9 -> 107.1).  Tried: softmax rows of K copied behind the slices' rows instead of ahead of them, N = 15600, 16 heads 85.5 -> 87.5.
+constexpr int P1R_THREADS = 320;          // warps 0-7: epilogue (two threads per token row, each half of a slice's columns); 8: TMA; 9: MMA
+constexpr int P1R_RING = 3;               // tiles of K in shared memory
+
+struct P1RLayout {
+  static constexpr int D = 128, NH = 2;
+  static constexpr int TILE = 128 * D * 2;
+  static constexpr int W_OFF = 0, X_OFF = NH * TILE, OUT_OFF = X_OFF + P1R_RING * TILE, BAR_OFF = OUT_OFF + 2 * TILE;
+  static constexpr int BIAS_OFF = BAR_OFF + 128;                // NH * D floats
+  static constexpr int TOTAL = BIAS_OFF + NH * D * 4 + 1024;
+  static constexpr int COLS = 2 * NH * D;                       // tensor memory: two tiles' products
+  static_assert(TOTAL <= 227 * 1024 && COLS == 512);
+};
+
+__global__ void __launch_bounds__(P1R_THREADS)
+phi1_run_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
+            const __grid_constant__ CUtensorMap tmH, const P1Params p) {
+  using L = P1RLayout;
+  constexpr int D = L::D, NH = L::NH;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const uint32_t sbase = smem_u32(smem);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::BAR_OFF);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::BAR_OFF + 120);
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::BAR_OFF + 124);
+  float* sBias = reinterpret_cast<float*>(smem + L::BIAS_OFF);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int t0 = (int)((long long)blockIdx.x * p.total / gridDim.x), t1 = (int)((long long)(blockIdx.x + 1) * p.total / gridDim.x);
+  const WaitCtx wc{p.status, abort_flag};
+  auto bar_x = [&](int s) { return smem_u32(bars + s); };                            // ring slot s: its tile has arrived
+  auto bar_x_empty = [&](int s) { return smem_u32(bars + P1R_RING + s); };            // read by the products and, for softmax rows, by the eight warps
+  auto bar_w = [&](int j) { return smem_u32(bars + 2 * P1R_RING + j); };              // a head's weights of slice j
+  const uint32_t bar_w_free = smem_u32(bars + 2 * P1R_RING + 2);                      // the last product with them has completed
+  auto bar_done = [&](int b, int j) { return smem_u32(bars + 2 * P1R_RING + 3 + 2 * b + j); };   // accumulators b: slice j's product has completed
+  auto bar_free = [&](int b) { return smem_u32(bars + 2 * P1R_RING + 7 + b); };       // accumulators b have been read
+  static_assert((2 * P1R_RING + 9) * 8 <= 120);
+
+  const int quad = warp & 3, hf = (warp >> 2) & 1, r = quad * 32 + lane;
+  auto head_of = [&](int t) { return t / p.tiles % p.H; };
+  auto rank_of = [&](int t) {            // of the sixteen rows of tile t whose softmax rows this warp copies
+    const int row = t % p.tiles * 128 + r;
+    return p.ks_w != nullptr && warp < 8 && lane / 16 == hf && t < t1 && row < p.N ? p.sm_rank[row] : -1;
+  };
+  auto load_bias = [&](int h) {          // by the eight warps
+    for (int i = threadIdx.x; i < NH * D; i += 256)
+      sBias[i] = (p.bias != nullptr && i < p.hid) ? __bfloat162float(p.bias[(size_t)h * p.hid + i]) : 0.f;
+  };
+  __shared__ uint32_t s_skip;
+  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (threadIdx.x == 0) {
+    *abort_flag = 0u;
+    for (int s = 0; s < P1R_RING; ++s) { mbar_init(bar_x(s), 1); mbar_init(bar_x_empty(s), p.ks_w != nullptr ? 9 : 1); }
+    for (int j = 0; j < 2; ++j) {
+      mbar_init(bar_w(j), 1);
+      mbar_init(bar_free(j), 8);
+      for (int b = 0; b < 2; ++b) mbar_init(bar_done(b, j), 1);
+    }
+    mbar_init(bar_w_free, 1);
+    fence_barrier_init();
+    fence_proxy_async();
+  }
+  if (warp == 8 && lane == 0) { tma_prefetch_desc(&tmX); tma_prefetch_desc(&tmW); tma_prefetch_desc(&tmH); }
+  if (warp == 9) { tmem_alloc(smem_u32(tmem_slot), L::COLS); tmem_relinquish(); }   // (dependents let in early gain nothing)
+  int rank_now = rank_of(t0), rank_next = rank_of(t0 + 1);     // two tiles ahead: a load behind copies of tiles takes microseconds
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  griddep_wait();                                    // the set-up above ran beside the kernel before this one
+  if (s_skip != 0u) {                                // an earlier launch timed out: do nothing
+    if (warp == 9) tmem_dealloc(tmem, L::COLS);
+    return;
+  }
+
+  if (warp == 8) {
+    if (lane == 0) {
+      uint32_t n_w = 0;
+      for (int t = t0, i = 0; t < t1; ++t, ++i) {
+        const int bh = t / p.tiles, h = bh % p.H, s = i % P1R_RING;
+        if (i >= P1R_RING && !mbar_wait(bar_x_empty(s), (i / P1R_RING - 1) & 1, wc)) break;
+        mbar_expect_tx(bar_x(s), L::TILE);
+        load_tile<D>(sbase + L::X_OFF + s * L::TILE, &tmX, bar_x(s), (t - bh * p.tiles) * 128, bh);
+        if (i > 0 && h == head_of(t - 1)) continue;
+        if (i > 0 && !mbar_wait(bar_w_free, (n_w - 1) & 1, wc)) break;
+        for (int j = 0; j < NH; ++j) {
+          mbar_expect_tx(bar_w(j), L::TILE);
+          load_tile<D>(sbase + L::W_OFF + j * L::TILE, &tmW, bar_w(j), j * 128, h);   // W_1[h] rows of slice j (past hid: zeros)
+        }
+        ++n_w;
+      }
+    }
+    __syncwarp();
+  } else if (warp == 9) {
+    uint32_t n_w = 0;
+    bool ok = true;
+    for (int t = t0, i = 0; ok && t < t1; ++t, ++i) {
+      const int s = i % P1R_RING, b = i & 1;
+      const bool first = i == 0 || head_of(t) != head_of(t - 1), last = t + 1 < t1 && head_of(t) != head_of(t + 1);
+      if (i >= 2) ok = mbar_wait_warp(bar_free(b), ((i >> 1) - 1) & 1, wc);
+      ok = ok && mbar_wait_warp(bar_x(s), (i / P1R_RING) & 1, wc);
+      for (int j = 0; j < NH; ++j) {         // X W_1^T: the D hidden units of slice j
+        if (first) ok = ok && mbar_wait_warp(bar_w(j), n_w & 1, wc);
+        if (!ok) break;
+        tc_fence_after();
+        if (elect_one()) {
+          issue_kmajor<D>(tmem + (b * NH + j) * D, kmajor_desc(sbase + L::X_OFF + s * L::TILE), kmajor_desc(sbase + L::W_OFF + j * L::TILE),
+                          make_idesc(128, D, 0, 0), false);
+          tc_commit(bar_done(b, j));
+          if (j == NH - 1 && t + P1R_RING < t1) tc_commit(bar_x_empty(s));
+          if (j == NH - 1 && last) tc_commit(bar_w_free);
+        }
+        __syncwarp();
+      }
+      n_w += first ? 1 : 0;
+    }
+  } else {
+    const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
+    bool ok = true;
+    load_bias(head_of(t0));                                     // (they meet below before the first look at it)
+    for (int t = t0, i = 0; t < t1; ++t, ++i) {
+      const int bh = t / p.tiles, s = i % P1R_RING, b = i & 1, row0 = (t - bh * p.tiles) * 128;
+      const int rank = rank_now;
+      rank_now = rank_next;
+      rank_next = rank_of(t + 2);
+      if (i > 0 && p.bias != nullptr && bh % p.H != head_of(t - 1)) {
+        load_bias(bh % p.H);                                    // (all have read the old one: they met behind it)
+      }
+      if (p.ks_w != nullptr) {
+        // sixteen rows of the K tile; D / 8 lanes a row
+        constexpr int CH = D / 8, RPI = 32 / CH;
+        uint32_t bits = __ballot_sync(0xffffffffu, rank >= 0);
+        if (ok) ok = mbar_wait_warp(bar_x(s), (i / P1R_RING) & 1, wc);
+        while (ok && bits) {
+          int src = -1;
+#pragma unroll
+          for (int i = 0; i < RPI; ++i) {
+            if (bits) {
+              if (lane / CH == i) src = __ffs(bits) - 1;
+              bits &= bits - 1;
+            }
+          }
+          const int to = __shfl_sync(0xffffffffu, rank, src < 0 ? 0 : src);
+          if (src >= 0) {
+            const int c = lane % CH;
+            const uint4 val = *reinterpret_cast<const uint4*>(smem + L::X_OFF + s * L::TILE + (c / 8) * BOX_BYTES +
+                                                              swz128_chunk_offset(quad * 32 + src, c % 8));
+            *reinterpret_cast<uint4*>(p.ks_w + ((size_t)bh * p.n_s + to) * D + c * 8) = val;
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_x_empty(s));
+      }
+      uint32_t x[32];
+#pragma unroll
+      for (int j = 0; j < NH; ++j) {
+        const int out = L::OUT_OFF + ((i * NH + j) & 1) * L::TILE;
+        if (ok) ok = mbar_wait_warp(bar_done(b, j), (i >> 1) & 1, wc);
+        if (threadIdx.x == 0) tma_store_wait_read_but_last();   // the store before the last one has read its tile, which is `out`
+        named_barrier_sync(1, 256);                             // these two are reached by every epilogue thread, also after a failed wait
+        if (ok) {
+          tc_fence_after();
+#pragma unroll
+          for (int c = 0; c < D / 64; ++c) {
+            const int col = hf * (D / 2) + c * 32;
+            tmem_ld32(tmem + lane_off + (b * NH + j) * D + col, x);
+            tmem_ld_wait(x);
+            const float* bb = sBias + j * D + col;
+            uint32_t w[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              w[i] = pack_bf16(fmaxf(__uint_as_float(x[2 * i]) + bb[2 * i], 0.f), fmaxf(__uint_as_float(x[2 * i + 1]) + bb[2 * i + 1], 0.f));
+            store_row_chunk(smem + out, r, col, w);
+          }
+          fence_proxy_async();
+          if (j == NH - 1) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_free(b));
+          }
+        }
+        named_barrier_sync(1, 256);
+        if (ok && threadIdx.x == 0) {
+#pragma unroll
+          for (int q = 0; q < D / 64; ++q) tma_store_3d(&tmH, sbase + out + q * BOX_BYTES, j * D + q * 64, row0, bh);
+          tma_store_commit();
+        }
+      }
+    }
+    if (threadIdx.x == 0) tma_store_wait_read();              // (the writes land by the end of the kernel)
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 9) {
+    tc_fence_after();
+    tmem_dealloc(tmem, L::COLS);
   }
 }
 
@@ -654,9 +848,9 @@ cudaError_t as_tensor_init_kpass() {
   if ((e = opt_in_smem(kpass_kernel<128, 2, 1>, KLayout<128, 2, 1>::TOTAL)) != cudaSuccess) return e;
   if ((e = opt_in_smem(kpass_kernel<128, 2, 2>, KLayout<128, 2, 2>::TOTAL)) != cudaSuccess) return e;
   if ((e = opt_in_smem(kpass_kernel<64, 2, 1>, KLayout<64, 2, 1>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(phi1_kernel<128, 1>, P1Layout<128, 1>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(phi1_kernel<128, 2>, P1Layout<128, 2>::TOTAL)) != cudaSuccess) return e;
-  if ((e = opt_in_smem(phi1_kernel<64, 1>, P1Layout<64, 1>::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(phi1_kernel<128>, P1Layout<128>::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(phi1_run_kernel, P1RLayout::TOTAL)) != cudaSuccess) return e;
+  if ((e = opt_in_smem(phi1_kernel<64>, P1Layout<64>::TOTAL)) != cudaSuccess) return e;
   return cudaSuccess;
 }
 
@@ -667,11 +861,17 @@ cudaError_t as_tensor_phi1(const as_launch_args& a, cudaStream_t st) {
   if (!make_map(&tmX, a.k, a.d, a.N, BH, 128) || !make_map(&tmW, a.wk, a.d, a.hid, a.H, 128) ||
       !make_map(&tmH, a.h1k, a.hid, a.N, BH, 128))
     return cudaErrorInvalidValue;
-  P1Params p{a.H, a.hid, a.N, a.n_s, a.bk1, a.sm_rank, a.ks_w, a.status};
-  dim3 grid((a.N + 127) / 128, BH, 1);
-  if (a.d == 128 && a.hid == 256) return as_launch_dependent(phi1_kernel<128, 2>, grid, dim3(P1_THREADS), P1Layout<128, 2>::TOTAL, st, tmX, tmW, tmH, p);
-  if (a.d == 128) return as_launch_dependent(phi1_kernel<128, 1>, grid, dim3(P1_THREADS), P1Layout<128, 1>::TOTAL, st, tmX, tmW, tmH, p);
-  return as_launch_dependent(phi1_kernel<64, 1>, grid, dim3(P1_THREADS), P1Layout<64, 1>::TOTAL, st, tmX, tmW, tmH, p);
+  const int tiles = (a.N + 127) / 128;
+  P1Params p{a.H, a.hid, a.N, a.n_s, tiles, tiles * BH, a.bk1, a.sm_rank, a.ks_w, a.status};
+  if (a.d == 128 && a.hid == 256) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
+      return cudaErrorInvalidValue;
+    return as_launch_dependent(phi1_run_kernel, dim3(std::min(p.total, sms)), dim3(P1R_THREADS), P1RLayout::TOTAL, st, tmX, tmW, tmH, p);
+  }
+  dim3 grid(tiles, BH, 1);
+  if (a.d == 128) return as_launch_dependent(phi1_kernel<128>, grid, dim3(P1_THREADS), P1Layout<128>::TOTAL, st, tmX, tmW, tmH, p);
+  return as_launch_dependent(phi1_kernel<64>, grid, dim3(P1_THREADS), P1Layout<64>::TOTAL, st, tmX, tmW, tmH, p);
 }
 
 cudaError_t as_tensor_kpass(const as_launch_args& a, cudaStream_t st) {

@@ -48,3 +48,37 @@ def test_rows_and_state(B, H, N, d, F, layers, tokens):
             assert bool((diff <= 2.0 ** -8 * size + 1e-5 * size.max()).all()), float((diff / (size + 1e-9)).max())
         else:
             assert float(diff.norm()) <= 2.0 ** -8 * float(size.norm())
+
+
+# (B, H, N, d, width): one tile; fewer tiles than SMs; two tiles a head, so that a run of tiles goes through several heads (of one batch row and the next);
+# runs of a few tiles and of ten, which end inside heads
+@pytest.mark.parametrize("B,H,N,d,width", [(1, 1, 128, 64, 64), (2, 3, 300, 128, 128), (3, 50, 130, 128, 128), (2, 97, 200, 64, 64), (2, 40, 701, 64, 64),
+                                           (1, 60, 1031, 128, 256), (2, 1, 20001, 128, 256), (1, 12, 15600, 128, 256)])
+@pytest.mark.parametrize("bias", [False, True])
+def test_first_layer_over_runs_of_tiles(B, H, N, d, width, bias):
+    import torch
+    from paper_2509_24899_b200 import HybridAttention
+    g = torch.Generator(device="cuda").manual_seed(N + d)
+
+    def draw(*shape):
+        return torch.randn(shape, device="cuda", generator=g).bfloat16()
+
+    k, v, w1, w2 = draw(B, H, N, d), draw(B, H, N, d), draw(H, width, d) * 0.1, draw(H, width, width) * 0.1
+    b1 = draw(H, width)
+    biases = {n: b1 if n == "bk1" else torch.zeros_like(b1) for n in ("bq1", "bk1", "bq2", "bk2")} if bias else None
+    idx = list(range(0, N, 3))
+    op = HybridAttention(B, H, N, d, (1, 1, N), (1, 1, N), 3, softmax_idx=idx, phi_dim=width, phi_layers=2, phi_hidden=width)
+    for _ in range(2):
+        ks, vs, S, z = op.key_pass(k, v, w1, w1, wk2=w2, wq2=w2, biases=biases)
+    assert op.last_status() == 0
+    at = torch.tensor(idx, device="cuda")
+    assert torch.equal(ks, k[:, :, at].reshape(B * H, len(idx), d)) and torch.equal(vs, v[:, :, at].reshape(B * H, len(idx), d))
+    linear = torch.ones(N, device="cuda", dtype=torch.float64)
+    linear[at] = 0
+    h1 = torch.relu(k.double() @ w1.double().transpose(-1, -2) + (b1.double()[:, None] if bias else 0)).bfloat16().double()
+    phi = torch.relu(h1 @ w2.double().transpose(-1, -2)) * linear[:, None]
+    phi[..., width // 2:] **= 2
+    # features rounded to bf16, 2^-8 of themselves at most; head by head, so that one head with another's weights cannot hide among the others
+    for got, ref, size in ((S, phi.transpose(-1, -2) @ v.double(), phi.transpose(-1, -2) @ v.double().abs()), (z, phi.sum(2), phi.sum(2))):
+        diff = (got.double().reshape(ref.shape) - ref).flatten(2).norm(dim=2)
+        assert bool((diff <= 2.0 ** -8 * size.flatten(2).norm(dim=2)).all())
