@@ -309,7 +309,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     const int part = p.F / p.P;
     const int pw = min(f / part, p.P - 1) + 1;                 // power of this feature's part (the same in a whole warp
                                                                // whenever the part width is a multiple of 32)
-    const float bias = (p.bias != nullptr && f < p.F) ? __bfloat162float(p.bias[(size_t)h * p.F + f]) : 0.f;
+    float bias = 0.f;                                          // the caller's: not before the wait for the kernel before this one
     float z0 = 0.f, z1 = 0.f;
     bool ok = true;
     uint32_t x[32];
@@ -362,6 +362,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       if (t < 0) {
         z0 = 0.f; z1 = 0.f;
         griddep_wait();
+        if (p.bias != nullptr && f < p.F) bias = __bfloat162float(p.bias[(size_t)h * p.F + f]);
         continue;
       }
       mbar_arrive(bar(B_PK + b));

@@ -43,6 +43,47 @@ def test_a_forward_right_behind_the_kernel_that_writes_its_input(name):
         assert torch.equal(got, want), n
 
 
+@pytest.mark.parametrize("name", ["hybrid_d128", "hybrid_d64", "linear_d128", "linear_d64", "two_layers"])
+def test_a_forward_right_behind_the_kernel_that_writes_its_weights(name):
+    """Weights and biases written by an ordinary kernel, and by one of the library's, which lets dependents in long before it writes: a query stage of a
+    few CTAs beside which the whole call finds room to set up."""
+    import torch
+    from paper_2509_24899_b200 import HybridAttention
+    wl, dev, op, second = _layer(**LAYERS[name])
+    g = torch.Generator(device="cuda").manual_seed(7)
+    before = HybridAttention(1, 1, 4096, 64, (1, 1, 4096), (1, 1, 4096), 1)
+    x = [torch.randn((1, 1, 4096, 64), device="cuda", generator=g).bfloat16() for _ in range(2)] + \
+        [torch.randn((1, 1, 4096, 64), device="cuda", generator=g).bfloat16() * 8]
+    written = before.forward(*x).clone()
+    H, hid, F = wl.H, wl.hidden or op.F, op.F
+    sizes = {"wq": (H, hid, wl.d), "wk": (H, hid, wl.d), "bq1": (H, hid), "bk1": (H, hid)}
+    if second:
+        sizes.update(wq2=(H, F, hid), wk2=(H, F, hid), bq2=(H, F), bk2=(H, F))
+
+    def run(w):
+        bias = {n: w[n] for n in sizes if n[0] == "b"}
+        out = op.forward(dev["q"], dev["k"], dev["v"], w["wq"], w["wk"], biases=bias, **{n: w[n] for n in second})
+        return out.view(torch.int16)                             # (bits: a row without a feature above 0 is no number)
+
+    w = {n: dev[n] if n in dev else torch.randn(size, device="cuda", generator=g).bfloat16() for n, size in sizes.items()}
+    for n, size in sizes.items():
+        late = dict(w, **{n: torch.full_like(w[n], 3.0)})
+        want = run(w).clone()
+        torch.cuda.synchronize()
+        _late(late[n], w[n])
+        got = run(late)
+        assert op.last_status() == 0
+        assert torch.equal(got, want), n
+        count = late[n].numel()
+        want = run(dict(w, **{n: written.flatten()[-count:].view(size)})).clone()
+        out = torch.full_like(written, 3.0)
+        torch.cuda.synchronize()
+        before.forward(*x, out=out)
+        got = run(dict(w, **{n: out.flatten()[-count:].view(size)}))
+        assert op.last_status() == 0
+        assert torch.equal(got, want), n
+
+
 @pytest.mark.parametrize("with_state", [False, True])
 @pytest.mark.parametrize("d", [64, 128])
 def test_a_query_pass_right_behind_the_kernel_that_writes_its_input(d, with_state):
