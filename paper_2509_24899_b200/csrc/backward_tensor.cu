@@ -171,7 +171,7 @@ btq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (threadIdx.x == 32) *skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (threadIdx.x == 32) *skip = status_now(p.status);
   if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   if (threadIdx.x == 17 * 32) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmY); tma_prefetch_desc(&tmH); tma_prefetch_desc(&tmW); tma_prefetch_desc(&tmS); }
   tc_fence_before();
@@ -363,9 +363,10 @@ btq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
       }
     }
     // ---- the chunk's partial results
+    const uint32_t late = status_now(p.status);      // behind the wait, ahead of the first write: not 0, and nothing is written
     if (ok && nt > 0) ok = mbar_wait_warp(bar(Q_END), 0, wc);
     const size_t slot = (size_t)bh * p.chunks + chunk;
-    if (ok && nt > 0) {
+    if (ok && late == 0u && nt > 0) {
       tc_fence_after();
       bt_store_acc(tdS + lane_off + cg * 32, p.part_dS + (slot * 128 + r) * 128 + cg * 32);
       bt_store_acc(tdW + lane_off + cg * 32, p.part_dW + (slot * 128 + r) * 128 + cg * 32);
@@ -377,8 +378,8 @@ btq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, off);
     if (lane == 0 && warp >= 8) red[256 + warp - 8] = loss;
     named_barrier_sync(1, BT_COMPUTE);
-    if (cg == 0) p.part_dz[slot * 128 + r] = red[r] + red[128 + r];
-    if (threadIdx.x == 128) {
+    if (cg == 0 && late == 0u) p.part_dz[slot * 128 + r] = red[r] + red[128 + r];
+    if (threadIdx.x == 128 && late == 0u) {
       float l = 0.f;
       for (int w = 0; w < 8; ++w) l += red[256 + w];
       p.part_loss[slot] = l;
@@ -455,7 +456,7 @@ btk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (threadIdx.x == 32) *skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (threadIdx.x == 32) *skip = status_now(p.status);
   if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   if (threadIdx.x == 17 * 32) { tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); tma_prefetch_desc(&tmW); tma_prefetch_desc(&tmS); }
   tc_fence_before();
@@ -557,8 +558,9 @@ btk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
       }
       mbar_arrive(bar(K_PRDY + grp));
     }
+    const uint32_t late = status_now(p.status);      // behind the wait, ahead of the first write: not 0, and nothing is written
     if (ok && nt > 0) ok = mbar_wait_warp(bar(K_END), 0, wc);
-    if (ok && nt > 0) {
+    if (ok && late == 0u && nt > 0) {
       tc_fence_after();
       const size_t slot = (size_t)bh * p.chunks + chunk;
       bt_store_acc(tmem + 256 + lane_off + cg * 32, p.part_dW + (slot * 128 + r) * 128 + cg * 32);

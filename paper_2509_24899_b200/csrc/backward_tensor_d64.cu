@@ -152,7 +152,7 @@ bsq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     fence_proxy_async();
   }
   __shared__ uint32_t s_skip;
-  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (threadIdx.x == 32) s_skip = status_now(p.status);
   if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 256); tmem_relinquish(); griddep_launch(); }
   if (threadIdx.x == 15 * 32) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmY); tma_prefetch_desc(&tmH); tma_prefetch_desc(&tmW); }
   tc_fence_before();
@@ -300,13 +300,15 @@ bsq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
       mbar_arrive(bar(Q_XRDY));
     }
     // ---- the chunk's partial results
+    const uint32_t late = status_now(p.status);      // behind the wait, ahead of the first write: not 0, and nothing is written
     if (ok && nt > 0) ok = mbar_wait_warp(bar(Q_DONE), (nt - 1) & 1, wc);
     const size_t slot = (size_t)bh * p.chunks + chunk;
     if (ok && nt > 0) {
       add_acc16(t_own, acc);
       float* dst = (r < 64 ? p.part_dS : p.part_dW) + (slot * 64 + (r & 63)) * 64 + cg * 16;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) reinterpret_cast<float4*>(dst)[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
+      for (int i = 0; i < 4; ++i)
+        if (late == 0u) reinterpret_cast<float4*>(dst)[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
     }
     // dz: over the warp's 32 rows by shuffles, then the four row blocks in order; the loss: the warps' sums in order
     float* red = reinterpret_cast<float*>(smem + L::X_OFF);       // idle: the last product has read it
@@ -320,9 +322,9 @@ bsq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, off);
     if (lane == 0) red[256 + warp] = loss;
     named_barrier_sync(1, BS_COMPUTE);
-    if (threadIdx.x < 64)
+    if (threadIdx.x < 64 && late == 0u)
       p.part_dz[slot * 64 + threadIdx.x] = (red[threadIdx.x] + red[64 + threadIdx.x]) + (red[128 + threadIdx.x] + red[192 + threadIdx.x]);
-    if (threadIdx.x == 64) {
+    if (threadIdx.x == 64 && late == 0u) {
       float l = 0.f;
       for (int i = 0; i < 16; ++i) l += red[256 + i];
       p.part_loss[slot] = l;
@@ -382,7 +384,7 @@ bsk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
     fence_proxy_async();
   }
   __shared__ uint32_t s_skip;
-  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (threadIdx.x == 32) s_skip = status_now(p.status);
   if (warp == 16) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   if (threadIdx.x == 15 * 32) { tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); tma_prefetch_desc(&tmW); }
   tc_fence_before();
@@ -489,6 +491,7 @@ bsk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
       fence_proxy_async();
       mbar_arrive(bar(K_XRDY + (t & 1)));
     }
+    const uint32_t late = status_now(p.status);      // behind the wait, ahead of the first write: not 0, and nothing is written
     for (int t = nt > 1 ? nt - 2 : 0; t < nt; ++t) {
       if (ok) ok = mbar_wait_warp(bar(K_DONE + (t & 1)), (t >> 1) & 1, wc);
       if (ok) add_tile(t);
@@ -500,7 +503,7 @@ bsk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUte
       for (int i = 0; i < 16; ++i) red[(cg * 16 + i) * 64 + (r - 64)] = acc[i] + accl[i];
     }
     named_barrier_sync(1, BS_COMPUTE);
-    if (ok && nt > 0 && r < 64) {
+    if (ok && late == 0u && nt > 0 && r < 64) {
       float* dst = p.part_dW + ((((size_t)bh * p.chunks + chunk) * 64) + r) * 64 + cg * 16;
 #pragma unroll
       for (int i = 0; i < 16; ++i) dst[i] = acc[i] + red[(cg * 16 + i) * 64 + r];

@@ -47,6 +47,30 @@ struct WaitCtx {
   volatile uint32_t* abort;     // shared-memory flag of this CTA
 };
 constexpr long long kWaitLimitCycles = 2000ll * 1000ll * 1000ll;
+// The status word as it stands: not 0 where a wait has run out, in an earlier launch or in another CTA of this one.  A dependent launch looks at it beside the
+// kernel before it, so as to return at once, and AGAIN behind griddep_wait, ahead of what it writes first: a time-out of that kernel comes after the first
+// look, and nothing may be written after one.
+AS_DEV uint32_t status_now(const uint32_t* status) { return *reinterpret_cast<const volatile uint32_t*>(status); }
+// The second look: asked for by one thread of a CTA as a copy of 16 bytes into shared memory, told by `bar` (one arrival) ...
+AS_DEV void status_again(uint32_t smem16, const uint32_t* status, uint32_t bar) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n\tcp.async.mbarrier.arrive.noinc.shared::cta.b64 [%2];" ::"r"(smem16), "l"(status), "r"(bar) : "memory");
+}
+// ... and whether it was 0: asked by those who write, while they have no tile yet.  (A load by every warp that writes - two thousand of one address while the first
+// tiles come - cost calls of 15 - 20 us 2 - 4 %, a copy by the producer as long, a look ahead of each first store or by the warp that issues the first products 1 %.)
+AS_DEV bool status_clear(uint32_t bar, uint32_t smem16) {
+  for (uint32_t it = 0; !mbar_try_wait(bar, 0); ++it)
+    if (it > 1000000u) return false;                 // (the other roles report it, where they wait for who asked)
+  uint32_t word;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(word) : "r"(smem16) : "memory");
+  return word == 0u;
+}
+// If it was not, by the same: the other roles of the CTA find the abort flag where they wait for these, and the CTA stays until the copies that have been asked for have
+// landed (20 us: they take two).
+AS_DEV void status_give_up(const WaitCtx& w) {
+  *w.abort = 1u;
+  const long long t0 = clock64();
+  while (clock64() - t0 < 40000) {}
+}
 
 AS_DEV bool mbar_wait_limit(uint32_t bar, uint32_t parity, const WaitCtx& w, long long limit_cycles) {
   if (mbar_try_wait(bar, parity)) return true;

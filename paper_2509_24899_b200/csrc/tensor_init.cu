@@ -35,6 +35,7 @@ namespace {
 __global__ void expire_wait_kernel(uint32_t* status, long long limit_cycles) {
   __shared__ uint64_t bar;
   __shared__ uint32_t abort_flag;
+  sm100::griddep_launch();               // as the kernels of a forward: what comes next sets up, and looks at the status word, before this wait runs out
   if (threadIdx.x == 0) {
     abort_flag = 0u;
     sm100::mbar_init(sm100::smem_u32(&bar), 1);

@@ -132,7 +132,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   // ---- Set-up that runs beside the kernel before this one.  The table of softmax ranks is the handle's and does not change; and the status word is asked
   // for here because small loads that come behind the first tiles' wait as long as these do (4 us at N = 7800, 12 heads).
   __shared__ uint32_t s_skip;
-  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (threadIdx.x == 32) s_skip = status_now(p.status);
   if (warp == 9) {
     // the query stage's CTAs may then set up as these ones end
     tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch();
@@ -177,6 +177,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     if (warp == 9) tmem_dealloc(*tmem_slot, 512);
     return;
   }
+  __shared__ volatile uint32_t s_late;                       // the status word behind the wait: not 0, and nothing is written
   if (warp >= 8) griddep_wait();                             // (the feature warps: see their loop)
   const uint32_t tmem = *tmem_slot;
   const uint32_t tD1[2] = {tmem + 0u, tmem + 128u};          // Phi^T of a tile, fp32
@@ -247,6 +248,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     }
   } else if (warp >= 11) {
     // ------------------------------------------------------------ gather of softmax-token rows
+    const uint32_t late = gathers || warp == 11 ? status_now(p.status) : 0u;
     if (gathers) {
       const int gw = warp & 1 ? 0 : 1;
       // rows handled by this warp: gw*64 .. gw*64+63; two ranks per lane
@@ -273,7 +275,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
         const uint8_t* from = (is_v ? vt : kt) + (c / 8) * BOX_BYTES;
         __nv_bfloat16* to = (is_v ? p.vs_w : p.ks_w) + (size_t)bh * p.n_s * D + c * 8;
         for (int e = 0; e < 2; ++e) {
-          const int mine = e == 0 ? rk[0] : rk[1];
+          const int mine = late != 0u ? -1 : e == 0 ? rk[0] : rk[1];
           uint32_t bits = __ballot_sync(0xffffffffu, mine >= 0);
           while (bits) {
             int src[AHEAD], rank[AHEAD];
@@ -299,6 +301,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
           for (int i = LAYERS == 1 ? 0 : NX; i < IPT; ++i) mbar_arrive(bar(B_EMPTY + (t * IPT + i) % SLOTS));
       }
     }
+    if (threadIdx.x == 11 * 32) s_late = late;
     named_barrier_arrive(2, K_FEATURE_THREADS + 64);           // the feature warps may reuse the ring for the partial S
   } else {
     // ------------------------------------------------------------ feature warps: lane of TMEM = feature
@@ -391,7 +394,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       }
     }
     named_barrier_sync(1, K_FEATURE_THREADS);
-    if (ok) {
+    if (ok && s_late == 0u) {
       constexpr int LPR = D / 4, RPW = 32 / LPR;               // lanes a row, rows an instruction
       const size_t slot = ((size_t)bh * p.n_chunks + chunk) * p.F + fc * 128;
       const int nf = min(128, p.F - fc * 128);
@@ -409,6 +412,7 @@ kpass_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
+  if (s_late != 0u) return;
   // ---- The chunks' partial states are added up here, in chunk order (fixed order, no float atomics): every CTA of
   // a (batch, head, feature chunk) takes a slice of the [F x (D + 1)] entries once all of them have stored theirs.
   // The CTAs of a launch are resident together where nothing else is on the GPU (one per SM at most).  A CTA that has waited for kSumPatience for
@@ -523,23 +527,27 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::BAR_OFF + 36);
   float* sBias = reinterpret_cast<float*>(smem + L::BIAS_OFF);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t s_late = sbase + L::BAR_OFF + 48;               // the status word behind the wait: not 0, and nothing is written
   const int bh = blockIdx.y, h = bh % p.H, row0 = blockIdx.x * 128;
   const WaitCtx wc{p.status, abort_flag};
   const uint32_t bar_full = smem_u32(bars);
   const uint32_t bar_done = smem_u32(bars + 1);                  // the product has completed
+  const uint32_t bar_late = smem_u32(bars + 2);                  // the status word is there
   constexpr int TM_COLS = 128;
 
   __shared__ uint32_t s_skip;
-  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (threadIdx.x == 32) s_skip = status_now(p.status);
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
     mbar_init(bar_full, 1);
     mbar_init(bar_done, 1);
+    mbar_init(bar_late, 1);
     fence_barrier_init();
     fence_proxy_async();
   }
   if (warp == 8) { tmem_alloc(smem_u32(tmem_slot), TM_COLS); tmem_relinquish(); }
   griddep_wait();                                    // the set-up above ran beside the kernel before this one
+  if (threadIdx.x == 0) status_again(s_late, p.status, bar_late);   // (the thread that has made the barrier)
   for (int i = threadIdx.x; i < D; i += P1_THREADS)
     sBias[i] = (p.bias != nullptr && i < p.hid) ? __bfloat162float(p.bias[(size_t)h * p.hid + i]) : 0.f;
   tc_fence_before();
@@ -571,8 +579,9 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
   } else {
     const int quad = warp & 3, hf = warp >> 2, r = quad * 32 + lane;
     const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
+    const bool live = __all_sync(0xffffffffu, status_clear(bar_late, s_late));
     bool ok = true;
-    if (p.ks_w != nullptr) {
+    if (live && p.ks_w != nullptr) {
       // sixteen rows of the K tile; D / 8 lanes a row
       constexpr int CH = D / 8, RPI = 32 / CH;
       const int rank = lane / 16 == hf && row0 + r < p.N ? p.sm_rank[row0 + r] : -1;
@@ -615,7 +624,7 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
       fence_proxy_async();
     }
     named_barrier_sync(1, 256);                               // reached by every epilogue thread, also after a failed wait
-    if (ok && threadIdx.x == 0) {
+    if (ok && live && threadIdx.x == 0) {
 #pragma unroll
       for (int b = 0; b < D / 64; ++b) tma_store_3d(&tmH, sW + b * BOX_BYTES, b * 64, row0, bh);
       tma_store_commit();
@@ -644,7 +653,7 @@ struct P1RLayout {
   static constexpr int D = 128, NH = 2;
   static constexpr int TILE = 128 * D * 2;
   static constexpr int W_OFF = 0, X_OFF = NH * TILE, OUT_OFF = X_OFF + P1R_RING * TILE, BAR_OFF = OUT_OFF + 2 * TILE;
-  static constexpr int BIAS_OFF = BAR_OFF + 128;                // NH * D floats
+  static constexpr int BIAS_OFF = BAR_OFF + 192;                // NH * D floats
   static constexpr int TOTAL = BIAS_OFF + NH * D * 4 + 1024;
   static constexpr int COLS = 2 * NH * D;                       // tensor memory: two tiles' products
   static_assert(TOTAL <= 227 * 1024 && COLS == 512);
@@ -659,8 +668,9 @@ phi1_run_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::BAR_OFF);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::BAR_OFF + 120);
-  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::BAR_OFF + 124);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::BAR_OFF + 160);
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::BAR_OFF + 164);
+  __shared__ __align__(16) volatile uint32_t s_late[4];        // the status word behind the wait: not 0, and nothing is written
   float* sBias = reinterpret_cast<float*>(smem + L::BIAS_OFF);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t0 = (int)((long long)blockIdx.x * p.total / gridDim.x), t1 = (int)((long long)(blockIdx.x + 1) * p.total / gridDim.x);
@@ -671,7 +681,8 @@ phi1_run_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   const uint32_t bar_w_free = smem_u32(bars + 2 * P1R_RING + 2);                      // the last product with them has completed
   auto bar_done = [&](int b, int j) { return smem_u32(bars + 2 * P1R_RING + 3 + 2 * b + j); };   // accumulators b: slice j's product has completed
   auto bar_free = [&](int b) { return smem_u32(bars + 2 * P1R_RING + 7 + b); };       // accumulators b have been read
-  static_assert((2 * P1R_RING + 9) * 8 <= 120);
+  const uint32_t bar_late = smem_u32(bars + 2 * P1R_RING + 9);                        // the status word is there
+  static_assert((2 * P1R_RING + 10) * 8 <= 160);
 
   const int quad = warp & 3, hf = (warp >> 2) & 1, r = quad * 32 + lane;
   auto head_of = [&](int t) { return t / p.tiles % p.H; };
@@ -684,7 +695,7 @@ phi1_run_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       sBias[i] = (p.bias != nullptr && i < p.hid) ? __bfloat162float(p.bias[(size_t)h * p.hid + i]) : 0.f;
   };
   __shared__ uint32_t s_skip;
-  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);
+  if (threadIdx.x == 32) s_skip = status_now(p.status);
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
     for (int s = 0; s < P1R_RING; ++s) { mbar_init(bar_x(s), 1); mbar_init(bar_x_empty(s), p.ks_w != nullptr ? 9 : 1); }
@@ -694,6 +705,7 @@ phi1_run_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       for (int b = 0; b < 2; ++b) mbar_init(bar_done(b, j), 1);
     }
     mbar_init(bar_w_free, 1);
+    mbar_init(bar_late, 1);
     fence_barrier_init();
     fence_proxy_async();
   }
@@ -729,6 +741,8 @@ phi1_run_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     }
     __syncwarp();
   } else if (warp == 9) {
+    if (lane == 0) status_again(smem_u32(const_cast<uint32_t*>(s_late)), p.status, bar_late);
+    __syncwarp();
     uint32_t n_w = 0;
     bool ok = true;
     for (int t = t0, i = 0; ok && t < t1; ++t, ++i) {
@@ -753,8 +767,9 @@ phi1_run_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     }
   } else {
     const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
-    bool ok = true;
     load_bias(head_of(t0));                                     // (they meet below before the first look at it)
+    bool ok = __all_sync(0xffffffffu, status_clear(bar_late, smem_u32(const_cast<uint32_t*>(s_late))));
+    if (!ok) status_give_up(wc);                                // the launch before has timed out: nothing is written
     for (int t = t0, i = 0; t < t1; ++t, ++i) {
       const int bh = t / p.tiles, s = i % P1R_RING, b = i & 1, row0 = (t - bh * p.tiles) * 128;
       const int rank = rank_now;

@@ -116,6 +116,7 @@ struct QLayout {
   static constexpr int P_OFF = 2 * TILE;                   // per group: phi_q, then the output rows
   static constexpr int KV_OFF = P_OFF + 2 * PTILE;
   static constexpr int BAR_OFF = KV_OFF + KV_STAGES * TILE;
+  static constexpr int LATE_OFF = BAR_OFF + 240;           // the status word behind the wait for the kernel before
   static constexpr int TOTAL = BAR_OFF + 256 + 1024;       // + slack for the 1024-byte alignment
 };
 
@@ -180,13 +181,14 @@ struct QRing {
   // barrier indices; per group: S (scores, hidden activations or Phi landed in the score columns), SF (score
   // columns read out), P (P in tensor memory, phi_q in shared memory), PF (the product that reads it has completed),
   // O (output accumulator final), QF (nothing of the unit reads the Q tile any more), H (two layers: the
-  // hidden activations are in shared memory); for both, a tail in columns of their own: PL (nothing reads the unit's P in tensor memory any more)
+  // hidden activations are in shared memory); for both, a tail in columns of their own: PL (nothing reads the unit's P in tensor memory any more); once: LATE (the status word is there, cf. status_again)
   // Whether a ring slot is full is told on a barrier of the warp that will use the item: KFULL for what is multiplied into the score columns (K,
   // weights), VFULL for what is added to O (V, S).  Each warp looks at every phase of its own barriers, in order.  (With one barrier for both a
   // warp would look at some of its phases only, and a wait by parity for a phase two ahead of the last one looked at passes while
   // the one between - a copy still under way for the other warp - is not over.)
   static constexpr int B_Q0 = 0, B_KFULL = 2, B_VFULL = B_KFULL + KV_STAGES, B_EMPTY = B_VFULL + KV_STAGES, B_S = B_EMPTY + KV_STAGES, B_SF = B_S + 2,
-                       B_P = B_SF + 2, B_PF = B_P + 2, B_O = B_PF + 2, B_QF = B_O + 2, B_H = B_QF + 2, B_PL = B_H + 2, B_COUNT = B_PL + 1;
+                       B_P = B_SF + 2, B_PF = B_P + 2, B_O = B_PF + 2, B_QF = B_O + 2, B_H = B_QF + 2, B_PL = B_H + 2, B_LATE = B_PL + 1, B_COUNT = B_LATE + 1;
+  static_assert(8 * B_COUNT + 8 <= L::LATE_OFF - L::BAR_OFF, "two words follow the barriers");
   const QCtx c;              // by value: nothing here is re-read from memory after a barrier or an MMA
   int nkv, lin, two, fc, nh, vl;
   int n_stream, n_items;
@@ -1143,7 +1145,7 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
-    mbar_init(bar(R::B_Q0), 1); mbar_init(bar(R::B_Q0 + 1), 1);
+    mbar_init(bar(R::B_Q0), 1); mbar_init(bar(R::B_Q0 + 1), 1); mbar_init(bar(R::B_LATE), 1);
     for (int s = 0; s < KV_STAGES; ++s) { mbar_init(bar(R::B_KFULL + s), 1); mbar_init(bar(R::B_VFULL + s), 1); mbar_init(bar(R::B_EMPTY + s), 1); }
     for (int g = 0; g < 2; ++g) {
       mbar_init(bar(R::B_S + g), 1); mbar_init(bar(R::B_SF + g), 256); mbar_init(bar(R::B_P + g), 256);
@@ -1154,7 +1156,7 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     fence_proxy_async();
   }
   __shared__ uint32_t s_skip;
-  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);    // (ahead of the wait: behind the first copies it would wait for these)
+  if (threadIdx.x == 32) s_skip = status_now(p.status);   // (ahead of the wait: behind the first copies it would wait for these)
   if (warp == 17) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   if (warp == 16 && (threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmW); tma_prefetch_desc(&tmSt); tma_prefetch_desc(&tmO); }
   tc_fence_before();
@@ -1167,6 +1169,8 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     if (warp == 17) tmem_dealloc(c.tmem, 512);
     return;
   }
+
+  if (threadIdx.x == 18 * 32) status_again(sbase + L::LATE_OFF, p.status, bar(R::B_LATE));
 
   if (warp == 16) {
     if ((threadIdx.x & 31) == 0) q_first_loads<D, MAP_ONE>(p, c, q_unit(p, 0), &tmQ, &tmQ, &tmW, &tmW);
@@ -1183,7 +1187,10 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     const int g = (warp >> 2) & 1;
     // a unit worked on by one group only is the CTA's last one: group 1 stops before it
     const int n_grp = (n_mine > p.n_rounds && g == 1 && q_unit(p, p.n_rounds).ng == 1) ? p.n_rounds : n_mine;
-    for (int u = 0; u < n_grp; ++u)
+    // not where the launch before has timed out behind the set-up's look at the status word
+    const bool start = __all_sync(0xffffffffu, status_clear(bar(R::B_LATE), sbase + L::LATE_OFF));
+    if (!start) status_give_up(c.wc);
+    for (int u = 0; start && u < n_grp; ++u)
       if (!q_linear_unit<D, GEN>(p, c, &tmO, smem, sDl, u)) break;
     if ((threadIdx.x & 31) == 0) tma_store_wait_read();
   }
@@ -1244,7 +1251,7 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 
   if (threadIdx.x == 0) {
     *abort_flag = 0u;
-    mbar_init(bar(R::B_Q0), 1); mbar_init(bar(R::B_Q0 + 1), 1);
+    mbar_init(bar(R::B_Q0), 1); mbar_init(bar(R::B_Q0 + 1), 1); mbar_init(bar(R::B_LATE), 1);
     for (int s = 0; s < KV_STAGES; ++s) { mbar_init(bar(R::B_KFULL + s), 1); mbar_init(bar(R::B_VFULL + s), 1); mbar_init(bar(R::B_EMPTY + s), 1); }
     for (int g = 0; g < 2; ++g) {
       mbar_init(bar(R::B_S + g), 1); mbar_init(bar(R::B_SF + g), X::GROUP); mbar_init(bar(R::B_P + g), X::GROUP);
@@ -1259,7 +1266,7 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   __shared__ QParams s_part[KS ? 2 : 1];
   __shared__ int s_parts;
   if (KS && threadIdx.x == 64) s_parts = q_parts<D>(p, s_part);
-  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);    // (ahead of the wait: behind the first copies it would wait for these)
+  if (threadIdx.x == 32) s_skip = status_now(p.status);   // (ahead of the wait: behind the first copies it would wait for these)
   if (warp == X::W_SCORE) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   if (warp == X::W_TMA && (threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); tma_prefetch_desc(&tmO); }
   tc_fence_before();
@@ -1273,6 +1280,8 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   const QCtx c{sbase, *tmem_slot, WaitCtx{p.status, abort_flag}};
   const int n_mine = KS ? p.n_rounds + s_parts : q_units_of_cta(p);   // units of this CTA
   auto of = [&](int u) -> const QParams& { return KS && u >= p.n_rounds ? s_part[KS ? u - p.n_rounds : 0] : p; };
+
+  if (threadIdx.x == X::W_ACCUM * 32) status_again(sbase + L::LATE_OFF, p.status, bar(R::B_LATE));
 
   if (warp == X::W_TMA) {
     if ((threadIdx.x & 31) == 0) q_first_loads<D, MAP, KS>(of(0), c, q_unit<KS>(of(0), 0), &tmQ, &tmK, &tmW, &tmW1);
@@ -1288,7 +1297,10 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   } else {
     // a unit worked on by one group only is the CTA's last one: group 1 stops before it
     const int n_grp = (!KS && n_mine > p.n_rounds && ((warp >> 2) & 1) == 1 && q_unit(p, p.n_rounds).ng == 1) ? p.n_rounds : n_mine;
-    for (int u = 0; u < n_grp; ++u)
+    // not where the launch before has timed out behind the set-up's look at the status word
+    const bool start = __all_sync(0xffffffffu, status_clear(bar(R::B_LATE), sbase + L::LATE_OFF));
+    if (!start) status_give_up(c.wc);
+    for (int u = 0; start && u < n_grp; ++u)
       if (!q_softmax_unit<D, T, MAP, GEN, KS>(of(u), c, &tmO, smem, u)) break;
     if ((threadIdx.x & 31) == 0) tma_store_wait_read();  // this warp's output stores have read their rows (the writes land by the end of the kernel)
   }

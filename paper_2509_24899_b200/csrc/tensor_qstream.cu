@@ -40,11 +40,12 @@ struct QSParams {
 struct QSLayout {
   static constexpr int W_OFF = 0, ST_OFF = TILE, Q_OFF = 2 * TILE, PHI_OFF = Q_OFF + QS_SLOTS * TILE;
   static constexpr int BAR_OFF = PHI_OFF + 2 * TILE;
+  static constexpr int LATE_OFF = BAR_OFF + 240;             // the status word behind the wait for the kernel before
   static constexpr int TOTAL = BAR_OFF + 256 + 1024;         // + slack for the 1024-byte alignment
 };
 // barriers
 constexpr int B_QFULL = 0, B_QEMPTY = B_QFULL + QS_SLOTS, B_WFULL = B_QEMPTY + QS_SLOTS, B_WFREE = B_WFULL + 1,
-              B_PHI = B_WFREE + 1, B_PHIF = B_PHI + 2, B_P = B_PHIF + 2, B_O = B_P + 2, B_OF = B_O + 2, B_COUNT = B_OF + 2;
+              B_PHI = B_WFREE + 1, B_PHIF = B_PHI + 2, B_P = B_PHIF + 2, B_O = B_P + 2, B_OF = B_O + 2, B_LATE = B_OF + 2, B_COUNT = B_LATE + 1;
 
 struct QSCtx {
   uint32_t sbase, tmem;
@@ -228,7 +229,7 @@ qstream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     *abort_flag = 0u;
     auto bar = [&](int i) { return sbase + QSLayout::BAR_OFF + 8 * i; };
     for (int s = 0; s < QS_SLOTS; ++s) { mbar_init(bar(B_QFULL + s), 1); mbar_init(bar(B_QEMPTY + s), 1); }
-    mbar_init(bar(B_WFULL), 1); mbar_init(bar(B_WFREE), 1);
+    mbar_init(bar(B_WFULL), 1); mbar_init(bar(B_WFREE), 1); mbar_init(bar(B_LATE), 1);
     for (int g = 0; g < 2; ++g) {
       mbar_init(bar(B_PHI + g), 1); mbar_init(bar(B_PHIF + g), 128); mbar_init(bar(B_P + g), 128);
       mbar_init(bar(B_O + g), 1); mbar_init(bar(B_OF + g), 128);
@@ -237,7 +238,7 @@ qstream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     fence_proxy_async();
   }
   __shared__ uint32_t s_skip;
-  if (threadIdx.x == 32) s_skip = *reinterpret_cast<volatile uint32_t*>(p.status);    // (ahead of the wait: behind the first copies it would wait for these)
+  if (threadIdx.x == 32) s_skip = status_now(p.status);   // (ahead of the wait: behind the first copies it would wait for these)
   if (warp == 9) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   if (warp == 8 && (threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmW); tma_prefetch_desc(&tmSt); tma_prefetch_desc(&tmO); }
   tc_fence_before();
@@ -266,6 +267,8 @@ qstream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     return;
   }
 
+  if (threadIdx.x == 10 * 32) status_again(sbase + QSLayout::LATE_OFF, p.status, c.bar(B_LATE));
+
   if (warp == 8) {
     // the first copies in line: as a part of qs_produce they go out 2500 clk later, which is what its instructions take to arrive
     if ((threadIdx.x & 31) == 0) {
@@ -282,7 +285,9 @@ qstream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     if ((threadIdx.x & 31) == 0) qs_issue_out(p, c);
     __syncwarp();
   } else {
-    qs_compute(p, c, &tmO, smem);
+    // not where the launch before has timed out behind the set-up's look at the status word
+    if (__all_sync(0xffffffffu, status_clear(c.bar(B_LATE), sbase + QSLayout::LATE_OFF))) qs_compute(p, c, &tmO, smem);
+    else status_give_up(c.wc);
   }
 
   tc_fence_before();

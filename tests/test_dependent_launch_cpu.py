@@ -70,3 +70,30 @@ def test_the_rule_sees_an_early_load():
     assert _early("k", "k(const P p) {\n const float b = p.bias[0];\n griddep_wait();") == {"bias"}
     assert _early("k", "k(const P p) {\n auto get = [&](int i) { return p.bias[i]; };\n get(1);\n griddep_wait();") == {"bias"}
     assert _early("k", "k(const P p) {\n auto get = [&](int i) { return p.bias[i]; };\n griddep_wait();\n get(1);") == set()
+
+
+# kernels that look at the status word, and what has to stand between their second look and all that they write
+SECOND_LOOK = {
+    "kpass_kernel": r"late = gathers \|\| warp == 11 \? status_now\(p\.status\)[^}]*", "phi1_kernel": r"bool live = __all_sync\(0xffffffffu, status_clear\(",
+    "phi1_run_kernel": r"bool ok = __all_sync\(0xffffffffu, status_clear\(", "qlin_kernel": r"start && u < n_grp; \+\+u\)\s*if \(!q_linear_unit<",
+    "qpass_kernel": r"start && u < n_grp; \+\+u\)\s*if \(!q_softmax_unit<", "qstream_kernel": r"if \(__all_sync\(0xffffffffu, status_clear\([^;]*\)\) qs_compute\(",
+    "btq_kernel": r"late = status_now\(p\.status\)", "btk_kernel": r"late = status_now\(p\.status\)", "bsq_kernel": r"late = status_now\(p\.status\)",
+    "bsk_kernel": r"late = status_now\(p\.status\)"}
+WRITES = r"tma_store_3d\(|\bout\[\(size_t\)r \* LPR|p\.part_z\[|\(to \+ \(size_t\)rank|\(p\.ks_w \+|\batomicAdd\(cnt|bt_store_acc\(\w|p\.part_\w+\[slot|" \
+         r"reinterpret_cast<float4\*>\(dst\)\[|\bdst\[i\] =|q_softmax_unit<|q_linear_unit<|qs_compute\("
+
+
+def test_a_time_out_of_the_kernel_before_is_seen_ahead_of_the_first_write():
+    """The status word is looked at again behind the wait (the look beside the kernel before it may come too early), by all that write and before they do."""
+    kernels = dict(_kernels())
+    assert {name for name, body in kernels.items() if "s_skip" in body or "*skip" in body} == set(SECOND_LOOK)
+    for name, look in sorted(SECOND_LOOK.items()):
+        body = kernels[name]
+        body = body[body.index("if (warp >= 8) griddep_wait();") if name == "kpass_kernel" else body.rindex("griddep_wait()"):]
+        at = re.search(look, body)
+        writes = [m.start() for m in re.finditer(WRITES, body)]
+        assert at and writes and at.start() < min(writes), (name, at, writes[:3])
+        for x in writes:
+            assert "s_late != 0u) return" in body[:x] or re.search(r"late == 0u|late != 0u \? -1|live && |\bif \(ok && |while \(ok && |start &&|status_clear\(", body[:x][-1300:]), (
+                name, body[:x][-300:])
+        assert ("status_again(" in body) == ("status_clear(" in body), name

@@ -156,3 +156,57 @@ def test_a_captured_step_gives_the_results_of_the_calls(name):
     got = list(captured) + [out, aux]
     assert all(torch.equal(a, b) for a, b in zip(got, want))
     del graph
+
+
+@pytest.mark.parametrize("name", sorted(LAYERS) + ["two_layers_128", "two_layers_d64", "biased_linear"])
+def test_nothing_is_written_behind_a_time_out_of_the_kernel_before(name):
+    """The kernel whose wait runs out lets dependents in first: they have looked at the status word when it is raised.  Neither outputs nor the workspace change, and
+    the handle works again once the status has been read."""
+    import torch
+    from paper_2509_24899_b200 import binding
+    layers = dict(LAYERS, two_layers_128=dict(d=128, rate=4, F=128, hidden=128), two_layers_d64=dict(d=64, rate=4, F=64, hidden=64),
+                  biased_linear=dict(d=128, rate=0))
+    wl, dev, op, second = _layer(**layers[name])
+    bias = {n: torch.ones((wl.H, op.F), dtype=torch.bfloat16, device="cuda") for n in ("bq1", "bk1")} if name == "biased_linear" else None
+    args = [dev[n] for n in ("q", "k", "v", "wq", "wk")]
+    aux = torch.empty((wl.B, wl.H, wl.N, 3), dtype=torch.float32, device="cuda")
+
+    def run(out=None, k=args[1]):
+        return op.forward(args[0], k, *args[2:], out=out, aux=aux, biases=bias, **second)
+
+    good, stats = run().clone(), aux.clone()
+    assert op.last_status() == 0
+    out, other = torch.full_like(good, 7.0), torch.randn_like(args[1])
+    aux.fill_(7.0)
+    before = op.workspace().clone()
+    torch.cuda.synchronize()
+    binding.as_hybrid_attn_debug_expire_wait(op.handle, 2_000_000, torch.cuda.current_stream().cuda_stream)
+    for _ in range(2):
+        run(out, other)
+    torch.cuda.synchronize()
+    assert torch.equal(out, torch.full_like(good, 7.0)) and torch.equal(aux, torch.full_like(aux, 7.0))
+    assert torch.equal(op.workspace(), before)
+    assert op.last_status() == binding.AS_ERR_DEVICE_TIMEOUT and op.last_status() == 0
+    assert torch.equal(run(out), good) and torch.equal(aux, stats)
+    assert op.last_status() == 0
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_no_partial_gradient_is_written_behind_a_time_out(d):
+    import torch
+    from paper_2509_24899_b200 import binding
+    wl, dev, op, _ = _layer(d, 4)
+    args = [dev[n] for n in ("q", "k", "v", "wq", "wk")]
+    y = to_cuda_bf16(W.teacher_output(wl))
+    aux = torch.empty((wl.B, wl.H, wl.N, 3), dtype=torch.float32, device="cuda")
+    y_hat = op.forward(*args, aux=aux)
+    want = [x.clone() for x in op.backward_phi(*args, y, y_hat, aux)]
+    assert op.last_status() == 0
+    other, before = args[0].flip(2).contiguous(), op._bws.clone()
+    torch.cuda.synchronize()
+    binding.as_hybrid_attn_debug_expire_wait(op.handle, 2_000_000, torch.cuda.current_stream().cuda_stream)
+    op.backward_phi(other, *args[1:], y, y_hat, aux)             # (sums over the chunks of dS and dz, formed again from the same partials, are the same)
+    torch.cuda.synchronize()
+    assert torch.equal(op._bws, before)
+    assert op.last_status() == binding.AS_ERR_DEVICE_TIMEOUT and op.last_status() == 0
+    assert all(torch.equal(a, b) for a, b in zip(op.backward_phi(*args, y, y_hat, aux), want))
