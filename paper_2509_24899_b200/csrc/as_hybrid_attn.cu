@@ -97,7 +97,7 @@ void layout_workspace(as_hybrid_attn_s* h) {
 }
 
 // the K pass's arrival counters, then the flags of the query stage's unfinished units
-size_t n_counters(const as_hybrid_attn_s* h) { return 8 * (size_t)h->desc.B * h->desc.H + 2 * (size_t)h->sms; }
+size_t n_counters(const as_hybrid_attn_s* h) { return 8 * (size_t)h->desc.B * h->desc.H + AS_PART_FLAGS * (size_t)h->sms; }
 
 struct ProfileScope {
   as_hybrid_attn_s* h; cudaStream_t st; int slot = -1;

@@ -44,7 +44,7 @@ struct as_launch_args {
   uint32_t* counters;                   // [B*H*4][2], zero between launches: K-pass CTAs of a (batch, head, feature chunk)
                                         // that have stored their partial state (and given up) / that have left
   float* parts;                         // where the query stage's CTAs leave unfinished units (NULL: they do not), and the flags that go with it
-  uint32_t* part_flags;                 // [SMs][2], zero between launches
+  uint32_t* part_flags;                 // [SMs][AS_PART_FLAGS], zero between launches
   int B, H, N, d, F, P;
   int n_s, n_l;
   int n_chunks, chunk_tiles;            // K-pass split of the token axis
@@ -112,6 +112,9 @@ cudaError_t as_launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, siz
   cfg.attrs = &attr; cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
+
+// Flags of a CTA of the query stage, one a compute warp.
+constexpr int AS_PART_FLAGS = 16;
 
 // Status bits written by kernels into as_launch_args::status.
 constexpr uint32_t AS_DEV_TIMEOUT = 1u;

@@ -45,7 +45,7 @@ struct QParams {
   // ---- key loops in parts (cf. plan_parts; only the kernels compiled for them look at these)
   int share;                 // key tiles of a CTA in the last round; 0: units are whole
   float* parts;              // [CTAs]: what a CTA leaves of a unit that another one finishes, see QPart
-  uint32_t* part_flags;      // [CTAs][2 groups]: it is there; zero between launches
+  uint32_t* part_flags;      // [CTAs][compute warps, AS_PART_FLAGS at most]: what the warp leaves is there; zero between launches
   // of one part (0 / unused in the launch's own parameters): in place of nkv, n_s and lin above those of the part, and
   int part;                  // 1: a part
   int bh, row0, key0;        // its unit; its first key
@@ -737,9 +737,11 @@ struct QPart {
   AS_DEV static float4* of(const QParams& p, int cta, int g) { return reinterpret_cast<float4*>(p.parts + (size_t)cta * TOTAL + (size_t)g * GROUP); }
 };
 
-// By the threads of a group, whose last product into O has completed.
+// By the threads of a group, whose last product into O has completed.  Every warp has a flag of its own and the warp of that index of the other CTA, with the
+// same rows, waits for that alone: where a wait runs out its warp leaves, and no other one is waiting for it at a barrier that has no limit.
 template <int D, int T>
 __device__ __noinline__ void q_leave_part(const QParams& p, uint32_t tOg, int g, int r, int hc, float m_ref, float m_true, float l) {
+  static_assert(8 * T <= AS_PART_FLAGS);
   float4* to = QPart<D>::of(p, (int)blockIdx.x, g);
 #pragma unroll 1
   for (int o = 0; o < D / T; o += 16) {
@@ -752,9 +754,9 @@ __device__ __noinline__ void q_leave_part(const QParams& p, uint32_t tOg, int g,
                                                                 __uint_as_float(y[4 * i + 3]));
   }
   if (hc == 0) to[QPart<D>::O / 4 + r] = make_float4(m_ref, m_true, l, 0.f);
-  named_barrier_sync(1 + g, 128 * T);
-  if ((threadIdx.x & 127) == 0 && threadIdx.x < 256)           // (one thread of either group; what the barrier has ordered before it goes with it)
-    asm volatile("st.release.gpu.global.u32 [%0], 1;" ::"l"(p.part_flags + 2 * blockIdx.x + g) : "memory");
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0)                                 // (what the warp's lanes have stored goes with it)
+    asm volatile("st.release.gpu.global.u32 [%0], 1;" ::"l"(p.part_flags + AS_PART_FLAGS * blockIdx.x + (threadIdx.x >> 5)) : "memory");
 }
 
 // Adds to O, and to the row's maxima and sum, what the p.merges CTAs right before this one have left.  CTAs start in the order of their index, so
@@ -765,7 +767,7 @@ __device__ __noinline__ float4 q_merge_parts(const QParams& p, const WaitCtx& wc
   constexpr int STEP = 32, N = STEP / 4;                       // columns and loads at once
   for (int n = 1; n <= p.merges; ++n) {
     const int cta = (int)blockIdx.x - n;
-    uint32_t* flag = p.part_flags + 2 * cta + g;
+    uint32_t* flag = p.part_flags + AS_PART_FLAGS * cta + (threadIdx.x >> 5);
     bool ok = true;
     if ((threadIdx.x & 31) == 0) {
       uint32_t there, it = 0;
@@ -780,6 +782,8 @@ __device__ __noinline__ float4 q_merge_parts(const QParams& p, const WaitCtx& wc
       }
     }
     if (!__all_sync(0xffffffffu, ok)) return make_float4(0.f, 0.f, -1.f, 0.f);
+    if ((threadIdx.x & 31) == 0) *reinterpret_cast<volatile uint32_t*>(flag) = 0u;   // nobody else looks at it before the next launch
+    __syncwarp();                                              // (the lanes' loads come behind lane 0's)
     const float4* from = QPart<D>::of(p, cta, g);
     const float4* mine_from = from + hc * (D / T / 4) * 128 + r;
     const float4 st = __ldcg(from + QPart<D>::O / 4 + r);
@@ -818,8 +822,6 @@ __device__ __noinline__ float4 q_merge_parts(const QParams& p, const WaitCtx& wc
     l = l * mine + st.z * theirs;
     m_true = fmaxf(m_true, st.y);
     m_ref = m;
-    named_barrier_sync(1 + g, 128 * T);                        // every warp has seen the flag: zero for the next launch
-    if ((threadIdx.x & 127) == 0 && threadIdx.x < 256) *reinterpret_cast<volatile uint32_t*>(flag) = 0u;
   }
   tc_fence_before();
   return make_float4(m_ref, m_true, l, 0.f);
