@@ -96,8 +96,8 @@ void layout_workspace(as_hybrid_attn_s* h) {
   w.total_host = off;
 }
 
-// the K pass's arrival counters, then the flags of the query stage's unfinished units
-size_t n_counters(const as_hybrid_attn_s* h) { return 8 * (size_t)h->desc.B * h->desc.H + AS_PART_FLAGS * (size_t)h->sms; }
+// the K pass's arrival counters, then the flags of the query stage's unfinished units and the counter of its CTAs
+size_t n_counters(const as_hybrid_attn_s* h) { return 8 * (size_t)h->desc.B * h->desc.H + AS_PART_FLAGS * (size_t)h->sms + 1; }
 
 struct ProfileScope {
   as_hybrid_attn_s* h; cudaStream_t st; int slot = -1;

@@ -44,7 +44,7 @@ struct as_launch_args {
   uint32_t* counters;                   // [B*H*4][2], zero between launches: K-pass CTAs of a (batch, head, feature chunk)
                                         // that have stored their partial state (and given up) / that have left
   float* parts;                         // where the query stage's CTAs leave unfinished units (NULL: they do not), and the flags that go with it
-  uint32_t* part_flags;                 // [SMs][AS_PART_FLAGS], zero between launches
+  uint32_t* part_flags;                 // [SMs][AS_PART_FLAGS], then the counter of the CTAs that have started; zero between launches
   int B, H, N, d, F, P;
   int n_s, n_l;
   int n_chunks, chunk_tiles;            // K-pass split of the token axis

@@ -100,7 +100,7 @@ AS_DEV bool mbar_wait_warp(uint32_t bar, uint32_t parity, const WaitCtx& w) {
 // A kernel launched by as_launch_dependent may start while the kernel before it in the stream is still running, once
 // every CTA of that one has called griddep_launch or ended.  griddep_wait returns when that kernel has completed and
 // its writes are visible: no access to global memory comes before it, but to what is the handle's own - its table of softmax ranks, which never
-// changes, and its status word.
+// changes, its status word, and the counter of the CTAs that have started, which a CTA uses ahead of griddep_launch only.
 // In a kernel that allocates tensor memory the allocating warp alone calls griddep_launch, behind the allocation (one thread's call
 // counts for its CTA): a dependent CTA on the same SM could otherwise take the columns first and then wait for this kernel, which
 // would wait in its allocation (the one wait without a limit) for that CTA.

@@ -46,8 +46,10 @@ struct QParams {
   int share;                 // key tiles of a CTA in the last round; 0: units are whole
   float* parts;              // [CTAs]: what a CTA leaves of a unit that another one finishes, see QPart
   uint32_t* part_flags;      // [CTAs][compute warps, AS_PART_FLAGS at most]: what the warp leaves is there; zero between launches
+  uint32_t* part_ticket;     // which CTA of the last round a CTA is: the order in which they have started; zero between launches
   // of one part (0 / unused in the launch's own parameters): in place of nkv, n_s and lin above those of the part, and
   int part;                  // 1: a part
+  int cta;                   // the CTA's index in the last round
   int bh, row0, key0;        // its unit; its first key
   int at_items, at_s, at_p, at_pf, at_tail;   // ring items, phases and tails of the CTA before it
   int leaves, merges;        // 1: leaves what it has to another CTA; number of CTAs right before this one that have left it theirs
@@ -742,7 +744,7 @@ struct QPart {
 template <int D, int T>
 __device__ __noinline__ void q_leave_part(const QParams& p, uint32_t tOg, int g, int r, int hc, float m_ref, float m_true, float l) {
   static_assert(8 * T <= AS_PART_FLAGS);
-  float4* to = QPart<D>::of(p, (int)blockIdx.x, g);
+  float4* to = QPart<D>::of(p, p.cta, g);
 #pragma unroll 1
   for (int o = 0; o < D / T; o += 16) {
     uint32_t y[16];
@@ -756,17 +758,17 @@ __device__ __noinline__ void q_leave_part(const QParams& p, uint32_t tOg, int g,
   if (hc == 0) to[QPart<D>::O / 4 + r] = make_float4(m_ref, m_true, l, 0.f);
   __syncwarp();
   if ((threadIdx.x & 31) == 0)                                 // (what the warp's lanes have stored goes with it)
-    asm volatile("st.release.gpu.global.u32 [%0], 1;" ::"l"(p.part_flags + AS_PART_FLAGS * blockIdx.x + (threadIdx.x >> 5)) : "memory");
+    asm volatile("st.release.gpu.global.u32 [%0], 1;" ::"l"(p.part_flags + AS_PART_FLAGS * p.cta + (threadIdx.x >> 5)) : "memory");
 }
 
-// Adds to O, and to the row's maxima and sum, what the p.merges CTAs right before this one have left.  CTAs start in the order of their index, so
-// those are running or through, and their parts that are left come first in them and wait for nothing: the wait ends whatever else is on the GPU (and is bounded
-// like every other).  Returns (m_ref, m_true, l); the sum is negative when a wait ran out.
+// Adds to O, and to the row's maxima and sum, what the p.merges CTAs right before this one have left.  A CTA's index is the order in which it has started (see
+// the kernel), so those are running or through, and their parts that are left come first in them and wait for nothing: the wait ends whatever else is on the GPU, in
+// whatever order CTAs are started (and is bounded like every other).  Returns (m_ref, m_true, l); the sum is negative when a wait ran out.
 template <int D, int T>
 __device__ __noinline__ float4 q_merge_parts(const QParams& p, const WaitCtx& wc, uint32_t tOg, int g, int r, int hc, float m_ref, float m_true, float l) {
   constexpr int STEP = 32, N = STEP / 4;                       // columns and loads at once
   for (int n = 1; n <= p.merges; ++n) {
-    const int cta = (int)blockIdx.x - n;
+    const int cta = p.cta - n;
     uint32_t* flag = p.part_flags + AS_PART_FLAGS * cta + (threadIdx.x >> 5);
     bool ok = true;
     if ((threadIdx.x & 31) == 0) {
@@ -1207,8 +1209,8 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 
 // The parts of CTA c in the last round (see plan_parts): at most two, the one that it leaves to the next CTA first.  Written by one thread.
 template <int D>
-AS_DEV int q_parts(const QParams& p, QParams* to) {
-  const int c = (int)blockIdx.x, n = (int)gridDim.x, left = p.n_pairs - p.n_rounds * n, all = left * p.nkv;
+AS_DEV int q_parts(const QParams& p, int c, QParams* to) {
+  const int n = (int)gridDim.x, left = p.n_pairs - p.n_rounds * n, all = left * p.nkv;
   const int r0 = c * p.share, r1 = min(all, r0 + p.share);
   if (r0 >= r1) return 0;
   const bool tailed = p.lin != 0;
@@ -1219,7 +1221,7 @@ AS_DEV int q_parts(const QParams& p, QParams* to) {
     QParams& q = to[np++];
     const int w = p.n_rounds * n + unit;
     q = p;
-    q.part = 1;
+    q.part = 1; q.cta = c;
     q.bh = w / p.nx; q.row0 = (w % p.nx) * 256; q.key0 = k0 * 128;
     q.nkv = k1 - k0; q.n_s = p.n_s - q.key0;
     q.leaves = k1 < p.nkv ? 1 : 0;
@@ -1267,8 +1269,10 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   __shared__ uint32_t s_skip;
   __shared__ QParams s_part[KS ? 2 : 1];
   __shared__ int s_parts;
-  if (KS && threadIdx.x == 64) s_parts = q_parts<D>(p, s_part);
   if (threadIdx.x == 32) s_skip = status_now(p.status);   // (ahead of the wait: behind the first copies it would wait for these)
+  // The CTA's index in the last round is the order in which it has started, by a counter that goes back to 0 with the launch's last CTA.  Ahead of the wait for the kernel
+  // before, and of griddep_launch: a later launch starts when all CTAs of this one have come past that, and so have taken theirs.
+  if (KS && threadIdx.x == X::W_SCORE * 32) s_parts = q_parts<D>(p, (int)atomicInc(p.part_ticket, gridDim.x - 1u), s_part);
   if (warp == X::W_SCORE) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   if (warp == X::W_TMA && (threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); tma_prefetch_desc(&tmO); }
   tc_fence_before();
@@ -1444,7 +1448,7 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
     return cudaErrorInvalidValue;
   dim3 grid(plan_units(p, BH, sms), 1, 1);
-  p.parts = a.parts; p.part_flags = a.part_flags;
+  p.parts = a.parts; p.part_flags = a.part_flags; p.part_ticket = a.part_flags + AS_PART_FLAGS * sms;
   const int ctas = a.parts != nullptr && !qlin ? plan_parts(p, BH, sms, p.nh) : 0;
   const bool ks = ctas > 0;
   if (ks) grid.x = ctas;

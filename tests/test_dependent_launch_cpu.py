@@ -4,8 +4,8 @@ import os
 import re
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2509_24899_b200", "csrc")
-# the handle's own memory: a table that does not change, and the status word
-OWN = {"sm_rank", "status"}
+# the handle's own memory: a table that does not change, the status word, and a counter that only CTAs use that have not yet let dependents in
+OWN = {"sm_rank", "status", "part_ticket"}
 # reached by warps only that have waited where the rest have not yet (the key stage's gather warps)
 BEHIND_A_WAIT_OF_THEIR_WARPS = {"kpass_kernel": {"ks_w", "vs_w"}}
 
