@@ -2,7 +2,7 @@
 // projection, linear apply and merge, fused in one persistent kernel.
 //
 //   persistent, one CTA per SM (what is left over after the full rounds is dealt out in one last round, in
-//   units of two 128-row tiles or of one, see plan_units, or by key tiles, see plan_parts); per unit a flash-style loop over 128-key tiles
+//   units of two 128-row tiles or of one, see as_plan_units, or by key tiles, see as_plan_parts); per unit a flash-style loop over 128-key tiles
 //   of K_S / V_S:        S = Q K_S^T -> TMEM; the softmax threads (one or two per row) read their row and
 //                        release the score columns at once, so the next product into them runs under the
 //                        exponentials; running max / sum per row; P = exp2(.) as bf16 -> TMEM,
@@ -16,8 +16,7 @@
 //                        (128 hidden units at a time) and kept as bf16 in the group's phi_q tile and, once nothing reads
 //                        Q any more, in the Q tile; Phi_c = sum over the hidden slices of h1_j W_q2[c, j]^T.
 // All tiles are staged by TMA with the 128-byte swizzle; every mbarrier wait is bounded.
-#include <algorithm>
-
+#include "query_plan.h"
 #include "tensor_common.cuh"
 
 namespace {
@@ -42,7 +41,7 @@ struct QParams {
   const float* z;            // [B*H][F]
   float* aux;                // [B*H][N][3] or nullptr
   uint32_t* status;
-  // ---- key loops in parts (cf. plan_parts; only the kernels compiled for them look at these)
+  // ---- key loops in parts (cf. as_plan_parts; only the kernels compiled for them look at these)
   int share;                 // key tiles of a CTA in the last round; 0: units are whole
   float* parts;              // [CTAs]: what a CTA leaves of a unit that another one finishes, see QPart
   uint32_t* part_flags;      // [CTAs][compute warps, AS_PART_FLAGS at most]: what the warp leaves is there; zero between launches
@@ -56,7 +55,7 @@ struct QParams {
 };
 
 // How the compute threads share a 128-row tile: T = 1, one thread per row (eight warps), or T = 2, threads t and t + 16 of a warp, each
-// with half of the row's columns (sixteen warps; the two share their maxima and sums by one shuffle).  cf. q_threads_per_row.
+// with half of the row's columns (sixteen warps; the two share their maxima and sums by one shuffle).  cf. as_threads_per_row.
 template <int T>
 struct QShape {
   static constexpr int COLS = 128 / T;                     // score columns of a thread
@@ -123,7 +122,7 @@ struct QLayout {
 };
 
 // Persistent: one CTA per SM walks over units of two 128-row tiles (unit w = blockIdx.x + u * gridDim.x, the last one
-// as plan_units deals it out; the units of one (batch, head) are consecutive, so the CTAs that run at the same time
+// from as_plan_units; the units of one (batch, head) are consecutive, so the CTAs that run at the same time
 // share K_S / V_S in L2).
 // Barrier phases and the K/V ring run on across units.
 //
@@ -154,7 +153,7 @@ struct QCtx {
 // Unit u of this CTA: which (batch, head), the row it starts at, and how many of the two 128-row groups work on it.  In
 // the rounds every CTA takes part in, CTA c has two-tile unit c + u * gridDim.x.  Last, each CTA takes at most one of what
 // is left: two-tile units - cut into their two tiles where CTAs enough are left for that - and the last tiles of heads with
-// an odd number of them (see plan_units).  A group that has the tensor and XU pipes to itself needs about two thirds of
+// an odd number of them (see as_plan_units).  A group that has the tensor and XU pipes to itself needs about two thirds of
 // the time that the two of a two-tile unit take.
 struct QUnit { int bh, row0, ng; };
 template <bool KS = false>
@@ -1207,32 +1206,24 @@ qlin_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   }
 }
 
-// The parts of CTA c in the last round (see plan_parts): at most two, the one that it leaves to the next CTA first.  Written by one thread.
-template <int D>
+// The parts of CTA c in the last round (see as_deal_parts), each as the parameters of a unit.  Written by one thread.
 AS_DEV int q_parts(const QParams& p, int c, QParams* to) {
-  const int n = (int)gridDim.x, left = p.n_pairs - p.n_rounds * n, all = left * p.nkv;
-  const int r0 = c * p.share, r1 = min(all, r0 + p.share);
-  if (r0 >= r1) return 0;
-  const bool tailed = p.lin != 0;
-  const int fc = tailed ? p.fc : 0, slices = tailed && p.layers == 2 ? p.nh : 0, tail_items = slices ? slices + fc * slices + fc : 2 * fc;
-  int at_items = p.n_rounds * (2 * p.nkv + tail_items), at_s = p.n_rounds * (p.nkv + slices + fc), at_p = p.n_rounds * (p.nkv + fc);
-  int at_pf = p.n_rounds * (p.nkv + (slices ? 1 : fc)), at_tail = p.n_rounds, np = 0;
-  auto add = [&](int unit, int k0, int k1) {
-    QParams& q = to[np++];
-    const int w = p.n_rounds * n + unit;
+  AsPart part[2];
+  const int n = (int)gridDim.x, np = as_deal_parts(p.n_pairs, p.n_rounds, p.share, p.nkv, p.lin, p.fc, p.layers == 2 ? p.nh : 0, n, c, part);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    if (i >= np) break;
+    const AsPart& a = part[i];
+    QParams& q = to[i];
+    const int w = p.n_rounds * n + a.unit;
     q = p;
     q.part = 1; q.cta = c;
-    q.bh = w / p.nx; q.row0 = (w % p.nx) * 256; q.key0 = k0 * 128;
-    q.nkv = k1 - k0; q.n_s = p.n_s - q.key0;
-    q.leaves = k1 < p.nkv ? 1 : 0;
-    q.lin = q.leaves ? 0 : p.lin;
-    q.merges = q.leaves || k0 == 0 ? 0 : c - unit * p.nkv / p.share;
-    q.at_items = at_items; q.at_s = at_s; q.at_p = at_p; q.at_pf = at_pf; q.at_tail = at_tail;
-    at_items += 2 * q.nkv; at_s += q.nkv; at_p += q.nkv; at_pf += q.nkv;       // (of one that is left; nothing comes behind another)
-  };
-  const int unit = r0 / p.nkv, k0 = r0 - unit * p.nkv, over = r1 - (unit + 1) * p.nkv;
-  if (over > 0) add(unit + 1, 0, over);
-  add(unit, k0, over > 0 ? p.nkv : r1 - unit * p.nkv);
+    q.bh = w / p.nx; q.row0 = (w % p.nx) * 256; q.key0 = a.k0 * 128;
+    q.nkv = a.k1 - a.k0; q.n_s = p.n_s - q.key0;
+    q.leaves = a.leaves; q.merges = a.merges;
+    q.lin = a.leaves ? 0 : p.lin;
+    q.at_items = a.at_items; q.at_s = a.at_s; q.at_p = a.at_p; q.at_pf = a.at_pf; q.at_tail = a.at_tail;
+  }
   return np;
 }
 
@@ -1272,7 +1263,7 @@ qpass_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   if (threadIdx.x == 32) s_skip = status_now(p.status);   // (ahead of the wait: behind the first copies it would wait for these)
   // The CTA's index in the last round is the order in which it has started, by a counter that goes back to 0 with the launch's last CTA.  Ahead of the wait for the kernel
   // before, and of griddep_launch: a later launch starts when all CTAs of this one have come past that, and so have taken theirs.
-  if (KS && threadIdx.x == X::W_SCORE * 32) s_parts = q_parts<D>(p, (int)atomicInc(p.part_ticket, gridDim.x - 1u), s_part);
+  if (KS && threadIdx.x == X::W_SCORE * 32) s_parts = q_parts(p, (int)atomicInc(p.part_ticket, gridDim.x - 1u), s_part);
   if (warp == X::W_SCORE) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); griddep_launch(); }
   if (warp == X::W_TMA && (threadIdx.x & 31) == 0) { tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); tma_prefetch_desc(&tmO); }
   tc_fence_before();
@@ -1343,86 +1334,12 @@ cudaError_t as_tensor_init_qpass() {
   return cudaSuccess;
 }
 
-// How the 128-row tiles of a launch are dealt out to the CTAs: full rounds of two-tile units, then one last round.  A head
-// with an odd number of tiles either has its last tile in a unit of its own, or in a two-tile unit whose other half is
-// past the end; which is better depends on what the last round comes to (N = 7800, 61 tiles in each of 12 heads, 148 SMs:
-// 360 units and 12 single tiles are two rounds and 140 tiles alone, 372 units are two rounds and 76 units: layer 92.8 -> 88.6
-// us; N = 1024 with 2 heads on 16 CTAs instead of 8: 22.5 -> 21.4).  Returns the
-// number of CTAs.
-namespace {
-int plan_units(QParams& p, int BH, int sms) {
-  const int tiles = (p.N + 127) / 128;
-  double best = 0.;
-  int grid = 0;
-  for (int alone = 0; alone <= (tiles & 1); ++alone) {
-    const int nx = (tiles + 1 - alone) / 2, pairs = nx * BH, single = alone * BH;
-    const int rounds = pairs / sms, left = pairs - rounds * sms;
-    const bool cut = 2 * left + single <= sms;
-    const int last = (cut ? 2 * left : left) + single;
-    if (last > sms) continue;                        // one last round only
-    const double t = rounds + (last == 0 ? 0. : (cut || left == 0) ? 0.7 : 1.);
-    if (grid != 0 && t > best) continue;             // (no worse: without empty tiles)
-    best = t;
-    p.nx = nx; p.n_pairs = pairs; p.n_single = single; p.n_rounds = rounds; p.split_last = cut ? 1 : 0;
-    grid = rounds > 0 ? sms : last;
-  }
-  return grid;
-}
-// The last round with the key loops of its units cut across CTAs: the key tiles of what is left after the full rounds, unit after unit, are dealt out in equal
-// shares, so that a CTA finishes one unit and leaves the beginning of the next one to the CTA after it (q_parts).  Whole units, or lone tiles, leave
-// much of the GPU idle where a little more than half of a round is left, or little work in long loops.  What it costs: O of a part through L2, the wait for it, a
-// unit's fixed work twice, 5 - 8 us in all (the 10000 or 14000 and 2500 clk below).  Taken where the rounds as plan_units deals them out take longer by more than
-// that, in the clocks that a key tile of a unit, one of a lone tile and a unit's tail were measured at.  Whole calls, units whole -> in parts (us): full softmax,
-// d = 128, 2 heads of N = 10000 135 -> 86, 1 of 15000 126 -> 96, 1 of 8000 72 -> 49, 4 of 5600 79 -> 61, 7 of 3999 59 -> 57; d = 64, 1 of 8000 70 -> 38, 4 of
-// 5600 76 -> 57; one key in two, 2 of 12288 102 -> 87, d = 64 94 -> 80; one rank of four of the 81-frame layer (two rounds and 88 units) 205 -> 202.  Below
-// the line: 5 heads of N = 5000, one key in two (0.96 by this rule with 10000) 56.5 -> 59.6.  Returns the number of CTAs, 0: units stay whole.
-int plan_parts(QParams& p, int BH, int sms, int slices) {
-  if (p.nkv < 2) return 0;
-  const int nx = ((p.N + 127) / 128 + 1) / 2, pairs = nx * BH, rounds = pairs / sms, left = pairs - rounds * sms;
-  if (left == 0) return 0;
-  const int all = left * p.nkv, share = std::max(2, (all + sms - 1) / sms);
-  if (share >= p.nkv) return 0;
-  const int merges = (p.nkv - 1) / share + 1;                 // the most that a CTA adds up
-  if (merges > 8) return 0;
-  const double tail = p.lin ? 9000. + 4500. * ((p.fc - 1) + (slices ? slices * (1 + p.fc) : 0)) : 4000.;
-  const double unit = p.nkv * 2900. + tail, lone = p.nkv * 1800. + 0.7 * tail;
-  const int last = p.split_last ? (p.n_pairs > p.n_rounds * sms || p.n_single > 0) : 2 * (p.n_pairs > p.n_rounds * sms);   // 0: none, 1: lone tiles, 2: units
-  const double now = p.n_rounds * unit + (last == 2 ? unit : last == 1 ? lone : 0.);
-  const double then = rounds * unit + share * 2900. + tail + (p.lin ? 14000. : 10000.) + 2500. * merges;
-  if (then > 0.96 * now) return 0;
-  p.nx = nx; p.n_pairs = pairs; p.n_single = 0; p.n_rounds = rounds; p.split_last = 0; p.share = share;
-  return rounds > 0 ? sms : (all + share - 1) / share;
-}
-// no CTA has more than one tile: one group works, the other one has nothing to do
-bool one_tile_each(const QParams& p) { return p.n_rounds == 0 && p.split_last; }
-// Threads per row of the kernel with a key loop (after plan_units).  Two (sixteen compute warps) hide more of the latencies; one draws less power per
-// exponential and has 168 registers where two have 96.  At d = 64 always two.  At d = 128 the gain of two over one in the query stage, on layers that differ
-// in the number of key tiles only (12 heads, N = 32760, 16384, 7800, 1560; 2 - 46 heads of 20140 - 442 rows; in bursts of 3 ms / in runs of 0.06 - 0.12 s,
-// which the power cap slows down where a CTA has several units):
-//   a CTA has one tile at most (2 heads, N = 4096), so that one group has the SM to itself: 4 - 10 % at any length with one layer, 0 - 5 % with two;
-//   one layer without biases: 4 tiles 0 - 8 % / 0 - 8 %, 16 0 - 3 / -1 - +3, 31 0 - 2 / -2 - +3, 40 -1 - +2 / -2 - +3, 96 -1 - +1 / -3 - -1; F = 256 alike;
-//   one layer with biases or powers beyond 2: 8 tiles 4 - 12 / 2 - 13, 16 2 - 7 / 2 - 6, 31 2 - 5 / -3 - +3, 48 1 - 4 / 0 - 2, 64 0 - 4 / -1 - +2;
-//   two layers with one feature chunk: 0 tiles -14 - 0 / -11 - 0, 4 and more -7 - 0 / -8 - 0, biased or not; with two, which one thread has
-//   to keep in its registers: 0 tiles -5 - 0 / -6 - 0, else -3 - +1 / -4 - +3, with biases or powers beyond 2 4 - 30 at few tiles, 16 4 - 16 / 2 - 12, 48 1 - 10 / -1 - +5.
-// That is the query stage over and over.  In a whole layer its instructions arrive cold, which costs one thread's longer code more: of two-layer
-// maps of few rounds 256 / 256 are 2 - 7 % faster with two (N = 1560 ... 9360, 0 to 10 tiles), 128 / 128 0 - 3 %.
-int q_threads_per_row(const QParams& p, int d, bool two, bool gen) {
-  if (d == 64 || one_tile_each(p)) return 2;
-  if (p.share > 0) return 1;                         // (with parts the key loop does not stay in 96 registers: full softmax, 4 heads of N = 5600 61 -> 67 us)
-  if (!two) return p.nkv <= (gen ? 48 : 31) ? 2 : 1;
-  if (gen && p.fc > 1) return p.nkv <= 48 ? 2 : 1;
-  if (p.fc == 1 && p.nkv == 0) return 1;
-  return p.nkv <= 16 && p.n_rounds < 4 ? 2 : 1;
-}
-}  // namespace
-
 size_t as_qpass_parts_bytes(int N, int BH, int d, int sms) {
-  QParams p{};
-  p.N = N;
-  plan_units(p, BH, sms);
+  AsUnits p;
+  as_plan_units(p, N, BH, sms);
   const int pairs = ((N + 127) / 128 + 1) / 2 * BH, rounds = pairs / sms;
   const double now = p.n_rounds + (p.split_last ? (p.n_pairs > p.n_rounds * sms || p.n_single > 0 ? 0.62 : 0.) : p.n_pairs > p.n_rounds * sms ? 1. : 0.);
-  if (pairs == rounds * sms || (double)pairs / sms > 0.96 * now) return 0;   // as plan_parts with a key loop without an end
+  if (pairs == rounds * sms || (double)pairs / sms > 0.96 * now) return 0;   // what as_plan_parts says of a key loop without an end
   return sizeof(float) * (size_t)(d == 128 ? QPart<128>::TOTAL : QPart<64>::TOTAL) * sms;
 }
 
@@ -1447,14 +1364,17 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
     return cudaErrorInvalidValue;
-  dim3 grid(plan_units(p, BH, sms), 1, 1);
-  p.parts = a.parts; p.part_flags = a.part_flags; p.part_ticket = a.part_flags + AS_PART_FLAGS * sms;
-  const int ctas = a.parts != nullptr && !qlin ? plan_parts(p, BH, sms, p.nh) : 0;
-  const bool ks = ctas > 0;
-  if (ks) grid.x = ctas;
   // the general kernels carry the bias and the powers beyond 2; the common case does without them
   const bool gen = lin && (a.P > 2 || p.b1 != nullptr || p.b2 != nullptr);
-  const int tpr = q_threads_per_row(p, a.d, two, gen);
+  const AsLoop loop{a.d, p.nkv, p.lin, p.fc, p.nh, gen ? 1 : 0};
+  AsUnits plan;
+  dim3 grid(as_plan_units(plan, a.N, BH, sms), 1, 1);
+  const int ctas = a.parts != nullptr && !qlin ? as_plan_parts(plan, loop, a.N, BH, sms) : 0;
+  const bool ks = ctas > 0;
+  if (ks) grid.x = ctas;
+  p.nx = plan.nx; p.n_pairs = plan.n_pairs; p.n_single = plan.n_single; p.n_rounds = plan.n_rounds; p.split_last = plan.split_last; p.share = plan.share;
+  p.parts = a.parts; p.part_flags = a.part_flags; p.part_ticket = a.part_flags + AS_PART_FLAGS * sms;
+  const int tpr = as_threads_per_row(plan, loop);
   // the output is stored warp by warp: boxes of a warp's rows
   if (!make_map(&tmQ, a.q, a.d, a.N, BH, 128) || !make_map(&tmO, a.out, a.d, a.N, BH, qlin ? 32 : 32 / tpr)) return cudaErrorInvalidValue;
   if (a.n_s > 0) {
@@ -1491,7 +1411,7 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
     const int threads = QShape<T_>::THREADS, smem = QLayout<D_>::TOTAL; \
     if (gen) AS_LAUNCH_Q(D_, T_, MAP_, true, true); else AS_LAUNCH_Q(D_, T_, MAP_, false, true); \
   } while (0)
-  const int map = two ? MAP_TWO : lin && p.fc > 1 && !one_tile_each(p) ? MAP_WIDE : MAP_ONE;
+  const int map = two ? MAP_TWO : lin && p.fc > 1 && !as_one_tile_each(plan) ? MAP_WIDE : MAP_ONE;
   if (ks) {
     if (a.d == 64) { if (two) AS_LAUNCH_QP(64, 2, MAP_TWO); else AS_LAUNCH_QP(64, 2, MAP_ONE); }
     if (map == MAP_TWO) AS_LAUNCH_QP(128, 1, MAP_TWO);
