@@ -845,7 +845,8 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
   const uint32_t tSg = q.tS(g) + lane_off, tOg = q.tO(g) + lane_off, tPg = q.tP(g) + lane_off;
   uint8_t* sPg = smem + L::P_OFF + g * L::PTILE;    // this group's phi_q / output staging tile
   const int ps = KS && p.part ? p.at_s : u * q.n_s, ppf = KS && p.part ? p.at_pf : u * q.n_pf;   // first phases of the unit (cf. QRing)
-  float m_ref = 0.f, m_true = -INFINITY, l = 0.f;
+  // (a part behind a unit's first starts from a finite maximum: keys with scores of -infinity weigh nothing, as they do behind others in an unbroken key loop)
+  float m_ref = KS ? (p.key0 > 0 ? -3.402823466e38f : -INFINITY) : 0.f, m_true = -INFINITY, l = 0.f;
 
   for (int j = 0; j < nkv; ++j) {
     if (!q.wait(R::B_S + g, ps + j)) return false;
@@ -874,7 +875,7 @@ __device__ __noinline__ bool q_softmax_unit(const QParams& p, const QCtx& c, con
     // are rescaled (once the previous tile's P V has completed, before this tile's P is handed over).
     const bool need = (j > 0) && (mx > m_ref + RESCALE_THRESHOLD);
     const float resc = need ? ex2(m_ref - mx) : 1.f;
-    if (j == 0 || need) m_ref = mx;
+    if (j == 0 || need) m_ref = KS ? fmaxf(mx, m_ref) : mx;
     // P = exp2(s * scale_log2 - m_ref) as bf16 into the group's columns of tensor memory
     const float neg_m = -m_ref;
     // packed fp32x2 arithmetic halves the instruction count of the scaling and of the row sum
