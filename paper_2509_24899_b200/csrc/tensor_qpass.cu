@@ -45,6 +45,8 @@ struct QParams {
   int share;                 // key tiles of a CTA in the last round; 0: units are whole
   float* parts;              // [CTAs]: what a CTA leaves of a unit that another one finishes, see QPart
   uint32_t* part_flags;      // [CTAs][compute warps, AS_PART_FLAGS at most]: what the warp leaves is there; zero between launches
+  const __nv_bfloat16* v;    // the keys' values [B*H][v_rows][D]
+  int v_rows;
   uint32_t* part_ticket;     // which CTA of the last round a CTA is: the order in which they have started; zero between launches
   // of one part (0 / unused in the launch's own parameters): in place of nkv, n_s and lin above those of the part, and
   int part;                  // 1: a part
@@ -760,6 +762,37 @@ __device__ __noinline__ void q_leave_part(const QParams& p, uint32_t tOg, int g,
     asm volatile("st.release.gpu.global.u32 [%0], 1;" ::"l"(p.part_flags + AS_PART_FLAGS * p.cta + (threadIdx.x >> 5)) : "memory");
 }
 
+// Where a part that weighs nothing against another one had a sum that is no number or past the end of the range (`bad`: in this thread's row).  Values near the end of the
+// range, many of them, are one cause: their sum is left out, as each of them would be in an unbroken key loop.  The other is a value that is infinite or no
+// number itself: 0 times that is no number there, and so it is here, in its column.  By a whole warp; on ordinary input never.
+template <int D, int T>
+__device__ __noinline__ void q_weightless(const QParams& p, uint32_t tOg, int hc, bool bad) {
+  const int lane = threadIdx.x & 31;
+  const uint16_t* v = reinterpret_cast<const uint16_t*>(p.v) + (size_t)p.bh * p.v_rows * D;
+  uint32_t mine = 0u;                                          // bit i: column lane + 32 i has such a value
+  for (int k = 0; k < p.v_rows; ++k)
+#pragma unroll
+    for (int i = 0; i < D / 32; ++i) mine |= (v[(size_t)k * D + i * 32 + lane] & 0x7f80u) == 0x7f80u ? 1u << i : 0u;
+#pragma unroll 1
+  for (int o = 0; o < D / T; o += 16) {
+    uint32_t y[16];
+    q_ld16<T, D / 2>(tOg + o, y);
+    tmem_ld16_wait(y);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      bool there[T];
+#pragma unroll
+      for (int h = 0; h < T; ++h) {                            // (every lane asks for the columns of either share)
+        const int col = h * (D / T) + o + i;
+        there[h] = (__shfl_sync(0xffffffffu, mine, col & 31) >> (col / 32) & 1u) != 0u;
+      }
+      if (bad && there[T == 1 ? 0 : hc] && fabsf(__uint_as_float(y[i])) < INFINITY) y[i] = 0x7fc00000u;
+    }
+    q_st16<T, D / 2>(tOg + o, y);
+  }
+  tmem_st_wait();
+}
+
 // Adds to O, and to the row's maxima and sum, what the p.merges CTAs right before this one have left.  A CTA's index is the order in which it has started (see
 // the kernel), so those are running or through, and their parts that are left come first in them and wait for nothing: the wait ends whatever else is on the GPU, in
 // whatever order CTAs are started (and is bounded like every other).  Returns (m_ref, m_true, l); the sum is negative when a wait ran out.
@@ -792,6 +825,8 @@ __device__ __noinline__ float4 q_merge_parts(const QParams& p, const WaitCtx& wc
 #pragma unroll
     for (int i = 0; i < N; ++i) x[i] = __ldcg(mine_from + i * 128);
     const float m = fmaxf(m_ref, st.x), mine = ex2(m_ref - m), theirs = ex2(st.x - m);
+    const bool weightless = !(mine > 0.f) || !(theirs > 0.f);
+    float odd = 0.f;                                           // no number if a weightless sum is past the end of the range or none
 #pragma unroll 1
     for (int o = 0; o < D / T; o += STEP) {
       uint32_t y[32];
@@ -800,9 +835,12 @@ __device__ __noinline__ float4 q_merge_parts(const QParams& p, const WaitCtx& wc
 #pragma unroll
       for (int i = 0; i < N; ++i) {
         const float part[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
+        if (weightless)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) odd = fmaf(part[e], 0.f, fmaf(__uint_as_float(y[4 * i + e]), 0.f, odd));
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          // a sum that weighs nothing is left out, also where it is past the end of the range (many keys with values near it)
+          // a sum that weighs nothing is left out, also where it is past the end of the range (cf. q_weightless)
           const float own = mine > 0.f ? __uint_as_float(y[4 * i + e]) * mine : 0.f;
           y[4 * i + e] = __float_as_uint(theirs > 0.f ? fmaf(part[e], theirs, own) : own);
         }
@@ -820,6 +858,7 @@ __device__ __noinline__ float4 q_merge_parts(const QParams& p, const WaitCtx& wc
       }
     }
     tmem_st_wait();
+    if (__any_sync(0xffffffffu, odd != odd)) q_weightless<D, T>(p, tOg, hc, odd != odd);
     l = l * mine + st.z * theirs;
     m_true = fmaxf(m_true, st.y);
     m_ref = m;
@@ -1374,6 +1413,7 @@ cudaError_t as_tensor_qpass(const as_launch_args& a, cudaStream_t st) {
   const bool ks = ctas > 0;
   if (ks) grid.x = ctas;
   p.nx = plan.nx; p.n_pairs = plan.n_pairs; p.n_single = plan.n_single; p.n_rounds = plan.n_rounds; p.split_last = plan.split_last; p.share = plan.share;
+  p.v = a.vs; p.v_rows = a.n_s;
   p.parts = a.parts; p.part_flags = a.part_flags; p.part_ticket = a.part_flags + AS_PART_FLAGS * sms;
   const int tpr = as_threads_per_row(plan, loop);
   // the output is stored warp by warp: boxes of a warp's rows

@@ -62,3 +62,22 @@ def test_values_at_the_end_of_the_range_under_keys_that_weigh_nothing(layer):
         v[:, :, run] = torch.finfo(torch.bfloat16).min
     out, scores, v = _run(layer, change)
     _close(out, torch.softmax(scores, -1) @ v)
+
+
+@pytest.mark.parametrize("layer", LAYERS)
+@pytest.mark.parametrize("value", ["inf", "nan"])
+@pytest.mark.parametrize("at", [0.1, 0.9])
+def test_a_value_that_is_no_number_shows_in_its_column(layer, value, at):
+    """Under a key that weighs nothing: 0 times it, wherever in the loop it comes.  The other columns are right, and finite."""
+    import torch
+    col = 5
+
+    def change(k, v, keys):
+        # all keys but the last tenth - or, for a value there, but the first tenth - weigh nothing
+        n = len(keys)
+        k[:, :, keys[:int(0.85 * n)] if at < 0.5 else keys[int(0.15 * n):]] = -1e4
+        v[:, :, keys[int(at * n)], col] = float(value)
+    out, scores, v = _run(layer, change)
+    assert not bool(out[..., col].isfinite().any())
+    rest = [c for c in range(out.shape[-1]) if c != col]
+    _close(out[..., rest], torch.softmax(scores, -1) @ v[..., rest])
