@@ -1081,13 +1081,14 @@ __device__ __noinline__ bool q_linear_unit(const QParams& p, const QCtx& c, cons
   const int part = p.F / p.P;
   uint32_t x[32];
   float dl = 0.f;
+  bool ok = true;                                   // a warp whose wait has run out still comes to the group's barriers, which have no limit
   for (int ch = 0; ch < q.fc; ++ch) {
-    if (!q.wait(R::B_S + g, ps + ch)) return false;
+    ok = ok && q.wait(R::B_S + g, ps + ch);
     tc_fence_after();
     // the phi_q tile may be written once the product that read it has completed and the previous unit's output store
     // has been read out (the stores are issued by the warps of column half 0)
     if (hf == 0 && lane == 0) tma_store_wait_read();
-    if (ppf + ch > 0 && !q.wait(R::B_PF + g, ppf + ch - 1)) return false;
+    if (ppf + ch > 0) ok = ok && q.wait(R::B_PF + g, ppf + ch - 1);
     named_barrier_sync(1 + g, 256);
     const float2* zrow = reinterpret_cast<const float2*>(p.z + (size_t)bh * p.F + ch * 128 + hf * half);
     const uint32_t* brow = nullptr;
@@ -1136,7 +1137,7 @@ __device__ __noinline__ bool q_linear_unit(const QParams& p, const QCtx& c, cons
   if (hf == 0) dl += *dl_slot;
   named_barrier_sync(1 + g, 256);
   if (hf == 0) *dl_slot = dl;
-  if (!q.wait(R::B_O + g, u)) return false;          // (the products run meanwhile)
+  ok = ok && q.wait(R::B_O + g, u);                  // (the products run meanwhile)
   named_barrier_sync(1 + g, 256);
   const float den = *dl_slot;
   tc_fence_after();
@@ -1157,6 +1158,7 @@ __device__ __noinline__ bool q_linear_unit(const QParams& p, const QCtx& c, cons
   fence_proxy_async();
   tc_fence_before();
   named_barrier_sync(1 + g, 256);                    // both halves of every row are staged
+  if (!ok) return false;
   const int wrow0 = row - lane;
   if (hf == 0 && lane == 0 && wrow0 < p.N) {
 #pragma unroll

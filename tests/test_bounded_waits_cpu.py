@@ -23,3 +23,9 @@ def test_no_warp_returns_ahead_of_a_barrier_of_its_group():
         returns = [m.start() for m in re.finditer(r"\breturn (?:false|make_float4\(0\.f, 0\.f, -1\.f)", body)]
         barriers = [m.start() for m in re.finditer(r"named_barrier_sync|" + "|".join(r"\b%s<" % f for f in with_barrier if f != name) or "$^", body)]
         assert not [b for b in barriers if (returns and min(returns) < b) or name != "q_softmax_unit"], name
+
+
+def test_the_linear_unit_comes_to_all_its_barriers():
+    """There the threads of a row's two halves meet: whoever's wait has run out goes on to the last barrier."""
+    body = dict(_functions("tensor_qpass.cu"))["q_linear_unit"]
+    assert body.rindex("named_barrier_sync") < body.index("return false") and body.count("return false") == 1
