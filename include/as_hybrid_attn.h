@@ -124,7 +124,7 @@ AS_API as_status_t as_hybrid_attn_create(const as_hybrid_attn_desc_t* desc, as_h
 AS_API as_status_t as_hybrid_attn_destroy(as_hybrid_attn_t h);
 
 /* Bytes of scratch `forward` needs (compacted softmax K/V, partial and final linear state, the keys' hidden
- * activations of a two-layer map).  (Utility: no counterpart in the paper.) */
+ * activations of a two-layer map, and the query stage's unfinished units: up to 20 MB where it may cut key loops across CTAs).  (Utility: no counterpart in the paper.) */
 AS_API as_status_t as_hybrid_attn_workspace_bytes(as_hybrid_attn_t h, size_t* bytes);
 
 /* Bytes of scratch `forward_host` needs: the above plus device staging for q, k, v and out.
@@ -141,9 +141,10 @@ AS_API as_status_t as_hybrid_attn_workspace_bytes_host(as_hybrid_attn_t h, size_
  *   cuda_stream  a cudaStream_t (NULL = default stream)
  * Enqueues its kernels and returns; errors found on the host are returned at once, a device
  * time-out is reported later by as_hybrid_attn_last_status.  Calls on one handle must be ordered on the device (one
- * stream, or events between streams): the handle's status word and the arrival counters of the key stage are shared
- * by its calls.  On AS_PATH_TENSOR the key stage's CTAs (at most one per SM) add their chunks of a head up together; where other
- * work holds SMs, so that they are not all on the device at once, the last of them does it alone: slower, the same bits. */
+ * stream, or events between streams): the handle's status word, the arrival counters of the key stage, and the query stage's flags and counter for key
+ * loops that are cut across CTAs are shared by its calls.  On AS_PATH_TENSOR the key stage's CTAs (at most one per SM) add their chunks of a head up together; where
+ * other work holds SMs, so that they are not all on the device at once, the last of them does it alone: slower, the same bits.  A CTA of the query stage waits only for
+ * CTAs that have started before it. */
 AS_API as_status_t as_hybrid_attn_forward(as_hybrid_attn_t h, const void* q, const void* k, const void* v,
                                    const as_phi_weights_t* w, void* out, float* aux,
                                    void* workspace, size_t workspace_bytes, void* cuda_stream);

@@ -123,12 +123,6 @@ AS_DEV void tma_store_3d(const CUtensorMap* m, uint32_t src, int x, int y, int z
                ::"l"(reinterpret_cast<uint64_t>(m)), "r"(src), "r"(x), "r"(y), "r"(z)
                : "memory");
 }
-// Untiled bulk copy shared -> global: both addresses 16-byte aligned, size a multiple of 16 bytes.
-AS_DEV void bulk_store_1d(void* dst_global, uint32_t src_smem, uint32_t bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-               ::"l"(reinterpret_cast<uint64_t>(dst_global)), "r"(src_smem), "r"(bytes)
-               : "memory");
-}
 AS_DEV void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 AS_DEV void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // Only until the sources of all committed stores have been read: the shared memory can be reused.

@@ -514,6 +514,26 @@ struct P1Layout {
   static constexpr int TOTAL = BIAS_OFF + D * 4 + 1024;
 };
 
+// Copies rows row0 + i of a K tile, i the set bits, to the rows of the compact K_S that their lanes i hold in `rank`.  By a warp, D / 8 lanes a row.
+template <int D>
+AS_DEV void copy_rows(const uint8_t* tile, int row0, uint32_t bits, int rank, __nv_bfloat16* ks) {
+  constexpr int CH = D / 8, RPI = 32 / CH;
+  const int lane = threadIdx.x & 31, c = lane % CH;
+  while (bits) {
+    int src = -1;
+#pragma unroll
+    for (int i = 0; i < RPI; ++i) {
+      if (bits) {
+        if (lane / CH == i) src = __ffs(bits) - 1;
+        bits &= bits - 1;
+      }
+    }
+    const int to = __shfl_sync(0xffffffffu, rank, src < 0 ? 0 : src);
+    if (src >= 0)
+      *reinterpret_cast<uint4*>(ks + (size_t)to * D + c * 8) = *reinterpret_cast<const uint4*>(tile + (c / 8) * BOX_BYTES + swz128_chunk_offset(row0 + src, c % 8));
+  }
+}
+
 template <int D>
 __global__ void __launch_bounds__(P1_THREADS)
 phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
@@ -582,27 +602,10 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
     const bool live = __all_sync(0xffffffffu, status_clear(bar_late, s_late));
     bool ok = true;
     if (live && p.ks_w != nullptr) {
-      // sixteen rows of the K tile; D / 8 lanes a row
-      constexpr int CH = D / 8, RPI = 32 / CH;
       const int rank = lane / 16 == hf && row0 + r < p.N ? p.sm_rank[row0 + r] : -1;
-      uint32_t bits = __ballot_sync(0xffffffffu, rank >= 0);
+      const uint32_t bits = __ballot_sync(0xffffffffu, rank >= 0);
       if (bits) ok = mbar_wait_warp(bar_full, 0, wc);
-      while (ok && bits) {
-        int src = -1;
-#pragma unroll
-        for (int i = 0; i < RPI; ++i) {
-          if (bits) {
-            if (lane / CH == i) src = __ffs(bits) - 1;
-            bits &= bits - 1;
-          }
-        }
-        const int to = __shfl_sync(0xffffffffu, rank, src < 0 ? 0 : src);
-        if (src >= 0) {
-          const int c = lane % CH;
-          const uint4 val = *reinterpret_cast<const uint4*>(smem + L::X_OFF + (c / 8) * BOX_BYTES + swz128_chunk_offset(quad * 32 + src, c % 8));
-          *reinterpret_cast<uint4*>(p.ks_w + ((size_t)bh * p.n_s + to) * D + c * 8) = val;
-        }
-      }
+      if (ok) copy_rows<D>(smem + L::X_OFF, quad * 32, bits, rank, p.ks_w + (size_t)bh * p.n_s * D);
       __syncwarp();
     }
     uint32_t x[32];
@@ -643,7 +646,7 @@ phi1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUt
 // head's weights stay in shared memory, three tiles of K are in flight, the products of a tile run under the rows of the one before (two sets of
 // accumulators), and a slice of h1 is stored while the next one is formed.  Where a run goes on into the next head, its weights come when the last
 // product with the old ones has completed; its first tile of K is asked for before that.  N = 32760, 12 heads, no softmax tokens: this stage 65 -> 56 us (floor
-// 46), the call 310 -> 300; rate 1/8 990 -> 980, N = 7800 140.5 -> 138.1, 8 heads of N = 1560 38.4 -> 37.7.  Narrower maps keep the kernel above, which has
+// 46), the call 314 -> 304; rate 1/8 990 -> 980, N = 7800 140.5 -> 138.1, 8 heads of N = 1560 38.4 -> 37.7.  Narrower maps keep the kernel above, which has
 // several CTAs on an SM there: in runs of tiles, 128 / 128 with 2 heads of N = 1560 27.4 -> 28.2 us, d = 64 with 12 of 7800 78.4 -> 79.5 (24 of 15600 without
 // softmax tokens 110.9 -> 107.1).  Tried: softmax rows of K copied behind the slices' rows instead of ahead of them, N = 15600, 16 heads 85.5 -> 87.5.
 constexpr int P1R_THREADS = 320;          // warps 0-7: epilogue (two threads per token row, each half of a slice's columns); 8: TMA; 9: MMA
@@ -779,27 +782,9 @@ phi1_run_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         load_bias(bh % p.H);                                    // (all have read the old one: they met behind it)
       }
       if (p.ks_w != nullptr) {
-        // sixteen rows of the K tile; D / 8 lanes a row
-        constexpr int CH = D / 8, RPI = 32 / CH;
-        uint32_t bits = __ballot_sync(0xffffffffu, rank >= 0);
+        const uint32_t bits = __ballot_sync(0xffffffffu, rank >= 0);
         if (ok) ok = mbar_wait_warp(bar_x(s), (i / P1R_RING) & 1, wc);
-        while (ok && bits) {
-          int src = -1;
-#pragma unroll
-          for (int i = 0; i < RPI; ++i) {
-            if (bits) {
-              if (lane / CH == i) src = __ffs(bits) - 1;
-              bits &= bits - 1;
-            }
-          }
-          const int to = __shfl_sync(0xffffffffu, rank, src < 0 ? 0 : src);
-          if (src >= 0) {
-            const int c = lane % CH;
-            const uint4 val = *reinterpret_cast<const uint4*>(smem + L::X_OFF + s * L::TILE + (c / 8) * BOX_BYTES +
-                                                              swz128_chunk_offset(quad * 32 + src, c % 8));
-            *reinterpret_cast<uint4*>(p.ks_w + ((size_t)bh * p.n_s + to) * D + c * 8) = val;
-          }
-        }
+        if (ok) copy_rows<D>(smem + L::X_OFF + s * L::TILE, quad * 32, bits, rank, p.ks_w + (size_t)bh * p.n_s * D);
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_x_empty(s));
       }

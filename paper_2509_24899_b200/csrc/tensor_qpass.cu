@@ -261,9 +261,9 @@ struct QRing {
 };
 
 // ---------------------------------------------------------------- TMA producer
-// The first copies of a CTA, by one thread: ring item 0 (the first key tile, else the first weights) and the first unit's Q tiles.  In line, right behind the wait for
-// the kernel before: as a part of q_produce_unit they went out 2500 - 3500 clk later, which is what its
-// instructions and its parameters take to arrive in a CTA that has just started.
+// The first copies of a CTA, by one thread: ring item 0 (the first key tile, else the first weights) and the first unit's Q tiles.  Right behind the wait for the kernel
+// before, and a few lines of instructions of their own: as a part of q_produce_unit they went out 2500 - 3500 clk later, which is what its instructions and its
+// parameters take to arrive in a CTA that has just started.  (Compiled into the kernel itself it moves q_softmax_unit's registers, N = 7800 + 2 us.)
 template <int D, int MAP, bool KS = false>
 __device__ __noinline__ void q_first_loads(const QParams& p, const QCtx& c, const QUnit& un, const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmW,
                           const CUtensorMap* tmW1) {

@@ -79,8 +79,8 @@ SECOND_LOOK = {
     "qpass_kernel": r"start && u < n_grp; \+\+u\)\s*if \(!q_softmax_unit<", "qstream_kernel": r"if \(__all_sync\(0xffffffffu, status_clear\([^;]*\)\) qs_compute\(",
     "btq_kernel": r"late = status_now\(p\.status\)", "btk_kernel": r"late = status_now\(p\.status\)", "bsq_kernel": r"late = status_now\(p\.status\)",
     "bsk_kernel": r"late = status_now\(p\.status\)"}
-WRITES = r"tma_store_3d\(|\bout\[\(size_t\)r \* LPR|p\.part_z\[|\(to \+ \(size_t\)rank|\(p\.ks_w \+|\batomicAdd\(cnt|bt_store_acc\(\w|p\.part_\w+\[slot|" \
-         r"reinterpret_cast<float4\*>\(dst\)\[|\bdst\[i\] =|q_softmax_unit<|q_linear_unit<|qs_compute\("
+WRITES = r"tma_store_3d\(|\bout\[\(size_t\)r \* LPR|p\.part_z\[|\(to \+ \(size_t\)rank|\\batomicAdd\(cnt|bt_store_acc\(\w|p\.part_\w+\[slot|" \
+         r"reinterpret_cast<float4\*>\(dst\)\[|\bdst\[i\] =|copy_rows<D>\(|q_softmax_unit<|q_linear_unit<|qs_compute\("
 
 
 def test_a_time_out_of_the_kernel_before_is_seen_ahead_of_the_first_write():
@@ -94,6 +94,6 @@ def test_a_time_out_of_the_kernel_before_is_seen_ahead_of_the_first_write():
         writes = [m.start() for m in re.finditer(WRITES, body)]
         assert at and writes and at.start() < min(writes), (name, at, writes[:3])
         for x in writes:
-            assert "s_late != 0u) return" in body[:x] or re.search(r"late == 0u|late != 0u \? -1|live && |\bif \(ok && |while \(ok && |start &&|status_clear\(", body[:x][-1300:]), (
+            assert "s_late != 0u) return" in body[:x] or re.search(r"late == 0u|late != 0u \? -1|live && |\bif \(ok(?: && |\) copy_rows)|while \(ok && |start &&|status_clear\(", body[:x][-1300:]), (
                 name, body[:x][-300:])
         assert ("status_again(" in body) == ("status_clear(" in body), name
