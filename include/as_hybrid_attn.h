@@ -231,7 +231,8 @@ AS_API as_status_t as_hybrid_attn_backward_phi(as_hybrid_attn_t h, const void* q
  * every kernel of the library uses, on a barrier nobody arrives at; no copy and no tensor-core operation is
  * in flight.  After about `limit_cycles` SM clocks (1 .. 1e8) the wait gives up, the kernel returns and the
  * handle's status word is set exactly as by a time-out inside `forward`: as_hybrid_attn_last_status then
- * returns AS_ERR_DEVICE_TIMEOUT once, and the handle is usable again afterwards. */
+ * returns AS_ERR_DEVICE_TIMEOUT once, and the handle is usable again afterwards.  Like the kernels of a `forward` it lets
+ * the launch behind it set up before it waits. */
 AS_API as_status_t as_hybrid_attn_debug_expire_wait(as_hybrid_attn_t h, int64_t limit_cycles, void* cuda_stream);
 
 /* Profiling aid (no counterpart in the paper): after `profile_enable(h, 1)` every kernel launch is bracketed by CUDA events on

@@ -210,3 +210,29 @@ def test_no_partial_gradient_is_written_behind_a_time_out(d):
     assert torch.equal(op._bws, before)
     assert op.last_status() == binding.AS_ERR_DEVICE_TIMEOUT and op.last_status() == 0
     assert all(torch.equal(a, b) for a, b in zip(op.backward_phi(*args, y, y_hat, aux), want))
+
+
+@pytest.mark.parametrize("H,N,rate,d", [(2, 10000, 1, 128), (1, 8000, 1, 64), (5, 9467, 2, 64)])
+def test_key_loops_in_parts_write_nothing_behind_a_time_out(H, N, rate, d):
+    import torch
+    from paper_2509_24899_b200 import HybridAttention, binding
+    from _query_plan import plan
+    assert plan(N, H, rate, d, d)["parts"]
+    g = torch.Generator(device="cuda").manual_seed(N)
+    q, k, v = (torch.randn((1, H, N, d), device="cuda", generator=g).bfloat16() for _ in range(3))
+    w = {} if rate == 1 else {n: (torch.randn((H, d, d), device="cuda", generator=g) * 0.05).bfloat16() for n in ("wq", "wk")}
+    op = HybridAttention(1, H, N, d, (1, 1, N), (1, 1, N), rate)
+    good = op.forward(q, k, v, **w).clone()
+    assert op.last_status() == 0
+    out, before = torch.full_like(good, 7.0), op.workspace().clone()
+    other = q.flip(2).contiguous()
+    torch.cuda.synchronize()
+    binding.as_hybrid_attn_debug_expire_wait(op.handle, 2_000_000, torch.cuda.current_stream().cuda_stream)
+    for _ in range(2):
+        op.forward(other, k, v, out=out, **w)
+    torch.cuda.synchronize()
+    assert torch.equal(out, torch.full_like(good, 7.0)) and torch.equal(op.workspace(), before)
+    assert op.last_status() == binding.AS_ERR_DEVICE_TIMEOUT
+    for _ in range(2):
+        assert torch.equal(op.forward(q, k, v, out=out, **w), good)
+    assert op.last_status() == 0
